@@ -55,8 +55,9 @@ struct AttnArgs {
     bool cache_fresh;           // the kernel launched just before may have written cache_k/v
     long lo;                    // split bf16: lo planes of q, K/V and out sit lo elements on (0: none)
 };
-template <typename T>
-void launch_attention(const AttnArgs<T> &a, cudaStream_t s);
+// fp32 contexts (CUDA cores); rows come in blocks of rows_per_req rows of one
+// request. Returns false if the shape is unsupported or the launch failed.
+bool launch_attention(const AttnArgs<float> &a, int rows_per_req, cudaStream_t s);
 
 // Scratch of the chunked top-k: per-chunk records and per-row tickets
 // (tickets must start at zero; the kernel leaves them at zero).
@@ -96,8 +97,8 @@ struct GemmW {
 };
 enum { EPI_STORE = 0, EPI_ADD = 1, EPI_SWIGLU = 2, EPI_ROPE_KV = 3 };
 
-template <typename T>
-void launch_gemm_simt(const T *X, int ldx, int M, int K, const GemmW &W, int O,
-                      float *Y, int ldy, int epi, cudaStream_t s);
+// fp32 contexts (CUDA cores)
+void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int O, float *Y, int ldy, int epi,
+                      cudaStream_t s);
 
 }  // namespace msd

@@ -181,7 +181,7 @@ void gemm(msd_ctx *c, const T *X, int ldx, int M, int K, const GemmW &W, int O, 
 template <>
 void gemm<float>(msd_ctx *c, const float *X, int ldx, int M, int K, const GemmW &W, int O,
                  float *Y, int ldy, int epi, cudaStream_t s, bool) {
-    launch_gemm_simt<float>(X, ldx, M, K, W, O, Y, ldy, epi, s);
+    launch_gemm_simt(X, ldx, M, K, W, O, Y, ldy, epi, s);
 }
 
 template <>
@@ -200,8 +200,11 @@ template <typename T>
 void attention(msd_ctx *c, const AttnArgs<T> &a, int rows_per_req, cudaStream_t s);
 
 template <>
-void attention<float>(msd_ctx *c, const AttnArgs<float> &a, int, cudaStream_t s) {
-    launch_attention<float>(a, s);
+void attention<float>(msd_ctx *c, const AttnArgs<float> &a, int rows_per_req, cudaStream_t s) {
+    if (!launch_attention(a, rows_per_req, s)) {
+        c->err = "fp32 attention: unsupported shape or launch failure";
+        launch_flag(c->status, ST_RANGE, s);     // reported by the next call
+    }
 }
 
 template <>

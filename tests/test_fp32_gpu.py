@@ -1,0 +1,73 @@
+"""The fp32 kernels at the edges of their tiles: the CUDA-core GEMM against
+float64 products, and the attention (row tiles of 16 and 64, key splits, tree
+tiles, both head dims) through whole steps against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2505_14260_gb300 import msd, synth
+from tests.gpu_support import open_engine
+from tests.parity_support import run_parity
+
+pytestmark = pytest.mark.gpu
+
+TINY = synth.WORKLOADS["tiny"]
+
+# (m, k, o, x row padding, x offset in elements): tile edges of the 16-, 32- and
+# 64-row tiles, K below, at and past a 64-k stage and over several K splits,
+# rows and pointers that are not 16-byte aligned
+GEMM = [(1, 1, 1, 0, 0), (1, 64, 33, 0, 0), (16, 256, 256, 0, 0), (17, 260, 65, 4, 0), (32, 2816, 64, 0, 0),
+        (33, 127, 129, 0, 0), (64, 8192, 16, 0, 0), (65, 66, 700, 1, 0), (5, 4096, 1024, 0, 1),
+        (200, 1028, 500, 0, 0), (7, 3, 2000, 2, 3)]
+
+
+@pytest.mark.parametrize("m,k,o,pad,off", GEMM)
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_fp32_linear_matches_float64(m, k, o, pad, off, accumulate):
+    eng, _ = open_engine(TINY, steps=1)
+    g = torch.Generator(device="cuda").manual_seed(m * 7 + k * 3 + o)
+    buf = torch.randn(off + m * (k + pad), generator=g, device="cuda")
+    x = buf[off:].view(m, k + pad)[:, :k]
+    w = torch.randn(o, k, generator=g, device="cuda")
+    y = torch.randn(m, o, generator=g, device="cuda")
+    ref = x.double() @ w.double().T + (y.double() if accumulate else 0.0)
+    mag = x.double().abs() @ w.double().abs().T + (y.double().abs() if accumulate else 0.0)
+    st = msd.lib().msd_linear(eng.ctx, x.data_ptr(), k + pad, m, k, w.data_ptr(), o, y.data_ptr(), o,
+                              int(accumulate), 0)
+    assert st == msd.MSD_OK
+    torch.cuda.synchronize()
+    # any order of k fp32 products and sums: (k + 1) rounding errors of 2^-24
+    assert bool(((y.double() - ref).abs() <= (k + 1) * 2.0 ** -24 * mag + 1e-30).all())
+    eng.close()
+
+
+# N over the 16-row tiles (one, two, a remainder) and the 64-row ones, prefixes
+# below a key tile, at its edge, past it, and over every split; hd 64 and 128
+@pytest.mark.parametrize("hd,nodes,vis,text", [(64, 7, 0, 9), (64, 33, 100, 28), (64, 70, 600, 41),
+                                               (128, 16, 30, 34), (128, 31, 700, 69), (128, 65, 64, 64)])
+def test_fp32_steps_match_oracle(hd, nodes, vis, text):
+    wl = TINY.with_(n_heads=256 // hd, head_dim=hd, tree_nodes=nodes, tree_depth=4, topk=5, n_vis=(vis,),
+                    n_text=(text, text))
+    run_parity(wl, 2, None)
+
+
+def test_fp32_ragged_batch_matches_oracle():
+    wl = TINY.with_(batch=3, n_vis=(8, 150), n_text=(5, 90), tree_nodes=20)
+    run_parity(wl, 2, None)
+
+
+def test_fp32_linear_rows_do_not_depend_on_each_other():
+    """A row of X alone gives the values it gives among others of the same tile
+    count (fixed summation order)."""
+    eng, _ = open_engine(TINY, steps=1)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(48, 512, generator=g, device="cuda")
+    w = torch.randn(300, 512, generator=g, device="cuda")
+    y = torch.zeros(48, 300, device="cuda")
+    eng.linear(x, w, y)
+    x2 = torch.randn(48, 512, generator=g, device="cuda")
+    x2[17] = x[17]
+    y2 = torch.zeros(48, 300, device="cuda")
+    eng.linear(x2, w, y2)
+    assert np.array_equal(y[17].cpu().numpy(), y2[17].cpu().numpy())
+    eng.close()
