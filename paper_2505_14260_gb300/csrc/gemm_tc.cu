@@ -203,6 +203,55 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+// Warp-wide forms. The TMA and MMA issue loops run in whole warps: tensor
+// instructions take their descriptors, addresses and barriers from uniform
+// registers, which a warp in step computes on the uniform datapath, while a loop
+// in one diverged lane moves every operand over on its own (about 0.4 us of
+// issue a 64-wide K stage, more than the MMAs of a 256 x 176 tile take). Only the
+// lane that elect_one() names (`on`) issues.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t on;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}" : "=r"(on));
+    return on;
+}
+
+__device__ __forceinline__ void w_expect_tx(uint32_t on, uint32_t bar, uint32_t bytes) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
+        "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(bar),
+        "r"(bytes), "r"(on)
+        : "memory");
+}
+
+__device__ __forceinline__ void w_tma_load_2d_pair(uint32_t on, uint32_t dst, const CUtensorMap *map, int x, int y,
+                                                   uint32_t cluster_bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3}], [%4];\n}" ::"r"(dst),
+        "l"(map), "r"(x), "r"(y), "r"(cluster_bar), "r"(on)
+        : "memory");
+}
+
+__device__ __forceinline__ void w_mma_bf16_pair(uint32_t on, uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
+                                                uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p, q;\n"
+        "setp.ne.b32 q, %5, 0;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on));
+}
+
+__device__ __forceinline__ void w_mma_commit_pair(uint32_t on, uint32_t bar, uint16_t cta_mask) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}" ::
+            "r"(bar),
+        "h"(cta_mask), "r"(on)
+        : "memory");
+}
+
 // Arrive (release, cluster scope) on an mbarrier of another CTA of the cluster.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -233,6 +282,17 @@ __device__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *a
             return false;
         }
     }
+}
+
+// The bounded waits for a whole warp (every lane waits; the answer is uniform).
+__device__ __forceinline__ bool w_mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
+}
+__device__ __forceinline__ bool w_mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                    int *status) {
+    if (__all_sync(0xffffffffu, mbar_try_cluster(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait_cluster(bar, parity, abort_flag, status));
 }
 
 // TMEM loads of this warp's 32 lanes, 16 or 32 columns, each waited for in
@@ -441,19 +501,24 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
-// Persistent stream-K variant (the context GEMM).
+// Persistent two-SM variant (the context GEMM for many token rows).
 //
-// The work is the list of (tile, K-block) units, tile-major; CTA c of G takes
-// units [c*U/G, (c+1)*U/G), so every CTA streams about the same number of
-// weight bytes through one continuously running TMA -> MMA pipeline, across
-// tile boundaries. Roles (192 threads): warp 0 lane 0 issues TMA, warp 1
-// allocates TMEM and its lane 0 issues the MMAs, warps 2-5 drain the
+// CTAs 2j and 2j+1 are a cluster that runs 256 x BN tiles with
+// tcgen05.mma.cta_group::2: each CTA holds 128 weight rows and half of the
+// token columns, so an SM reads half the token bytes per flop of a single-SM
+// 128 x BN tile (whose two token planes, 2 x BN x 128 bytes a stage, bounded the
+// kernel through L2: 66% of the burst rate in issued flops at 640 rows).
+// The work is the list of (tile, K-block) units, tile-major; pair c of G takes
+// units [c*U/G, (c+1)*U/G) of the cut tiles, then whole tiles, so every pair
+// streams through one continuously running TMA -> MMA pipeline, across tile
+// boundaries. Roles (192 threads): warp 0 lane 0 issues TMA, warp 1
+// allocates TMEM and the even CTA's lane 0 issues the MMAs, warps 2-5 drain the
 // accumulators. Two TMEM accumulators let the epilogue of one tile overlap the
-// MMAs of the next. A tile whose K range is cut between CTAs ("pieces") is
-// fixed up through the workspace: each piece is written to its CTA's slot (a
-// CTA has at most two cut tiles, its first and its last), and the CTA that
-// takes the tile's last ticket sums the pieces in CTA order (deterministic)
-// and applies the epilogue. No CTA ever waits on another.
+// MMAs of the next. A tile whose K range is cut between pairs ("pieces") is
+// fixed up through the workspace, each CTA its own 128 rows: each piece is
+// written to its CTA's slot (a CTA has at most two cut tiles, its first and its
+// last), and the CTA that takes the tile's last ticket sums the pieces in pair
+// order (deterministic) and applies the epilogue. No CTA waits on another pair.
 // ---------------------------------------------------------------------------
 constexpr int P_THREADS = 192;
 constexpr int P_MAX_STAGES = 12;
@@ -464,10 +529,12 @@ struct PkParams {
     int seg_tiles[3];
     int seg_rows[3];
     int seg_out[3];
-    int M, kblocks, BN, n_tiles_n, stages, acc_stride, tmem_cols, grid;
+    int M, kblocks, BN, n_tiles_n, stages, acc_stride, tmem_cols, grid;   // grid: CTA pairs
+    int tiles;              // 128-row weight tiles
     long long units;        // stream-K units: T_sk tiles x K-blocks
-    int T_sk, dp_rounds;    // stream-K tiles; whole-tile rounds of G tiles after them
-    const bf16 *wpacked;    // pre-packed weights (tile-contiguous, pre-swizzled)
+    int T_sk, dp_rounds;    // stream-K tiles; rounds of whole tiles after them
+    int T_all;              // all 256-row tiles x token tiles
+    int kb_chunk;           // K-blocks of a whole tile accumulated before they are added to Y
     float *Y;
     int ldy, epi;
     float *ws;
@@ -486,17 +553,17 @@ __device__ __forceinline__ float swiglu_fused(float g, float u) {
     return __fdividef(g, 1.f + __expf(-g)) * u;
 }
 
-// CTA owning unit u under the balanced partition u0(c) = floor(c * U / G).
+// CTA pair owning unit u under the balanced partition u0(c) = floor(c * U / G).
 __device__ __forceinline__ int owner_cta(long long u, long long U, int G) {
     return (int)(((u + 1) * (long long)G - 1) / U);
 }
 
-// The work items of one CTA, in order: its share of the stream-K tiles
+// The work items of one CTA pair, in order: its share of the stream-K tiles
 // [0, T_sk) (a contiguous range of (tile, K-block) units, cut at tile
-// boundaries), then its whole data-parallel tiles T_sk + cta + j*G.
+// boundaries), then its whole tiles T_sk + cta + j*G, each in chunks of K.
 struct ItemIter {
     long long u, u1;
-    int KB, T_sk, G, cta, dp_j, dp_rounds;
+    int KB, T_sk, G, cta, dp_j, dp_rounds, T_all, chunk, dp_kb;
     __device__ bool next(int &t, int &kb_b, int &kb_e) {
         if (u < u1) {
             t = (int)(u / KB);
@@ -505,20 +572,45 @@ struct ItemIter {
             u += kb_e - kb_b;
             return true;
         }
-        if (dp_j < dp_rounds) {
+        if (dp_j < dp_rounds && T_sk + cta + dp_j * G < T_all) {
             t = T_sk + cta + dp_j * G;
-            kb_b = 0;
-            kb_e = KB;
-            ++dp_j;
+            kb_b = dp_kb;
+            kb_e = min(KB, dp_kb + chunk);
+            dp_kb = kb_e;
+            if (kb_e == KB) {
+                dp_kb = 0;
+                ++dp_j;
+            }
             return true;
         }
         return false;
     }
 };
 
+// all threads of both CTAs of the pair
+__device__ __forceinline__ void c_cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t c_cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ uint32_t c_mapa(uint32_t local, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
+    return a;
+}
+
+// RAW: mw maps the caller's row-major weight (128-byte swizzle), read only after
+// the wait on the previous kernel; otherwise the packed blocks.
+template <bool RAW>
 __global__ void __launch_bounds__(P_THREADS, 1)
     gemm_persist_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mxl,
-                        const PkParams p) {
+                        const __grid_constant__ CUtensorMap mw, const PkParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[2 * P_MAX_STAGES + 5];
     __shared__ uint32_t tmem_base;
@@ -527,14 +619,16 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     __shared__ int s_slot[P_MAX_PIECES];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cta = blockIdx.x;
+    const int half = (int)(blockIdx.x & 1u);          // cluster rank: the even CTA leads
+    const int cta = (int)(blockIdx.x >> 1);           // the pair
     const long long U = p.units;                      // stream-K units
     const long long u0 = (long long)cta * U / p.grid, u1 = (long long)(cta + 1) * U / p.grid;
     const int KB = p.kblocks, stages = p.stages, BN = p.BN;
     const bool has_lo = p.has_lo != 0;
-    const uint32_t b_bytes = (uint32_t)BN * BK * 2;           // one plane of a token stage
+    const uint32_t b_bytes = (uint32_t)(BN / 2) * BK * 2;     // one plane of this CTA's token columns
     const uint32_t bs_bytes = has_lo ? 2 * b_bytes : b_bytes;  // hi, then lo
-    const ItemIter items0{u0, u1, KB, p.T_sk, p.grid, cta, 0, p.dp_rounds};
+    const uint32_t stage_tx = 2u * (A_BYTES + bs_bytes);       // both CTAs' copies
+    const ItemIter items0{u0, u1, KB, p.T_sk, p.grid, cta, 0, p.dp_rounds, p.T_all, p.kb_chunk, 0};
 
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_base = sbase, b_base = sbase + stages * A_BYTES;
@@ -551,27 +645,29 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(accf0 + 8 * a, 1);
-            mbar_init(acce0 + 8 * a, 128);
+            mbar_init(acce0 + 8 * a, 8);        // the epilogue warps of both CTAs
         }
         mbar_init(drain, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+    if (warp == 1) {        // both CTAs allocate together (the same columns in each)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_base)),
                      "r"(p.tmem_cols)
                      : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
+    c_cluster_sync();       // both CTAs' barriers are initialised before either signals the other's
 
-    // (tile) -> weight segment, weight rows, token rows
-    auto tile_geom = [&](int t, int &seg, int &row0, int &n0) {
-        const int wt = t / p.n_tiles_n, nt = t - wt * p.n_tiles_n;
+    // (tile) -> this CTA's weight tile, its segment and rows; token rows
+    auto tile_geom = [&](int t, int &wt, int &seg, int &row0, int &n0) {
+        const int pt = t / p.n_tiles_n, nt = t - pt * p.n_tiles_n;
+        wt = 2 * pt + half;             // (== tiles: the odd CTA past an odd tile count; no rows)
         int w = wt;
         seg = 0;
         while (seg < p.n_seg - 1 && w >= p.seg_tiles[seg]) {
@@ -581,100 +677,119 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         row0 = w * BM;
         n0 = nt * BN;
     };
-    const size_t blk_elems = A_BYTES / 2;
 
     if (warp == 0) {
+        const uint32_t on = elect_one();
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&mx) : "memory");
             if (has_lo) asm volatile("prefetch.tensormap [%0];" ::"l"(&mxl) : "memory");
-            // Weights never depend on the previous kernel: the first stages'
-            // weight blocks are requested before waiting for it.
-            int n_pre = 0;
-            {
-                ItemIter it = items0;
-                int t, kb_b, kb_e;
-                while (n_pre < stages && it.next(t, kb_b, kb_e)) {
-                    const bf16 *w = p.wpacked + ((size_t)(t / p.n_tiles_n) * KB + kb_b) * blk_elems;
-                    for (int kb = kb_b; kb < kb_e && n_pre < stages; ++kb, ++n_pre, w += blk_elems) {
-                        mbar_expect_tx(full0 + 8 * n_pre, A_BYTES + bs_bytes);
-                        bulk_load(a_base + n_pre * A_BYTES, w, A_BYTES, full0 + 8 * n_pre);
-                    }
-                }
-            }
-            pdl_wait();
-            stamp_min(p.stamp, 1);
-            pdl_trigger();
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&mw) : "memory");
+        }
+        __syncwarp();
+        const uint32_t sig0 = c_mapa(full0, 0);         // copies complete on the even CTA's barriers
+        const uint32_t on_expect = half == 0 ? on : 0u;
+        // the weight block of (weight tile, kb): x, y in the weight map (rows past
+        // the last weight tile read as zeros)
+        auto load_w = [&](int wt, int kb, int st) {
+            w_expect_tx(on_expect, full0 + 8 * st, stage_tx);
+            const int x = RAW ? kb * BK : 0, y = RAW ? wt * BM : (wt * KB + kb) * BM;
+            w_tma_load_2d_pair(on, a_base + st * A_BYTES, &mw, x, y, sig0 + 8 * st);
+        };
+        // Packed weights never depend on the previous kernel: the first stages'
+        // weight blocks are requested before waiting for it.
+        int n_pre = 0;
+        if constexpr (!RAW) {
             ItemIter it = items0;
-            int t, kb_b, kb_e, s = 0, i = 0;
-            uint32_t ph = 0;
-            bool stop = false;
-            while (!stop && it.next(t, kb_b, kb_e)) {
-                int seg, row0, n0;
-                tile_geom(t, seg, row0, n0);
-                const bf16 *w = p.wpacked + ((size_t)(t / p.n_tiles_n) * KB + kb_b) * blk_elems;
-                for (int kb = kb_b; kb < kb_e; ++kb, ++i, w += blk_elems) {
-                    if (i >= n_pre) {
-                        if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, &abort_flag, p.status)) {
-                            stop = true;
-                            break;
-                        }
-                        mbar_expect_tx(full0 + 8 * s, A_BYTES + bs_bytes);
-                        bulk_load(a_base + s * A_BYTES, w, A_BYTES, full0 + 8 * s);
+            int t, kb_b, kb_e;
+            while (n_pre < stages && it.next(t, kb_b, kb_e)) {
+                const int wt = 2 * (t / p.n_tiles_n) + half;
+                for (int kb = kb_b; kb < kb_e && n_pre < stages; ++kb, ++n_pre) load_w(wt, kb, n_pre);
+            }
+        }
+        pdl_wait();
+        if (lane == 0) stamp_min(p.stamp, 1);
+        pdl_trigger();
+        ItemIter it = items0;
+        int t, kb_b, kb_e, s = 0, i = 0;
+        uint32_t ph = 0;
+        bool stop = false;
+        while (!stop && it.next(t, kb_b, kb_e)) {
+            const int pt = t / p.n_tiles_n, wt = 2 * pt + half;
+            const int ny = (t - pt * p.n_tiles_n) * BN + half * (BN / 2);
+            for (int kb = kb_b; kb < kb_e; ++kb, ++i) {
+                if (i >= n_pre) {
+                    if (!w_mbar_wait(empty0 + 8 * s, ph ^ 1u, &abort_flag, p.status)) {
+                        stop = true;
+                        break;
                     }
-                    tma_load_2d(b_base + s * bs_bytes, &mx, kb * BK, n0, full0 + 8 * s);
-                    if (has_lo) tma_load_2d(b_base + s * bs_bytes + b_bytes, &mxl, kb * BK, n0, full0 + 8 * s);
-                    if (++s == stages) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                    load_w(wt, kb, s);
+                }
+                w_tma_load_2d_pair(on, b_base + s * bs_bytes, &mx, kb * BK, ny, sig0 + 8 * s);
+                if (has_lo)
+                    w_tma_load_2d_pair(on, b_base + s * bs_bytes + b_bytes, &mxl, kb * BK, ny, sig0 + 8 * s);
+                if (++s == stages) {
+                    s = 0;
+                    ph ^= 1u;
                 }
             }
-            if (abort_flag) {
-                volatile int never = 0;
-                for (int j = (i > stages ? i - stages : 0); j < i; ++j)
-                    mbar_wait(full0 + 8 * (j % stages), (uint32_t)(j / stages) & 1u, &never,
-                              p.status);
-            }
+        }
+        if (abort_flag && half == 0) {      // (its barriers count both CTAs' copies)
+            volatile int never = 0;
+            for (int j = (i > stages ? i - stages : 0); j < i; ++j)
+                mbar_wait(full0 + 8 * (j % stages), (uint32_t)(j / stages) & 1u, &never, p.status);
         }
         __syncwarp();
     } else if (warp == 1) {
         pdl_wait();
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc(BN);
+        if (half == 0) {                    // the even CTA issues for both
+            const uint32_t on = elect_one();
+            const uint32_t idesc = instr_desc(BN, 2 * BM);
             ItemIter it = items0;
             int t, kb_b, kb_e, s = 0;
             uint32_t ph = 0;
-            for (int item = 0; !abort_flag && it.next(t, kb_b, kb_e); ++item) {
+            bool stop = false;
+            for (int item = 0; !stop && it.next(t, kb_b, kb_e); ++item) {
                 const int a = item & 1;
-                if (!mbar_wait(acce0 + 8 * a, (uint32_t)((item >> 1) & 1) ^ 1u, &abort_flag,
-                               p.status))
+                if (!w_mbar_wait_cluster(acce0 + 8 * a, (uint32_t)((item >> 1) & 1) ^ 1u, &abort_flag, p.status))
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem + a * p.acc_stride;
-                for (int j = 0; j < kb_e - kb_b; ++j) {
-                    if (!mbar_wait(full0 + 8 * s, ph, &abort_flag, p.status)) break;
+                uint32_t more = 0;          // the item's first MMA starts the accumulator
+                for (int j = kb_b; j < kb_e; ++j) {
+                    if (!w_mbar_wait_cluster(full0 + 8 * s, ph, &abort_flag, p.status)) {
+                        stop = true;
+                        break;
+                    }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t ad = smem_desc(a_base + s * A_BYTES);
                     const uint64_t bd = smem_desc(b_base + s * bs_bytes);
                     const uint64_t bl = smem_desc(b_base + s * bs_bytes + b_bytes);
+                    if (has_lo) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        mma_bf16(acc, ad + 2 * kk, bd + 2 * kk, idesc, (j != 0) || (kk != 0));
-                        if (has_lo) mma_bf16(acc, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            w_mma_bf16_pair(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                            w_mma_bf16_pair(on, acc, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                        }
+                    } else {
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk)
+                            w_mma_bf16_pair(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
                     }
-                    mma_commit(empty0 + 8 * s);
+                    more = 1;
+                    w_mma_commit_pair(on, empty0 + 8 * s, (uint16_t)3);
                     if (++s == stages) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
-                mma_commit(accf0 + 8 * a);
+                w_mma_commit_pair(on, accf0 + 8 * a, (uint16_t)3);
             }
-            // every MMA issued above completes before the CTA frees its TMEM
-            mma_commit(drain);
-            volatile int never = 0;
-            mbar_wait(drain, 0, &never, p.status);
+            // every MMA issued above completes before either CTA frees its TMEM
+            w_mma_commit_pair(on, drain, (uint16_t)3);
+            __syncwarp();
         }
+        volatile int never = 0;
+        mbar_wait_cluster(drain, 0, &never, p.status);
         __syncwarp();
     } else {
         // epilogue warps: TMEM lane quarter (warp % 4)
@@ -686,25 +801,41 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         int t, kb_b, kb_e;
         for (int item = 0; it.next(t, kb_b, kb_e); ++item) {
             const int a = item & 1;
-            const bool ok = mbar_wait(accf0 + 8 * a, (uint32_t)(item >> 1) & 1u, &abort_flag,
-                                      p.status) && !abort_flag;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            int seg, row0, n0;
-            tile_geom(t, seg, row0, n0);
+            int wt, seg, row0, n0;
+            tile_geom(t, wt, seg, row0, n0);
             const int o_local = row0 + row;
-            const bool row_ok = ok && o_local < p.seg_rows[seg];
+            const bool row_in = wt < p.tiles && o_local < p.seg_rows[seg];
             const int o = p.seg_out[seg] + o_local;
-            const bool whole = kb_b == 0 && kb_e == KB;
+            const bool whole = t >= p.T_sk || (kb_b == 0 && kb_e == KB);
             const uint32_t taddr = tmem + a * p.acc_stride + ((uint32_t)(q * 32) << 16);
             // a CTA cuts at most two stream-K tiles: its first item and its last
-            const int slot = 2 * cta + (item == 0 ? 0 : 1);
+            const int slot = 2 * (2 * cta + (item == 0 ? 0 : 1)) + half;
             float *part = p.ws + (size_t)slot * BN * BM;
-            const bool add = p.epi == EPI_ADD;
+            // (a whole tile's later chunks add to what this thread stored for the first)
+            const bool add = p.epi == EPI_ADD || (whole && kb_b > 0);
             const bool glu = p.epi == EPI_SWIGLU;
             float *stg = reinterpret_cast<float *>(smem_raw + p.stg_off);   // [32 columns][128 rows]
+            // residual rows of 32 columns, requested one group ahead (the first
+            // group's before the accumulator is waited for)
+            auto residual = [&](int g0, float *yin) {
+                const float *yb = p.Y + (size_t)(n0 + g0) * p.ldy + o;
+                const int lim = min(min(32, BN - g0), p.M - (n0 + g0));
+#pragma unroll
+                for (int j = 0; j < 32; ++j) yin[j] = add && whole && row_in && j < lim ? yb[(size_t)j * p.ldy] : 0.f;
+            };
+            float ynext[32];
+            residual(0, ynext);
+            const bool landed = mbar_wait_cluster(accf0 + 8 * a, (uint32_t)(item >> 1) & 1u, &abort_flag,
+                                                  p.status) && !abort_flag;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const bool ok = landed && wt < p.tiles, row_ok = landed && row_in;
             for (int g0 = 0; g0 < BN; g0 += 32) {
                 // up to 32 accumulator columns with one TMEM round trip
                 const int gw = min(32, BN - g0);
+                float yin[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) yin[j] = ynext[j];
+                if (g0 + 32 < BN) residual(g0 + 32, ynext);
                 uint32_t r[32];
                 tmem_ld_cols(taddr + g0, r, gw);
                 if (whole && glu) {
@@ -733,11 +864,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 } else if (row_ok) {
                     float *yb = p.Y + (size_t)(n0 + g0) * p.ldy + o;
                     const int mlim = p.M - (n0 + g0);
-                    if (add) {               // residual: every load in flight, then the stores
-                        float yin[32];
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            yin[j] = (j < gw && j < mlim) ? yb[(size_t)j * p.ldy] : 0.f;
+                    if (add) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j)
                             if (j < gw && j < mlim) yb[(size_t)j * p.ldy] = yin[j] + __uint_as_float(r[j]);
@@ -749,7 +876,8 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acce0 + 8 * a) : "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(c_mapa(acce0 + 8 * a, 0));
             if (whole) continue;
             // ticket for the cut tile; the last piece reduces all pieces in CTA order
             __threadfence();
@@ -758,13 +886,13 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             const int c_last = owner_cta((long long)(t + 1) * KB - 1, U, p.grid);
             const int np = c_last - c_first + 1;
             if (et == 0) {
-                const int prev = atomicAdd(&p.counters[t], 1);
+                const int prev = atomicAdd(&p.counters[2 * t + half], 1);
                 s_reduce = prev == np - 1;
             }
             if (et < np && et < P_MAX_PIECES) {
                 const int cc = c_first + et;
                 const long long cu0 = (long long)cc * U / p.grid;
-                s_slot[et] = 2 * cc + (cu0 >= (long long)t * KB ? 0 : 1);
+                s_slot[et] = 2 * (2 * cc + (cu0 >= (long long)t * KB ? 0 : 1)) + half;
             }
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (!s_reduce) continue;
@@ -773,37 +901,52 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 continue;
             }
             __threadfence();
-            // flat float4 view of the [BN][128] pieces; 16 float4 loads in flight per thread
+            // flat float4 view of the [BN][128] pieces; 16 float4 loads of two pieces
+            // (a cut tile mostly has two or three) in flight per thread
+            constexpr int GR = 8, PI = 2;
             const int n4 = BN * BM / 4;
             const size_t piece4 = (size_t)BN * BM / 4;
             const float4 *ws4 = reinterpret_cast<const float4 *>(p.ws);
-            for (int base4 = et; base4 < n4; base4 += 4 * 128) {
-                float4 acc[4];
+            for (int base4 = et; base4 < n4; base4 += GR * 128) {
+                float4 acc[GR];
 #pragma unroll
-                for (int g = 0; g < 4; ++g) acc[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int i0 = 0; i0 < np; i0 += 4) {
-                    float4 v[4][4];
+                for (int g = 0; g < GR; ++g) acc[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i0 = 0; i0 < np; i0 += PI) {
+                    float4 v[PI][GR];
 #pragma unroll
-                    for (int pi = 0; pi < 4; ++pi) {
+                    for (int pi = 0; pi < PI; ++pi) {
                         const bool have = i0 + pi < np;
                         const float4 *src = ws4 + (size_t)s_slot[have ? i0 + pi : 0] * piece4;
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
+                        for (int g = 0; g < GR; ++g) {
                             const int e4 = base4 + g * 128;
                             v[pi][g] = (have && e4 < n4) ? __ldcg(src + e4)
                                                          : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
                     }
 #pragma unroll
-                    for (int pi = 0; pi < 4; ++pi)
+                    for (int pi = 0; pi < PI; ++pi)
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
+                        for (int g = 0; g < GR; ++g) {
                             acc[g].x += v[pi][g].x; acc[g].y += v[pi][g].y;
                             acc[g].z += v[pi][g].z; acc[g].w += v[pi][g].w;
                         }
                 }
+                // (the residual's loads of all groups before any store)
+                float4 yin[GR];
+                if (p.epi == EPI_ADD) {
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
+                    for (int g = 0; g < GR; ++g) {
+                        const int e4 = base4 + g * 128, col = (e4 * 4) / BM, r4 = (e4 * 4) - col * BM;
+                        const float *y = p.Y + (size_t)(n0 + col) * p.ldy + p.seg_out[seg] + row0 + r4;
+                        yin[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (e4 < n4 && n0 + col < p.M && ok && row0 + r4 + 4 <= p.seg_rows[seg] &&
+                            ((reinterpret_cast<uintptr_t>(y) & 15u) == 0))
+                            yin[g] = *reinterpret_cast<const float4 *>(y);
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < GR; ++g) {
                     const int e4 = base4 + g * 128;
                     if (p.epi == EPI_SWIGLU) {
                         // lane l < 16 holds gate rows 4l..4l+3 of a column, lane
@@ -834,8 +977,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                         ((reinterpret_cast<uintptr_t>(y) & 15u) == 0)) {      // one 16-byte access
                         float4 out = acc[g];
                         if (p.epi == EPI_ADD) {
-                            const float4 yi = *reinterpret_cast<const float4 *>(y);
-                            out.x += yi.x; out.y += yi.y; out.z += yi.z; out.w += yi.w;
+                            out.x += yin[g].x; out.y += yin[g].y; out.z += yin[g].z; out.w += yin[g].w;
                         }
                         *reinterpret_cast<float4 *>(y) = out;
                     } else {
@@ -849,16 +991,19 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                     }
                 }
             }
-            if (et == 0) p.counters[t] = 0;
+            if (et == 0) p.counters[2 * t + half] = 0;
         }
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (threadIdx.x == 0) stamp_max(p.stamp, 2);
+    // neither CTA leaves, or frees its tensor memory, while the other may still
+    // signal its barriers or read its own accumulators
+    c_cluster_sync();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(p.tmem_cols)
                      : "memory");
     }
@@ -895,22 +1040,6 @@ struct CkParams {
     GemmNorm nout, nin;     // folded RMSNorm: producer / consumer side (ss null: off)
     unsigned long long *stamp;   // launch stamps (entry, wait, exit ns) or null
 };
-
-__device__ __forceinline__ void c_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t c_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ uint32_t c_mapa(uint32_t local, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
-    return a;
-}
 
 // Where a CTA finds the S partials of the token columns it owns, [c_lo,
 // c_hi) = [rank * BN / S, (rank + 1) * BN / S): its own partial ([BN][128]
@@ -2157,6 +2286,65 @@ bool gemm_bf16(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int
     return true;
 }
 
+// How the persistent GEMM cuts its work: token tiles of BN columns, G CTA
+// pairs, T_sk of the T_all tiles stream-K, the others whole in chunks of
+// kb_chunk K-blocks.
+struct PersistShape {
+    int BN, nt, G, T_all, T_sk, dp_rounds, kb_chunk;
+};
+constexpr uint32_t P_BUDGET = 220u * 1024u;     // ring and staging bytes of a CTA
+constexpr int P_STAGES = 6;
+
+// Clocks, measured at 333 to 1024 rows and K = 4096, 11008. A K-block of a 256 x
+// BN tile takes 2.08 nb BN (4% above the MMAs' own time: 0.35 us at 160 columns
+// and two planes, 0.48 us at 224), and not less than 420 + 0.8 nb BN (0.26 to
+// 0.32 us at 96 to 112, by the clock the power limit leaves). For each count of token tiles that keeps BN <= 256: whole tiles
+// alone take ceil(T / G) rounds; with the remainder cut stream-K the units are
+// even, but the pieces' round trip through the workspace then costs 330 BN
+// where every tile is cut (O at 640 rows, 224 columns: 68 us against 40 in whole
+// tiles), about 180 BN where whole tiles follow to hide part of it.
+// A one-plane product (msd_linear) accumulates at most 40 K-blocks of a whole
+// tile in tensor memory before it adds them to Y: the accumulators truncate, so
+// the error grows with the chain (4096-long products: 2.2e-6 relative in pieces
+// of 40 blocks, 4.4e-6 in one of 64).
+static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int pairs) {
+    const int kblocks = (K + BK - 1) / BK, wt = (tiles + 1) / 2;
+    PersistShape best{};
+    double best_cost = 1e300;
+    for (int nt = (M + 255) / 256, n = 0; n < 6; ++nt, ++n) {
+        const int BN = ((M + nt - 1) / nt + 15) / 16 * 16;
+        if (n > 0 && BN < 64) break;
+        const long long T = (long long)wt * nt;
+        const double tk = std::max(2.08 * nb * BN, 420.0 + 0.8 * nb * BN);
+        // at least 4 K-blocks a pair
+        const long long G = std::max<long long>(1, std::min<long long>(pairs, T * kblocks / 4));
+        const int chunk = nb == 1 && !glu ? (kblocks + (kblocks + 39) / 40 - 1) / ((kblocks + 39) / 40) : kblocks;
+        PersistShape g{BN, nt, (int)G, (int)T, 0, (int)((T + G - 1) / G), chunk};
+        double cost = g.dp_rounds * tk * kblocks;
+        int rounds = (int)(T / G), T_sk = (int)(T - rounds * G);
+        if (T_sk > 0) {
+            const bool few = rounds > 0 && G > 8LL * T_sk;
+            // a few short-K tiles join a round of whole tiles: every tile in two
+            // or three pieces, fixed up at the end of the launch
+            if (few && kblocks <= 64 && !glu) {
+                --rounds;
+                T_sk += (int)G;
+            }
+            const double sk = T * tk * kblocks / G + (rounds == 0 ? 330.0 : 180.0) * BN;
+            if (sk < cost && (long long)T_sk * kblocks >= G) {      // (every pair holds a unit)
+                g.T_sk = T_sk;
+                g.dp_rounds = rounds;
+                cost = sk;
+            }
+        }
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = g;
+        }
+    }
+    return best;
+}
+
 static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
                          int O, float *Y, int ldy, int epi, const GemmFused *fx, int *status, cudaStream_t s) {
     const bool glu = fx && fx->epi == EPI_SWIGLU;
@@ -2172,44 +2360,17 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         tiles += pk.seg_tiles[i];
     }
     const int nb = X_lo ? 2 : 1;
+    const PersistShape g = persist_shape(tiles, M, K, nb, glu, p->num_sms / 2);
+    const int BN = g.BN, nt = g.nt, kblocks = (K + BK - 1) / BK, G = g.G;
     // the fused SwiGLU epilogue takes 16 KB of staging from the ring's budget
     const uint32_t stg_bytes = glu ? 32u * BM * 4u : 0u;
-    constexpr uint32_t BUDGET = 208u * 1024u;
-    // token tiles: the widest (fewest tiles, most weight reuse) that keeps three
-    // stages in shared memory; five stages measured best on decode shapes
-    int nt = (M + 255) / 256, BN = 0;
-    for (;; ++nt) {
-        BN = ((M + nt - 1) / nt + 15) / 16 * 16;
-        const uint32_t st = A_BYTES + (uint32_t)nb * BN * BK * 2;
-        if (3u * st + stg_bytes <= BUDGET || BN <= 16) break;
-    }
-    const int kblocks = (K + BK - 1) / BK;
-    const uint32_t stage_bytes = A_BYTES + (uint32_t)nb * BN * BK * 2;
-    int stages = (int)((BUDGET - stg_bytes) / stage_bytes);
-    stages = stages < 2 ? 2 : (stages > 5 ? 5 : stages);
+    const uint32_t stage_bytes = A_BYTES + (uint32_t)nb * (BN / 2) * BK * 2;
+    const int stages = std::max(2, std::min((int)((P_BUDGET - stg_bytes) / stage_bytes), P_STAGES));
     const size_t smem = 1024 + (size_t)stages * stage_bytes + stg_bytes;
-    const long long tiles_total = (long long)tiles * nt;
-    const long long all_units = tiles_total * kblocks;
-    // one CTA per SM, at least 4 K-blocks each
-    long long G = all_units / 4;
-    if (G > p->num_sms) G = p->num_sms;
-    if (G < 1) G = 1;
-    // whole tiles in rounds of G, the remainder split stream-K across all CTAs
-    // (its fix-ups overlap the whole tiles that follow). A remainder of a few
-    // short-K tiles would cut each into more than eight pieces, summed by one
-    // CTA: there one round of whole tiles joins it (every tile in two or three
-    // pieces, fixed up at the end). Measured on the 960-row verify GEMMs: O
-    // (K = 4096) 89 -> 75 us; down (K = 11008) 106 -> 140 us and the SwiGLU
-    // launches slower, so those keep the rounds.
-    int dp_rounds = (int)(tiles_total / G);
-    int T_sk = (int)(tiles_total - (long long)dp_rounds * G);
-    if (T_sk > 0 && dp_rounds > 0 && G > 8LL * T_sk && kblocks <= 64 && !glu) {
-        --dp_rounds;
-        T_sk += (int)G;
-    }
-    const long long units = (long long)T_sk * kblocks;
-    const size_t ws_need = 2ull * G * BN * BM * sizeof(float);
-    if (ws_need > WS_BYTES || tiles_total > N_COUNTERS) {
+    const long long units = (long long)g.T_sk * kblocks;
+    const long long all_units = (long long)g.T_all * kblocks;
+    const size_t ws_need = 4ull * G * BN * BM * sizeof(float);
+    if (ws_need > WS_BYTES || 2ll * g.T_sk > N_COUNTERS) {
         flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
         fprintf(stderr, "msd: GEMM shape M=%d K=%d O=%d exceeds the workspace\n", M, K, O);
         return;
@@ -2223,17 +2384,19 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     pk.stages = stages;
     pk.acc_stride = acc;
     pk.tmem_cols = 2 * acc;
-    pk.grid = (int)G;
+    pk.grid = G;
+    pk.tiles = tiles;
     pk.units = units;
-    pk.T_sk = T_sk;
-    pk.dp_rounds = dp_rounds;
+    pk.T_sk = g.T_sk;
+    pk.dp_rounds = g.dp_rounds;
+    pk.T_all = g.T_all;
+    pk.kb_chunk = g.kb_chunk;
     pk.Y = Y;
     pk.ldy = ldy;
     pk.epi = epi;
     pk.ws = p->ws;
     pk.counters = p->counters;
     pk.status = status;
-    pk.wpacked = static_cast<const bf16 *>(W.packed);
     pk.has_lo = X_lo ? 1 : 0;
     if (glu) {
         pk.epi = EPI_SWIGLU;
@@ -2247,13 +2410,14 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         fprintf(stderr, "msd: GEMM weights were not packed\n");
         return;
     }
-    const CUtensorMap *mx = get_map(p, X, M, K, ldx, BN, status);
-    const CUtensorMap *mxl = X_lo ? get_map(p, X_lo, M, K, ldx, BN, status) : mx;
-    if (!mx || !mxl) return;
+    const CUtensorMap *mx = get_map(p, X, M, K, ldx, BN / 2, status);
+    const CUtensorMap *mxl = X_lo ? get_map(p, X_lo, M, K, ldx, BN / 2, status) : mx;
+    const CUtensorMap *mw = get_wmap(p, W.packed, (long)tiles * kblocks * BM);
+    if (!mx || !mxl || !mw) return;
     pk.stamp = stamp_slot(p);
     if (!p->smem_set) {
-        cudaFuncSetAttribute(gemm_persist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(BUDGET + 1024));
+        cudaFuncSetAttribute(gemm_persist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(P_BUDGET + 1024));
         p->smem_set = true;
     }
     const bool prof = p->profile;
@@ -2270,16 +2434,24 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     // touching anything but weights.
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof lc);
-    lc.gridDim = dim3((unsigned)G);
+    lc.gridDim = dim3((unsigned)(2 * G));
     lc.blockDim = dim3(P_THREADS);
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     lc.attrs = at;
-    lc.numAttrs = 1;
-    cudaLaunchKernelEx(&lc, gemm_persist_kernel, *mx, *mxl, pk);
+    lc.numAttrs = 2;
+    if (cudaLaunchKernelEx(&lc, gemm_persist_kernel<false>, *mx, *mxl, *mw, pk) != cudaSuccess) {
+        cudaGetLastError();
+        flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
+        fprintf(stderr, "msd: persistent GEMM launch failed (M=%d K=%d O=%d)\n", M, K, O);
+    }
     note_launch();
     if (prof) {
         cudaEventRecord(p->ev[p->ev_used + 1], s);
@@ -2288,7 +2460,7 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     const double wb = (double)O * K * 2.0;
     account(p, wb, wb + (double)M * K * 2.0 * nb +
                        (glu ? (double)M * fx->F * 2.0 * nb : (double)M * O * 4.0 * (epi == EPI_ADD ? 2 : 1)),
-            M, O, K, nb, std::min(wb, (double)G * std::min<long long>(stages, all_units / G) * A_BYTES));
+            M, O, K, nb, std::min(wb, 2.0 * G * std::min<long long>(stages, all_units / G) * A_BYTES));
 }
 
 }  // namespace msd
