@@ -243,6 +243,41 @@ __device__ __forceinline__ void w_mma_bf16_pair(uint32_t on, uint32_t tmem_d, ui
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on));
 }
 
+__device__ __forceinline__ void w_tma_load_2d(uint32_t on, uint32_t dst, const CUtensorMap *map, int x, int y,
+                                              uint32_t bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];\n}" ::"r"(dst),
+        "l"(map), "r"(x), "r"(y), "r"(bar), "r"(on)
+        : "memory");
+}
+
+__device__ __forceinline__ void w_bulk_load(uint32_t on, uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %4, 0;\n"
+        "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(bar), "r"(on)
+        : "memory");
+}
+
+__device__ __forceinline__ void w_mma_bf16(uint32_t on, uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
+                                           uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p, q;\n"
+        "setp.ne.b32 q, %5, 0;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(on));
+}
+
+__device__ __forceinline__ void w_mma_commit(uint32_t on, uint32_t bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar), "r"(on)
+        : "memory");
+}
+
 __device__ __forceinline__ void w_mma_commit_pair(uint32_t on, uint32_t bar, uint16_t cta_mask) {
     asm volatile(
         "{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
@@ -1427,90 +1462,102 @@ __global__ void __launch_bounds__(C_THREADS)
     if constexpr (pair) c_cluster_sync();
 
     if (warp == 0) {
+        const uint32_t on = elect_one();
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&mx) : "memory");
             if (has_lo) asm volatile("prefetch.tensormap [%0];" ::"l"(&mxl) : "memory");
             if (pair) asm volatile("prefetch.tensormap [%0];" ::"l"(&mw) : "memory");
-            // the weight block of pipeline step i: a bulk copy, or (pair) a tensor
-            // copy of its 128 rows that completes on the even CTA's barrier
-            auto load_w = [&](int i, int st) {
-                if (!pair || half == 0) mbar_expect_tx(full0 + 8 * st, stage_tx);
-                if constexpr (pair)
-                    tma_load_2d_pair(a_base + st * A_BYTES, &mw, 0, (int)(((size_t)blockIdx.x * KB + kb0 + i) * BM),
-                                     sig0 + 8 * st);
-                else
-                    bulk_load(a_base + st * A_BYTES, wblk + (size_t)i * blk_elems, A_BYTES, full0 + 8 * st);
-            };
-            // weights first (they never depend on the previous kernel), then wait
-            const int n_pre = min(stages, nk);
-            for (int j = 0; j < n_pre; ++j) load_w(j, j);
-            pdl_wait();
-            stamp_min(p.stamp, 1);
-            pdl_trigger();
-            int s = 0;
-            uint32_t ph = 0;
-            int i = 0;
-            for (; i < nk; ++i) {
-                if (i >= n_pre) {
-                    if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, &abort_flag, p.status)) break;
-                    load_w(i, s);
-                }
-                if constexpr (pair) {
-                    const int ny = n0 + (int)half * BNs;
-                    tma_load_2d_pair(b_base + s * bs_bytes, &mx, (kb0 + i) * BK, ny, sig0 + 8 * s);
-                    if (has_lo) tma_load_2d_pair(b_base + s * bs_bytes + b_bytes, &mxl, (kb0 + i) * BK, ny, sig0 + 8 * s);
-                } else {
-                    tma_load_2d(b_base + s * bs_bytes, &mx, (kb0 + i) * BK, n0, full0 + 8 * s);
-                    if (has_lo) tma_load_2d(b_base + s * bs_bytes + b_bytes, &mxl, (kb0 + i) * BK, n0, full0 + 8 * s);
-                }
-                if (++s == stages) {
-                    s = 0;
-                    ph ^= 1u;
-                }
+        }
+        __syncwarp();
+        const uint32_t on_expect = !pair || half == 0 ? on : 0u;
+        // the weight block of pipeline step i: a bulk copy, or (pair) a tensor
+        // copy of its 128 rows that completes on the even CTA's barrier
+        auto load_w = [&](int i, int st) {
+            w_expect_tx(on_expect, full0 + 8 * st, stage_tx);
+            if constexpr (pair)
+                w_tma_load_2d_pair(on, a_base + st * A_BYTES, &mw, 0, ((int)blockIdx.x * KB + kb0 + i) * BM,
+                                   sig0 + 8 * st);
+            else
+                w_bulk_load(on, a_base + st * A_BYTES, wblk + (size_t)i * blk_elems, A_BYTES, full0 + 8 * st);
+        };
+        // weights first (they never depend on the previous kernel), then wait
+        const int n_pre = min(stages, nk);
+        for (int j = 0; j < n_pre; ++j) load_w(j, j);
+        pdl_wait();
+        if (lane == 0) stamp_min(p.stamp, 1);
+        pdl_trigger();
+        const int ny = pair ? n0 + (int)half * BNs : n0;
+        int s = 0;
+        uint32_t ph = 0;
+        int i = 0;
+        for (; i < nk; ++i) {
+            if (i >= n_pre) {
+                if (!w_mbar_wait(empty0 + 8 * s, ph ^ 1u, &abort_flag, p.status)) break;
+                load_w(i, s);
             }
-            if (abort_flag && (!pair || half == 0)) {   // (pair: the even CTA's barriers count both CTAs' copies)
-                volatile int never = 0;
-                for (int j = (i > stages ? i - stages : 0); j < i; ++j)
-                    mbar_wait(full0 + 8 * (j % stages), (uint32_t)(j / stages) & 1u, &never, p.status);
+            if constexpr (pair) {
+                w_tma_load_2d_pair(on, b_base + s * bs_bytes, &mx, (kb0 + i) * BK, ny, sig0 + 8 * s);
+                if (has_lo)
+                    w_tma_load_2d_pair(on, b_base + s * bs_bytes + b_bytes, &mxl, (kb0 + i) * BK, ny, sig0 + 8 * s);
+            } else {
+                w_tma_load_2d(on, b_base + s * bs_bytes, &mx, (kb0 + i) * BK, ny, full0 + 8 * s);
+                if (has_lo)
+                    w_tma_load_2d(on, b_base + s * bs_bytes + b_bytes, &mxl, (kb0 + i) * BK, ny, full0 + 8 * s);
             }
+            if (++s == stages) {
+                s = 0;
+                ph ^= 1u;
+            }
+        }
+        if (abort_flag && (!pair || half == 0)) {   // (pair: the even CTA's barriers count both CTAs' copies)
+            volatile int never = 0;
+            for (int j = (i > stages ? i - stages : 0); j < i; ++j)
+                mbar_wait(full0 + 8 * (j % stages), (uint32_t)(j / stages) & 1u, &never, p.status);
         }
         __syncwarp();
     } else if (warp == 1) {
         pdl_wait();
-        if (lane == 0 && (!pair || half == 0)) {      // (pair: the even CTA issues for both)
+        if (!pair || half == 0) {      // (pair: the even CTA issues for both)
+            const uint32_t on = elect_one();
             const uint32_t idesc = instr_desc(BN, pair ? 2 * BM : BM);
             int s = 0;
             uint32_t ph = 0;
             for (int i = 0; i < nk; ++i) {
-                if (pair ? !mbar_wait_cluster(full0 + 8 * s, ph, &abort_flag, p.status)
-                         : !mbar_wait(full0 + 8 * s, ph, &abort_flag, p.status))
+                if (pair ? !w_mbar_wait_cluster(full0 + 8 * s, ph, &abort_flag, p.status)
+                         : !w_mbar_wait(full0 + 8 * s, ph, &abort_flag, p.status))
                     break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint64_t ad = smem_desc(a_base + s * A_BYTES);
                 const uint64_t bd = smem_desc(b_base + s * bs_bytes);
                 const uint64_t bl = smem_desc(b_base + s * bs_bytes + b_bytes);
-                if constexpr (pair) {
+                const uint32_t more = i != 0;
+                if (has_lo) {
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk) {
-                        mma_bf16_pair(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (i != 0) || (kk != 0));
-                        if (has_lo) mma_bf16_pair(tmem, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                        if constexpr (pair) {
+                            w_mma_bf16_pair(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                            w_mma_bf16_pair(on, tmem, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                        } else {
+                            w_mma_bf16(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                            w_mma_bf16(on, tmem, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                        }
                     }
-                    mma_commit_pair(empty0 + 8 * s, pair_mask);
                 } else {
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk) {
-                        mma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (i != 0) || (kk != 0));
-                        if (has_lo) mma_bf16(tmem, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                        if constexpr (pair) w_mma_bf16_pair(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                        else w_mma_bf16(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
                     }
-                    mma_commit(empty0 + 8 * s);
                 }
+                if constexpr (pair) w_mma_commit_pair(on, empty0 + 8 * s, pair_mask);
+                else w_mma_commit(on, empty0 + 8 * s);
                 if (++s == stages) {
                     s = 0;
                     ph ^= 1u;
                 }
             }
-            if constexpr (pair) mma_commit_pair(done, pair_mask);
-            else mma_commit(done);
+            if constexpr (pair) w_mma_commit_pair(on, done, pair_mask);
+            else w_mma_commit(on, done);
             volatile int never = 0;     // (as gemm_tc_kernel: no MMA outlives the CTA's TMEM)
             mbar_wait(done, 0, &never, p.status);
         }
