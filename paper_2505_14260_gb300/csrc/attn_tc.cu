@@ -126,18 +126,6 @@ __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void bar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void bar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void tma2d(uint32_t dst, const CUtensorMap *m, int x, int y, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(m), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
 // Shared-memory matrix descriptor (sm100 version 1, 128-byte swizzle): start
 // address, leading byte offset (MN-major: the stride between 64-element
 // atoms along M/N) and stride byte offset (the stride between 8-row groups).
@@ -153,17 +141,47 @@ __device__ __forceinline__ uint32_t idesc(int M, int N, int b_mn) {
            ((uint32_t)(M >> 4) << 24);
 }
 
-// D (+)= A B^T with A read from tensor memory and B from shared memory.
-__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
-        "r"(a), "l"(b), "r"(id), "r"(acc));
+// Warp-wide forms: the TMA and MMA loops run in whole warps, in step, and only
+// the lane that elect_one() names (`on`) issues, so that descriptors, addresses
+// and barriers stay on the uniform datapath (a loop in one diverged lane took
+// 36 to 46 ns to issue an MMA of 64 x 64 x 16 or 64 x 128 x 16, more than it runs).
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t on;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}" : "=r"(on));
+    return on;
 }
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+__device__ __forceinline__ void w_expect_tx(uint32_t on, uint32_t bar, uint32_t bytes) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
+        "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(bar),
+        "r"(bytes), "r"(on)
+        : "memory");
+}
+__device__ __forceinline__ void w_tma2d(uint32_t on, uint32_t dst, const CUtensorMap *m, int x, int y, uint32_t bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];\n}" ::"r"(dst),
+        "l"(m), "r"(x), "r"(y), "r"(bar), "r"(on)
+        : "memory");
+}
+// D (+)= A B^T with A read from tensor memory and B from shared memory.
+__device__ __forceinline__ void w_mma_ts(uint32_t on, uint32_t d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.b32 q, %5, 0;\nsetp.ne.b32 p, %4, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
+        "r"(a), "l"(b), "r"(id), "r"(acc), "r"(on));
+}
+__device__ __forceinline__ void w_commit(uint32_t on, uint32_t bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar), "r"(on)
+        : "memory");
+}
+// Bounded wait of a whole warp (every lane waits; the answer is uniform).
+__device__ __forceinline__ bool w_bar_wait(uint32_t bar, uint32_t parity, volatile int *abort, int *status) {
+    if (__all_sync(0xffffffffu, bar_try(bar, parity))) return true;
+    return __all_sync(0xffffffffu, bar_wait(bar, parity, abort, status));
 }
 
 // 32 columns of this warp's lanes, waited for in the same asm statement: the
@@ -352,28 +370,30 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int row_base_c = (req * p.nh + h) * p.cache_slots;
     const int row_base_t = (req * p.nh + h) * p.tree_slots;
 
-    auto issue = [&](int i) {
-        const int s = i % STAGES;
+    auto issue = [&](uint32_t on, int i, int s) {
         const uint32_t bar = full0 + 8 * s;
         const uint32_t kd = base + s * L::STAGE;
-        bar_expect_tx(bar, L::STAGE);
+        w_expect_tx(on, bar, L::STAGE);
         const bool cache = i < nc;
         const CUtensorMap *mk = cache ? &mkc : &mkt, *mv = cache ? &mvc : &mvt;
         const int y = cache ? row_base_c + k_lo + i * KT : row_base_t + (i - nc) * KT;
 #pragma unroll
         for (int b = 0; b < L::NB; ++b) {
-            tma2d(kd + b * L::BOX, mk, b * 64, y, bar);
-            tma2d(kd + L::TILE + b * L::BOX, mk, b * 64, y + p.lo_rows, bar);
-            tma2d(kd + 2 * L::TILE + b * L::BOX, mv, b * 64, y, bar);
-            tma2d(kd + 3 * L::TILE + b * L::BOX, mv, b * 64, y + p.lo_rows, bar);
+            w_tma2d(on, kd + b * L::BOX, mk, b * 64, y, bar);
+            w_tma2d(on, kd + L::TILE + b * L::BOX, mk, b * 64, y + p.lo_rows, bar);
+            w_tma2d(on, kd + 2 * L::TILE + b * L::BOX, mv, b * 64, y, bar);
+            w_tma2d(on, kd + 3 * L::TILE + b * L::BOX, mv, b * 64, y + p.lo_rows, bar);
         }
     };
     // the cache tiles of the first stages may go out before the wait; tree
     // K/V is the previous kernel's output
     const int n_pre = min(STAGES, ntiles);
     const int n_early = p.cache_early ? min(n_pre, nc) : 0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < n_early; ++i) issue(i);
+    uint32_t prod_on = 0;
+    if (warp == 0) {
+        prod_on = elect_one();
+        for (int i = 0; i < n_early; ++i) issue(prod_on, i, i);
+    }
     wait_prior();
     if (threadIdx.x == 0 && p.stamp) atomicMin(p.stamp + 1, gtime());
     allow_dependents();
@@ -383,50 +403,60 @@ __global__ void __launch_bounds__(THREADS, 1)
 
     if (warp == 0) {
         // ---- producer ------------------------------------------------------
-        if (lane == 0) {
-            for (int i = n_early; i < n_pre; ++i) issue(i);
-            int i = n_pre;
-            for (; i < ntiles; ++i) {
-                const int s = i % STAGES;
-                if (!bar_wait(empty0 + 8 * s, (uint32_t)(i / STAGES - 1) & 1u, &abort_flag, p.status)) break;
-                issue(i);
+        __syncwarp();
+        for (int i = n_early; i < n_pre; ++i) issue(prod_on, i, i);
+        int i = n_pre, s = n_pre % STAGES;
+        uint32_t ph = 0;
+        for (; i < ntiles; ++i) {
+            if (!w_bar_wait(empty0 + 8 * s, ph, &abort_flag, p.status)) break;
+            issue(prod_on, i, s);
+            if (++s == STAGES) {
+                s = 0;
+                ph ^= 1u;
             }
-            if (abort_flag) {       // the copies still in flight land before the CTA exits
-                volatile int never = 0;
-                for (int j = (i > STAGES ? i - STAGES : 0); j < i; ++j)
-                    bar_wait(full0 + 8 * (j % STAGES), (uint32_t)(j / STAGES) & 1u, &never, p.status);
-            }
+        }
+        if (abort_flag) {           // the copies still in flight land before the CTA exits
+            volatile int never = 0;
+            for (int j = (i > STAGES ? i - STAGES : 0); j < i; ++j)
+                bar_wait(full0 + 8 * (j % STAGES), (uint32_t)(j / STAGES) & 1u, &never, p.status);
         }
         __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issue -----------------------------------------------------
-        if (lane == 0 && ntiles > 0) {
+        if (ntiles > 0) {
+            const uint32_t on = elect_one();
             const uint32_t id_qk = idesc(ROWS, KT, 0), id_pv = idesc(ROWS, HD, 1);
+            int qs = 0;                     // stage and phase of the next Q K^T tile
+            uint32_t qph = 0;
             auto qk = [&](int t) -> bool {
-                const int s = t % STAGES;
-                if (!bar_wait(full0 + 8 * s, (uint32_t)(t / STAGES) & 1u, &abort_flag, p.status)) return false;
+                if (!w_bar_wait(full0 + 8 * qs, qph, &abort_flag, p.status)) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t kd = base + s * L::STAGE;
+                const uint32_t kd = base + qs * L::STAGE;
                 const uint32_t sd = tmem + L::T_S + (t & 1) * KT;
 #pragma unroll
                 for (int kk = 0; kk < HD / 16; ++kk) {
                     const uint32_t ko = (kk >> 2) * L::BOX + (kk & 3) * 32;
                     const uint64_t kh = sdesc(kd + ko, 16, 1024), kl = sdesc(kd + L::TILE + ko, 16, 1024);
-                    mma_ts(sd, tmem + L::T_QH + kk * 8, kh, id_qk, kk > 0);
-                    mma_ts(sd, tmem + L::T_QL + kk * 8, kh, id_qk, 1u);
-                    mma_ts(sd, tmem + L::T_QH + kk * 8, kl, id_qk, 1u);
+                    w_mma_ts(on, sd, tmem + L::T_QH + kk * 8, kh, id_qk, kk > 0);
+                    w_mma_ts(on, sd, tmem + L::T_QL + kk * 8, kh, id_qk, 1u);
+                    w_mma_ts(on, sd, tmem + L::T_QH + kk * 8, kl, id_qk, 1u);
                 }
-                mma_commit(s_full0 + 8 * (t & 1));
+                w_commit(on, s_full0 + 8 * (t & 1));
+                if (++qs == STAGES) {
+                    qs = 0;
+                    qph ^= 1u;
+                }
                 return true;
             };
-            bool ok = bar_wait(q_ready, 0, &abort_flag, p.status);
+            bool ok = w_bar_wait(q_ready, 0, &abort_flag, p.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (ok) ok = qk(0);
             if (ok && ntiles > 1) ok = qk(1);
+            int vs = 0;                     // stage of tile j
             for (int j = 0; ok && j < ntiles; ++j) {
-                if (!bar_wait(p_full0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, &abort_flag, p.status)) break;
+                if (!w_bar_wait(p_full0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, &abort_flag, p.status)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t vd = base + (j % STAGES) * L::STAGE + 2 * L::TILE;
+                const uint32_t vd = base + vs * L::STAGE + 2 * L::TILE;
                 // P of keys 32h .. 32h+31 sits in S columns 32h .. 32h+31: hi pairs
                 // in the first 16, lo pairs in the next 16
                 const uint32_t pd = tmem + L::T_S + (j & 1) * KT;
@@ -435,16 +465,17 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const uint32_t ph = pd + (kk >> 1) * 32 + (kk & 1) * 8, pl = ph + 16;
                     const uint64_t vh = sdesc(vd + kk * 2048, L::BOX, 1024);
                     const uint64_t vl = sdesc(vd + L::TILE + kk * 2048, L::BOX, 1024);
-                    mma_ts(tmem + L::T_O, ph, vh, id_pv, (j > 0) || (kk > 0));
-                    mma_ts(tmem + L::T_O, pl, vh, id_pv, 1u);
-                    mma_ts(tmem + L::T_O, ph, vl, id_pv, 1u);
+                    w_mma_ts(on, tmem + L::T_O, ph, vh, id_pv, kk > 0 ? 1u : (uint32_t)(j > 0));
+                    w_mma_ts(on, tmem + L::T_O, pl, vh, id_pv, 1u);
+                    w_mma_ts(on, tmem + L::T_O, ph, vl, id_pv, 1u);
                 }
-                mma_commit(empty0 + 8 * (j % STAGES));
-                mma_commit(o_ready);
+                w_commit(on, empty0 + 8 * vs);
+                w_commit(on, o_ready);
+                if (++vs == STAGES) vs = 0;
                 if (j + 2 < ntiles) ok = qk(j + 2);
             }
             // no MMA outlives the CTA's tensor memory
-            mma_commit(drain);
+            w_commit(on, drain);
             volatile int never = 0;
             bar_wait(drain, 0, &never, p.status);
         }
