@@ -290,11 +290,10 @@ msd_status msd_ar_step(msd_ctx *ctx, int32_t *token_dev, void *stream);
  * y[i][j] (= or, if accumulate != 0, +=) sum_t x[i][t] * w[j][t] for i < m,
  * j < o, t < k. x [m][ldx] and w [o][k] are in the context dtype (bf16 rows
  * 16-byte aligned: ldx and k multiples of 8), y [m][ldy] is fp32; all device.
- * bf16 runs on the tcgen05 tensor-core GEMM of the step: w is first re-laid
- * into the context's packing scratch (grown on demand, so this call may
- * allocate), then multiplied; fp32 runs on the CUDA-core GEMM.
- * Errors: MSD_ERR_INVALID on null pointers, non-positive sizes or bad strides,
- * MSD_ERR_OOM if the packing scratch cannot grow. */
+ * bf16 runs on the tcgen05 tensor-core GEMMs of the step, which read w as it
+ * is; fp32 runs on the CUDA-core GEMM.
+ * Errors: MSD_ERR_INVALID on null pointers, non-positive sizes, bad strides or
+ * alignment. */
 msd_status msd_linear(msd_ctx *ctx, const void *x_dev, int32_t ldx, int32_t m, int32_t k,
                       const void *w_dev, int32_t o, float *y_dev, int32_t ldy,
                       int32_t accumulate, void *stream);
@@ -305,23 +304,24 @@ msd_status msd_linear(msd_ctx *ctx, const void *x_dev, int32_t ldx, int32_t m, i
  * where an allocation would synchronise the device or is not permitted, a
  * plug-in handed buffers but no allocator). It needs no context and allocates
  * nothing: its scratch is one static device array (a 256-byte status word,
- * 4096 int tile tickets and 16 MiB of fp32 split-K partials) which every GPU
+ * 4096 int tile tickets and 16 MiB of fp32 pieces of cut tiles) which every GPU
  * that loads this library holds until the process exits. The paper has no
  * counterpart; this is a service of the library, not a step of the method.
  * Arguments are those of msd_linear (x [m][ldx], w [o][k] bf16 with ldx and k
  * multiples of 8, y [m][ldy] fp32, all device memory on the current device).
- * The split-K choice is limited to what the array holds: a shape whose best
- * split would need more partials or tickets runs with fewer splits (none at
- * worst), so no shape is refused for its scratch. The first call made on a
- * device looks up the array's device address on that device
- * (cudaGetSymbolAddress) and sets the kernel's shared-memory limit; make that
+ * Up to 128 rows need none of it; with more, a shape whose best cut would need
+ * more than the array holds runs in whole tiles, so no shape is refused for its
+ * scratch. The first call made on a device looks up the array's device address
+ * on that device (cudaGetSymbolAddress), page-locks one page of the library's
+ * own host memory for the status word (where it cannot, the array's word is
+ * copied back by each call) and sets the kernels' shared-memory limits; make that
  * first call before any stream capture. Every call shares the array and it
  * keeps the last call's contents; the tile tickets are cleared on `stream`
  * before each launch that uses them. Calls that overlap on the GPU (other
  * streams, other host threads) race on the array: serialise them.
  * Device-side errors: a bounded wait of the kernel that runs out (2 s) sets the
- * array's status word. Each call first reads that word back on `stream` (so it
- * returns only after the work queued before it on `stream` has finished); if it
+ * status word. Each call first waits for the work queued before it on `stream`
+ * and reads that word; if it
  * is set, the call clears it, launches nothing and returns MSD_ERR_DEVICE: the
  * failed call's y is not to be trusted.
  * Errors: MSD_ERR_INVALID (null pointer, non-positive size, bad stride or

@@ -1,23 +1,15 @@
-// bf16 GEMM for the decode step on the sm_103a tensor cores.
+// bf16 GEMMs on the sm_103a tensor cores.
 //
-// Decode GEMMs multiply a few token rows (M = 7 .. 960) by large weight
-// matrices, so they stream weights from HBM. The kernel swaps operands: a
-// 128-row weight tile is the MMA's A operand (M = 128) and the token rows are
-// its B operand (N = 16 .. 256), so the accumulator D^T[128 weight rows][N
-// tokens] sits in TMEM, one weight row per TMEM lane.
-//
-// Per CTA (128 threads):
-//   warp 0 lane 0  TMA producer: 128x64 weight tile + Nx64 token tile per
-//                  stage, 128-byte swizzle, completion on a full[] mbarrier
-//   warp 1         allocates TMEM; lane 0 issues tcgen05.mma (K = 16 per
-//                  instruction, 4 per stage) and frees stages via
-//                  tcgen05.commit -> empty[]
-//   all 4 warps    epilogue: tcgen05.ld of their 32 TMEM lanes, fp32 store
-//                  or accumulate into Y (coalesced along the output dim)
-// Split-K: when there are too few weight tiles to cover the SMs, K is split;
-// every split writes its fp32 partial to a workspace and the last CTA to
-// finish a tile (atomic counter) sums the partials in split order, so results
-// are deterministic, and resets the counter. No CTA waits on another.
+// Operands are swapped: a 128-row weight tile is the MMA's A operand (M = 128,
+// or 256 over a CTA pair) and the token rows are its B operand (N = 16 .. 256), so
+// the accumulator D^T[128 weight rows][N tokens] sits in TMEM, one weight row per
+// TMEM lane. Two kernels share the building blocks below:
+//   gemm_cluster_kernel  up to 128 token rows: weight streaming from HBM, K split
+//                        over a cluster, fused epilogues
+//   gemm_persist_kernel  more token rows: tensor-bound, two-SM tiles
+// Both take the context's packed weights, or the caller's row-major weight
+// (msd_linear, msd_linear_noalloc) through a tensor map whose 128-byte swizzle
+// leaves the same blocks in shared memory, so nothing is re-laid first.
 // Every mbarrier wait is bounded (2 s of %globaltimer); on timeout the CTA
 // sets the device status word and winds down.
 #include <cuda.h>
@@ -39,25 +31,10 @@ namespace {
 
 constexpr int BM = 128;          // weight rows per tile (MMA M)
 constexpr int BK = 64;           // K per stage: one 128-byte swizzle row of bf16
-constexpr int THREADS = 128;
-constexpr int MAX_STAGES = 8;
 constexpr uint32_t A_BYTES = BM * BK * 2;          // 16 KB
 constexpr unsigned long long TIMEOUT_NS = 2000000000ull;
 constexpr size_t WS_BYTES = 64ull << 20;
 constexpr int N_COUNTERS = 16384;
-
-struct TcParams {
-    int n_seg;
-    int seg_tiles[3];
-    int seg_rows[3];
-    int seg_out[3];
-    int M, kblocks, splits, kb_per_split, BN, n_tiles_n, stages, tmem_cols;
-    float *Y;
-    int ldy, epi;
-    float *ws;
-    int *counters;
-    int *status;
-};
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -118,24 +95,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y,
-                                            uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
-// Contiguous global -> shared copy completing on an mbarrier (16-byte aligned).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            dst),
-        "l"(src), "r"(bytes), "r"(bar)
-        : "memory");
-}
-
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 
@@ -151,56 +110,6 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
 __device__ __forceinline__ uint32_t instr_desc(int BN, int M = BM) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-}
-
-// Two-SM tiles (tcgen05 cta_group::2; CTAs 2j and 2j+1 of a cluster are a
-// pair). The even CTA issues M = 256 MMAs: each CTA's own 128 weight rows are A,
-// at the same shared-memory offset in both; each CTA holds BN/2 token columns
-// of B (the even CTA the first half); each CTA's TMEM receives its own 128 rows
-// x BN. Both CTAs' copies complete on the even CTA's stage barrier.
-__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
-                                              uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
-// Arrives, once the pair's MMAs issued so far complete, on the mbarrier at the
-// same offset in each CTA of cta_mask (cluster ranks).
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t cta_mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            bar),
-        "h"(cta_mask)
-        : "memory");
-}
-
-// 2-D tensor copy into this CTA's shared memory completing on an mbarrier of
-// either CTA of the pair (a shared::cluster address).
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int x, int y,
-                                                 uint32_t cluster_bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(map), "r"(x), "r"(y), "r"(cluster_bar)
-        : "memory");
 }
 
 // Warp-wide forms. The TMA and MMA issue loops run in whole warps: tensor
@@ -223,6 +132,13 @@ __device__ __forceinline__ void w_expect_tx(uint32_t on, uint32_t bar, uint32_t 
         : "memory");
 }
 
+// Two-SM tiles (tcgen05 cta_group::2; CTAs 2j and 2j+1 of a cluster are a
+// pair). The even CTA issues M = 256 MMAs: each CTA's own 128 weight rows are A,
+// at the same shared-memory offset in both; each CTA holds BN/2 token columns
+// of B (the even CTA the first half); each CTA's TMEM receives its own 128 rows
+// x BN. Both CTAs' copies complete on the even CTA's stage barrier.
+// 2-D tensor copy into this CTA's shared memory completing on an mbarrier of
+// either CTA of the pair (a shared::cluster address).
 __device__ __forceinline__ void w_tma_load_2d_pair(uint32_t on, uint32_t dst, const CUtensorMap *map, int x, int y,
                                                    uint32_t cluster_bar) {
     asm volatile(
@@ -253,6 +169,7 @@ __device__ __forceinline__ void w_tma_load_2d(uint32_t on, uint32_t dst, const C
         : "memory");
 }
 
+// Contiguous global -> shared copy completing on an mbarrier (16-byte aligned).
 __device__ __forceinline__ void w_bulk_load(uint32_t on, uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
     asm volatile(
         "{\n.reg .pred q;\nsetp.ne.b32 q, %4, 0;\n"
@@ -278,6 +195,8 @@ __device__ __forceinline__ void w_mma_commit(uint32_t on, uint32_t bar) {
         : "memory");
 }
 
+// Arrives, once the pair's MMAs issued so far complete, on the mbarrier at the
+// same offset in each CTA of cta_mask (cluster ranks).
 __device__ __forceinline__ void w_mma_commit_pair(uint32_t on, uint32_t bar, uint16_t cta_mask) {
     asm volatile(
         "{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
@@ -363,176 +282,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *r) {
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t *r, int gw) {
     if (gw > 16) tmem_ld32(taddr, r);
     else tmem_ld16(taddr, r);
-}
-
-__global__ void __launch_bounds__(THREADS, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap mw0, const __grid_constant__ CUtensorMap mw1,
-                   const __grid_constant__ CUtensorMap mw2, const __grid_constant__ CUtensorMap mx,
-                   const TcParams p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 1];
-    __shared__ uint32_t tmem_base;
-    __shared__ volatile int abort_flag;
-    __shared__ int is_last;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int tile = blockIdx.x, seg = 0;
-    while (seg < p.n_seg - 1 && tile >= p.seg_tiles[seg]) {
-        tile -= p.seg_tiles[seg];
-        ++seg;
-    }
-    const CUtensorMap *mw = seg == 0 ? &mw0 : (seg == 1 ? &mw1 : &mw2);
-    const int row0 = tile * BM;
-    const int ntile = blockIdx.y, n0 = ntile * p.BN;
-    const int split = blockIdx.z;
-    const int kb0 = split * p.kb_per_split;
-    const int kb1 = min(p.kblocks, kb0 + p.kb_per_split);
-    const int nk = kb1 - kb0;
-    const int stages = p.stages;
-    const uint32_t b_bytes = (uint32_t)p.BN * BK * 2;
-
-    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t a_base = sbase, b_base = sbase + stages * A_BYTES;
-    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[MAX_STAGES]);
-    const uint32_t done = smem_u32(&bars[2 * MAX_STAGES]);
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(full0 + 8 * s, 1);
-            mbar_init(empty0 + 8 * s, 1);
-        }
-        mbar_init(done, 1);
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(mw) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&mx) : "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base)),
-                     "r"(p.tmem_cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            int issued = 0;
-            for (int i = 0; i < nk; ++i) {
-                const int s = i % stages;
-                const uint32_t ph = (uint32_t)(i / stages) & 1u;
-                if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, &abort_flag, p.status)) break;
-                mbar_expect_tx(full0 + 8 * s, A_BYTES + b_bytes);
-                tma_load_2d(a_base + s * A_BYTES, mw, (kb0 + i) * BK, row0, full0 + 8 * s);
-                tma_load_2d(b_base + s * b_bytes, &mx, (kb0 + i) * BK, n0, full0 + 8 * s);
-                issued = i + 1;
-            }
-            if (abort_flag) {
-                // let the copies still in flight land before the CTA exits
-                volatile int never = 0;
-                for (int i = (issued > stages ? issued - stages : 0); i < issued; ++i)
-                    mbar_wait(full0 + 8 * (i % stages), (uint32_t)(i / stages) & 1u, &never,
-                              p.status);
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc(p.BN);
-            for (int i = 0; i < nk; ++i) {
-                const int s = i % stages;
-                const uint32_t ph = (uint32_t)(i / stages) & 1u;
-                if (!mbar_wait(full0 + 8 * s, ph, &abort_flag, p.status)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t ad = smem_desc(a_base + s * A_BYTES);
-                const uint64_t bd = smem_desc(b_base + s * b_bytes);
-#pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    mma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (i | kk) != 0);
-                mma_commit(empty0 + 8 * s);
-            }
-            mma_commit(done);   // arrives once every MMA issued above has completed
-            // after an abort the epilogue may skip its wait: the tensor memory is
-            // freed only once every MMA issued here has completed
-            volatile int never = 0;
-            mbar_wait(done, 0, &never, p.status);
-        }
-        __syncwarp();
-    }
-
-    // ---- epilogue -----------------------------------------------------------
-    const bool ok = mbar_wait(done, 0, &abort_flag, p.status) && !abort_flag;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int row = warp * 32 + lane;
-    const int o_local = row0 + row;
-    const bool row_ok = o_local < p.seg_rows[seg];
-    const int o = p.seg_out[seg] + o_local;
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    const int M = p.M;
-
-    if (p.splits == 1) {
-        for (int c0 = 0; c0 < p.BN; c0 += 16) {
-            uint32_t r[16];
-            tmem_ld16(taddr + c0, r);
-            if (ok && row_ok) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int m = n0 + c0 + j;
-                    if (m < M) {
-                        float *y = p.Y + (size_t)m * p.ldy + o;
-                        const float v = __uint_as_float(r[j]);
-                        *y = p.epi == EPI_ADD ? *y + v : v;
-                    }
-                }
-            }
-        }
-    } else {
-        const int tile_id = blockIdx.x * p.n_tiles_n + ntile;
-        const size_t tile_elems = (size_t)p.BN * BM;
-        float *part = p.ws + ((size_t)tile_id * p.splits + split) * tile_elems;
-        for (int c0 = 0; c0 < p.BN; c0 += 16) {
-            uint32_t r[16];
-            tmem_ld16(taddr + c0, r);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) part[(size_t)(c0 + j) * BM + row] = __uint_as_float(r[j]);
-        }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int prev = atomicAdd(&p.counters[tile_id], 1);
-            is_last = prev == p.splits - 1;
-        }
-        __syncthreads();
-        if (is_last) {
-            __threadfence();
-            const float *tb = p.ws + (size_t)tile_id * p.splits * tile_elems;
-            for (int c = 0; c < p.BN; ++c) {
-                const int m = n0 + c;
-                if (m >= M) break;
-                float v = 0.f;
-                for (int s = 0; s < p.splits; ++s)
-                    v += __ldcg(tb + (size_t)s * tile_elems + (size_t)c * BM + row);
-                if (ok && row_ok) {
-                    float *y = p.Y + (size_t)m * p.ldy + o;
-                    *y = p.epi == EPI_ADD ? *y + v : v;
-                }
-            }
-            if (threadIdx.x == 0) p.counters[tile_id] = 0;
-        }
-    }
-
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 1) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(p.tmem_cols)
-                     : "memory");
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1066,6 +815,7 @@ struct CkParams {
     int seg_out[3];
     int M, kblocks, BN, n_tiles_n, splits, tmem_cols;
     int stages;             // ring depth (<= C_STAGES)
+    int n_acc, acc_stride;  // accumulators that take turns over the K-blocks (summed in the epilogue)
     int has_lo;             // X is a split pair: its lo plane comes through the second map
     const bf16 *wpacked;
     float *Y;
@@ -1378,7 +1128,9 @@ __device__ __forceinline__ void c_reduce_norm(const CkParams &p, const PartSrc &
     }
 }
 
-template <bool PAIR>
+// RAW: mw maps the caller's row-major weight, read only after the wait on the
+// previous kernel (which may have written it); otherwise the packed blocks.
+template <bool PAIR, bool RAW>
 __global__ void __launch_bounds__(C_THREADS)
     gemm_cluster_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mxl,
                         const __grid_constant__ CUtensorMap mw, const CkParams p) {
@@ -1466,7 +1218,7 @@ __global__ void __launch_bounds__(C_THREADS)
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&mx) : "memory");
             if (has_lo) asm volatile("prefetch.tensormap [%0];" ::"l"(&mxl) : "memory");
-            if (pair) asm volatile("prefetch.tensormap [%0];" ::"l"(&mw) : "memory");
+            if (pair || RAW) asm volatile("prefetch.tensormap [%0];" ::"l"(&mw) : "memory");
         }
         __syncwarp();
         const uint32_t on_expect = !pair || half == 0 ? on : 0u;
@@ -1477,11 +1229,13 @@ __global__ void __launch_bounds__(C_THREADS)
             if constexpr (pair)
                 w_tma_load_2d_pair(on, a_base + st * A_BYTES, &mw, 0, ((int)blockIdx.x * KB + kb0 + i) * BM,
                                    sig0 + 8 * st);
+            else if constexpr (RAW)
+                w_tma_load_2d(on, a_base + st * A_BYTES, &mw, (kb0 + i) * BK, row0, full0 + 8 * st);
             else
                 w_bulk_load(on, a_base + st * A_BYTES, wblk + (size_t)i * blk_elems, A_BYTES, full0 + 8 * st);
         };
         // weights first (they never depend on the previous kernel), then wait
-        const int n_pre = min(stages, nk);
+        const int n_pre = RAW ? 0 : min(stages, nk);
         for (int j = 0; j < n_pre; ++j) load_w(j, j);
         pdl_wait();
         if (lane == 0) stamp_min(p.stamp, 1);
@@ -1520,7 +1274,7 @@ __global__ void __launch_bounds__(C_THREADS)
         if (!pair || half == 0) {      // (pair: the even CTA issues for both)
             const uint32_t on = elect_one();
             const uint32_t idesc = instr_desc(BN, pair ? 2 * BM : BM);
-            int s = 0;
+            int s = 0, a = 0;
             uint32_t ph = 0;
             for (int i = 0; i < nk; ++i) {
                 if (pair ? !w_mbar_wait_cluster(full0 + 8 * s, ph, &abort_flag, p.status)
@@ -1530,23 +1284,24 @@ __global__ void __launch_bounds__(C_THREADS)
                 const uint64_t ad = smem_desc(a_base + s * A_BYTES);
                 const uint64_t bd = smem_desc(b_base + s * bs_bytes);
                 const uint64_t bl = smem_desc(b_base + s * bs_bytes + b_bytes);
-                const uint32_t more = i != 0;
+                const uint32_t more = i >= p.n_acc, acc = tmem + a * p.acc_stride;
+                if (++a == p.n_acc) a = 0;
                 if (has_lo) {
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk) {
                         if constexpr (pair) {
-                            w_mma_bf16_pair(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
-                            w_mma_bf16_pair(on, tmem, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                            w_mma_bf16_pair(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                            w_mma_bf16_pair(on, acc, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
                         } else {
-                            w_mma_bf16(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
-                            w_mma_bf16(on, tmem, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
+                            w_mma_bf16(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                            w_mma_bf16(on, acc, ad + 2 * kk, bl + 2 * kk, idesc, 1u);
                         }
                     }
                 } else {
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk) {
-                        if constexpr (pair) w_mma_bf16_pair(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
-                        else w_mma_bf16(on, tmem, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                        if constexpr (pair) w_mma_bf16_pair(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
+                        else w_mma_bf16(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
                     }
                 }
                 if constexpr (pair) w_mma_commit_pair(on, empty0 + 8 * s, pair_mask);
@@ -1558,7 +1313,7 @@ __global__ void __launch_bounds__(C_THREADS)
             }
             if constexpr (pair) w_mma_commit_pair(on, done, pair_mask);
             else w_mma_commit(on, done);
-            volatile int never = 0;     // (as gemm_tc_kernel: no MMA outlives the CTA's TMEM)
+            volatile int never = 0;     // (no MMA outlives the CTA's TMEM)
             mbar_wait(done, 0, &never, p.status);
         }
         __syncwarp();
@@ -1599,11 +1354,22 @@ __global__ void __launch_bounds__(C_THREADS)
     const int o_base = p.seg_out[seg] + row0;
     const bool paired = p.epi >= EPI_SWIGLU;
     const bool norm_out = p.nout.ss != nullptr;
+    // columns [g0, g0 + gw) of the tile, the accumulators that took a K-block added in order
+    const int n_acc = min(p.n_acc, nk);
+    auto acc_cols = [&](int g0, uint32_t *r, int gw) {
+        tmem_ld_cols(taddr + g0, r, gw);
+        for (int q = 1; q < n_acc; ++q) {
+            uint32_t t[32];
+            tmem_ld_cols(taddr + q * p.acc_stride + g0, t, gw);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(t[j]));
+        }
+    };
     if (S == 1 && !paired && !norm_out) {
         for (int g0 = 0; g0 < BN; g0 += 32) {
             const int gw = min(32, BN - g0);
             uint32_t r[32];
-            tmem_ld_cols(taddr + g0, r, gw);
+            acc_cols(g0, r, gw);
             if (ok && row < rows_here) {
                 float *yb = p.Y + (size_t)(n0 + g0) * p.ldy + o_base + row;
                 const int mlim = p.M - (n0 + g0);
@@ -1628,7 +1394,7 @@ __global__ void __launch_bounds__(C_THREADS)
         for (int g0 = 0; g0 < BN; g0 += 32) {
             const int gw = min(32, BN - g0);
             uint32_t r[32];
-            tmem_ld_cols(taddr + g0, r, gw);
+            acc_cols(g0, r, gw);
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 if (j < gw) part[(g0 + j) * BM + row] = __uint_as_float(r[j]);
@@ -1905,8 +1671,11 @@ __global__ void stamp_collect_kernel(unsigned long long *st, int n, int xn, doub
 }
 
 struct GemmPlan {
-    float *ws = nullptr;
+    float *ws = nullptr;        // stream-K pieces and their tickets
     int *counters = nullptr;
+    size_t ws_bytes = WS_BYTES;
+    int n_counters = N_COUNTERS;
+    bool clear_counters = false;    // tickets are cleared before each launch that uses them
     int num_sms = 148;
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     std::unordered_map<MapKey, CUtensorMap, MapKeyHash> maps;
@@ -2099,26 +1868,29 @@ GemmProfile gemm_profile_read(GemmPlan *p) {
     return r;
 }
 
-static const CUtensorMap *get_map(GemmPlan *p, const void *ptr, long rows, long cols, long ld,
-                                  long box_rows, int *status) {
-    MapKey key{ptr, rows, cols, ld, box_rows};
-    auto it = p->maps.find(key);
-    if (it != p->maps.end()) return &it->second;
-    CUtensorMap m;
-    memset(&m, 0, sizeof m);
+// Tensor map over rows of `cols` bf16, boxes of 64 columns x box_rows rows in the
+// 128-byte swizzle (columns and rows past the end read as zeros).
+static bool make_map(GemmPlan *p, const void *ptr, long rows, long cols, long ld, long box_rows, CUtensorMap *m) {
+    memset(m, 0, sizeof *m);
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
     cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = p->encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims,
-                           strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        fprintf(stderr, "msd: cuTensorMapEncodeTiled failed (%d) rows=%ld cols=%ld ld=%ld\n", (int)r,
-                rows, cols, ld);
-        return nullptr;
-    }
+    const CUresult r = p->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box,
+                                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS)
+        fprintf(stderr, "msd: cuTensorMapEncodeTiled failed (%d) rows=%ld cols=%ld ld=%ld\n", (int)r, rows, cols, ld);
+    return r == CUDA_SUCCESS;
+}
+
+// The map of a context buffer, cached.
+static const CUtensorMap *get_map(GemmPlan *p, const void *ptr, long rows, long cols, long ld, long box_rows) {
+    MapKey key{ptr, rows, cols, ld, box_rows};
+    auto it = p->maps.find(key);
+    if (it != p->maps.end()) return &it->second;
+    CUtensorMap m;
+    if (!make_map(p, ptr, rows, cols, ld, box_rows, &m)) return nullptr;
     return &p->maps.emplace(key, m).first->second;
 }
 
@@ -2175,7 +1947,7 @@ void gemm_pack_glu(const void *gate, const void *up, int F, int K, void *dst, cu
 // shared memory (token tiles of up to 64 split rows), otherwise one with up to
 // four stages; the split count keeps every split's partial slices within the
 // stage memory they reuse.
-static void gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
+static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
                          int tiles, int BN, int kblocks, float *Y, int ldy, int epi, int *status,
                          cudaStream_t s, int O, const GemmFused *fx = nullptr,
                          const GemmNorm *nout = nullptr, const GemmNorm *nin = nullptr) {
@@ -2200,13 +1972,21 @@ static void gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     stages = std::max(2, std::min(stages, C_STAGES));
     int S = (per_sm * p->num_sms) / tiles;
     S = std::max(1, std::min(S, 8));
+    // One-plane products (msd_linear): the accumulators truncate, so a chain of at
+    // most 16 K-blocks each -- as many of them as 256 TMEM columns hold take turns,
+    // and K is split further where that is not enough (17 x 4096 x 11008: 1.1e-6
+    // relative in chains of 22, below 0.8e-6 in chains of 3)
+    int acc_stride = 32;
+    while (acc_stride < BN) acc_stride <<= 1;
+    const int n_acc = nb == 1 ? 256 / acc_stride : 1;
+    if (nb == 1) S = std::max(S, std::min(8, (kblocks + 16 * n_acc - 1) / (16 * n_acc)));
     while (S > 1 && kblocks / S < 2) --S;
     // own partial [BN][128] fp32 plus the other ranks' slices of this rank's columns
     while (S > 1 && (size_t)BN * BM * 4 + (size_t)(S - 1) * ((BN + S - 1) / S) * BM * 4 > stages * stage) --S;
     // Two-SM tiles for unsplit launches whose token stage is as large as the
     // weight block (split token rows, 32 or more): each CTA of a pair holds
     // half the token columns, so the ring gets a fourth stage.
-    const bool pair = S == 1 && nb == 2 && BN >= 32 && tiles % 2 == 0 && per_sm == 2;
+    const bool pair = S == 1 && nb == 2 && BN >= 32 && tiles % 2 == 0 && per_sm == 2 && W.packed;
     const int BNs = pair ? BN / 2 : BN;
     if (pair) {
         stage = A_BYTES + (size_t)nb * BNs * BK * 2;
@@ -2219,23 +1999,36 @@ static void gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     ck.splits = S;
     ck.stages = stages;
     ck.has_lo = X_lo ? 1 : 0;
-    ck.tmem_cols = BN <= 32 ? 32 : (BN <= 64 ? 64 : 128);
+    ck.n_acc = n_acc;
+    ck.acc_stride = acc_stride;
+    ck.tmem_cols = n_acc * acc_stride;
     ck.wpacked = static_cast<const bf16 *>(W.packed);
     ck.Y = Y;
     ck.ldy = ldy;
     ck.epi = epi;
     ck.status = status;
-    const CUtensorMap *mx = get_map(p, X, M, K, ldx, BNs, status);
+    // a caller's row-major weight and rows: maps of this call alone
+    const bool raw = !W.packed;
+    CUtensorMap rawx, raww;
+    const CUtensorMap *mx = raw ? (make_map(p, X, M, K, ldx, BNs, &rawx) ? &rawx : nullptr)
+                                : get_map(p, X, M, K, ldx, BNs);
     ck.stamp = stamp_slot(p);
-    const CUtensorMap *mxl = X_lo ? get_map(p, X_lo, M, K, ldx, BNs, status) : mx;
-    const CUtensorMap *mw = pair ? get_wmap(p, W.packed, (long)tiles * kblocks * BM) : mx;
-    if (!mx || !mxl || !mw) return;
+    const CUtensorMap *mxl = X_lo ? get_map(p, X_lo, M, K, ldx, BNs) : mx;
+    const CUtensorMap *mw = raw    ? (make_map(p, W.w[0], O, K, K, BM, &raww) ? &raww : nullptr)
+                            : pair ? get_wmap(p, W.packed, (long)tiles * kblocks * BM)
+                                   : mx;
+    if (!mx || !mxl || !mw) {
+        flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
+        return false;
+    }
     const size_t smem = 1024 + (size_t)stages * stage;
     if (!p->cluster_attr_set) {
-        cudaFuncSetAttribute(gemm_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(1024 + FULL_SM));
-        cudaFuncSetAttribute(gemm_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(1024 + FULL_SM));
+        auto set = [](const void *f) {
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(1024 + FULL_SM));
+        };
+        set((const void *)gemm_cluster_kernel<false, false>);
+        set((const void *)gemm_cluster_kernel<true, false>);
+        set((const void *)gemm_cluster_kernel<false, true>);
         p->cluster_attr_set = true;
     }
     const bool prof = p->profile;
@@ -2262,8 +2055,10 @@ static void gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     at[1].val.clusterDim.z = (unsigned)S;
     lc.attrs = at;
     lc.numAttrs = 2;
-    if ((pair ? cudaLaunchKernelEx(&lc, gemm_cluster_kernel<true>, *mx, *mxl, *mw, ck)
-              : cudaLaunchKernelEx(&lc, gemm_cluster_kernel<false>, *mx, *mxl, *mw, ck)) != cudaSuccess) {
+    const auto kernel = raw ? gemm_cluster_kernel<false, true>
+                            : (pair ? gemm_cluster_kernel<true, false> : gemm_cluster_kernel<false, false>);
+    const bool launched = cudaLaunchKernelEx(&lc, kernel, *mx, *mxl, *mw, ck) == cudaSuccess;
+    if (!launched) {
         cudaGetLastError();
         flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
         fprintf(stderr, "msd: cluster GEMM launch failed (M=%d K=%d O=%d S=%d)\n", M, K, O, S);
@@ -2281,12 +2076,14 @@ static void gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     for (int z = 0; z < S; ++z)
         pre += (double)tiles * std::min(stages, (int)((long long)(z + 1) * kblocks / S - (long long)z * kblocks / S)) *
                A_BYTES;
+    if (raw) pre = 0.0;
     account(p, wb, wb + (double)M * K * 2.0 * nb + yb, M, O, K, nb, std::min(pre, wb));
+    return launched;
 }
 
 // The persistent stream-K GEMM (many token rows). fx: EPI_SWIGLU writes
 // act = silu(g) * u from glu-packed gate/up weights instead of Y.
-static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
+static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
                          int O, float *Y, int ldy, int epi, const GemmFused *fx, int *status, cudaStream_t s);
 
 bool gemm_bf16_fused(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
@@ -2298,7 +2095,7 @@ bool gemm_bf16_fused(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int 
         // epilogue (RoPE/KV stays a separate kernel there: fused, its
         // per-column gathers outlasted the main loop, measured slower)
         if (fx.epi != EPI_SWIGLU || norm_in || !fx.act) return false;
-        gemm_persist(p, X, X_lo, ldx, M, K, W, O, nullptr, 0, EPI_SWIGLU, &fx, status, s);
+        gemm_persist(p, X, X_lo, ldx, M, K, W, O, nullptr, 0, EPI_SWIGLU, &fx, status, s);   // (or flags the status)
         return true;
     }
     if (fx.epi == EPI_ROPE_KV &&
@@ -2322,7 +2119,8 @@ bool gemm_bf16(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int
     if (norm_out && (M > 128 || !W.packed || W.nseg != 1 || !norm_out->ss || !norm_out->xg || !norm_out->g ||
                      (O + BM - 1) / BM > norm_out->ld || O % 4 || ldy % 4))
         return false;
-    if (M <= 128 && W.packed) {
+    if (!W.packed && W.nseg != 1) return false;
+    if (M <= 128) {
         int tiles = 0;
         for (int i = 0; i < W.nseg; ++i) tiles += (W.rows[i] + BM - 1) / BM;
         gemm_cluster(p, X, X_lo, ldx, M, K, W, tiles, ((M + 15) / 16) * 16, (K + BK - 1) / BK, Y, ldy, epi,
@@ -2350,11 +2148,12 @@ constexpr int P_STAGES = 6;
 // even, but the pieces' round trip through the workspace then costs 330 BN
 // where every tile is cut (O at 640 rows, 224 columns: 68 us against 40 in whole
 // tiles), about 180 BN where whole tiles follow to hide part of it.
-// A one-plane product (msd_linear) accumulates at most 40 K-blocks of a whole
+// A one-plane product (msd_linear) accumulates at most 24 K-blocks of a whole
 // tile in tensor memory before it adds them to Y: the accumulators truncate, so
 // the error grows with the chain (4096-long products: 2.2e-6 relative in pieces
-// of 40 blocks, 4.4e-6 in one of 64).
-static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int pairs) {
+// of 32 to 40 blocks, 4.4e-6 in one of 64).
+static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int pairs, size_t ws_bytes,
+                                  int n_counters) {
     const int kblocks = (K + BK - 1) / BK, wt = (tiles + 1) / 2;
     PersistShape best{};
     double best_cost = 1e300;
@@ -2365,7 +2164,7 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
         const double tk = std::max(2.08 * nb * BN, 420.0 + 0.8 * nb * BN);
         // at least 4 K-blocks a pair
         const long long G = std::max<long long>(1, std::min<long long>(pairs, T * kblocks / 4));
-        const int chunk = nb == 1 && !glu ? (kblocks + (kblocks + 39) / 40 - 1) / ((kblocks + 39) / 40) : kblocks;
+        const int chunk = nb == 1 && !glu ? (kblocks + (kblocks + 23) / 24 - 1) / ((kblocks + 23) / 24) : kblocks;
         PersistShape g{BN, nt, (int)G, (int)T, 0, (int)((T + G - 1) / G), chunk};
         double cost = g.dp_rounds * tk * kblocks;
         int rounds = (int)(T / G), T_sk = (int)(T - rounds * G);
@@ -2378,7 +2177,9 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
                 T_sk += (int)G;
             }
             const double sk = T * tk * kblocks / G + (rounds == 0 ? 330.0 : 180.0) * BN;
-            if (sk < cost && (long long)T_sk * kblocks >= G) {      // (every pair holds a unit)
+            // (every pair holds a unit, and the pieces and tickets have their place)
+            if (sk < cost && (long long)T_sk * kblocks >= G && 16ull * G * BN * BM <= ws_bytes &&
+                2LL * T_sk <= n_counters) {
                 g.T_sk = T_sk;
                 g.dp_rounds = rounds;
                 cost = sk;
@@ -2392,7 +2193,7 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
     return best;
 }
 
-static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
+static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
                          int O, float *Y, int ldy, int epi, const GemmFused *fx, int *status, cudaStream_t s) {
     const bool glu = fx && fx->epi == EPI_SWIGLU;
     PkParams pk;
@@ -2407,7 +2208,7 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         tiles += pk.seg_tiles[i];
     }
     const int nb = X_lo ? 2 : 1;
-    const PersistShape g = persist_shape(tiles, M, K, nb, glu, p->num_sms / 2);
+    const PersistShape g = persist_shape(tiles, M, K, nb, glu, p->num_sms / 2, p->ws_bytes, p->n_counters);
     const int BN = g.BN, nt = g.nt, kblocks = (K + BK - 1) / BK, G = g.G;
     // the fused SwiGLU epilogue takes 16 KB of staging from the ring's budget
     const uint32_t stg_bytes = glu ? 32u * BM * 4u : 0u;
@@ -2416,12 +2217,6 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     const size_t smem = 1024 + (size_t)stages * stage_bytes + stg_bytes;
     const long long units = (long long)g.T_sk * kblocks;
     const long long all_units = (long long)g.T_all * kblocks;
-    const size_t ws_need = 4ull * G * BN * BM * sizeof(float);
-    if (ws_need > WS_BYTES || 2ll * g.T_sk > N_COUNTERS) {
-        flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
-        fprintf(stderr, "msd: GEMM shape M=%d K=%d O=%d exceeds the workspace\n", M, K, O);
-        return;
-    }
     int acc = 32;
     while (acc < BN) acc <<= 1;
     pk.M = M;
@@ -2452,21 +2247,28 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         pk.lo = fx->lo;
         pk.stg_off = (uint32_t)(1024 + (size_t)stages * stage_bytes);
     }
-    if (!W.packed) {
+    const bool raw = !W.packed;
+    CUtensorMap rawx, raww;
+    const CUtensorMap *mx = raw ? (make_map(p, X, M, K, ldx, BN / 2, &rawx) ? &rawx : nullptr)
+                                : get_map(p, X, M, K, ldx, BN / 2);
+    const CUtensorMap *mxl = X_lo ? get_map(p, X_lo, M, K, ldx, BN / 2) : mx;
+    const CUtensorMap *mw = raw ? (make_map(p, W.w[0], O, K, K, BM, &raww) ? &raww : nullptr)
+                                : get_wmap(p, W.packed, (long)tiles * kblocks * BM);
+    if (!mx || !mxl || !mw) {
         flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
-        fprintf(stderr, "msd: GEMM weights were not packed\n");
-        return;
+        return false;
     }
-    const CUtensorMap *mx = get_map(p, X, M, K, ldx, BN / 2, status);
-    const CUtensorMap *mxl = X_lo ? get_map(p, X_lo, M, K, ldx, BN / 2, status) : mx;
-    const CUtensorMap *mw = get_wmap(p, W.packed, (long)tiles * kblocks * BM);
-    if (!mx || !mxl || !mw) return;
     pk.stamp = stamp_slot(p);
     if (!p->smem_set) {
         cudaFuncSetAttribute(gemm_persist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(P_BUDGET + 1024));
+        cudaFuncSetAttribute(gemm_persist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(P_BUDGET + 1024));
         p->smem_set = true;
     }
+    if (p->clear_counters && g.T_sk > 0 &&
+        cudaMemsetAsync(p->counters, 0, sizeof(int) * 2 * g.T_sk, s) != cudaSuccess)
+        return false;
     const bool prof = p->profile;
     if (prof) {
         while (p->ev.size() < p->ev_used + 2) {
@@ -2494,7 +2296,9 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     at[1].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = 2;
-    if (cudaLaunchKernelEx(&lc, gemm_persist_kernel<false>, *mx, *mxl, *mw, pk) != cudaSuccess) {
+    const auto kernel = raw ? gemm_persist_kernel<true> : gemm_persist_kernel<false>;
+    const bool launched = cudaLaunchKernelEx(&lc, kernel, *mx, *mxl, *mw, pk) == cudaSuccess;
+    if (!launched) {
         cudaGetLastError();
         flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
         fprintf(stderr, "msd: persistent GEMM launch failed (M=%d K=%d O=%d)\n", M, K, O);
@@ -2507,7 +2311,8 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     const double wb = (double)O * K * 2.0;
     account(p, wb, wb + (double)M * K * 2.0 * nb +
                        (glu ? (double)M * fx->F * 2.0 * nb : (double)M * O * 4.0 * (epi == EPI_ADD ? 2 : 1)),
-            M, O, K, nb, std::min(wb, 2.0 * G * std::min<long long>(stages, all_units / G) * A_BYTES));
+            M, O, K, nb, raw ? 0.0 : std::min(wb, 2.0 * G * std::min<long long>(stages, all_units / G) * A_BYTES));
+    return launched;
 }
 
 }  // namespace msd
@@ -2523,15 +2328,20 @@ static void gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
 // by every GPU that loads it until the process exits.
 //
 // Layout of the array: a status word (padded to 256 bytes), NOALLOC_COUNTERS
-// int tile tickets, then the fp32 split-K partials (NOALLOC_PARTIAL_BYTES). In
-// host code the array's name is only a host-side stand-in; the device address
+// int tile tickets, then the fp32 pieces of stream-K tiles (NOALLOC_PARTIAL_BYTES).
+// In host code the array's name is only a host-side stand-in; the device address
 // comes from cudaGetSymbolAddress, taken once per device (with that device
 // current) on the first call made on it. Every call shares the array and it
 // keeps the last call's contents: the tickets are cleared on the caller's
 // stream before each launch that uses them, and calls that overlap on the GPU
-// race on the array. The split-K choice is limited to what the array holds, so
-// a shape that would split further on the context GEMM runs with fewer splits
-// (none at worst) instead of being refused.
+// race on the array. A product of up to 128 rows splits K over a cluster and
+// needs none of it; with more rows, a shape whose pieces would not fit runs in
+// whole tiles.
+// The status word that kernels set is a word of this library's own host memory,
+// page-locked on the first call and written by the GPU in place, so that a call
+// reads it after a stream synchronisation alone (a copy back to pageable memory
+// took most of a small call: 66 us for 17 x 4096 x 11008 before, with the rows'
+// kernel at 30); where it cannot be mapped, the array's word is copied back.
 // ---------------------------------------------------------------------------
 namespace msd {
 namespace {
@@ -2540,7 +2350,6 @@ constexpr int NOALLOC_COUNTERS = 4096;
 constexpr size_t NOALLOC_PARTIAL_BYTES = 16ull << 20;
 constexpr size_t NOALLOC_BYTES = NOALLOC_STATUS_BYTES + NOALLOC_COUNTERS * sizeof(int) + NOALLOC_PARTIAL_BYTES;
 constexpr int NOALLOC_MAX_DEVICES = 64;
-constexpr size_t NOALLOC_MAX_MAPS = 256;   // cached weight tensor maps per process
 constexpr long NOALLOC_MAX_ROWS = 65535L * 256;   // token-tile grid dimension limit
 }  // namespace
 
@@ -2550,12 +2359,14 @@ namespace {
 struct NoAllocDevice {
     bool ready = false;
     unsigned char *scratch = nullptr;   // device address of g_noalloc_scratch
-    int num_sms = 0;
-    int status_host = 0;                // last value read back from the status word
+    GemmPlan *plan = nullptr;           // maps nothing and owns nothing: scratch is the array's
+    int *status = nullptr;              // device address of the status word
+    volatile int *host = nullptr;       // the same word in host memory (null: copied back)
+    int status_copy = 0;
 };
 std::mutex g_noalloc_mu;
 NoAllocDevice g_noalloc_dev[NOALLOC_MAX_DEVICES];
-GemmPlan g_noalloc_maps;                // host-side tensor-map cache only (no device memory)
+alignas(4096) unsigned char g_noalloc_host[NOALLOC_MAX_DEVICES * 64];   // one cache line per device
 
 // One-time set-up of the current device (caller holds g_noalloc_mu).
 bool noalloc_setup(int dev) {
@@ -2563,36 +2374,47 @@ bool noalloc_setup(int dev) {
     if (d.ready) return true;
     void *ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) return false;
-    if (cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
-    if (cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024 + 1024) !=
-        cudaSuccess)
+    if (!d.plan) d.plan = new GemmPlan();
+    GemmPlan *p = d.plan;
+    if (cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    cudaDriverEntryPointQueryResult q;
+    void *fn = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess || !fn)
         return false;
-    if (!g_noalloc_maps.encode) {
-        cudaDriverEntryPointQueryResult q;
-        void *fn = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess || !fn)
-            return false;
-        g_noalloc_maps.encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
+    p->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
     d.scratch = static_cast<unsigned char *>(ptr);
+    p->counters = reinterpret_cast<int *>(d.scratch + NOALLOC_STATUS_BYTES);
+    p->ws = reinterpret_cast<float *>(d.scratch + NOALLOC_STATUS_BYTES + NOALLOC_COUNTERS * sizeof(int));
+    p->ws_bytes = NOALLOC_PARTIAL_BYTES;
+    p->n_counters = NOALLOC_COUNTERS;
+    p->clear_counters = true;
+    d.status = reinterpret_cast<int *>(d.scratch);
+    void *mapped = nullptr;
+    const cudaError_t e = cudaHostRegister(g_noalloc_host, sizeof g_noalloc_host,
+                                           cudaHostRegisterMapped | cudaHostRegisterPortable);
+    if ((e == cudaSuccess || e == cudaErrorHostMemoryAlreadyRegistered) &&
+        cudaHostGetDevicePointer(&mapped, g_noalloc_host, 0) == cudaSuccess && mapped) {
+        d.status = reinterpret_cast<int *>(static_cast<unsigned char *>(mapped) + 64 * dev);
+        d.host = reinterpret_cast<volatile int *>(g_noalloc_host + 64 * dev);
+    }
+    cudaGetLastError();
     d.ready = true;
     return true;
 }
 
-// Tensor map of an activation operand: encoded on every call (a host-only
-// computation), so the cache holds weight maps alone.
-bool encode_x_map(const void *x, long rows, long cols, long ld, long box_rows, CUtensorMap *m) {
-    memset(m, 0, sizeof *m);
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return g_noalloc_maps.encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(x), dims, strides, box,
-                                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
+// Waits for the work queued before on `s`, then takes (and clears) the status word.
+cudaError_t noalloc_take_status(NoAllocDevice &d, cudaStream_t s, int *code) {
+    if (!d.host) {
+        cudaError_t e = cudaMemcpyAsync(&d.status_copy, d.status, sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        *code = e == cudaSuccess ? d.status_copy : 0;
+        return e == cudaSuccess && *code ? cudaMemsetAsync(d.status, 0, sizeof(int), s) : e;
+    }
+    const cudaError_t e = cudaStreamSynchronize(s);
+    *code = e == cudaSuccess ? *d.host : 0;
+    if (*code) *d.host = 0;
+    return e;
 }
 }  // namespace
 
@@ -2603,7 +2425,7 @@ int *noalloc_status_word() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NOALLOC_MAX_DEVICES) return nullptr;
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
     if (!noalloc_setup(dev)) return nullptr;
-    return reinterpret_cast<int *>(g_noalloc_dev[dev].scratch);
+    return g_noalloc_dev[dev].status;
 }
 
 // Test hook of the bounded waits: one CTA waits on an mbarrier that nothing
@@ -2644,76 +2466,18 @@ extern "C" msd_status msd_linear_noalloc(const void *x, int32_t ldx, int32_t m, 
     if (!noalloc_setup(dev)) return CUDA_ERR;
     NoAllocDevice &d = g_noalloc_dev[dev];
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int *status = reinterpret_cast<int *>(d.scratch);
     // The status word left by earlier launches on this device (a bounded wait
-    // that ran out): read back into pageable host memory, so the copy returns
-    // once the work queued before it on `stream` has finished; a set word is
-    // cleared and reported once.
-    if (cudaMemcpyAsync(&d.status_host, status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return CUDA_ERR;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return CUDA_ERR;
-    if (d.status_host != 0) {
-        d.status_host = 0;
-        if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) return CUDA_ERR;
-        return DEVICE;
-    }
-    // The same tile shape and stages as the context GEMM; the split-K choice is
-    // limited to what the array holds.
-    const int M = m, K = k, O = o;
-    const int tiles = (O + BM - 1) / BM;
-    const int nt = (M + 255) / 256;
-    int BN = (M + nt - 1) / nt;
-    BN = ((BN + 15) / 16) * 16;
-    const int kblocks = (K + BK - 1) / BK;
-    const uint32_t stage_bytes = A_BYTES + (uint32_t)BN * BK * 2;
-    const int ctas_per_sm = BN <= 128 ? 2 : 1;
-    int stages = (int)((ctas_per_sm == 2 ? 100u * 1024u : 200u * 1024u) / stage_bytes);
-    stages = stages < 2 ? 2 : (stages > MAX_STAGES ? MAX_STAGES : stages);
-    const size_t smem = 1024 + (size_t)stages * stage_bytes;
-    const long base = (long)tiles * nt;
-    const long slots = (long)d.num_sms * ctas_per_sm;
-    const size_t tile_bytes = (size_t)BN * BM * sizeof(float);
-    int best_s = 1;
-    double best = 1e30;
-    for (int sp = 1; sp <= 16 && sp <= kblocks; ++sp) {
-        const int kps = (kblocks + sp - 1) / sp;
-        const int se = (kblocks + kps - 1) / kps;
-        if (se > 1 && ((size_t)base * se * tile_bytes > NOALLOC_PARTIAL_BYTES || base > NOALLOC_COUNTERS))
-            continue;
-        const long waves = (base * se + slots - 1) / slots;
-        const double cost = (double)waves * kps + (se > 1 ? 2.0 : 0.0);
-        if (cost < best - 1e-9) { best = cost; best_s = se; }
-    }
-    const int kps = (kblocks + best_s - 1) / best_s;
-    const int splits = (kblocks + kps - 1) / kps;
-
-    TcParams tp;
-    memset(&tp, 0, sizeof tp);
-    tp.n_seg = 1;
-    tp.seg_tiles[0] = tiles;
-    tp.seg_rows[0] = O;
-    tp.seg_out[0] = 0;
-    tp.M = M;
-    tp.kblocks = kblocks;
-    tp.splits = splits;
-    tp.kb_per_split = kps;
-    tp.BN = BN;
-    tp.n_tiles_n = nt;
-    tp.stages = stages;
-    tp.tmem_cols = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
-    tp.Y = y;
-    tp.ldy = ldy;
-    tp.epi = accumulate ? EPI_ADD : EPI_STORE;
-    tp.counters = reinterpret_cast<int *>(d.scratch + NOALLOC_STATUS_BYTES);
-    tp.ws = reinterpret_cast<float *>(d.scratch + NOALLOC_STATUS_BYTES + NOALLOC_COUNTERS * sizeof(int));
-    tp.status = status;
-    if (g_noalloc_maps.maps.size() >= NOALLOC_MAX_MAPS) g_noalloc_maps.maps.clear();
-    const CUtensorMap *mw = get_map(&g_noalloc_maps, w, O, K, K, BM, nullptr);
-    CUtensorMap mx;
-    if (!mw || !encode_x_map(x, M, K, ldx, BN, &mx)) return INVALID;
-    if (splits > 1 && cudaMemsetAsync(tp.counters, 0, sizeof(int) * base, s) != cudaSuccess)
-        return CUDA_ERR;
-    gemm_tc_kernel<<<dim3(tiles, nt, splits), THREADS, smem, s>>>(*mw, *mw, *mw, mx, tp);
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? OK : CUDA_ERR;
+    // that ran out), once the work queued before on `stream` has finished; a set
+    // word is cleared and reported once.
+    int code = 0;
+    if (noalloc_take_status(d, s, &code) != cudaSuccess) return CUDA_ERR;
+    if (code != 0) return DEVICE;
+    if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w)) & 15) return INVALID;
+    const GemmW W{{w, nullptr, nullptr}, {o, 0, 0}, 1, nullptr};
+    const bf16 *X = static_cast<const bf16 *>(x);
+    const int epi = accumulate ? EPI_ADD : EPI_STORE;
+    const bool ok = m <= 128 ? gemm_cluster(d.plan, X, nullptr, ldx, m, k, W, (o + BM - 1) / BM, (m + 15) / 16 * 16,
+                                            (k + BK - 1) / BK, y, ldy, epi, d.status, s, o)
+                             : gemm_persist(d.plan, X, nullptr, ldx, m, k, W, o, y, ldy, epi, nullptr, d.status, s);
+    return ok && cudaGetLastError() == cudaSuccess ? OK : CUDA_ERR;
 }

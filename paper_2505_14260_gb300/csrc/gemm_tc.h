@@ -19,6 +19,8 @@ void gemm_plan_destroy(GemmPlan *p);
 // norm_out (nullable, decode shapes M <= 128 with packed W only): the
 // producer side of a folded RMSNorm (GemmNorm below); returns false (nothing
 // launched) when it is given for a shape off the decode path.
+// W is packed (below), or one row-major segment (packed null): then X, X's rows
+// and W are the caller's, 16-byte aligned.
 bool gemm_bf16(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W, int O,
                float *Y, int ldy, int epi, int *status, cudaStream_t s, const GemmNorm *norm_out = nullptr);
 

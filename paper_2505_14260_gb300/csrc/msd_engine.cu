@@ -78,8 +78,6 @@ struct msd_ctx {
     std::vector<LayerPack> lpack;
     LayerPack dpack;
     const void *pk_lm = nullptr, *pk_fc = nullptr;
-    void *pk_scratch = nullptr;     // msd_linear: its weight, packed per call
-    size_t pk_scratch_bytes = 0;
     std::vector<void *> allocs;
     std::vector<long> L_bound;
     bool prefilled = false;
@@ -912,7 +910,6 @@ msd_status msd_destroy(msd_ctx *c) {
     if (c->status_ev) MSD_TEARDOWN(cudaEventDestroy(c->status_ev));
     if (c->gplan) gemm_plan_destroy(c->gplan);
     if (c->aplan) attn_tc_plan_destroy(c->aplan);
-    if (c->pk_scratch) MSD_TEARDOWN(cudaFree(c->pk_scratch));
     for (auto &g : c->graphs)
         if (g.exec) MSD_TEARDOWN(cudaGraphExecDestroy(g.exec));
     if (c->cap_stream) {
@@ -1199,25 +1196,13 @@ msd_status msd_linear(msd_ctx *c, const void *x, int32_t ldx, int32_t m, int32_t
         return fail(c, MSD_ERR_CUDA, "a CUDA error was pending before the call");
     if (!x || !w || !y || m <= 0 || k <= 0 || o <= 0 || ldx < k || ldy < o)
         return fail(c, MSD_ERR_INVALID, "bad msd_linear arguments");
-    if (c->cfg.dtype == MSD_BF16 && (ldx % 8 || k % 8))
+    if (c->cfg.dtype == MSD_BF16 &&
+        (ldx % 8 || k % 8 || ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w)) & 15)))
         return fail(c, MSD_ERR_INVALID, "bf16 rows must be 16-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     GemmW W = one(w, o);
     const int epi = accumulate ? EPI_ADD : EPI_STORE;
     if (c->cfg.dtype == MSD_BF16) {
-        // pack w into the context's scratch (grown on demand), then the GEMM
-        const size_t need = gemm_pack_bytes(W, k);
-        if (need > c->pk_scratch_bytes) {
-            CU(cudaStreamSynchronize(s));
-            if (c->pk_scratch) CU(cudaFree(c->pk_scratch));
-            c->pk_scratch = nullptr;
-            c->pk_scratch_bytes = 0;
-            if (cudaMalloc(&c->pk_scratch, need) != cudaSuccess)
-                return fail(c, MSD_ERR_OOM, "msd_linear: packing scratch");
-            c->pk_scratch_bytes = need;
-        }
-        gemm_pack(W, k, c->pk_scratch, s);
-        W.packed = c->pk_scratch;
         gemm<bf16>(c, static_cast<const bf16 *>(x), ldx, m, k, W, o, y, ldy, epi, s, false);
     } else
         gemm<float>(c, static_cast<const float *>(x), ldx, m, k, W, o, y, ldy, epi, s);
