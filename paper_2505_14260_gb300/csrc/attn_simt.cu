@@ -300,10 +300,8 @@ cudaError_t launch_as(AsArgs p, int num_sms, cudaStream_t s) {
     const int row_tiles = a.R / p.rows_per_req * p.tiles_per_req;
     // splits while they fit one wave of CTAs: a function of the launch's shape
     const long base = (long)row_tiles * a.nh;
-    p.nsplit = (int)std::max<long>(1, std::min<long>(AS_MAX_SPLITS, num_sms / base));
-    const cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel<HD, QR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               AsLay<HD, QR>::SMEM);
-    if (e != cudaSuccess) return e;
+    p.nsplit = (int)std::max<long>(
+        1, std::min<long>(std::min<long>(AS_MAX_SPLITS, (a.cache_slots + AS_KT - 1) / AS_KT), num_sms / base));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)a.nh, (unsigned)row_tiles, (unsigned)p.nsplit);
     lc.blockDim = dim3(AS_THREADS);
@@ -319,15 +317,19 @@ cudaError_t launch_as(AsArgs p, int num_sms, cudaStream_t s) {
     return cudaLaunchKernelEx(&lc, attn_simt_kernel<HD, QR>, (const AsArgs)p);
 }
 
+template <int HD, int QR>
+bool set_as() {
+    return cudaFuncSetAttribute(attn_simt_kernel<HD, QR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                AsLay<HD, QR>::SMEM) == cudaSuccess;
+}
+
 }  // namespace
 
-bool launch_attention(const AttnArgs<float> &a, int rows_per_req, cudaStream_t s) {
+bool attention_setup() { return set_as<64, 16>() && set_as<64, 64>() && set_as<128, 16>() && set_as<128, 64>(); }
+
+bool launch_attention(const AttnArgs<float> &a, int rows_per_req, int num_sms, cudaStream_t s) {
     if (a.R <= 0) return true;
     if (rows_per_req < 1 || a.R % rows_per_req || (a.hd != 64 && a.hd != 128)) return false;
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-        n = 148;
     AsArgs p;
     p.a = a;
     p.rows_per_req = rows_per_req;
@@ -336,9 +338,9 @@ bool launch_attention(const AttnArgs<float> &a, int rows_per_req, cudaStream_t s
     if ((long)(a.R / 16 + a.R / rows_per_req) > 65535) return false;     // the grid's row tiles
     cudaError_t e;
     if (rows_per_req <= 32)
-        e = a.hd == 128 ? launch_as<128, 16>(p, n, s) : launch_as<64, 16>(p, n, s);
+        e = a.hd == 128 ? launch_as<128, 16>(p, num_sms, s) : launch_as<64, 16>(p, num_sms, s);
     else
-        e = a.hd == 128 ? launch_as<128, 64>(p, n, s) : launch_as<64, 64>(p, n, s);
+        e = a.hd == 128 ? launch_as<128, 64>(p, num_sms, s) : launch_as<64, 64>(p, num_sms, s);
     note_launch();
     return e == cudaSuccess;
 }

@@ -780,7 +780,10 @@ bool launch_attention_tc(AttnTcPlan *p, const AttnArgs<bf16> &a, int B, int rows
     const int has_tree = a.mask != nullptr;
     // One CTA fills an SM: as many splits per (row tile, head) as keep the
     // launch within one wave (a function of the launch's shape alone).
-    const int nsplit = (int)std::max<long>(1, std::min<long>(MAX_SPLITS, p->num_sms / base));
+    // (and no more than the cache has key tiles: a cluster of empty splits only
+    // makes the combine longer)
+    const int nsplit = (int)std::max<long>(
+        1, std::min<long>(std::min<long>(MAX_SPLITS, (a.cache_slots + KT - 1) / KT), p->num_sms / base));
     const long lo_rows = a.lo / a.hd;
     const long kc_rows = (long)B * a.nh * a.cache_slots + lo_rows;
     const CUtensorMap *mkc = kv_map(p, a.cache_k, kc_rows, a.hd);

@@ -8,9 +8,9 @@
 // at once: packed fp32 FMAs (f32x2) keep the even-k and the odd-k sums of each
 // output in one 64-bit register, added at the end. Rows are padded to 68
 // floats, so the 8 rows a warp reads together sit in different banks.
-// Tiles: 16 token rows x 32 outputs, 32 x 64 or 64 x 64, always 256 threads:
-// the smaller the tile, the more warps share it by taking different k of a
-// stage (their sums meet in shared memory). When the tiles leave SMs idle, K is
+// Tiles of 32 x 16 to 128 outputs x 64 token rows, always 256 threads: the
+// smaller the tile, the more warps share it by taking different k of a stage
+// (their sums meet in shared memory). When the tiles leave SMs idle, K is
 // split over the CTAs of a cluster (at most 8), whose partial tiles are summed
 // through distributed shared memory in rank order. Every order is fixed by the
 // launch's shape, so results are reproducible and an output depends only on
@@ -62,6 +62,7 @@ struct Tile {
     static constexpr int KS = SG_THREADS / GROUP;
     static constexpr int STAGE = (BO + BM) * SG_LD;                        // floats
     static constexpr int SMEM = STAGES * STAGE * 4;
+    static constexpr int PER_SM = TO * TM >= 64 ? 1 : 2;                   // CTAs an SM holds (registers)
     static_assert(GROUP % 32 == 0 && (SG_BK / 4) % KS == 0, "whole warps, whole 4-k chunks");
     static_assert(KS * BO * BM <= STAGES * STAGE, "the k groups' partial tiles reuse the ring");
 };
@@ -207,12 +208,11 @@ template <class TL, bool VEC>
 void launch_tile(SgArgs a, int num_sms, cudaStream_t s) {
     const int to = (a.O + TL::BO - 1) / TL::BO, tm = (a.M + TL::BM - 1) / TL::BM;
     const int nb = (a.K + SG_BK - 1) / SG_BK;
-    // split K while that still fills idle SMs (two CTAs each) and leaves every
-    // split two or more k blocks
-    long S = 2L * num_sms / std::max(1L, (long)to * tm);
+    // split K while that still fills idle SMs and leaves every split two or more
+    // k blocks
+    long S = (long)TL::PER_SM * num_sms / std::max(1L, (long)to * tm);
     S = std::max(1L, std::min(std::min(S, 8L), (long)nb / 2));
     a.splits = (int)S;
-    cudaFuncSetAttribute(gemm_simt_kernel<TL, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::SMEM);
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)to, (unsigned)tm, (unsigned)S);
     lc.blockDim = dim3(SG_THREADS);
@@ -235,18 +235,25 @@ void launch_vec(const SgArgs &a, bool vec, int num_sms, cudaStream_t s) {
     else launch_tile<TL, false>(a, num_sms, s);
 }
 
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-        n = 148;
-    return n;
+template <class TL>
+bool set_tile() {
+    return cudaFuncSetAttribute(gemm_simt_kernel<TL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::SMEM) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(gemm_simt_kernel<TL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::SMEM) ==
+               cudaSuccess;
 }
+
+typedef Tile<32, 16, 4, 4, 4> T32x16;
+typedef Tile<32, 32, 4, 4, 4> T32x32;
+typedef Tile<64, 64, 8, 8, 3> T64x64;
+typedef Tile<128, 64, 8, 8, 3> T128x64;
 
 }  // namespace
 
+bool gemm_simt_setup() { return set_tile<T32x16>() && set_tile<T32x32>() && set_tile<T64x64>() && set_tile<T128x64>(); }
+
 void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int O, float *Y, int ldy, int epi,
-                      cudaStream_t s) {
+                      int num_sms, cudaStream_t s) {
     if (M <= 0 || O <= 0) return;
     SgArgs a;
     a.X = X; a.ldx = ldx; a.M = M; a.K = K;
@@ -259,13 +266,17 @@ void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int
     uintptr_t bits = reinterpret_cast<uintptr_t>(X);
     for (int i = 0; i < W.nseg; ++i) bits |= reinterpret_cast<uintptr_t>(w[i]);
     const bool vec = (bits & 15) == 0 && K % 4 == 0 && ldx % 4 == 0;
-    const int n = sm_count();
-    // token rows per tile: the smallest that holds them all, since weights are
-    // read once per row of tiles; 64 at most (larger tiles leave SMs idle at
-    // the widths fp32 contexts run)
-    if (M <= 16) launch_vec<Tile<32, 16, 4, 4, 4>>(a, vec, n, s);
-    else if (M <= 32) launch_vec<Tile<64, 32, 8, 4, 3>>(a, vec, n, s);
-    else launch_vec<Tile<64, 64, 8, 4, 3>>(a, vec, n, s);
+    const int n = num_sms;
+    // The smallest tiles win while they all run at once (weights are read once per
+    // row of tiles, and small tiles share one among more warps): 24 x 1024 x 2816
+    // 12.5 us in 32 x 32 tiles, 22.6 in 64 x 32. Past two CTAs an SM, FMAs per
+    // shared-memory load decide: 333 x 3072 x 1024 57 us in 128 x 64 tiles, 66 to 81
+    // in smaller ones; 333 x 1024 x 1024 35 us in 64 x 64, 52 in 128 x 64 (48 tiles).
+    const long t32 = (long)((O + 31) / 32) * ((M + 31) / 32), t128 = (long)((O + 127) / 128) * ((M + 63) / 64);
+    if (M <= 16) launch_vec<T32x16>(a, vec, n, s);
+    else if (M <= 32 || t32 <= 2L * n) launch_vec<T32x32>(a, vec, n, s);
+    else if (8 * t128 < 7L * n) launch_vec<T64x64>(a, vec, n, s);
+    else launch_vec<T128x64>(a, vec, n, s);
 }
 
 }  // namespace msd

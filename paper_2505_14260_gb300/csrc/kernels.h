@@ -57,7 +57,10 @@ struct AttnArgs {
 };
 // fp32 contexts (CUDA cores); rows come in blocks of rows_per_req rows of one
 // request. Returns false if the shape is unsupported or the launch failed.
-bool launch_attention(const AttnArgs<float> &a, int rows_per_req, cudaStream_t s);
+// attention_setup sets the kernels' shared-memory limits on the current device,
+// once before its first launch.
+bool attention_setup();
+bool launch_attention(const AttnArgs<float> &a, int rows_per_req, int num_sms, cudaStream_t s);
 
 // Scratch of the chunked top-k: per-chunk records and per-row tickets
 // (tickets must start at zero; the kernel leaves them at zero).
@@ -68,8 +71,7 @@ struct TopkScratch {
 size_t topk_scratch_floats(int max_rows, int V);
 
 // out[r] = argmax_j logits[r][j] (ties: lower j)
-void launch_argmax(const float *logits, int R, int V, int *out, const TopkScratch &sc,
-                   cudaStream_t s);
+void launch_argmax(const float *logits, int R, int V, int *out, cudaStream_t s);
 
 // Top-k of each row (ties: lower id) and their log-softmax values (logp
 // nullable). k <= 16.
@@ -97,8 +99,9 @@ struct GemmW {
 };
 enum { EPI_STORE = 0, EPI_ADD = 1, EPI_SWIGLU = 2, EPI_ROPE_KV = 3 };
 
-// fp32 contexts (CUDA cores)
+// fp32 contexts (CUDA cores); gemm_simt_setup as attention_setup
+bool gemm_simt_setup();
 void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int O, float *Y, int ldy, int epi,
-                      cudaStream_t s);
+                      int num_sms, cudaStream_t s);
 
 }  // namespace msd

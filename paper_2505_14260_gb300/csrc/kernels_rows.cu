@@ -164,7 +164,7 @@ void launch_rope_kv(const float *qkv, const RowDesc *rows, int R, int nh, int hd
 }
 
 // ---------------------------------------------------------------------------
-// Top-k per row with log-softmax values (argmax = top-1). The row is cut into
+// Top-k per row with log-softmax values. The row is cut into
 // chunks, one CTA each: the CTA holds its chunk in shared memory, computes the
 // chunk max, the chunk sum of exp(z - max) and the chunk's top-k (k rounds of
 // a block-wide best-of with removal); the last CTA of the row (ticket) merges
@@ -346,6 +346,7 @@ __global__ void __launch_bounds__(TK_THREADS)
     if (lane == 0) { s_m[warp] = m; s_s[warp] = sum; }
     __syncthreads();
     float *rec = ws + ((size_t)r * nc + c) * TK_REC;
+    if (nc == 1 && warp != 0) return;
     if (warp == 0) {
         // the NW warps' k candidates, NW * TOPK_MAX / 32 slots per lane
         constexpr int NS = NW * TOPK_MAX / 32;
@@ -360,10 +361,18 @@ __global__ void __launch_bounds__(TK_THREADS)
         m = lane < NW ? s_m[lane] : -INFINITY;
         sum = lane < NW ? s_s[lane] : 0.f;
         warp_lse(m, sum);
-        if (lane == 0) { rec[0] = m; rec[1] = sum; }
         __syncwarp();                      // the candidates are in registers: reuse s_v / s_i
         warp_topk<NS>(cv, ci, k, s_v, s_i, s_cv, s_ci);
         __syncwarp();
+        if (nc == 1) {                     // one chunk: its result is the row's
+            const float lse = m + logf(sum);
+            if (lane < k) {
+                ids[(size_t)r * k + lane] = s_i[lane] == TK_NONE ? 0 : s_i[lane];
+                if (logp) logp[(size_t)r * k + lane] = s_v[lane] - lse;
+            }
+            return;
+        }
+        if (lane == 0) { rec[0] = m; rec[1] = sum; }
         if (lane < k) {
             rec[2 + lane] = s_v[lane];
             rec[2 + TOPK_MAX + lane] = __int_as_float(s_i[lane]);
@@ -421,9 +430,68 @@ bool topk_supported(int V, int k) {
     return k >= 1 && k <= TOPK_MAX && topk_chunks(V) * k <= 32 * TK_MERGE_SLOTS;
 }
 
-void launch_argmax(const float *logits, int R, int V, int *out, const TopkScratch &sc,
-                   cudaStream_t s) {
-    launch_topk_logp(logits, R, V, 1, out, nullptr, sc, s);
+// out[r] = the index of row r's largest logit (ties: lower index; NaN never
+// selected, 0 if there is nothing else): the order of better(). Bound by reading
+// the logits (960 x 32000 fp32: 123 MB; the top-k kernel above, with its
+// log-sum-exp, ranks and per-chunk tickets, took 96 us for them). One CTA per row,
+// 16-byte loads, 16 in flight per thread where a row is aligned.
+constexpr int AM_THREADS = 512;
+
+__global__ void __launch_bounds__(AM_THREADS) argmax_rows_kernel(const float *__restrict__ logits, int V,
+                                                                 int *__restrict__ out) {
+    wait_prior();
+    allow_dependents();
+    __shared__ unsigned s_k[AM_THREADS / 32];
+    __shared__ int s_i[AM_THREADS / 32];
+    const float *z = logits + (size_t)blockIdx.x * V;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float bv = -INFINITY;
+    int bi = TK_NONE;
+    auto take = [&](float v, int j) {           // (a thread's indices ascend)
+        if (v > bv || (bi == TK_NONE && v == v)) { bv = v; bi = j; }
+    };
+    const int head = (int)min((long long)V, (long long)(((16 - (reinterpret_cast<uintptr_t>(z) & 15)) & 15) >> 2));
+    const int n4 = (V - head) >> 2;
+    if (tid < head) take(z[tid], tid);
+    const float4 *z4 = reinterpret_cast<const float4 *>(z + head);
+    for (int g0 = tid; g0 < n4; g0 += 16 * AM_THREADS) {
+        float4 v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int g = g0 + u * AM_THREADS;
+            if (g < n4) v[u] = z4[g];
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int g = g0 + u * AM_THREADS, j = head + 4 * g;
+            if (g < n4) {
+                take(v[u].x, j);
+                take(v[u].y, j + 1);
+                take(v[u].z, j + 2);
+                take(v[u].w, j + 3);
+            }
+        }
+    }
+    for (int j = head + 4 * n4 + tid; j < V; j += AM_THREADS) take(z[j], j);
+    auto best = [&](unsigned key, int i, unsigned &k, int &ix) {     // of a whole warp
+        k = __reduce_max_sync(0xffffffffu, key);
+        ix = (int)__reduce_min_sync(0xffffffffu, key == k ? (unsigned)i : (unsigned)TK_NONE);
+    };
+    unsigned k;
+    int ix;
+    best(bi == TK_NONE ? 0u : tk_key(bv), bi, k, ix);
+    if (lane == 0) { s_k[warp] = k; s_i[warp] = ix; }
+    __syncthreads();
+    if (warp != 0) return;
+    constexpr int NW = AM_THREADS / 32;
+    best(lane < NW ? s_k[lane] : 0u, lane < NW ? s_i[lane] : TK_NONE, k, ix);
+    if (lane == 0) out[blockIdx.x] = ix == TK_NONE ? 0 : ix;
+}
+
+void launch_argmax(const float *logits, int R, int V, int *out, cudaStream_t s) {
+    if (R <= 0) return;
+    launch_chain(argmax_rows_kernel, R, AM_THREADS, 0, s, logits, V, out);
+    note_launch();
 }
 
 // ---------------------------------------------------------------------------

@@ -30,6 +30,7 @@ struct msd_ctx {
     msd_weights w;
     std::vector<msd_layer> layers;
     int dev = 0;
+    int sms = 148;
     size_t esz = 0;
     int B, S, N, D, D1, k, H, F, V, nh, hd, NL, W, C, Td, Wd, Rmax, chunk, Rlog;
 
@@ -179,7 +180,7 @@ void gemm(msd_ctx *c, const T *X, int ldx, int M, int K, const GemmW &W, int O, 
 template <>
 void gemm<float>(msd_ctx *c, const float *X, int ldx, int M, int K, const GemmW &W, int O,
                  float *Y, int ldy, int epi, cudaStream_t s, bool) {
-    launch_gemm_simt(X, ldx, M, K, W, O, Y, ldy, epi, s);
+    launch_gemm_simt(X, ldx, M, K, W, O, Y, ldy, epi, c->sms, s);
 }
 
 template <>
@@ -199,7 +200,7 @@ void attention(msd_ctx *c, const AttnArgs<T> &a, int rows_per_req, cudaStream_t 
 
 template <>
 void attention<float>(msd_ctx *c, const AttnArgs<float> &a, int rows_per_req, cudaStream_t s) {
-    if (!launch_attention(a, rows_per_req, s)) {
+    if (!launch_attention(a, rows_per_req, c->sms, s)) {
         c->err = "fp32 attention: unsupported shape or launch failure";
         launch_flag(c->status, ST_RANGE, s);     // reported by the next call
     }
@@ -434,7 +435,7 @@ msd_status prefill_impl(msd_ctx *c, int batch, const int32_t *seq_len_host, cons
         }
         const T *h_last = static_cast<const T *>(c->h_all) + (size_t)(L - 1) * H;
         gemm<T>(c, h_last, H, 1, H, one(c->w.lm_head, V, c->pk_lm), V, c->logits, V, EPI_STORE, s);
-        launch_argmax(c->logits, 1, V, c->argmax_tmp, c->tks, s);
+        launch_argmax(c->logits, 1, V, c->argmax_tmp, s);
         // draft cache over positions 0 .. L-2 with the decoupled input (Eq. 7): text
         // rows f_down(Concat(h, e_next)); visual rows e (MSD), the same
         // concatenation (Baseline) or h (Visual Feature), Sec. 5.3
@@ -576,7 +577,7 @@ msd_status verify_impl(msd_ctx *c, const msd_tree *tree, int32_t *argmax_dev, fl
     float *lg = logits_dev ? logits_dev : c->logits;
     gemm<T>(c, static_cast<const T *>(c->hT), H, R, H, one(c->w.lm_head, V, c->pk_lm), V, lg, V, EPI_STORE,
             s);
-    launch_argmax(lg, R, V, argmax_dev, c->tks, s);
+    launch_argmax(lg, R, V, argmax_dev, s);
     return post_status(c, s);
 }
 
@@ -772,6 +773,7 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     c->layers.assign(w->layers, w->layers + cfg->n_layers);
     c->w.layers = c->layers.data();
     cudaGetDevice(&c->dev);
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev);
     c->esz = cfg->dtype == MSD_BF16 ? 2 : 4;
     c->B = cfg->max_batch; c->S = cfg->max_seq; c->N = cfg->tree_nodes; c->D = cfg->tree_depth;
     c->D1 = c->D + 1; c->k = cfg->topk; c->H = cfg->hidden; c->F = cfg->ffn; c->V = cfg->vocab;
@@ -866,6 +868,7 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     ok &= dalloc(c, &c->status, sizeof(int));
     if (ok) ok = cudaMallocHost(&c->status_host, sizeof(int)) == cudaSuccess;
     if (ok) ok = cudaEventCreateWithFlags(&c->status_ev, cudaEventDisableTiming) == cudaSuccess;
+    if (ok && cfg->dtype == MSD_F32) ok = gemm_simt_setup() && attention_setup();
     if (ok && cfg->dtype == MSD_BF16) ok = gemm_plan_create(&c->gplan, c->Rmax, c->H, c->F, c->V);
     if (ok && cfg->dtype == MSD_BF16) ok = attn_tc_plan_create(&c->aplan);
     c->lpack.assign(c->NL, msd_ctx::LayerPack());

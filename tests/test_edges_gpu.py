@@ -166,3 +166,19 @@ def test_single_split_attention_matches_oracle():
     splits per head, the last one with the tree keys.)"""
     wl = synth.WORKLOADS["tiny"].with_(dtype="bf16", batch=40, n_text=(8, 90), steps=2)
     run_parity(wl, wl.steps, (0, 17, 39))
+
+
+@pytest.mark.parametrize("vocab,depth", [(1021, 2), (4097, 2), (8191, 1)])
+def test_argmax_of_unaligned_rows(vocab, depth):
+    """Verify's argmax over rows whose length is no multiple of four (rows start
+    at every alignment), one logit past a 16-byte tail and past a chunk: equal to
+    the lowest index of the largest logit of each row."""
+    wl = synth.WORKLOADS["tiny"].with_(dtype="f32", vocab=vocab, tree_depth=depth, tree_nodes=5)
+    eng, _ = open_engine(wl, steps=1)
+    ids, lens, vis, offs = msd.upload_prompts(synth.make_prompts(wl))
+    eng.prefill(ids, lens, vis, offs)
+    eng.draft_tree()
+    logits = torch.zeros(wl.tree_nodes, vocab, device="cuda")
+    am = eng.verify(logits=logits).cpu().numpy()
+    assert np.array_equal(am, np.argmax(logits.cpu().numpy(), 1))
+    eng.close()
