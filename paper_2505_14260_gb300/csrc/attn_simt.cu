@@ -76,9 +76,17 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
     allow_dependents();
     const AttnArgs<float> &a = p.a;
     const int tid = threadIdx.x;
-    const int h = blockIdx.x, blk = blockIdx.y / p.tiles_per_req, split = blockIdx.z;
-    const int r0 = blk * p.rows_per_req + (blockIdx.y - blk * p.tiles_per_req) * QR;
-    const int r_end = min(r0 + QR, (blk + 1) * p.rows_per_req), nrows = r_end - r0;
+    const int h = blockIdx.x, split = blockIdx.z;
+    int r0, nrows;
+    if (a.tiles) {
+        const int2 t = a.tiles[blockIdx.y];
+        r0 = t.x;
+        nrows = t.y;
+    } else {
+        const int blk = blockIdx.y / p.tiles_per_req;
+        r0 = blk * p.rows_per_req + (blockIdx.y - blk * p.tiles_per_req) * QR;
+        nrows = min(r0 + QR, (blk + 1) * p.rows_per_req) - r0;
+    }
     const int H = a.nh * HD;
     const int req = a.rows[r0].req;
 
@@ -297,7 +305,7 @@ template <int HD, int QR>
 cudaError_t launch_as(AsArgs p, int num_sms, cudaStream_t s) {
     const AttnArgs<float> &a = p.a;
     p.tiles_per_req = (p.rows_per_req + QR - 1) / QR;
-    const int row_tiles = a.R / p.rows_per_req * p.tiles_per_req;
+    const int row_tiles = a.tiles ? a.n_tiles : a.R / p.rows_per_req * p.tiles_per_req;
     // splits while they fit one wave of CTAs: a function of the launch's shape
     const long base = (long)row_tiles * a.nh;
     p.nsplit = (int)std::max<long>(
@@ -329,15 +337,15 @@ bool attention_setup() { return set_as<64, 16>() && set_as<64, 64>() && set_as<1
 
 bool launch_attention(const AttnArgs<float> &a, int rows_per_req, int num_sms, cudaStream_t s) {
     if (a.R <= 0) return true;
-    if (rows_per_req < 1 || a.R % rows_per_req || (a.hd != 64 && a.hd != 128)) return false;
+    if (rows_per_req < 1 || (!a.tiles && a.R % rows_per_req) || (a.hd != 64 && a.hd != 128)) return false;
     AsArgs p;
     p.a = a;
     p.rows_per_req = rows_per_req;
     p.tiles_per_req = p.nsplit = 1;
     p.scale_log2 = a.scale * 1.4426950408889634f;
-    if ((long)(a.R / 16 + a.R / rows_per_req) > 65535) return false;     // the grid's row tiles
+    if ((a.tiles ? (long)a.n_tiles : (long)a.R / 16 + a.R / rows_per_req) > 65535) return false;   // the grid's row tiles
     cudaError_t e;
-    if (rows_per_req <= 32)
+    if (!a.tiles && rows_per_req <= 32)
         e = a.hd == 128 ? launch_as<128, 16>(p, num_sms, s) : launch_as<64, 16>(p, num_sms, s);
     else
         e = a.hd == 128 ? launch_as<128, 64>(p, num_sms, s) : launch_as<64, 64>(p, num_sms, s);

@@ -71,6 +71,7 @@ struct Lay {
 struct AttnTcParams {
     const bf16 *q;
     const RowDesc *rows;
+    const int2 *tiles;        // row tiles (first row, rows), or null: blocks of rows_per_req rows
     const uint64_t *mask;
     bf16 *out;
     long lo;                  // lo planes of q and out (elements); K/V: lo_rows rows on
@@ -301,10 +302,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     // heads vary fastest in the launch order, then row tiles, request blocks in
     // p.order (the CTAs of the longest requests start first)
     const int h = blockIdx.x, tile = blockIdx.y, split = blockIdx.z;
-    const int pos = tile / p.tiles_per_req;
-    const int blk = p.n_order > 0 ? (int)p.order[pos] : pos;
-    const int r0 = blk * p.rows_per_req + (tile - pos * p.tiles_per_req) * ROWS;
-    const int r_end = min(r0 + ROWS, (blk + 1) * p.rows_per_req);
+    int r0, r_end;
+    if (p.tiles) {            // (written, like the row descriptors, at least two launches back)
+        const int2 t = p.tiles[tile];
+        r0 = t.x;
+        r_end = t.x + t.y;
+    } else {
+        const int pos = tile / p.tiles_per_req;
+        const int blk = p.n_order > 0 ? (int)p.order[pos] : pos;
+        r0 = blk * p.rows_per_req + (tile - pos * p.tiles_per_req) * ROWS;
+        r_end = min(r0 + ROWS, (blk + 1) * p.rows_per_req);
+    }
     const int H = p.nh * HD;
 
     const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;
@@ -774,7 +782,7 @@ bool launch_attention_tc(AttnTcPlan *p, const AttnArgs<bf16> &a, int B, int rows
     if (a.lo % a.hd) return false;
     const int tiles_per_req = (rows_per_req + ROWS - 1) / ROWS;
     const int n_blocks = a.R / rows_per_req;
-    const int row_tiles = n_blocks * tiles_per_req;
+    const int row_tiles = a.tiles ? a.n_tiles : n_blocks * tiles_per_req;
     if (row_tiles > 65535 || a.nh > 65535) return false;   // grid (heads, row tiles, splits)
     const long base = (long)row_tiles * a.nh;
     const int has_tree = a.mask != nullptr;
@@ -799,6 +807,7 @@ bool launch_attention_tc(AttnTcPlan *p, const AttnArgs<bf16> &a, int B, int rows
     memset(&tp, 0, sizeof tp);
     tp.q = a.q;
     tp.rows = a.rows;
+    tp.tiles = a.tiles;
     tp.mask = a.mask;
     tp.out = a.out;
     tp.lo = a.lo;
@@ -816,7 +825,7 @@ bool launch_attention_tc(AttnTcPlan *p, const AttnArgs<bf16> &a, int B, int rows
     tp.cache_early = a.cache_fresh ? 0 : 1;
     tp.scale_log2 = a.scale * 1.4426950408889634f;
     tp.stamp = stamp;
-    if (order && n_blocks > 1 && n_blocks <= ORDER_MAX) {
+    if (order && !a.tiles && n_blocks > 1 && n_blocks <= ORDER_MAX) {
         // the kernel indexes rows through it: only a permutation is taken
         uint64_t seen = 0;
         for (int i = 0; i < n_blocks; ++i) {

@@ -218,29 +218,6 @@ __device__ __forceinline__ void copy_row(TD *__restrict__ dst, const TS *__restr
     }
 }
 
-// One source row to two destinations (d2 nullable).
-template <typename TD1, typename TD2, typename TS>
-__device__ __forceinline__ void copy_row_2dst(TD1 *__restrict__ d1, TD2 *__restrict__ d2,
-                                              const TS *__restrict__ src, int n) {
-    const int n4 = n >> 2;
-    for (int g0 = threadIdx.x; g0 < n4; g0 += 4 * blockDim.x) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) v[u] = Vec4<TS>::load(src + 4 * g);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) {
-                Vec4<TD1>::store(d1 + 4 * g, v[u]);
-                if (d2) Vec4<TD2>::store(d2 + 4 * g, v[u]);
-            }
-        }
-    }
-}
-
 // Two independent row copies in one pass (s1 null: d1 gets zeros).
 template <typename TD1, typename TS1, typename TD2, typename TS2>
 __device__ __forceinline__ void copy_rows2(TD1 *__restrict__ d1, const TS1 *__restrict__ s1,

@@ -11,22 +11,18 @@ namespace msd {
 
 // ---- elementwise / row kernels (kernels_rows.cu) ---------------------------
 
-// x[r] = float(src[r] >= 0 ? E[src[r]] : vis[-1 - src[r]]); emb_out (nullable)
-// receives the same row in T.
+// x[r] = float(src[r] >= 0 ? E[src[r]] : vis[-1 - src[r]])
 template <typename T>
-void launch_embed_rows(const T *E, const T *vis, const int *src, int R, int H,
-                       float *x, T *emb_out, int V, int *status, cudaStream_t s);
+void launch_embed_rows(const T *E, const T *vis, const int *src, int R, int H, float *x, int V, int *status,
+                       cudaStream_t s);
 
 // out[r] = x[r] / sqrt(mean(x[r]^2) + eps) * g, split (lo plane at out + lo)
 template <typename T>
 void launch_rmsnorm(const float *x, const T *g, int R, int H, float eps, T *out, long lo,
                     cudaStream_t s);
 
-// act[r][j] = T(silu(g) * u) with g = gu[r][j], u = gu[r][F + j], or, for
-// glu-packed gate/up products (glu = true, rows of 128 * ceil(F / 64)),
-// g = gu[r][128 (j / 64) + j % 64] and u 64 columns further.
-template <typename T>
-void launch_swiglu(const float *gu, int R, int F, bool glu, T *act, long lo, cudaStream_t s);
+// act[r][j] = silu(g) * u with g = gu[r][j], u = gu[r][F + j] (fp32 contexts)
+void launch_swiglu(const float *gu, int R, int F, float *act, cudaStream_t s);
 
 // RoPE (rotate-half, table of (cos, sin) per position and pair) on q and k of
 // qkv [R][3H]; q -> q_out [R][H]; k, v -> kdst/vdst at slot rows[r].dst of
@@ -52,6 +48,10 @@ struct AttnArgs {
     int nh, hd;
     float scale;
     T *out;                     // [R][nh*hd]
+    // row tiles of a packed prefill chunk (first row, rows <= 64 of one request),
+    // longest prefix first; null: blocks of rows_per_req rows of one request
+    const int2 *tiles;
+    int n_tiles;
     bool cache_fresh;           // the kernel launched just before may have written cache_k/v
     long lo;                    // split bf16: lo planes of q, K/V and out sit lo elements on (0: none)
 };

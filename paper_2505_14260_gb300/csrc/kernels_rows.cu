@@ -16,8 +16,8 @@ void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void embed_rows_kernel(const T *__restrict__ E, const T *__restrict__ vis,
-                                  const int *__restrict__ src, int H, float *__restrict__ x,
-                                  T *__restrict__ emb_out, int V, int *status) {
+                                  const int *__restrict__ src, int H, float *__restrict__ x, int V,
+                                  int *status) {
     wait_prior();
     allow_dependents();
     const int r = blockIdx.x;
@@ -32,14 +32,14 @@ __global__ void embed_rows_kernel(const T *__restrict__ E, const T *__restrict__
     } else {
         row = vis + (size_t)(-1 - s) * H;
     }
-    copy_row_2dst(x + (size_t)r * H, emb_out ? emb_out + (size_t)r * H : nullptr, row, H);
+    copy_row(x + (size_t)r * H, row, H);
 }
 
 template <typename T>
-void launch_embed_rows(const T *E, const T *vis, const int *src, int R, int H, float *x,
-                       T *emb_out, int V, int *status, cudaStream_t s) {
+void launch_embed_rows(const T *E, const T *vis, const int *src, int R, int H, float *x, int V, int *status,
+                       cudaStream_t s) {
     if (R <= 0) return;
-    launch_chain(embed_rows_kernel<T>, R, 256, 0, s, E, vis, src, H, x, emb_out, V, status); note_launch();
+    launch_chain(embed_rows_kernel<T>, R, 256, 0, s, E, vis, src, H, x, V, status); note_launch();
 }
 
 // ---------------------------------------------------------------------------
@@ -88,32 +88,27 @@ void launch_rmsnorm(const float *x, const T *g, int R, int H, float eps, T *out,
 }
 
 // ---------------------------------------------------------------------------
-// SwiGLU: silu(gate) * up
+// SwiGLU of fp32 contexts: silu(gate) * up
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void swiglu_kernel(const float *__restrict__ gu, int F, int glu, T *__restrict__ act, long lo) {
+__global__ void swiglu_kernel(const float *__restrict__ gu, int F, float *__restrict__ act) {
     wait_prior();
     allow_dependents();
     const int r = blockIdx.y;
-    const int ld = glu ? 128 * ((F + 63) / 64) : 2 * F;
-    const float *row = gu + (size_t)r * ld;
+    const float *row = gu + (size_t)r * 2 * F;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < F; j += gridDim.x * blockDim.x) {
-        const int gi = glu ? ((j >> 6) << 7) + (j & 63) : j;
-        const float g = row[gi], u = row[gi + (glu ? 64 : F)];
-        const float sg = g / (1.f + __expf(-g));
-        Split<T>::store(act + (size_t)r * F + j, lo, sg * u);
+        const float g = row[j];
+        act[(size_t)r * F + j] = g / (1.f + __expf(-g)) * row[F + j];
     }
 }
 
-template <typename T>
-void launch_swiglu(const float *gu, int R, int F, bool glu, T *act, long lo, cudaStream_t s) {
+void launch_swiglu(const float *gu, int R, int F, float *act, cudaStream_t s) {
     if (R <= 0) return;
-    dim3 grid((F + 255) / 256, R);
-    launch_chain(swiglu_kernel<T>, grid, 256, 0, s, gu, F, glu ? 1 : 0, act, lo); note_launch();
+    launch_chain(swiglu_kernel, dim3((F + 255) / 256, R), 256, 0, s, gu, F, act); note_launch();
 }
 
 // ---------------------------------------------------------------------------
-// RoPE (rotate-half pairs (i, i + hd/2)) on q and k, and K/V placement.
+// RoPE (rotate-half pairs (i, i + hd/2)) on q and k, and K/V placement. Bound by
+// memory: 7B rows read 48 KB and write 48 KB (split pairs).
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void rope_kv_kernel(const float *__restrict__ qkv, const RowDesc *__restrict__ rows,
@@ -132,24 +127,38 @@ __global__ void rope_kv_kernel(const float *__restrict__ qkv, const RowDesc *__r
     }
     const bool write_kv = d.dst >= 0 && d.dst < slots;
     if (d.dst >= slots && threadIdx.x == 0) set_status(status, ST_RANGE);
+    // four frequencies of a head per thread: 16-byte loads of both halves of q, k
+    // and v, all requested before the first store
     const float *q = qkv + (size_t)r * 3 * H;
-    const float *k = q + H;
-    const float *v = q + 2 * H;
-    const float2 *cs = tab + (size_t)pos * half;
-    for (int t = threadIdx.x; t < nh * half; t += blockDim.x) {
-        const int h = t / half, i = t - h * half;
-        const float2 c = cs[i];
+    const float4 *cs = reinterpret_cast<const float4 *>(tab + (size_t)pos * half);
+    const int per = half >> 2;
+    for (int t = threadIdx.x; t < nh * per; t += blockDim.x) {
+        const int h = t / per, i = (t - h * per) * 4;
         const int a = h * hd + i, b = a + half;
-        const float qa = q[a], qb = q[b];
-        Split<T>::store(q_out + (size_t)r * H + a, lo, qa * c.x - qb * c.y);
-        Split<T>::store(q_out + (size_t)r * H + b, lo, qb * c.x + qa * c.y);
+        auto ld = [&](int o) { return *reinterpret_cast<const float4 *>(q + o); };
+        const float4 c0 = cs[i >> 1], c1 = cs[(i >> 1) + 1];        // (cos, sin) x 2 each
+        const float4 qa = ld(a), qb = ld(b);
+        float4 ka, kb, va, vb;
         if (write_kv) {
-            const float ka = k[a], kb = k[b];
-            const size_t base = ((size_t)(d.req * nh + h) * slots + d.dst) * hd;
-            Split<T>::store(kdst + base + i, lo, ka * c.x - kb * c.y);
-            Split<T>::store(kdst + base + i + half, lo, kb * c.x + ka * c.y);
-            Split<T>::store(vdst + base + i, lo, v[a]);
-            Split<T>::store(vdst + base + i + half, lo, v[b]);
+            ka = ld(H + a); kb = ld(H + b);
+            va = ld(2 * H + a); vb = ld(2 * H + b);
+        }
+        auto lo_half = [&](const float4 &x, const float4 &y) {
+            return make_float4(x.x * c0.x - y.x * c0.y, x.y * c0.z - y.y * c0.w, x.z * c1.x - y.z * c1.y,
+                               x.w * c1.z - y.w * c1.w);
+        };
+        auto hi_half = [&](const float4 &x, const float4 &y) {
+            return make_float4(y.x * c0.x + x.x * c0.y, y.y * c0.z + x.y * c0.w, y.z * c1.x + x.z * c1.y,
+                               y.w * c1.z + x.w * c1.w);
+        };
+        Split<T>::store4(q_out + (size_t)r * H + a, lo, lo_half(qa, qb));
+        Split<T>::store4(q_out + (size_t)r * H + b, lo, hi_half(qa, qb));
+        if (write_kv) {
+            const size_t base = ((size_t)(d.req * nh + h) * slots + d.dst) * hd + i;
+            Split<T>::store4(kdst + base, lo, lo_half(ka, kb));
+            Split<T>::store4(kdst + base + half, lo, hi_half(ka, kb));
+            Split<T>::store4(vdst + base, lo, va);
+            Split<T>::store4(vdst + base + half, lo, vb);
         }
     }
 }
@@ -520,10 +529,9 @@ void launch_flag(int *status, int code, cudaStream_t s) {
 
 #define MSD_INST(T)                                                                          \
     template void launch_embed_rows<T>(const T *, const T *, const int *, int, int, float *,  \
-                                       T *, int, int *, cudaStream_t);                       \
+                                       int, int *, cudaStream_t);                            \
     template void launch_rmsnorm<T>(const float *, const T *, int, int, float, T *, long,    \
                                     cudaStream_t);                                           \
-    template void launch_swiglu<T>(const float *, int, int, bool, T *, long, cudaStream_t);  \
     template void launch_rope_kv<T>(const float *, const RowDesc *, int, int, int,           \
                                     const float2 *, int, T *, T *, T *, int, long, int *,    \
                                     cudaStream_t);                                           \

@@ -799,45 +799,61 @@ __global__ void pend_h_kernel(const T *__restrict__ hT, const int *__restrict__ 
 // ---------------------------------------------------------------------------
 // Prefill helpers
 // ---------------------------------------------------------------------------
-// Decoupled draft input (Eq. 7): visual rows take the raw embedding.
+// The draft rows of a packed prefill chunk (all positions of a request but its
+// last). draft[r] >= 0: chunk row r is draft row draft[r], whose text input is
+// Concat(h_i, e_{i+1}) with e_{i+1} gathered by next[r] (a token id, or -1 - row of
+// the visual rows); draft[r] = -1 - b: r is the last position of request b, whose
+// feature is kept in h_last[b].
 template <typename T>
-__global__ void select_visual_kernel(float *__restrict__ x, const T *__restrict__ emb, long slo,
-                                     const int *__restrict__ src, int H) {
+__global__ void prefill_draft_in_kernel(const T *__restrict__ h, const T *__restrict__ E, const T *__restrict__ vis,
+                                        const int *__restrict__ draft, const int *__restrict__ next, int H,
+                                        T *__restrict__ xfc, T *__restrict__ h_last, long lo) {
     wait_prior();
     allow_dependents();
-    const int r = blockIdx.x;
-    if (src[r] >= 0) return;
-    copy_row_split(x + (size_t)r * H, 0, emb + (size_t)r * H, slo, H);
+    const int r = blockIdx.x, j = draft[r];
+    const T *hr = h + (size_t)r * H;
+    if (j < 0) {
+        copy_row_split(h_last + (size_t)(-1 - j) * H, lo, hr, lo, H);
+        return;
+    }
+    const int s = next[r];
+    const T *e = s >= 0 ? E + (size_t)s * H : vis + (size_t)(-1 - s) * H;
+    copy_rows2_split(xfc + (size_t)j * 2 * H, hr, lo, xfc + (size_t)j * 2 * H + H, e, H, lo);
 }
 
-// Concat(h_i, e_{i+1}) rows for the draft prefill (text positions; visual rows
-// are overwritten after f_down by select_visual_kernel).
+// Decoupled draft input (Eq. 7): draft rows of visual positions take the raw
+// embedding, or (feat) the target's feature.
 template <typename T>
-__global__ void concat_next_kernel(const T *__restrict__ h, const T *__restrict__ emb, int H,
-                                   T *__restrict__ xfc, long lo) {
+__global__ void select_visual_kernel(float *__restrict__ x, const T *__restrict__ h, const T *__restrict__ vis,
+                                     const int *__restrict__ draft, const int *__restrict__ src, int feat, long lo,
+                                     int H) {
     wait_prior();
     allow_dependents();
-    const int r = blockIdx.x;
-    copy_rows2_split(xfc + (size_t)r * 2 * H, h + (size_t)r * H, lo, xfc + (size_t)r * 2 * H + H,
-                     emb + (size_t)(r + 1) * H, H, lo);
+    const int r = blockIdx.x, j = draft[r], s = src[r];
+    if (s >= 0 || j < 0) return;
+    if (feat) copy_row_split(x + (size_t)j * H, 0, h + (size_t)r * H, lo, H);
+    else copy_row_split(x + (size_t)j * H, 0, vis + (size_t)(-1 - s) * H, 0, H);
 }
 
+// One CTA per request: its length, root token and pending draft row.
 template <typename T>
-__global__ void prefill_finish_kernel(const int *__restrict__ argmax1, const T *__restrict__ h_last,
-                                      int b, int L, int D1, int H, int *__restrict__ seq_len,
+__global__ void prefill_finish_kernel(const int *__restrict__ argmax, const T *__restrict__ h_last,
+                                      const int *__restrict__ L, int D1, int H, int *__restrict__ seq_len,
                                       int *__restrict__ n_pend, int *__restrict__ root,
                                       int *__restrict__ pend_next, T *__restrict__ pend_h, long lo,
                                       int *__restrict__ root_out) {
     wait_prior();
-    const int x = argmax1[0];
+    allow_dependents();
+    const int b = blockIdx.x;
     if (threadIdx.x == 0) {
-        seq_len[b] = L;
+        const int x = argmax[b];
+        seq_len[b] = L[b];
         n_pend[b] = 1;
         root[b] = x;
         pend_next[b * D1] = x;
         if (root_out) root_out[b] = x;
     }
-    copy_row_split(pend_h + (size_t)b * D1 * H, lo, h_last, lo, H);
+    copy_row_split(pend_h + (size_t)b * D1 * H, lo, h_last + (size_t)b * H, lo, H);
 }
 
 // ---------------------------------------------------------------------------
@@ -959,23 +975,25 @@ void launch_pend_h(const T *hT, const int *acc_path, const int *acc_a, int B, in
 }
 
 template <typename T>
-void launch_select_visual(float *x, const T *emb, long slo, const int *src, int R, int H, cudaStream_t s) {
+void launch_prefill_draft_in(const T *h, const T *E, const T *vis, const int *draft, const int *next, int R, int H,
+                             T *xfc, T *h_last, long lo, cudaStream_t s) {
     if (R <= 0) return;
-    launch_chain(select_visual_kernel<T>, R, 256, 0, s, x, emb, slo, src, H); note_launch();
+    launch_chain(prefill_draft_in_kernel<T>, R, 256, 0, s, h, E, vis, draft, next, H, xfc, h_last, lo); note_launch();
 }
 
 template <typename T>
-void launch_concat_next(const T *h, const T *emb, int R, int H, T *xfc, long lo, cudaStream_t s) {
+void launch_select_visual(float *x, const T *h, const T *vis, const int *draft, const int *src, bool feat, long lo,
+                          int R, int H, cudaStream_t s) {
     if (R <= 0) return;
-    launch_chain(concat_next_kernel<T>, R, 256, 0, s, h, emb, H, xfc, lo); note_launch();
+    launch_chain(select_visual_kernel<T>, R, 256, 0, s, x, h, vis, draft, src, feat ? 1 : 0, lo, H); note_launch();
 }
 
 template <typename T>
-void launch_prefill_finish(const int *argmax1, const T *h_last, int b, int L, int D1, int H,
-                           int *seq_len, int *n_pend, int *root, int *pend_next, T *pend_h, long lo,
-                           int *root_out, cudaStream_t s) {
-    launch_chain(prefill_finish_kernel<T>, 1, 256, 0, s, argmax1, h_last, b, L, D1, H, seq_len, n_pend,
-                                               root, pend_next, pend_h, lo, root_out); note_launch();
+void launch_prefill_finish(const int *argmax, const T *h_last, const int *L, int B, int D1, int H, int *seq_len,
+                           int *n_pend, int *root, int *pend_next, T *pend_h, long lo, int *root_out,
+                           cudaStream_t s) {
+    launch_chain(prefill_finish_kernel<T>, B, 256, 0, s, argmax, h_last, L, D1, H, seq_len, n_pend, root, pend_next,
+                 pend_h, lo, root_out); note_launch();
 }
 
 #define MSD_INST(T)                                                                             \
@@ -990,11 +1008,12 @@ void launch_prefill_finish(const int *argmax1, const T *h_last, int b, int L, in
     template void launch_tree_step<T>(const DraftArgs<T> &, int, int, cudaStream_t);            \
     template void launch_pend_h<T>(const T *, const int *, const int *, int, int, int, int, T *, \
                                    long, cudaStream_t);                                         \
-    template void launch_select_visual<T>(float *, const T *, long, const int *, int, int,      \
-                                          cudaStream_t);                                        \
-    template void launch_concat_next<T>(const T *, const T *, int, int, T *, long, cudaStream_t); \
-    template void launch_prefill_finish<T>(const int *, const T *, int, int, int, int, int *,   \
-                                           int *, int *, int *, T *, long, int *, cudaStream_t);
+    template void launch_prefill_draft_in<T>(const T *, const T *, const T *, const int *,      \
+                                             const int *, int, int, T *, T *, long, cudaStream_t); \
+    template void launch_select_visual<T>(float *, const T *, const T *, const int *, const int *, \
+                                          bool, long, int, int, cudaStream_t);                  \
+    template void launch_prefill_finish<T>(const int *, const T *, const int *, int, int, int,  \
+                                           int *, int *, int *, int *, T *, long, int *, cudaStream_t);
 MSD_INST(float)
 MSD_INST(bf16)
 #undef MSD_INST

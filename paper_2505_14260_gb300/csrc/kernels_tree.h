@@ -97,14 +97,17 @@ void launch_compact_kv(const void *tree_kv, void *cache, const int *acc_path, co
 template <typename T>
 void launch_pend_h(const T *hT, const int *acc_path, const int *acc_a, int B, int N, int D1,
                    int H, T *pend_h, long lo, cudaStream_t s);
-// slo: lo plane of emb (0: emb is exact, e.g. the embedding rows)
+// Packed prefill chunks of R rows: the draft rows' inputs (and the requests' last
+// features), the visual rows' inputs, and the requests' state (one row per request).
 template <typename T>
-void launch_select_visual(float *x, const T *emb, long slo, const int *src, int R, int H, cudaStream_t s);
+void launch_prefill_draft_in(const T *h, const T *E, const T *vis, const int *draft, const int *next, int R, int H,
+                             T *xfc, T *h_last, long lo, cudaStream_t s);
 template <typename T>
-void launch_concat_next(const T *h, const T *emb, int R, int H, T *xfc, long lo, cudaStream_t s);
+void launch_select_visual(float *x, const T *h, const T *vis, const int *draft, const int *src, bool feat, long lo,
+                          int R, int H, cudaStream_t s);
 template <typename T>
-void launch_prefill_finish(const int *argmax1, const T *h_last, int b, int L, int D1, int H,
-                           int *seq_len, int *n_pend, int *root, int *pend_next, T *pend_h, long lo,
-                           int *root_out, cudaStream_t s);
+void launch_prefill_finish(const int *argmax, const T *h_last, const int *L, int B, int D1, int H, int *seq_len,
+                           int *n_pend, int *root, int *pend_next, T *pend_h, long lo, int *root_out,
+                           cudaStream_t s);
 
 }  // namespace msd

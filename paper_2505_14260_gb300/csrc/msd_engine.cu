@@ -61,7 +61,12 @@ struct msd_ctx {
     int *ar_argmax = nullptr;
     bool draft_stale = false;   // msd_ar_step ran: the draft cache no longer follows the target's
     float2 *rope_tab = nullptr;
-    void *h_all = nullptr, *emb_all = nullptr;
+    void *h_all = nullptr;      // prefill: final-normed features of a chunk, [chunk][H]
+    // prefill metadata of all its chunks, built in page-locked host memory and
+    // copied at once: row descriptors of the target and the draft rows, embedding
+    // sources, draft row maps, attention tiles, lengths
+    char *pf_host = nullptr, *pf_dev = nullptr;
+    size_t pf_bytes = 0;
     // bf16 contexts: every bf16 buffer that feeds a tensor-core product (and the
     // KV caches) is carved from one arena whose upper half holds the lo planes
     // of the split pairs; lo = that half's size in elements (0: fp32 context)
@@ -212,7 +217,7 @@ void attention<bf16>(msd_ctx *c, const AttnArgs<bf16> &a, int rows_per_req, cuda
     // bound of each request's L orders them; only scheduling depends on it)
     int order[64];
     const int *ord = nullptr;
-    if (a.R == c->B * rows_per_req && c->B > 1 && c->B <= 64) {
+    if (!a.tiles && a.R == c->B * rows_per_req && c->B > 1 && c->B <= 64) {
         for (int b = 0; b < c->B; ++b) order[b] = b;
         std::stable_sort(order, order + c->B, [&](int x, int y) { return c->L_bound[x] > c->L_bound[y]; });
         ord = order;
@@ -271,15 +276,13 @@ void gate_up_swiglu(msd_ctx *c, const msd_layer &lw, const msd_ctx::LayerPack &l
         fx.act = static_cast<bf16 *>(c->act);
         fx.F = F;
         fx.lo = c->lo;
-        if (gemm_bf16_fused(c->gplan, static_cast<const bf16 *>(c->xn), lo_of(c, c->xn), H, R, H, wgu, O, fx,
-                            c->status, s, norm_in))
-            return;
-        gemm<T>(c, static_cast<const T *>(c->xn), H, R, H, wgu, O, c->gu, O, EPI_STORE, s);
-        launch_swiglu<T>(c->gu, R, F, true, static_cast<T *>(c->act), c->lo, s);
+        // (ffn is a multiple of 16 and the weights are packed: the fused GEMM takes every shape)
+        gemm_bf16_fused(c->gplan, static_cast<const bf16 *>(c->xn), lo_of(c, c->xn), H, R, H, wgu, O, fx, c->status, s,
+                        norm_in);
     } else {
         GemmW wgu = {{lw.w_gate, lw.w_up, nullptr}, {F, F, 0}, 2, nullptr};
         gemm<T>(c, static_cast<const T *>(c->xn), H, R, H, wgu, 2 * F, c->gu, 2 * F, EPI_STORE, s);
-        launch_swiglu<T>(c->gu, R, F, false, static_cast<T *>(c->act), c->lo, s);
+        launch_swiglu(c->gu, R, F, static_cast<float *>(c->act), s);
     }
 }
 
@@ -310,7 +313,7 @@ bool run_layer(msd_ctx *c, const msd_layer &lw, const msd_ctx::LayerPack &lp, in
                const RowDesc *rows, T *kdst, T *vdst, int dst_slots, const T *ck, const T *cv,
                int cslots, const T *tk, const T *tv, int tslots, const uint64_t *mask, int mw,
                int rows_per_req, cudaStream_t s, bool in_folded = false,
-               const void *out_norm_g = nullptr) {
+               const void *out_norm_g = nullptr, const int2 *tiles = nullptr, int n_tiles = 0) {
     const int H = c->H, F = c->F;
     const float eps = c->cfg.rms_eps;
     const bool fold = folds(c, R, lp.o) && lp.qkv && lp.gu && lp.down;
@@ -337,6 +340,8 @@ bool run_layer(msd_ctx *c, const msd_layer &lw, const msd_ctx::LayerPack &lp, in
     a.out = static_cast<T *>(c->attn);
     a.cache_fresh = kdst == ck;         // this layer's own K/V go into the cache it reads
     a.lo = c->lo;
+    a.tiles = tiles;
+    a.n_tiles = n_tiles;
     attention<T>(c, a, rows_per_req, s);
     GemmW wo = {{lw.wo, nullptr, nullptr}, {H, 0, 0}, 1, lp.o};
     GemmW wd = {{lw.w_down, nullptr, nullptr}, {H, 0, 0}, 1, lp.down};
@@ -388,6 +393,57 @@ bool draft_fc(msd_ctx *c, int R, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Prefill
 // ---------------------------------------------------------------------------
+// The prompts' rows are packed one request after another and run in chunks of up
+// to c->chunk rows of any requests: the GEMMs see full chunks whatever the
+// prompts' lengths (16 ragged prompts of 600 to 1660 rows in chunks of their own
+// cost a second, mostly empty chunk each), and large chunks fill the pairs of the
+// many-row GEMM (O at 7B: 64 of 76 in one round at 1024 rows, 304 in four at
+// 4864). A request's earlier rows are in the cache when a later chunk reads it.
+// The draft rows of a chunk follow its target pass, since e_{i+1} is a gather by
+// the next position's source. All row metadata is built on the host first and
+// copied at once, so the launches run without a synchronisation between.
+constexpr int PREFILL_CHUNK = 4864;
+
+// Byte offsets of the metadata arrays, for n rows in chunks of `chunk`, B requests.
+struct PrefillMeta {
+    size_t rows, drows, src, next, draft, len, tiles, dtiles, bytes;
+    long max_tiles;
+    PrefillMeta(long n, int chunk, int B) {
+        size_t off = 0;
+        auto take = [&](size_t b) {
+            const size_t at = off;
+            off += (b + 255) / 256 * 256;
+            return at;
+        };
+        max_tiles = n / 64 + 2L * B + 2 * (n / chunk + 1);      // a partial tile per request and chunk
+        rows = take(sizeof(RowDesc) * n);
+        drows = take(sizeof(RowDesc) * n);
+        src = take(sizeof(int) * n);
+        next = take(sizeof(int) * n);
+        draft = take(sizeof(int) * n);
+        len = take(sizeof(int) * B);
+        tiles = take(sizeof(int2) * max_tiles);
+        dtiles = take(sizeof(int2) * max_tiles);
+        bytes = off;
+    }
+};
+
+// Row tiles of up to 64 rows of one request over the n rows at rd, longest
+// prefix first (the CTAs that start last are the shortest). Returns their count.
+int row_tiles(const RowDesc *rd, int n, int2 *out) {
+    int k = 0;
+    for (int r = 0; r < n;) {
+        int e = r + 1;
+        while (e < n && e - r < 64 && rd[e].req == rd[r].req) ++e;
+        out[k++] = make_int2(r, e - r);
+        r = e;
+    }
+    std::stable_sort(out, out + k, [&](const int2 &a, const int2 &b) {
+        return rd[a.x + a.y - 1].plen > rd[b.x + b.y - 1].plen;
+    });
+    return k;
+}
+
 template <typename T>
 msd_status prefill_impl(msd_ctx *c, int batch, const int32_t *seq_len_host, const int32_t *ids_dev,
                         int ids_stride, const void *vis_dev, const int64_t *vis_off_host,
@@ -398,72 +454,114 @@ msd_status prefill_impl(msd_ctx *c, int batch, const int32_t *seq_len_host, cons
     CU(cudaMemsetAsync(c->seq_len, 0, sizeof(int) * c->B, s));
     CU(cudaMemsetAsync(c->n_pend, 0, sizeof(int) * c->B, s));
     for (int b = 0; b < c->B; ++b) c->L_bound[b] = 0;
-    std::vector<int> ids, src;
-    std::vector<RowDesc> rd;
-    for (int b = 0; b < batch; ++b) {
-        const int L = seq_len_host[b];
-        ids.resize(L);
-        CU(cudaMemcpy(ids.data(), ids_dev + (size_t)b * ids_stride, sizeof(int) * L,
-                      cudaMemcpyDeviceToHost));
-        if (ids[L - 1] < 0) return fail(c, MSD_ERR_INVALID, "a prompt must end with a text token");
-        src.resize(L);
-        long vrow = vis_off_host ? vis_off_host[b] : 0;
-        int n_vis = 0;
-        for (int i = 0; i < L; ++i) {
-            if (ids[i] >= V || ids[i] < -1) return fail(c, MSD_ERR_INVALID, "token id out of range");
-            if (ids[i] >= 0) src[i] = ids[i];
-            else { src[i] = (int)(-1 - (vrow + n_vis)); ++n_vis; }
-        }
-        if (n_vis > 0 && !vis) return fail(c, MSD_ERR_INVALID, "visual slots but no visual rows");
-        CU(cudaMemcpyAsync(c->src, src.data(), sizeof(int) * L, cudaMemcpyHostToDevice, s));
-        // target over the prompt, causal, in chunks
-        for (int r0 = 0; r0 < L; r0 += c->chunk) {
-            const int n = std::min(c->chunk, L - r0);
-            rd.resize(n);
-            for (int i = 0; i < n; ++i) rd[i] = RowDesc{b, r0 + i, r0 + i + 1, r0 + i};
-            CU(cudaMemcpyAsync(c->rows, rd.data(), sizeof(RowDesc) * n, cudaMemcpyHostToDevice, s));
-            launch_embed_rows<T>(E, vis, c->src + r0, n, H, c->x,
-                                 static_cast<T *>(c->emb_all) + (size_t)r0 * H, V, c->status, s);
-            for (int l = 0; l < c->NL; ++l) {
-                T *K = tkv<T>(c, c->target_kv, l, 0, c->S), *Vv = tkv<T>(c, c->target_kv, l, 1, c->S);
-                run_layer<T>(c, c->layers[l], c->lpack[l], n, c->rows, K, Vv, c->S, K, Vv, c->S, nullptr,
-                             nullptr, 0, nullptr, 0, n, s);
+    long total = 0;
+    for (int b = 0; b < batch; ++b) total += seq_len_host[b];
+    // equal chunks of at most c->chunk rows
+    const int n_chunks = (int)((total + c->chunk - 1) / c->chunk);
+    const int step = (int)((total + n_chunks - 1) / n_chunks);
+    const PrefillMeta m(total, step, batch);
+    if (m.bytes > c->pf_bytes) return fail(c, MSD_ERR_CAPACITY, "prefill metadata");    // (sized for B x max_seq)
+    RowDesc *rows = reinterpret_cast<RowDesc *>(c->pf_host + m.rows);
+    RowDesc *drows = reinterpret_cast<RowDesc *>(c->pf_host + m.drows);
+    int *src = reinterpret_cast<int *>(c->pf_host + m.src), *next = reinterpret_cast<int *>(c->pf_host + m.next),
+        *draft = reinterpret_cast<int *>(c->pf_host + m.draft), *len = reinterpret_cast<int *>(c->pf_host + m.len);
+    int2 *tiles = reinterpret_cast<int2 *>(c->pf_host + m.tiles), *dtiles = reinterpret_cast<int2 *>(c->pf_host + m.dtiles);
+    // the prompts' ids, into the place of the draft map (built after them); the
+    // copies queue behind the last prefill's use of the page-locked arrays
+    {
+        long r = 0;
+        for (int b = 0; b < batch; r += seq_len_host[b], ++b)
+            CU(cudaMemcpyAsync(draft + r, ids_dev + (size_t)b * ids_stride, sizeof(int) * seq_len_host[b],
+                               cudaMemcpyDeviceToHost, s));
+        CU(cudaStreamSynchronize(s));
+    }
+    {
+        long r = 0;
+        for (int b = 0; b < batch; ++b) {
+            const int L = seq_len_host[b];
+            const int *id = draft + r;
+            if (id[L - 1] < 0) return fail(c, MSD_ERR_INVALID, "a prompt must end with a text token");
+            const long vrow = vis_off_host ? vis_off_host[b] : 0;
+            int n_vis = 0;
+            for (int i = 0; i < L; ++i) {
+                if (id[i] >= V || id[i] < -1) return fail(c, MSD_ERR_INVALID, "token id out of range");
+                if (id[i] >= 0) src[r + i] = id[i];
+                else { src[r + i] = (int)(-1 - (vrow + n_vis)); ++n_vis; }
+                rows[r + i] = RowDesc{b, i, i + 1, i};
             }
-            launch_rmsnorm<T>(c->x, static_cast<const T *>(c->w.final_norm), n, H, c->cfg.rms_eps,
-                              static_cast<T *>(c->h_all) + (size_t)r0 * H, c->lo, s);
-            CU(cudaStreamSynchronize(s));   // rd/src host vectors are reused
+            if (n_vis > 0 && !vis) return fail(c, MSD_ERR_INVALID, "visual slots but no visual rows");
+            for (int i = 0; i < L; ++i) next[r + i] = i + 1 < L ? src[r + i + 1] : 0;
+            len[b] = L;
+            r += L;
         }
-        const T *h_last = static_cast<const T *>(c->h_all) + (size_t)(L - 1) * H;
-        gemm<T>(c, h_last, H, 1, H, one(c->w.lm_head, V, c->pk_lm), V, c->logits, V, EPI_STORE, s);
-        launch_argmax(c->logits, 1, V, c->argmax_tmp, s);
+    }
+    struct Chunk { long r0, d0; int n, nd, t0, nt, dt0, ndt; };
+    std::vector<Chunk> chunks;
+    long nd_all = 0;
+    int nt_all = 0, ndt_all = 0;
+    for (long r0 = 0; r0 < total; r0 += step) {
+        Chunk k{};
+        k.r0 = r0;
+        k.d0 = nd_all;
+        k.n = (int)std::min<long>(step, total - r0);
+        for (int i = 0; i < k.n; ++i) {
+            const RowDesc &d = rows[r0 + i];
+            if (d.plen == len[d.req]) {
+                draft[r0 + i] = -1 - d.req;
+            } else {
+                draft[r0 + i] = k.nd;
+                drows[nd_all + k.nd++] = d;
+            }
+        }
+        k.t0 = nt_all;
+        k.nt = row_tiles(rows + r0, k.n, tiles + nt_all);
+        k.dt0 = ndt_all;
+        k.ndt = row_tiles(drows + nd_all, k.nd, dtiles + ndt_all);
+        nt_all += k.nt;
+        ndt_all += k.ndt;
+        nd_all += k.nd;
+        chunks.push_back(k);
+    }
+    CU(cudaMemcpyAsync(c->pf_dev, c->pf_host, m.bytes, cudaMemcpyHostToDevice, s));
+    const RowDesc *rows_d = reinterpret_cast<const RowDesc *>(c->pf_dev + m.rows);
+    const RowDesc *drows_d = reinterpret_cast<const RowDesc *>(c->pf_dev + m.drows);
+    const int *src_d = reinterpret_cast<const int *>(c->pf_dev + m.src);
+    const int *next_d = reinterpret_cast<const int *>(c->pf_dev + m.next);
+    const int *draft_d = reinterpret_cast<const int *>(c->pf_dev + m.draft);
+    const int2 *tiles_d = reinterpret_cast<const int2 *>(c->pf_dev + m.tiles);
+    const int2 *dtiles_d = reinterpret_cast<const int2 *>(c->pf_dev + m.dtiles);
+    T *h = static_cast<T *>(c->h_all), *h_last = static_cast<T *>(c->xr);
+    const bool feat = c->cfg.draft_input == MSD_DRAFT_FEATURE;
+    for (const Chunk &k : chunks) {
+        // target over the chunk, causal
+        launch_embed_rows<T>(E, vis, src_d + k.r0, k.n, H, c->x, V, c->status, s);
+        for (int l = 0; l < c->NL; ++l) {
+            T *K = tkv<T>(c, c->target_kv, l, 0, c->S), *Vv = tkv<T>(c, c->target_kv, l, 1, c->S);
+            run_layer<T>(c, c->layers[l], c->lpack[l], k.n, rows_d + k.r0, K, Vv, c->S, K, Vv, c->S, nullptr, nullptr,
+                         0, nullptr, 0, k.n, s, false, nullptr, tiles_d + k.t0, k.nt);
+        }
+        launch_rmsnorm<T>(c->x, static_cast<const T *>(c->w.final_norm), k.n, H, c->cfg.rms_eps, h, c->lo, s);
         // draft cache over positions 0 .. L-2 with the decoupled input (Eq. 7): text
         // rows f_down(Concat(h, e_next)); visual rows e (MSD), the same
         // concatenation (Baseline) or h (Visual Feature), Sec. 5.3
-        for (int r0 = 0; r0 < L - 1; r0 += c->chunk) {
-            const int n = std::min(c->chunk, L - 1 - r0);
-            rd.resize(n);
-            for (int i = 0; i < n; ++i) rd[i] = RowDesc{b, r0 + i, r0 + i + 1, r0 + i};
-            CU(cudaMemcpyAsync(c->rows, rd.data(), sizeof(RowDesc) * n, cudaMemcpyHostToDevice, s));
-            launch_concat_next<T>(static_cast<const T *>(c->h_all) + (size_t)r0 * H,
-                                  static_cast<const T *>(c->emb_all) + (size_t)r0 * H, n, H,
-                                  static_cast<T *>(c->xfc), c->lo, s);
-            gemm<T>(c, static_cast<const T *>(c->xfc), 2 * H, n, 2 * H, one(c->w.draft_fc, H, c->pk_fc), H,
-                    c->x, H, EPI_STORE, s);
-            if (c->cfg.draft_input != MSD_DRAFT_CONCAT) {
-                const bool feat = c->cfg.draft_input == MSD_DRAFT_FEATURE;
-                const void *vis_rows = feat ? c->h_all : c->emb_all;
-                launch_select_visual<T>(c->x, static_cast<const T *>(vis_rows) + (size_t)r0 * H, feat ? c->lo : 0,
-                                        c->src + r0, n, H, s);
-            }
-            T *K = tkv<T>(c, c->draft_kv, 0, 0, c->S), *Vv = tkv<T>(c, c->draft_kv, 0, 1, c->S);
-            run_layer<T>(c, c->w.draft, c->dpack, n, c->rows, K, Vv, c->S, K, Vv, c->S, nullptr, nullptr, 0,
-                         nullptr, 0, n, s);
-            CU(cudaStreamSynchronize(s));
-        }
-        launch_prefill_finish<T>(c->argmax_tmp, h_last, b, L, D1, H, c->seq_len, c->n_pend, c->root,
-                                 c->pend_next, static_cast<T *>(c->pend_h), c->lo, root_out, s);
-        c->L_bound[b] = L;
+        launch_prefill_draft_in<T>(h, E, vis, draft_d + k.r0, next_d + k.r0, k.n, H, static_cast<T *>(c->xfc), h_last,
+                                   c->lo, s);
+        if (k.nd == 0) continue;
+        gemm<T>(c, static_cast<const T *>(c->xfc), 2 * H, k.nd, 2 * H, one(c->w.draft_fc, H, c->pk_fc), H, c->x, H,
+                EPI_STORE, s);
+        if (c->cfg.draft_input != MSD_DRAFT_CONCAT)
+            launch_select_visual<T>(c->x, h, vis, draft_d + k.r0, src_d + k.r0, feat, c->lo, k.n, H, s);
+        T *K = tkv<T>(c, c->draft_kv, 0, 0, c->S), *Vv = tkv<T>(c, c->draft_kv, 0, 1, c->S);
+        run_layer<T>(c, c->w.draft, c->dpack, k.nd, drows_d + k.d0, K, Vv, c->S, K, Vv, c->S, nullptr, nullptr, 0,
+                     nullptr, 0, k.nd, s, false, nullptr, dtiles_d + k.dt0, k.ndt);
     }
+    // the root tokens: one LM head over the requests' last features
+    gemm<T>(c, h_last, H, batch, H, one(c->w.lm_head, V, c->pk_lm), V, c->logits, V, EPI_STORE, s);
+    launch_argmax(c->logits, batch, V, c->argmax_tmp, s);
+    launch_prefill_finish<T>(c->argmax_tmp, h_last, reinterpret_cast<const int *>(c->pf_dev + m.len), batch, D1, H,
+                             c->seq_len, c->n_pend, c->root, c->pend_next, static_cast<T *>(c->pend_h), c->lo,
+                             root_out, s);
+    for (int b = 0; b < batch; ++b) c->L_bound[b] = seq_len_host[b];
     c->prefilled = true;
     c->draft_stale = false;
     return post_status(c, s);
@@ -562,8 +660,7 @@ msd_status verify_impl(msd_ctx *c, const msd_tree *tree, int32_t *argmax_dev, fl
     const int B = c->B, N = c->N, H = c->H, V = c->V, R = B * N;
     TreeIn t{tree->tokens, tree->parent, tree->depth, tree->mask, tree->n_nodes};
     launch_verify_setup(t, c->seq_len, c->root, B, N, V, c->rows, c->src, c->vmask, c->status, s);
-    launch_embed_rows<T>(static_cast<const T *>(c->w.embed), nullptr, c->src, R, H, c->x, nullptr,
-                         V, c->status, s);
+    launch_embed_rows<T>(static_cast<const T *>(c->w.embed), nullptr, c->src, R, H, c->x, V, c->status, s);
     bool folded = false;
     for (int l = 0; l < c->NL; ++l) {
         T *K = tkv<T>(c, c->target_kv, l, 0, c->S), *Vv = tkv<T>(c, c->target_kv, l, 1, c->S);
@@ -782,7 +879,7 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     c->C = c->k + (c->D - 1) * c->k * c->k;
     c->Td = std::max(1, (c->D - 1) * c->k);
     c->Wd = (c->Td + 63) / 64;
-    c->chunk = std::min(c->S, 1024);
+    c->chunk = (int)std::min<long>((long)c->B * c->S, PREFILL_CHUNK);
     c->Rmax = std::max(std::max(c->B * c->N, c->B * c->D1), std::max(c->B * c->k, c->chunk));
     c->Rlog = std::max(std::max(c->B * c->N, c->B * c->k), 1);
     c->L_bound.assign(c->B, 0);
@@ -804,7 +901,7 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
         {&c->xfc, R * 2 * H},
         {&c->xr, R * H},
         {&c->hT, (size_t)c->B * c->N * H},
-        {&c->h_all, (size_t)c->S * H},
+        {&c->h_all, (size_t)c->chunk * H},
     };
     if (cfg->dtype == MSD_BF16) {
         size_t total = 0;
@@ -832,11 +929,11 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     ok &= dalloc(c, &c->qkv, R * 3 * H * 4);
     c->ss_ld = (H + 127) / 128;
     ok &= dalloc(c, &c->ss_part, R * (size_t)c->ss_ld * 4);
-    ok &= dalloc(c, &c->gu, R * std::max<size_t>(2 * F, glu_rows(c->F)) * 4);
+    if (cfg->dtype == MSD_F32) ok &= dalloc(c, &c->gu, R * 2 * F * 4);
     ok &= dalloc(c, &c->logits, (size_t)c->Rlog * c->V * 4);
-    ok &= dalloc(c, &c->argmax_tmp, sizeof(int) * 4);
+    ok &= dalloc(c, &c->argmax_tmp, sizeof(int) * c->B);
     ok &= dalloc(c, &c->rows, sizeof(RowDesc) * R);
-    ok &= dalloc(c, &c->src, sizeof(int) * std::max<size_t>(R, c->S));
+    ok &= dalloc(c, &c->src, sizeof(int) * R);
     ok &= dalloc(c, &c->vmask, sizeof(uint64_t) * c->B * c->N * c->W);
     ok &= dalloc(c, &c->cand_tok, sizeof(int) * c->B * c->C);
     ok &= dalloc(c, &c->cand_par, sizeof(int) * c->B * c->C);
@@ -864,9 +961,11 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     ok &= dalloc(c, &c->ar_tree.n_nodes, sizeof(int) * c->B);
     ok &= dalloc(c, &c->ar_argmax, sizeof(int) * c->B * c->N);
     ok &= dalloc(c, &c->rope_tab, sizeof(float2) * (size_t)c->S * (c->hd / 2));
-    ok &= dalloc(c, &c->emb_all, (size_t)c->S * H * e);
+    c->pf_bytes = PrefillMeta((long)c->B * c->S, std::max(1, c->chunk / 2), c->B).bytes;
+    ok &= dalloc(c, &c->pf_dev, c->pf_bytes);
     ok &= dalloc(c, &c->status, sizeof(int));
-    if (ok) ok = cudaMallocHost(&c->status_host, sizeof(int)) == cudaSuccess;
+    if (ok) ok = cudaMallocHost(&c->pf_host, c->pf_bytes + sizeof(int)) == cudaSuccess;
+    if (ok) c->status_host = reinterpret_cast<int *>(c->pf_host + c->pf_bytes);
     if (ok) ok = cudaEventCreateWithFlags(&c->status_ev, cudaEventDisableTiming) == cudaSuccess;
     if (ok && cfg->dtype == MSD_F32) ok = gemm_simt_setup() && attention_setup();
     if (ok && cfg->dtype == MSD_BF16) ok = gemm_plan_create(&c->gplan, c->Rmax, c->H, c->F, c->V);
@@ -909,7 +1008,7 @@ msd_status msd_destroy(msd_ctx *c) {
     report_stale_error("msd_destroy");
     MSD_TEARDOWN(cudaDeviceSynchronize());
     for (void *p : c->allocs) MSD_TEARDOWN(cudaFree(p));
-    if (c->status_host) MSD_TEARDOWN(cudaFreeHost(c->status_host));
+    if (c->pf_host) MSD_TEARDOWN(cudaFreeHost(c->pf_host));
     if (c->status_ev) MSD_TEARDOWN(cudaEventDestroy(c->status_ev));
     if (c->gplan) gemm_plan_destroy(c->gplan);
     if (c->aplan) attn_tc_plan_destroy(c->aplan);
