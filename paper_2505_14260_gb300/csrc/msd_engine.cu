@@ -71,10 +71,11 @@ struct msd_ctx {
     // KV caches) is carved from one arena whose upper half holds the lo planes
     // of the split pairs; lo = that half's size in elements (0: fp32 context)
     long lo = 0;
-    int *status = nullptr;
-    int *status_host = nullptr;
-    cudaEvent_t status_ev = nullptr;
-    bool status_pending = false;
+    // the device status word lives in page-locked host memory, written by the GPU
+    // in place: no call copies it back
+    int *status = nullptr;                  // its device address
+    volatile int *status_host = nullptr;
+    bool status_pending = false;            // work that may set it has been launched since it was last reported
     GemmPlan *gplan = nullptr;
     AttnTcPlan *aplan = nullptr;
     // pre-packed GEMM weights (bf16 contexts)
@@ -145,23 +146,18 @@ bool report_stale_error(const char *where) {
 
 // The device status word of earlier calls, observed without blocking.
 msd_status check_status(msd_ctx *c) {
-    if (c->status_pending && cudaEventQuery(c->status_ev) == cudaSuccess) {
+    if (c->status_pending && *c->status_host != 0) {
         c->status_pending = false;
-        if (*c->status_host != 0) {
-            char buf[96];
-            snprintf(buf, sizeof buf, "device status word set (code %d)", *c->status_host);
-            return fail(c, MSD_ERR_DEVICE, buf);
-        }
+        char buf[96];
+        snprintf(buf, sizeof buf, "device status word set (code %d)", *c->status_host);
+        return fail(c, MSD_ERR_DEVICE, buf);
     }
     return MSD_OK;
 }
 
-msd_status post_status(msd_ctx *c, cudaStream_t s) {
+msd_status post_status(msd_ctx *c) {
     CU(cudaGetLastError());
-    if (c->capturing) return MSD_OK;    // the step's entry point posts after the replay
-    CU(cudaMemcpyAsync(c->status_host, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CU(cudaEventRecord(c->status_ev, s));
-    c->status_pending = true;
+    if (!c->capturing) c->status_pending = true;    // (recording: the step's entry point posts after the replay)
     return MSD_OK;
 }
 
@@ -564,7 +560,7 @@ msd_status prefill_impl(msd_ctx *c, int batch, const int32_t *seq_len_host, cons
     for (int b = 0; b < batch; ++b) c->L_bound[b] = seq_len_host[b];
     c->prefilled = true;
     c->draft_stale = false;
-    return post_status(c, s);
+    return post_status(c);
 }
 
 // ---------------------------------------------------------------------------
@@ -648,7 +644,7 @@ msd_status draft_impl(msd_ctx *c, const msd_tree *out, const msd_draft_record *r
     TreeOut t{out->tokens, out->parent, out->depth, out->mask, out->n_nodes};
     launch_tree_finalize(t, c->cand_tok, c->cand_par, c->cand_depth, c->cand_score, c->node_of,
                          c->root, B, c->C, c->N, c->status, s);
-    return post_status(c, s);
+    return post_status(c);
 }
 
 // ---------------------------------------------------------------------------
@@ -675,7 +671,7 @@ msd_status verify_impl(msd_ctx *c, const msd_tree *tree, int32_t *argmax_dev, fl
     gemm<T>(c, static_cast<const T *>(c->hT), H, R, H, one(c->w.lm_head, V, c->pk_lm), V, lg, V, EPI_STORE,
             s);
     launch_argmax(lg, R, V, argmax_dev, s);
-    return post_status(c, s);
+    return post_status(c);
 }
 
 // Compaction after an acceptance kernel has written acc_path / acc_L0 / acc_a:
@@ -689,7 +685,7 @@ msd_status compact_impl(msd_ctx *c, cudaStream_t s, int grow) {
                      static_cast<T *>(c->pend_h), c->lo, s);
     if (!c->capturing)
         for (int b = 0; b < c->B; ++b) c->L_bound[b] += grow < 0 ? c->D1 : grow;
-    return post_status(c, s);
+    return post_status(c);
 }
 
 template <typename T>
@@ -963,10 +959,14 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     ok &= dalloc(c, &c->rope_tab, sizeof(float2) * (size_t)c->S * (c->hd / 2));
     c->pf_bytes = PrefillMeta((long)c->B * c->S, std::max(1, c->chunk / 2), c->B).bytes;
     ok &= dalloc(c, &c->pf_dev, c->pf_bytes);
-    ok &= dalloc(c, &c->status, sizeof(int));
-    if (ok) ok = cudaMallocHost(&c->pf_host, c->pf_bytes + sizeof(int)) == cudaSuccess;
-    if (ok) c->status_host = reinterpret_cast<int *>(c->pf_host + c->pf_bytes);
-    if (ok) ok = cudaEventCreateWithFlags(&c->status_ev, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) ok = cudaHostAlloc(&c->pf_host, c->pf_bytes + sizeof(int), cudaHostAllocMapped) == cudaSuccess;
+    if (ok) {
+        c->status_host = reinterpret_cast<int *>(c->pf_host + c->pf_bytes);
+        *c->status_host = 0;
+        void *mapped = nullptr;
+        ok = cudaHostGetDevicePointer(&mapped, const_cast<int *>(c->status_host), 0) == cudaSuccess;
+        c->status = static_cast<int *>(mapped);
+    }
     if (ok && cfg->dtype == MSD_F32) ok = gemm_simt_setup() && attention_setup();
     if (ok && cfg->dtype == MSD_BF16) ok = gemm_plan_create(&c->gplan, c->Rmax, c->H, c->F, c->V);
     if (ok && cfg->dtype == MSD_BF16) ok = attn_tc_plan_create(&c->aplan);
@@ -977,7 +977,6 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
         cudaGetLastError();
         return MSD_ERR_OOM;
     }
-    *c->status_host = 0;
     // RoPE table: (cos, sin) of pos * base^(-2i/hd), computed in double.
     std::vector<float2> tab((size_t)c->S * (c->hd / 2));
     for (int p = 0; p < c->S; ++p)
@@ -1009,7 +1008,6 @@ msd_status msd_destroy(msd_ctx *c) {
     MSD_TEARDOWN(cudaDeviceSynchronize());
     for (void *p : c->allocs) MSD_TEARDOWN(cudaFree(p));
     if (c->pf_host) MSD_TEARDOWN(cudaFreeHost(c->pf_host));
-    if (c->status_ev) MSD_TEARDOWN(cudaEventDestroy(c->status_ev));
     if (c->gplan) gemm_plan_destroy(c->gplan);
     if (c->aplan) attn_tc_plan_destroy(c->aplan);
     for (auto &g : c->graphs)
@@ -1138,7 +1136,7 @@ msd_status run_step_graph(msd_ctx *c, int kind, const msd_tree *tree, int32_t *a
     // While GEMM profiling is on, steps run eagerly (events bracket each GEMM).
     if (c->cfg.dtype == MSD_BF16 && c->gplan && gemm_profile_on(c->gplan)) {
         st = step_kind_eager(c, kind, tree, argmax_dev, path_dev, accept_len_dev, bonus_dev, sa, s);
-        return st == MSD_OK ? post_status(c, s) : st;
+        return st == MSD_OK ? post_status(c) : st;
     }
     const bool stamped = c->gplan && gemm_stamp_on(c->gplan);
     msd_ctx::StepGraph *g = nullptr;
@@ -1194,7 +1192,7 @@ msd_status run_step_graph(msd_ctx *c, int kind, const msd_tree *tree, int32_t *a
     g->uses += 1;
     c->graph_kernels += g->kernels;
     for (int b = 0; b < c->B; ++b) c->L_bound[b] += grow;
-    return post_status(c, s);
+    return post_status(c);
 }
 
 }  // namespace
@@ -1308,7 +1306,7 @@ msd_status msd_linear(msd_ctx *c, const void *x, int32_t ldx, int32_t m, int32_t
         gemm<bf16>(c, static_cast<const bf16 *>(x), ldx, m, k, W, o, y, ldy, epi, s, false);
     } else
         gemm<float>(c, static_cast<const float *>(x), ldx, m, k, W, o, y, ldy, epi, s);
-    return post_status(c, s);
+    return post_status(c);
 }
 
 msd_status msd_profile_enable(msd_ctx *c, int32_t mode) {
@@ -1373,7 +1371,7 @@ msd_status msd_tree_complete(msd_ctx *c, const msd_tree *tree, int32_t request, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int b0 = request < 0 ? 0 : request, nb = request < 0 ? c->B : 1;
     launch_tree_complete(tree->parent, tree->depth, tree->mask, tree->n_nodes, b0, nb, c->N, c->status, s);
-    return post_status(c, s);
+    return post_status(c);
 }
 
 msd_status msd_test_wait_timeout(msd_ctx *c, int64_t limit_ns, void *stream) {
@@ -1384,7 +1382,7 @@ msd_status msd_test_wait_timeout(msd_ctx *c, int64_t limit_ns, void *stream) {
     int *status = c ? c->status : noalloc_status_word();
     if (!status) return MSD_ERR_CUDA;
     if (!launch_wait_probe(status, (long long)limit_ns, s)) return fail(c, MSD_ERR_CUDA, "probe launch failed");
-    return c ? post_status(c, s) : MSD_OK;
+    return c ? post_status(c) : MSD_OK;
 }
 
 msd_status msd_state(msd_ctx *c, msd_state_view *out) {
