@@ -315,13 +315,15 @@ cudaError_t launch_as(AsArgs p, int num_sms, cudaStream_t s) {
     lc.blockDim = dim3(AS_THREADS);
     lc.dynamicSmemBytes = AsLay<HD, QR>::SMEM;
     lc.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = (unsigned)p.nsplit;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
-    lc.numAttrs = 1;
+    lc.numAttrs = programmatic(s) ? 2 : 1;
     return cudaLaunchKernelEx(&lc, attn_simt_kernel<HD, QR>, (const AsArgs)p);
 }
 

@@ -56,11 +56,21 @@ __device__ __forceinline__ void wait_prior() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Launches a short kernel in plain stream order behind the previous one. (With
-// programmatic serialization these kernels' griddepcontrol.wait returned
-// later than a plain launch starts: measured slower.) The kernel still calls
-// wait_prior(), a no-op here, and allow_dependents(), which lets a following
-// programmatic launch (the tensor-core GEMMs) start early.
+// Whether a launch on `s` should use programmatic stream serialization. Behind
+// another kernel of a stream, a plain launch of a small kernel waited for the next
+// of about 2 us long intervals (6.2, 8.2, 10.3 us a launch back to back, whatever
+// the kernel did in between); a programmatic one starts when the kernel behind it
+// is done. In a recorded graph plain edges have no such step and the programmatic
+// wait returns later than a plain node starts, so launches being captured stay
+// plain.
+inline bool programmatic(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+}
+
+// Launches a short kernel behind the previous one (see programmatic). The kernel
+// calls wait_prior() before it reads or writes anything another may touch, and
+// allow_dependents() after that.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                 cudaStream_t s, Args &&...args) {
@@ -69,6 +79,11 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     lc.blockDim = block;
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = programmatic(s) ? 1 : 0;
     return cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
 }
 

@@ -81,6 +81,7 @@ template <class TL, bool VEC>
 __global__ void __launch_bounds__(SG_THREADS) gemm_simt_kernel(const SgArgs a) {
     extern __shared__ __align__(16) float sm[];
     wait_prior();
+    allow_dependents();
     const int tid = threadIdx.x;
     const int o0 = blockIdx.x * TL::BO, m0 = blockIdx.y * TL::BM, split = blockIdx.z;
     const int nb = (a.K + SG_BK - 1) / SG_BK;                     // k blocks
@@ -218,13 +219,15 @@ void launch_tile(SgArgs a, int num_sms, cudaStream_t s) {
     lc.blockDim = dim3(SG_THREADS);
     lc.dynamicSmemBytes = TL::SMEM;
     lc.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = (unsigned)S;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
-    lc.numAttrs = 1;
+    lc.numAttrs = programmatic(s) ? 2 : 1;
     cudaLaunchKernelEx(&lc, gemm_simt_kernel<TL, VEC>, (const SgArgs)a);
     note_launch();
 }
