@@ -1173,17 +1173,33 @@ __global__ void __launch_bounds__(C_THREADS)
     const uint32_t recv_bar = smem_u32(&bars[2 * C_STAGES + 1]);   // the other ranks' slices have landed
     const uint32_t pexit = smem_u32(&bars[2 * C_STAGES + 2]);      // (pair) the other CTA is done with its TMEM
 
-    if (threadIdx.x == 0) {
-        stamp_min(p.stamp, 0);
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(full0 + 8 * s, 1);
-            mbar_init(empty0 + 8 * s, 1);
+    // Warp 0's elected lane sets the barriers up and, where the copies complete on
+    // this CTA's own barriers, requests the first weight blocks at once (packed
+    // weights depend on no earlier kernel): not after the tensor-memory allocation,
+    // which waits while CTAs of the previous kernel still hold theirs.
+    uint32_t on = 0;
+    const int n_pre = RAW ? 0 : min(stages, nk);
+    const uint32_t stage_tx = (pair ? 2u : 1u) * (A_BYTES + bs_bytes);
+    if (warp == 0) {
+        on = elect_one();
+        if (on) {
+            stamp_min(p.stamp, 0);
+            for (int s = 0; s < stages; ++s) {
+                mbar_init(full0 + 8 * s, 1);
+                mbar_init(empty0 + 8 * s, 1);
+            }
+            mbar_init(done, 1);
+            mbar_init(recv_bar, 1);
+            mbar_init(pexit, 1);
+            abort_flag = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
-        mbar_init(done, 1);
-        mbar_init(recv_bar, 1);
-        mbar_init(pexit, 1);
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        __syncwarp();
+        if constexpr (!pair)
+            for (int j = 0; j < n_pre; ++j) {
+                w_expect_tx(on, full0 + 8 * j, stage_tx);
+                w_bulk_load(on, a_base + j * A_BYTES, wblk + (size_t)j * blk_elems, A_BYTES, full0 + 8 * j);
+            }
     }
     if (warp == 1) {
         if constexpr (pair) {   // both CTAs of the pair allocate together (the same columns in each)
@@ -1209,12 +1225,10 @@ __global__ void __launch_bounds__(C_THREADS)
     const uint16_t pair_mask = (uint16_t)(3u << lead_rank);
     // where this CTA's copies complete: its own barriers, or (pair) the even CTA's
     const uint32_t sig0 = pair ? c_mapa(full0, lead_rank) : full0;
-    const uint32_t stage_tx = (pair ? 2u : 1u) * (A_BYTES + bs_bytes);
     // (pair) both CTAs' barriers are initialised before either signals the other's
     if constexpr (pair) c_cluster_sync();
 
     if (warp == 0) {
-        const uint32_t on = elect_one();
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&mx) : "memory");
             if (has_lo) asm volatile("prefetch.tensormap [%0];" ::"l"(&mxl) : "memory");
@@ -1234,9 +1248,9 @@ __global__ void __launch_bounds__(C_THREADS)
             else
                 w_bulk_load(on, a_base + st * A_BYTES, wblk + (size_t)i * blk_elems, A_BYTES, full0 + 8 * st);
         };
-        // weights first (they never depend on the previous kernel), then wait
-        const int n_pre = RAW ? 0 : min(stages, nk);
-        for (int j = 0; j < n_pre; ++j) load_w(j, j);
+        // (pair) the first weight blocks, then the wait on the previous kernel
+        if constexpr (pair)
+            for (int j = 0; j < n_pre; ++j) load_w(j, j);
         pdl_wait();
         if (lane == 0) stamp_min(p.stamp, 1);
         pdl_trigger();
