@@ -306,6 +306,7 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t *r, int gw
 // ---------------------------------------------------------------------------
 constexpr int P_THREADS = 192;
 constexpr int P_MAX_STAGES = 12;
+constexpr int P_MAX_ACC = 8;
 constexpr int P_MAX_PIECES = 128;   // pieces of one cut tile (CTAs sharing it)
 
 struct PkParams {
@@ -319,6 +320,8 @@ struct PkParams {
     int T_sk, dp_rounds;    // stream-K tiles; rounds of whole tiles after them
     int T_all;              // all 256-row tiles x token tiles
     int kb_chunk;           // K-blocks of a whole tile accumulated before they are added to Y
+    int n_acc;              // accumulators the items take in turn
+    int fold;               // a pair's only tile: its chunks stay in their accumulators and are summed at the end
     float *Y;
     int ldy, epi;
     float *ws;
@@ -396,7 +399,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     gemm_persist_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mxl,
                         const __grid_constant__ CUtensorMap mw, const PkParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * P_MAX_STAGES + 5];
+    __shared__ __align__(8) uint64_t bars[2 * P_MAX_STAGES + 2 * P_MAX_ACC + 1];
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
     __shared__ int s_reduce;
@@ -418,8 +421,8 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     const uint32_t a_base = sbase, b_base = sbase + stages * A_BYTES;
     const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[P_MAX_STAGES]);
     const uint32_t accf0 = smem_u32(&bars[2 * P_MAX_STAGES]);
-    const uint32_t acce0 = smem_u32(&bars[2 * P_MAX_STAGES + 2]);
-    const uint32_t drain = smem_u32(&bars[2 * P_MAX_STAGES + 4]);
+    const uint32_t acce0 = smem_u32(&bars[2 * P_MAX_STAGES + P_MAX_ACC]);
+    const uint32_t drain = smem_u32(&bars[2 * P_MAX_STAGES + 2 * P_MAX_ACC]);
 
     if (threadIdx.x == 0) {
         stamp_min(p.stamp, 0);
@@ -427,7 +430,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             mbar_init(full0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < p.n_acc; ++a) {
             mbar_init(accf0 + 8 * a, 1);
             mbar_init(acce0 + 8 * a, 8);        // the epilogue warps of both CTAs
         }
@@ -532,10 +535,10 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             int t, kb_b, kb_e, s = 0;
             uint32_t ph = 0;
             bool stop = false;
-            for (int item = 0; !stop && it.next(t, kb_b, kb_e); ++item) {
-                const int a = item & 1;
-                if (!w_mbar_wait_cluster(acce0 + 8 * a, (uint32_t)((item >> 1) & 1) ^ 1u, &abort_flag, p.status))
-                    break;
+            int a = 0;                      // the item's accumulator and its phase
+            uint32_t aph = 0;
+            for (; !stop && it.next(t, kb_b, kb_e); a = a + 1 == p.n_acc ? (aph ^= 1u, 0) : a + 1) {
+                if (!w_mbar_wait_cluster(acce0 + 8 * a, aph ^ 1u, &abort_flag, p.status)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem + a * p.acc_stride;
                 uint32_t more = 0;          // the item's first MMA starts the accumulator
@@ -583,8 +586,10 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         const int et = threadIdx.x - 64;     // 0..127
         ItemIter it = items0;
         int t, kb_b, kb_e;
-        for (int item = 0; it.next(t, kb_b, kb_e); ++item) {
-            const int a = item & 1;
+        int a = 0;
+        uint32_t aph = 0;
+        for (int item = 0; it.next(t, kb_b, kb_e); ++item, a = a + 1 == p.n_acc ? (aph ^= 1u, 0) : a + 1) {
+            if (p.fold && kb_e < KB) continue;      // (summed with the tile's last chunk)
             int wt, seg, row0, n0;
             tile_geom(t, wt, seg, row0, n0);
             const int o_local = row0 + row;
@@ -596,7 +601,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             const int slot = 2 * (2 * cta + (item == 0 ? 0 : 1)) + half;
             float *part = p.ws + (size_t)slot * BN * BM;
             // (a whole tile's later chunks add to what this thread stored for the first)
-            const bool add = p.epi == EPI_ADD || (whole && kb_b > 0);
+            const bool add = p.epi == EPI_ADD || (whole && kb_b > 0 && !p.fold);
             const bool glu = p.epi == EPI_SWIGLU;
             float *stg = reinterpret_cast<float *>(smem_raw + p.stg_off);   // [32 columns][128 rows]
             // residual rows of 32 columns, requested one group ahead (the first
@@ -609,8 +614,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             };
             float ynext[32];
             residual(0, ynext);
-            const bool landed = mbar_wait_cluster(accf0 + 8 * a, (uint32_t)(item >> 1) & 1u, &abort_flag,
-                                                  p.status) && !abort_flag;
+            bool landed = mbar_wait_cluster(accf0 + 8 * a, aph, &abort_flag, p.status) && !abort_flag;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const bool ok = landed && wt < p.tiles, row_ok = landed && row_in;
             for (int g0 = 0; g0 < BN; g0 += 32) {
@@ -622,6 +626,14 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 if (g0 + 32 < BN) residual(g0 + 32, ynext);
                 uint32_t r[32];
                 tmem_ld_cols(taddr + g0, r, gw);
+                if (p.fold)             // the earlier chunks' accumulators, in K order before this one's
+                    for (int q = a - 1; q >= 0; --q) {
+                        uint32_t e[32];
+                        tmem_ld_cols(tmem + q * p.acc_stride + ((uint32_t)(32 * (warp & 3)) << 16) + g0, e, gw);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            r[j] = __float_as_uint(__uint_as_float(e[j]) + __uint_as_float(r[j]));
+                    }
                 if (whole && glu) {
                     // gate row i and up row 64 + i of the tile sit in different
                     // warps: exchange through shared memory, then thread (i, h)
@@ -2165,10 +2177,12 @@ constexpr int P_STAGES = 6;
 // even, but the pieces' round trip through the workspace then costs 330 BN
 // where every tile is cut (O at 640 rows, 224 columns: 68 us against 40 in whole
 // tiles), about 180 BN where whole tiles follow to hide part of it.
-// A one-plane product (msd_linear) accumulates at most 24 K-blocks of a whole
-// tile in tensor memory before it adds them to Y: the accumulators truncate, so
-// the error grows with the chain (4096-long products: 2.2e-6 relative in pieces
-// of 32 to 40 blocks, 4.4e-6 in one of 64).
+// A one-plane product (msd_linear) accumulates short chains of K-blocks: the
+// accumulators truncate, so the error grows with the chain (4096-long products:
+// 2.2e-6 relative in chains of 32 to 40 blocks, 4.4e-6 in one of 64). A pair's only
+// tile keeps its chunks in accumulators of their own, up to the 512 TMEM columns,
+// summed by its epilogue; otherwise chunks of 24 blocks are added to Y one after
+// another (576 x 4096 x 4096: 34 us added, 22 us kept).
 static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int pairs, size_t ws_bytes,
                                   int n_counters) {
     const int kblocks = (K + BK - 1) / BK, wt = (tiles + 1) / 2;
@@ -2181,7 +2195,15 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
         const double tk = std::max(2.08 * nb * BN, 420.0 + 0.8 * nb * BN);
         // at least 4 K-blocks a pair
         const long long G = std::max<long long>(1, std::min<long long>(pairs, T * kblocks / 4));
-        const int chunk = nb == 1 && !glu ? (kblocks + (kblocks + 23) / 24 - 1) / ((kblocks + 23) / 24) : kblocks;
+        int n_ch = 1;
+        if (nb == 1 && !glu) {
+            int stride = 32;
+            while (stride < BN) stride <<= 1;
+            const int most = T <= G ? std::min(512 / stride, P_MAX_ACC) : 1;    // accumulators of a pair's only tile
+            n_ch = (kblocks + 15) / 16;
+            if (n_ch > most) n_ch = (kblocks + 31) / 32 <= most ? most : (kblocks + 23) / 24;
+        }
+        const int chunk = (kblocks + n_ch - 1) / n_ch;
         PersistShape g{BN, nt, (int)G, (int)T, 0, (int)((T + G - 1) / G), chunk};
         double cost = g.dp_rounds * tk * kblocks;
         int rounds = (int)(T / G), T_sk = (int)(T - rounds * G);
@@ -2242,7 +2264,14 @@ static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     pk.n_tiles_n = nt;
     pk.stages = stages;
     pk.acc_stride = acc;
-    pk.tmem_cols = 2 * acc;
+    pk.n_acc = 2;
+    const int chunks = (kblocks + g.kb_chunk - 1) / g.kb_chunk;
+    if (chunks > 1 && g.T_sk == 0 && g.dp_rounds == 1 && chunks <= std::min(512 / acc, P_MAX_ACC)) {
+        pk.fold = 1;
+        pk.n_acc = std::max(2, chunks);
+    }
+    pk.tmem_cols = 64;
+    while (pk.tmem_cols < pk.n_acc * acc) pk.tmem_cols <<= 1;
     pk.grid = G;
     pk.tiles = tiles;
     pk.units = units;

@@ -260,6 +260,10 @@ __device__ __forceinline__ void warp_topk_rounds(float (&v)[NS], int (&ix)[NS], 
 template <int NS>
 __device__ __forceinline__ void warp_topk(float (&v)[NS], int (&ix)[NS], int k, float *out_v, int *out_i,
                                           float *scr_v, int *scr_i) {
+    if (k <= 6) {       // few rounds are shorter than ranking the 32 heads and the compacted slots
+        warp_topk_rounds<NS>(v, ix, k, out_v, out_i);
+        return;
+    }
     const int lane = threadIdx.x & 31;
     float hv = -INFINITY;
     int hi = TK_NONE;
@@ -307,7 +311,8 @@ __device__ __forceinline__ void warp_topk(float (&v)[NS], int (&ix)[NS], int k, 
         const float cv = scr_v[lane];
         const int ci = scr_i[lane];
         int r = 0;
-        for (int j = 0; j < total; ++j) r += better(scr_v[j], scr_i[j], cv, ci);
+#pragma unroll 8
+        for (int j = 0; j < 32; ++j) r += j < total && better(scr_v[j], scr_i[j], cv, ci);
         if (r < k) { out_v[r] = cv; out_i[r] = ci; }
     } else if (lane < k) {
         out_v[lane] = -INFINITY;
