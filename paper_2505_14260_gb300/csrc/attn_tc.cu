@@ -13,7 +13,8 @@
 //                   swizzle) into a three-stage shared-memory ring
 //   warp 1          allocates tensor memory; lane 0 issues the MMAs
 //   warps 2-9       two per TMEM lane quarter (an M = 64 accumulator keeps
-//                   rows 16q .. 16q+15 in lanes 0-15 of quarter q), each
+//                   rows 16q .. 16q+15 in lanes 0-15 of quarter q, read in matrix
+//                   fragments so that all 32 threads of a warp have work), each
 //                   taking half of a tile's keys and of O's columns: load the
 //                   query rows into TMEM, then per key tile read S, mask it
 //                   (prefix length, tree bitmask), run the online softmax in
@@ -185,43 +186,69 @@ __device__ __forceinline__ bool w_bar_wait(uint32_t bar, uint32_t parity, volati
     return __all_sync(0xffffffffu, bar_wait(bar, parity, abort, status));
 }
 
-// 32 columns of this warp's lanes, waited for in the same asm statement: the
-// compiler sees the registers defined only once the data has landed.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *r) {
+// Tensor-memory access. An M = 64 accumulator keeps 16 rows in lanes 0-15 of
+// each lane quarter, so a row-per-lane load leaves half of a warp idle. The
+// 16-lane shapes give every thread work, in the fragment layout of a matrix
+// product: in each 8 columns of a 16x256b load, thread t holds columns 2 (t % 4)
+// and the next of row t / 4 in registers 0 and 1, of row t / 4 + 8 in 2 and 3; in
+// each 4 (32-bit) columns of a 16x128b store, column t % 4 of those two rows.
+// Each is waited for in the same asm statement: the compiler sees a load's
+// registers defined only once the data has landed, and reuses a store's only
+// after the tensor memory has taken them.
+__device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, uint32_t *r) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {"
+        "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
         "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-          "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+          "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
 }
-
-
-// Stores of 32 / 16 columns, waited for in the same asm statement, so the
-// source registers are not reused before the tensor memory has taken them.
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *r) {
+__device__ __forceinline__ void tmem_ld_frag64(uint32_t taddr, uint32_t *r) {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n"
+        "tcgen05.ld.sync.aligned.16x256b.x8.b32 {"
+        "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+          "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+          "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+          "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_frag32(uint32_t taddr, const uint32_t *r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {"
+        "%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
         "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
-        "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
-        "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
+        "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]),
+        "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_pairs16(uint32_t taddr, const uint32_t *r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {"
+        "%1,%2,%3,%4,%5,%6,%7,%8};\n"
+        "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
+        "r"(r[7])
         : "memory");
 }
 
+// 16 columns of this warp's 32 lanes (the query rows)
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *r) {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {"
+        "%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
         "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
+        "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]),
+        "r"(r[14]), "r"(r[15])
         : "memory");
 }
 
@@ -503,8 +530,25 @@ __global__ void __launch_bounds__(THREADS, 1)
     };
     const int hf = (warp - 2) >> 2;                   // column half of a softmax warp
     constexpr int OH = HD / 2;                        // O columns per half
-    uint32_t o_acc[OH];                               // this half of the row's O (fp32 bits)
-    float m_used = -INFINITY, l_sum = 0.f;
+    // fragment rows of this thread: t / 4 and t / 4 + 8 of its quarter's 16
+    const int fr = 16 * quarter + (lane >> 2), fc = 2 * (lane & 3);
+    // this half of O in fragments, 32 or 64 columns at a time
+    auto o_load = [&](uint32_t addr, uint32_t *r) {
+        if constexpr (OH == 64) tmem_ld_frag64(addr, r);
+        else tmem_ld_frag32(addr, r);
+    };
+    auto o_scale = [&](uint32_t addr, const float *f) {
+#pragma unroll
+        for (int c0 = 0; c0 < OH; c0 += 32) {
+            uint32_t r[16];
+            tmem_ld_frag32(addr + c0, r);
+#pragma unroll
+            for (int x = 0; x < 16; ++x) r[x] = __float_as_uint(__uint_as_float(r[x]) * f[(x >> 1) & 1]);
+            tmem_st_frag32(addr + c0, r);
+        }
+    };
+    uint32_t o_acc[OH / 2];                           // fragments of this half of O (fp32 bits)
+    float m_used[2] = {-INFINITY, -INFINITY}, l_sum[2] = {0.f, 0.f};
     bool dead = false;
     if (smx) {
         // query row (hi, lo) into tensor memory, the A operand of Q K^T: this
@@ -529,70 +573,97 @@ __global__ void __launch_bounds__(THREADS, 1)
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             bar_arrive(q_ready);
         }
-        const uint64_t *mrow = (has_tree_tiles && valid) ? p.mask + (size_t)row * p.mask_words : nullptr;
-        const int klim = valid ? min(k_hi, plen) : 0;        // cache keys visible by position
-        const int tlim = valid ? p.tree_slots : 0;           // tree keys: by the ancestor mask
+        int klim[2], tlim[2];                                // visible keys by position; tree slots
+        const uint64_t *mrow[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int rr = r0 + fr + 8 * i;
+            const bool in = rr < r_end;
+            klim[i] = in ? min(k_hi, p.rows[rr].plen) : 0;
+            tlim[i] = in ? p.tree_slots : 0;
+            mrow[i] = has_tree_tiles && in ? p.mask + (size_t)rr * p.mask_words : nullptr;
+        }
         for (int j = 0; j < ntiles; ++j) {
             if (!dead && !wwait(s_full0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u)) dead = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t sd = tq + L::T_S + (j & 1) * KT;
-            uint32_t sr[32];
-            tmem_ld32(sd + 32 * hf, sr);
+            uint32_t sr[16];
+            tmem_ld_frag32(sd + 32 * hf, sr);
             const bool tree_tile = j >= nc;
             const int key0 = (tree_tile ? (j - nc) * KT : k_lo + j * KT) + 32 * hf;
-            const int lim = (tree_tile ? tlim : klim) - key0;   // columns c < lim are inside the range
-            uint32_t bits = 0xffffffffu;
-            if (tree_tile) {
-                const int w = j - nc;                           // one mask word per 64 tree keys
-                bits = (mrow && w < p.mask_words) ? (uint32_t)(mrow[w] >> (32 * hf)) : 0u;
-            }
-            float v[32];
-            float mx = -INFINITY;
+            float mx[2] = {-INFINITY, -INFINITY};
+            float v[16];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-                const bool vis = c < lim && ((bits >> c) & 1u);
-                v[c] = vis ? __uint_as_float(sr[c]) * p.scale_log2 : -INFINITY;
-                mx = fmaxf(mx, v[c]);
+            for (int i = 0; i < 2; ++i) {
+                const int lim = (tree_tile ? tlim[i] : klim[i]) - key0;     // columns c < lim are inside the range
+                uint32_t bits = 0xffffffffu;
+                if (tree_tile) {
+                    const int w = j - nc;                                   // one mask word per 64 tree keys
+                    bits = mrow[i] && w < p.mask_words ? (uint32_t)(mrow[i][w] >> (32 * hf)) : 0u;
+                }
+                if (lim < 32) bits &= lim <= 0 ? 0u : (1u << lim) - 1u;
+                bits >>= fc;
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int x = 4 * n + 2 * i + e;
+                        v[x] = (bits >> (8 * n + e)) & 1u ? __uint_as_float(sr[x]) * p.scale_log2 : -INFINITY;
+                        mx[i] = fmaxf(mx[i], v[x]);
+                    }
             }
-            // the row's tile maximum over both halves
+            // the rows' tile maxima over the quad's columns, then over both halves
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 1));
+                mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 2));
+            }
             float *xm = s_xmax + ((j & 1) * 2 + hf) * ROWS;
-            if (lane < 16) xm[row_local] = mx;
+            if ((lane & 3) == 0) {
+                xm[fr] = mx[0];
+                xm[fr + 8] = mx[1];
+            }
             softmax_sync(quarter);
-            if (lane < 16) mx = fmaxf(mx, s_xmax[((j & 1) * 2 + (hf ^ 1)) * ROWS + row_local]);
+            const float *xo = s_xmax + ((j & 1) * 2 + (hf ^ 1)) * ROWS;
+            mx[0] = fmaxf(mx[0], xo[fr]);
+            mx[1] = fmaxf(mx[1], xo[fr + 8]);
             // move the reference maximum only when the tile's exceeds it by > 2^8
             // (and O already holds visible keys: otherwise O is exactly 0). The
             // rescale waits for P V of tile j-1 on o_ready: the completed Q K^T of
             // tile j implies P V of tile j-2, so the barrier is at most one phase
             // behind and its parity names the phase.
-            const bool need = m_used != -INFINITY && mx > m_used + RESCALE_LOG2;
-            if (__any_sync(0xffffffffu, need)) {
+            bool need[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) need[i] = m_used[i] != -INFINITY && mx[i] > m_used[i] + RESCALE_LOG2;
+            if (__any_sync(0xffffffffu, need[0] || need[1])) {
                 if (!dead && !wwait(o_ready, (uint32_t)(j - 1) & 1u)) dead = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const float f = need ? ex2_fast(m_used - mx) : 1.f;
+                float f[2];
 #pragma unroll
-                for (int c0 = 0; c0 < OH; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld32(tq + L::T_O + hf * OH + c0, r);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
-                    tmem_st32(tq + L::T_O + hf * OH + c0, r);
+                for (int i = 0; i < 2; ++i) {
+                    f[i] = need[i] ? ex2_fast(m_used[i] - mx[i]) : 1.f;
+                    l_sum[i] *= f[i];
+                    if (need[i]) m_used[i] = mx[i];
                 }
-                l_sum *= f;
-                if (need) m_used = mx;
+                o_scale(tq + L::T_O + hf * OH, f);
             }
-            if (m_used == -INFINITY) m_used = mx;
-            const float use = m_used == -INFINITY ? 0.f : m_used;
-            float rs = 0.f;
-            uint32_t ph[16], pl[16];
+            float use[2];
 #pragma unroll
-            for (int c = 0; c < 32; c += 2) {
-                const float e0 = ex2_fast(v[c] - use), e1 = ex2_fast(v[c + 1] - use);
-                rs += e0 + e1;
-                split_pair(e0, e1, ph[c / 2], pl[c / 2]);
+            for (int i = 0; i < 2; ++i) {
+                if (m_used[i] == -INFINITY) m_used[i] = mx[i];
+                use[i] = m_used[i] == -INFINITY ? 0.f : m_used[i];
             }
-            l_sum += rs;
-            tmem_st16(sd + 32 * hf, ph);                  // over this half's own S columns:
-            tmem_st16(sd + 32 * hf + 16, pl);             // hi pairs, then lo pairs
+            uint32_t ph[8], pl[8];
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float e0 = ex2_fast(v[4 * n + 2 * i] - use[i]), e1 = ex2_fast(v[4 * n + 2 * i + 1] - use[i]);
+                    l_sum[i] += e0 + e1;
+                    split_pair(e0, e1, ph[2 * n + i], pl[2 * n + i]);
+                }
+            tmem_st_pairs16(sd + 32 * hf, ph);            // over this half's own S columns:
+            tmem_st_pairs16(sd + 32 * hf + 16, pl);       // hi pairs, then lo pairs
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             bar_arrive(p_full0 + 8 * (j & 1));
         }
@@ -602,30 +673,47 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!dead && ntiles > 0 && !wwait(drain, 0u)) dead = true;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (ntiles > 0) {
-#pragma unroll
-            for (int c0 = 0; c0 < OH; c0 += 32) tmem_ld32(tq + L::T_O + hf * OH + c0, o_acc + c0);
+            o_load(tq + L::T_O + hf * OH, o_acc);
         } else {
 #pragma unroll
-            for (int c = 0; c < OH; ++c) o_acc[c] = 0u;
+            for (int c = 0; c < OH / 2; ++c) o_acc[c] = 0u;
         }
-        // the row's sum over both halves
-        if (lane < 16) s_xmax[(4 + hf) * ROWS + row_local] = l_sum;
+        // the rows' sums over the quad, then over both halves
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            l_sum[i] += __shfl_xor_sync(0xffffffffu, l_sum[i], 1);
+            l_sum[i] += __shfl_xor_sync(0xffffffffu, l_sum[i], 2);
+        }
+        if ((lane & 3) == 0) {
+            s_xmax[(4 + hf) * ROWS + fr] = l_sum[0];
+            s_xmax[(4 + hf) * ROWS + fr + 8] = l_sum[1];
+        }
         softmax_sync(quarter);
-        if (lane < 16) l_sum += s_xmax[(4 + (hf ^ 1)) * ROWS + row_local];
+        // (half 0's sum first, so both halves hold the same value)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            l_sum[i] = s_xmax[4 * ROWS + fr + 8 * i] + s_xmax[5 * ROWS + fr + 8 * i];
     }
     const bool ok = !dead && !abort_flag;
 
     const int nsplit = p.nsplit;
     if (nsplit == 1) {
-        if (valid && ok) {
-            const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
-            bf16 *dst = p.out + (size_t)row * H + h * HD + hf * OH;
+        if (smx && ok) {
 #pragma unroll
-            for (int c = 0; c < OH; c += 4)
-                Split<bf16>::store4(dst + c, p.lo,
-                                    make_float4(__uint_as_float(o_acc[c]) * inv, __uint_as_float(o_acc[c + 1]) * inv,
-                                                __uint_as_float(o_acc[c + 2]) * inv,
-                                                __uint_as_float(o_acc[c + 3]) * inv));
+            for (int i = 0; i < 2; ++i) {
+                const int rr = r0 + fr + 8 * i;
+                if (rr >= r_end) continue;
+                const float inv = l_sum[i] > 0.f ? 1.f / l_sum[i] : 0.f;
+                bf16 *dst = p.out + (size_t)rr * H + h * HD + hf * OH + fc;
+#pragma unroll
+                for (int n = 0; n < OH / 8; ++n) {
+                    uint32_t hi, lo;
+                    split_pair(__uint_as_float(o_acc[4 * n + 2 * i]) * inv,
+                               __uint_as_float(o_acc[4 * n + 2 * i + 1]) * inv, hi, lo);
+                    *reinterpret_cast<uint32_t *>(dst + 8 * n) = hi;
+                    if (p.lo) *reinterpret_cast<uint32_t *>(dst + p.lo + 8 * n) = lo;
+                }
+            }
         }
     } else {
         // Several splits: this (row tile, head)'s CTAs form one cluster. Each
@@ -636,17 +724,21 @@ __global__ void __launch_bounds__(THREADS, 1)
         float *s_o = reinterpret_cast<float *>(smem_raw + (base - su32(smem_raw)));   // [64][LD]
         float *s_ml = s_o + ROWS * L::LD;                                             // [64][2]
         __syncthreads();                  // every TMA into the ring has landed and been used
-        if (smx && lane < 16) {
-            const bool live = valid && ok;
+        if (smx) {
 #pragma unroll
-            for (int c = 0; c < OH; c += 4)
-                *reinterpret_cast<float4 *>(s_o + row_local * L::LD + hf * OH + c) =
-                    live ? make_float4(__uint_as_float(o_acc[c]), __uint_as_float(o_acc[c + 1]),
-                                       __uint_as_float(o_acc[c + 2]), __uint_as_float(o_acc[c + 3]))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (hf == 0)
-                *reinterpret_cast<float2 *>(s_ml + row_local * 2) =
-                    live ? make_float2(m_used, l_sum) : make_float2(-INFINITY, 0.f);
+            for (int i = 0; i < 2; ++i) {
+                const int rl = fr + 8 * i;
+                const bool live = r0 + rl < r_end && ok;
+#pragma unroll
+                for (int n = 0; n < OH / 8; ++n)
+                    *reinterpret_cast<float2 *>(s_o + rl * L::LD + hf * OH + 8 * n + fc) =
+                        live ? make_float2(__uint_as_float(o_acc[4 * n + 2 * i]),
+                                           __uint_as_float(o_acc[4 * n + 2 * i + 1]))
+                             : make_float2(0.f, 0.f);
+                if (hf == 0 && (lane & 3) == 0)
+                    *reinterpret_cast<float2 *>(s_ml + rl * 2) =
+                        live ? make_float2(m_used[i], l_sum[i]) : make_float2(-INFINITY, 0.f);
+            }
         }
         cluster_sync();
         const uint32_t rank = cluster_rank();
