@@ -306,10 +306,11 @@ cudaError_t launch_as(AsArgs p, int num_sms, cudaStream_t s) {
     const AttnArgs<float> &a = p.a;
     p.tiles_per_req = (p.rows_per_req + QR - 1) / QR;
     const int row_tiles = a.tiles ? a.n_tiles : a.R / p.rows_per_req * p.tiles_per_req;
-    // splits while they fit one wave of CTAs: a function of the launch's shape
+    // splits while they fit one wave of CTAs, two key tiles of the cache each: a
+    // function of the launch's shape
     const long base = (long)row_tiles * a.nh;
     p.nsplit = (int)std::max<long>(
-        1, std::min<long>(std::min<long>(AS_MAX_SPLITS, (a.cache_slots + AS_KT - 1) / AS_KT), num_sms / base));
+        1, std::min<long>(std::min<long>(AS_MAX_SPLITS, (a.cache_slots + 2 * AS_KT - 1) / (2 * AS_KT)), num_sms / base));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)a.nh, (unsigned)row_tiles, (unsigned)p.nsplit);
     lc.blockDim = dim3(AS_THREADS);

@@ -880,10 +880,10 @@ bool launch_attention_tc(AttnTcPlan *p, const AttnArgs<bf16> &a, int B, int rows
     const int has_tree = a.mask != nullptr;
     // One CTA fills an SM: as many splits per (row tile, head) as keep the
     // launch within one wave (a function of the launch's shape alone).
-    // (and no more than the cache has key tiles: a cluster of empty splits only
-    // makes the combine longer)
+    // No more than one per three key tiles of the cache: a tile takes about 1 us,
+    // the cluster's barriers and combine 3 us.
     const int nsplit = (int)std::max<long>(
-        1, std::min<long>(std::min<long>(MAX_SPLITS, (a.cache_slots + KT - 1) / KT), p->num_sms / base));
+        1, std::min<long>(std::min<long>(MAX_SPLITS, (a.cache_slots + 3 * KT - 1) / (3 * KT)), p->num_sms / base));
     const long lo_rows = a.lo / a.hd;
     const long kc_rows = (long)B * a.nh * a.cache_slots + lo_rows;
     const CUtensorMap *mkc = kv_map(p, a.cache_k, kc_rows, a.hd);

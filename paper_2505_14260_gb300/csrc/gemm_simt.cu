@@ -8,7 +8,7 @@
 // at once: packed fp32 FMAs (f32x2) keep the even-k and the odd-k sums of each
 // output in one 64-bit register, added at the end. Rows are padded to 68
 // floats, so the 8 rows a warp reads together sit in different banks.
-// Tiles of 32 x 16 to 128 outputs x 64 token rows, always 256 threads: the
+// Tiles of 32 x 8 to 128 outputs x 64 token rows, always 256 threads: the
 // smaller the tile, the more warps share it by taking different k of a stage
 // (their sums meet in shared memory). When the tiles leave SMs idle, K is
 // split over the CTAs of a cluster (at most 8), whose partial tiles are summed
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(SG_THREADS) gemm_simt_kernel(const SgArgs a) {
     const int b0 = (int)((long long)split * nb / a.splits), b1 = (int)((long long)(split + 1) * nb / a.splits);
 
     // the rows this thread copies: 16 threads per row of a stage
-    constexpr int RO = TL::BO / 16, RM = TL::BM / 16;
+    constexpr int RO = TL::BO / 16, RM = (TL::BM + 15) / 16;    // (an 8-row tile: half of its last pass is idle)
     const int crow = tid >> 4, cq = (tid & 15) * 4;
     const float *src[RO + RM];
 #pragma unroll
@@ -102,13 +102,14 @@ __global__ void __launch_bounds__(SG_THREADS) gemm_simt_kernel(const SgArgs a) {
 #pragma unroll
     for (int i = 0; i < RM; ++i) {
         const int m = m0 + crow + 16 * i;
-        src[RO + i] = m < a.M ? a.X + (size_t)m * a.ldx : nullptr;
+        src[RO + i] = m < a.M && crow + 16 * i < TL::BM ? a.X + (size_t)m * a.ldx : nullptr;
     }
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(sm) + (uint32_t)(crow * SG_LD + cq) * 4u;
     auto load = [&](int blk, int st) {
         const int k = blk * SG_BK + cq;
 #pragma unroll
         for (int i = 0; i < RO + RM; ++i) {
+            if (TL::BM < 16 && i == RO && crow >= TL::BM) break;
             const uint32_t d = s0 + (uint32_t)(st * TL::STAGE + 16 * i * SG_LD) * 4u;
             const float *p = src[i];
             if constexpr (VEC) {                  // K % 4 == 0: whole chunks
@@ -246,6 +247,7 @@ bool set_tile() {
                cudaSuccess;
 }
 
+typedef Tile<32, 8, 4, 2, 4> T32x8;
 typedef Tile<32, 16, 4, 4, 4> T32x16;
 typedef Tile<32, 32, 4, 4, 4> T32x32;
 typedef Tile<64, 64, 8, 8, 3> T64x64;
@@ -253,7 +255,7 @@ typedef Tile<128, 64, 8, 8, 3> T128x64;
 
 }  // namespace
 
-bool gemm_simt_setup() { return set_tile<T32x16>() && set_tile<T32x32>() && set_tile<T64x64>() && set_tile<T128x64>(); }
+bool gemm_simt_setup() { return set_tile<T32x8>() && set_tile<T32x16>() && set_tile<T32x32>() && set_tile<T64x64>() && set_tile<T128x64>(); }
 
 void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int O, float *Y, int ldy, int epi,
                       int num_sms, cudaStream_t s) {
@@ -276,7 +278,8 @@ void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int
     // shared-memory load decide: 333 x 3072 x 1024 57 us in 128 x 64 tiles, 66 to 81
     // in smaller ones; 333 x 1024 x 1024 35 us in 64 x 64, 52 in 128 x 64 (48 tiles).
     const long t32 = (long)((O + 31) / 32) * ((M + 31) / 32), t128 = (long)((O + 127) / 128) * ((M + 63) / 64);
-    if (M <= 16) launch_vec<T32x16>(a, vec, n, s);
+    if (M <= 8) launch_vec<T32x8>(a, vec, n, s);
+    else if (M <= 16) launch_vec<T32x16>(a, vec, n, s);
     else if (M <= 32 || t32 <= 2L * n) launch_vec<T32x32>(a, vec, n, s);
     else if (8 * t128 < 7L * n) launch_vec<T64x64>(a, vec, n, s);
     else launch_vec<T128x64>(a, vec, n, s);

@@ -2502,7 +2502,7 @@ extern "C" msd_status msd_linear_noalloc(const void *x, int32_t ldx, int32_t m, 
                                          int32_t accumulate, void *stream) {
     using namespace msd;
     constexpr msd_status OK = MSD_OK, INVALID = MSD_ERR_INVALID, CAPACITY = MSD_ERR_CAPACITY,
-                         CUDA_ERR = MSD_ERR_CUDA, DEVICE = MSD_ERR_DEVICE;
+                         CUDA_ERR = MSD_ERR_CUDA;
     if (!x || !w || !y || m <= 0 || k <= 0 || o <= 0 || ldx < k || ldy < o) return INVALID;
     if (ldx % 8 || k % 8) return INVALID;
     if ((long)m > NOALLOC_MAX_ROWS) return CAPACITY;
@@ -2517,7 +2517,7 @@ extern "C" msd_status msd_linear_noalloc(const void *x, int32_t ldx, int32_t m, 
     // word is cleared and reported once.
     int code = 0;
     if (noalloc_take_status(d, s, &code) != cudaSuccess) return CUDA_ERR;
-    if (code != 0) return DEVICE;
+    if (code != 0) return MSD_ERR_DEVICE;
     if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w)) & 15) return INVALID;
     const GemmW W{{w, nullptr, nullptr}, {o, 0, 0}, 1, nullptr};
     const bf16 *X = static_cast<const bf16 *>(x);
