@@ -1998,6 +1998,16 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     stages = std::max(2, std::min(stages, C_STAGES));
     int S = (per_sm * p->num_sms) / tiles;
     S = std::max(1, std::min(S, 8));
+    // Clusters stay within a GPC, so fewer CTAs run at once the larger they are, and
+    // a launch past that runs a second wave. Two CTAs per SM on 152 SMs: 32 clusters
+    // of 8, 40 of 6, 56 of 5 and 96 of 3 ran as one, 40 of 7 and 48 of 6 did not
+    // (60 x 5120 x 13824: 43.6 us in sevens, 29.6 in sixes; 60 x 6144 x 4096: 22.9
+    // in sixes, 14.8 in fives).
+    auto one_wave = [&](int c) {
+        const int slots = c >= 6 ? 256 : (c >= 4 ? 280 : (c == 3 ? 288 : 304));
+        return (long)tiles * c * 304 <= (long)slots * per_sm * p->num_sms;
+    };
+    while (S > 1 && !one_wave(S)) --S;
     // One-plane products (msd_linear): the accumulators truncate, so a chain of at
     // most 16 K-blocks each -- as many of them as 256 TMEM columns hold take turns,
     // and K is split further where that is not enough (17 x 4096 x 11008: 1.1e-6
