@@ -11,10 +11,11 @@ namespace msd {
 
 // ---- elementwise / row kernels (kernels_rows.cu) ---------------------------
 
-// x[r] = float(src[r] >= 0 ? E[src[r]] : vis[-1 - src[r]])
+// x[r] = float(src[r] >= 0 ? E[src[r]] : vis[-1 - src[r]]), xn[r] = its RMSNorm
+// with gain g, split (lo plane at xn + lo)
 template <typename T>
-void launch_embed_rows(const T *E, const T *vis, const int *src, int R, int H, float *x, int V, int *status,
-                       cudaStream_t s);
+void launch_embed_norm(const T *E, const T *vis, const int *src, const T *g, int R, int H, float eps, float *x, T *xn,
+                       long lo, int V, int *status, cudaStream_t s);
 
 // out[r] = x[r] / sqrt(mean(x[r]^2) + eps) * g, split (lo plane at out + lo)
 template <typename T>

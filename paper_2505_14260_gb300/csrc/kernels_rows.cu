@@ -1,6 +1,7 @@
-// Row-wise kernels of the MSD step: embedding gather (Eq. 1-3), RMSNorm,
+// Row-wise kernels of the MSD step: embedding gather (Eq. 1-3) and row set-up, RMSNorm,
 // SwiGLU, RoPE + K/V placement, argmax and top-k with log-softmax.
 #include "kernels.h"
+#include "kernels_tree.h"
 
 #include <algorithm>
 #include <atomic>
@@ -12,42 +13,35 @@ long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 // ---------------------------------------------------------------------------
-// Embedding gather (Eq. 1 for text, Eq. 2's projected rows for visual slots)
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void embed_rows_kernel(const T *__restrict__ E, const T *__restrict__ vis,
-                                  const int *__restrict__ src, int H, float *__restrict__ x, int V,
-                                  int *status) {
-    wait_prior();
-    allow_dependents();
-    const int r = blockIdx.x;
-    int s = src[r];
-    const T *row;
-    if (s >= 0) {
-        if (s >= V) {
-            if (threadIdx.x == 0) set_status(status, ST_BAD_TOKEN);
-            s = 0;
-        }
-        row = E + (size_t)s * H;
-    } else {
-        row = vis + (size_t)(-1 - s) * H;
-    }
-    copy_row(x + (size_t)r * H, row, H);
-}
-
-template <typename T>
-void launch_embed_rows(const T *E, const T *vis, const int *src, int R, int H, float *x, int V, int *status,
-                       cudaStream_t s) {
-    if (R <= 0) return;
-    launch_chain(embed_rows_kernel<T>, R, 256, 0, s, E, vis, src, H, x, V, status); note_launch();
-}
-
-// ---------------------------------------------------------------------------
-// RMSNorm: y = x / sqrt(mean(x^2) + eps) * g
+// RMSNorm: y = x / sqrt(mean(x^2) + eps) * g; the embedding gather (Eq. 1 for
+// text, Eq. 2's projected rows for visual slots) with the first layer's norm
 // ---------------------------------------------------------------------------
 // One CTA per row; the row stays in registers (H <= 8 * 4 * 256).
 constexpr int RMS_THREADS = 256;
 constexpr int RMS_VEC = 8;
+
+// y = x / rms(x) * g of the row held in v (thread t: groups t, t + 256, ...).
+template <typename T>
+__device__ __forceinline__ void rms_row(const float4 (&v)[RMS_VEC], const T *__restrict__ g, int H, float eps,
+                                        T *__restrict__ out, long lo, float *red) {
+    const int n4 = H >> 2;
+    float ss = 0.f;
+#pragma unroll
+    for (int i = 0; i < RMS_VEC; ++i)
+        ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+    ss = block_sum(ss, red);
+    const float inv = rsqrtf(ss / (float)H + eps);
+#pragma unroll
+    for (int i = 0; i < RMS_VEC; ++i) {
+        const int j = threadIdx.x + i * RMS_THREADS;
+        if (j < n4) {
+            const float4 gg = Vec4<T>::load(g + 4 * j);
+            Split<T>::store4(out + 4 * j, lo,
+                             make_float4(v[i].x * inv * gg.x, v[i].y * inv * gg.y,
+                                         v[i].z * inv * gg.z, v[i].w * inv * gg.w));
+        }
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(RMS_THREADS) rmsnorm_kernel(const float *__restrict__ x,
@@ -59,25 +53,119 @@ __global__ void __launch_bounds__(RMS_THREADS) rmsnorm_kernel(const float *__res
     const int r = blockIdx.x, n4 = H >> 2;
     const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)r * H);
     float4 v[RMS_VEC];
-    float ss = 0.f;
 #pragma unroll
     for (int i = 0; i < RMS_VEC; ++i) {
         const int j = threadIdx.x + i * RMS_THREADS;
         v[i] = j < n4 ? xr[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-        ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
     }
-    ss = block_sum(ss, red);
-    const float inv = rsqrtf(ss / (float)H + eps);
+    rms_row<T>(v, g, H, eps, out + (size_t)r * H, lo, red);
+}
+
+// The embedding row of source s (a token id, or -1 - row of the visual rows) as
+// x (fp32) and, normalised for the first layer, as xn: one launch for both.
+template <typename T>
+__device__ __forceinline__ void embed_norm_row(const T *__restrict__ E, const T *__restrict__ vis, int s,
+                                               const T *__restrict__ g, int H, float eps, float *__restrict__ x,
+                                               T *__restrict__ xn, long lo, float *red) {
+    const T *row = s >= 0 ? E + (size_t)s * H : vis + (size_t)(-1 - s) * H;
+    const int n4 = H >> 2;
+    float4 v[RMS_VEC];
 #pragma unroll
     for (int i = 0; i < RMS_VEC; ++i) {
         const int j = threadIdx.x + i * RMS_THREADS;
-        if (j < n4) {
-            const float4 gg = Vec4<T>::load(g + 4 * j);
-            Split<T>::store4(out + (size_t)r * H + 4 * j, lo,
-                             make_float4(v[i].x * inv * gg.x, v[i].y * inv * gg.y,
-                                         v[i].z * inv * gg.z, v[i].w * inv * gg.w));
-        }
+        v[i] = j < n4 ? Vec4<T>::load(row + 4 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+#pragma unroll
+    for (int i = 0; i < RMS_VEC; ++i) {
+        const int j = threadIdx.x + i * RMS_THREADS;
+        if (j < n4) reinterpret_cast<float4 *>(x)[j] = v[i];
+    }
+    rms_row<T>(v, g, H, eps, xn, lo, red);
+}
+
+// Prefill rows.
+template <typename T>
+__global__ void __launch_bounds__(RMS_THREADS) embed_norm_kernel(const T *__restrict__ E, const T *__restrict__ vis,
+                                                                 const int *__restrict__ src, const T *__restrict__ g,
+                                                                 int H, float eps, float *__restrict__ x,
+                                                                 T *__restrict__ xn, long lo, int V, int *status) {
+    wait_prior();
+    allow_dependents();
+    __shared__ float red[32];
+    const int r = blockIdx.x;
+    int s = src[r];
+    if (s >= V) {
+        if (threadIdx.x == 0) set_status(status, ST_BAD_TOKEN);
+        s = 0;
+    }
+    embed_norm_row<T>(E, vis, s, g, H, eps, x + (size_t)r * H, xn + (size_t)r * H, lo, red);
+}
+
+// Verify rows: the tree node's checks, row descriptor and mask words (thread 0),
+// then its embedding and first norm.
+template <typename T>
+__global__ void __launch_bounds__(RMS_THREADS) verify_rows_kernel(TreeIn t, const int *__restrict__ seq_len,
+                                                                  const int *__restrict__ root, int N, int V,
+                                                                  RowDesc *__restrict__ rows,
+                                                                  uint64_t *__restrict__ vmask,
+                                                                  const T *__restrict__ E, const T *__restrict__ g,
+                                                                  int H, float eps, float *__restrict__ x,
+                                                                  T *__restrict__ xn, long lo, int *status) {
+    wait_prior();
+    allow_dependents();
+    __shared__ float red[32];
+    const int r = blockIdx.x, b = r / N, i = r - b * N, W = (N + 63) / 64;
+    const int n = t.n_nodes ? t.n_nodes[b] : N;
+    const bool valid = i < n;
+    int tok = valid ? t.tokens[r] : 0;
+    const bool bad = tok < 0 || tok >= V;
+    if (bad) tok = 0;
+    if (threadIdx.x == 0) {
+        if (bad) set_status(status, ST_BAD_TOKEN);
+        const int L = seq_len[b];
+        int depth = valid ? t.depth[r] : 0;
+        if (valid) {
+            const int p = t.parent[r];
+            const bool ok = i == 0 ? (p == -1 && depth == 0 && tok == root[b])
+                                   : (p >= 0 && p < i && depth == t.depth[b * N + p] + 1);
+            if (!ok) { set_status(status, ST_BAD_TREE); depth = depth < 0 ? 0 : depth; }
+        }
+        RowDesc d;
+        d.req = b;
+        d.pos = L + depth;
+        d.plen = L;
+        d.dst = i;
+        rows[r] = d;
+    }
+    for (int w = threadIdx.x; w < W; w += blockDim.x) {
+        uint64_t m = 0;
+        if (valid) {
+            m = t.mask[(size_t)r * W + w];
+            const int lo_n = w * 64;
+            if (n - lo_n < 64) m &= n - lo_n <= 0 ? 0ull : ((1ull << (n - lo_n)) - 1ull);
+        } else if (w == i / 64) {
+            m = 1ull << (i % 64);
+        }
+        vmask[(size_t)r * W + w] = m;
+    }
+    embed_norm_row<T>(E, E, tok, g, H, eps, x + (size_t)r * H, xn + (size_t)r * H, lo, red);
+}
+
+template <typename T>
+void launch_embed_norm(const T *E, const T *vis, const int *src, const T *g, int R, int H, float eps, float *x, T *xn,
+                       long lo, int V, int *status, cudaStream_t s) {
+    if (R <= 0) return;
+    launch_chain(embed_norm_kernel<T>, R, RMS_THREADS, 0, s, E, vis, src, g, H, eps, x, xn, lo, V, status);
+    note_launch();
+}
+
+template <typename T>
+void launch_verify_rows(const TreeIn &t, const int *seq_len, const int *root, int B, int N, int V, RowDesc *rows,
+                        uint64_t *vmask, const T *E, const T *g, int H, float eps, float *x, T *xn, long lo,
+                        int *status, cudaStream_t s) {
+    launch_chain(verify_rows_kernel<T>, B * N, RMS_THREADS, 0, s, t, seq_len, root, N, V, rows, vmask, E, g, H, eps, x,
+                 xn, lo, status);
+    note_launch();
 }
 
 template <typename T>
@@ -533,8 +621,11 @@ void launch_flag(int *status, int code, cudaStream_t s) {
 }
 
 #define MSD_INST(T)                                                                          \
-    template void launch_embed_rows<T>(const T *, const T *, const int *, int, int, float *,  \
-                                       int, int *, cudaStream_t);                            \
+    template void launch_embed_norm<T>(const T *, const T *, const int *, const T *, int, int, float, float *, T *, \
+                                       long, int, int *, cudaStream_t);                      \
+    template void launch_verify_rows<T>(const TreeIn &, const int *, const int *, int, int, int, RowDesc *, \
+                                        uint64_t *, const T *, const T *, int, float, float *, T *, long, int *, \
+                                        cudaStream_t);                                       \
     template void launch_rmsnorm<T>(const float *, const T *, int, int, float, T *, long,    \
                                     cudaStream_t);                                           \
     template void launch_rope_kv<T>(const float *, const RowDesc *, int, int, int,           \

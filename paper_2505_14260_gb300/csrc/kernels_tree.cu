@@ -243,51 +243,6 @@ __global__ void tree_finalize_kernel(TreeOut t, const int *__restrict__ cand_tok
 }
 
 // ---------------------------------------------------------------------------
-// Verify set-up: row r = b*N + i at position L + depth(i), sees the prefix
-// [0, L) and the tree nodes of its mask (restricted to valid nodes).
-// ---------------------------------------------------------------------------
-__global__ void verify_setup_kernel(TreeIn t, const int *__restrict__ seq_len,
-                                    const int *__restrict__ root, int B, int N, int V,
-                                    RowDesc *__restrict__ rows, int *__restrict__ src,
-                                    uint64_t *__restrict__ vmask, int *status) {
-    wait_prior();
-    allow_dependents();
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= B * N) return;
-    const int b = r / N, i = r - b * N, W = (N + 63) / 64;
-    const int n = t.n_nodes ? t.n_nodes[b] : N;
-    const bool valid = i < n;
-    const int L = seq_len[b];
-    int tok = valid ? t.tokens[r] : 0;
-    if (tok < 0 || tok >= V) { set_status(status, ST_BAD_TOKEN); tok = 0; }
-    int depth = valid ? t.depth[r] : 0;
-    if (valid) {
-        const int p = t.parent[r];
-        bool ok = i == 0 ? (p == -1 && depth == 0 && tok == root[b])
-                         : (p >= 0 && p < i && depth == t.depth[b * N + p] + 1);
-        if (!ok) { set_status(status, ST_BAD_TREE); depth = depth < 0 ? 0 : depth; }
-    }
-    RowDesc d;
-    d.req = b;
-    d.pos = L + depth;
-    d.plen = L;
-    d.dst = i;
-    rows[r] = d;
-    src[r] = tok;
-    for (int w = 0; w < W; ++w) {
-        uint64_t m = 0;
-        if (valid) {
-            m = t.mask[(size_t)r * W + w];
-            const int lo = w * 64;
-            if (n - lo < 64) m &= n - lo <= 0 ? 0ull : ((1ull << (n - lo)) - 1ull);
-        } else if (w == i / 64) {
-            m = 1ull << (i % 64);
-        }
-        vmask[(size_t)r * W + w] = m;
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Root-only tree of plain greedy decoding: one thread per request.
 // ---------------------------------------------------------------------------
 __global__ void root_tree_kernel(const int *__restrict__ root, int B, int N, int W, int *__restrict__ tokens,
@@ -753,15 +708,27 @@ accept_sample_kernel(TreeIn t, const float *__restrict__ logits, const float *__
 
 // K/V of accepted node path[j] -> cache position L0 + j, all layers and heads.
 // grid (n_layers*2*nh, B); 16-byte vector copies.
-__global__ void compact_kv_kernel(const uint4 *__restrict__ tree_kv, uint4 *__restrict__ cache,
-                                  const int *__restrict__ acc_path, const int *__restrict__ acc_L0,
-                                  const int *__restrict__ acc_a, int B, int nh, int N, int S,
-                                  int D1, int vec_per_row, long tree_lo, long cache_lo, int *status) {
+// Blocks past the KV rows (kv_blocks of a request) copy its pending draft rows:
+// the target features h of the accepted nodes.
+template <typename T>
+__global__ void compact_kernel(const uint4 *__restrict__ tree_kv, uint4 *__restrict__ cache,
+                               const int *__restrict__ acc_path, const int *__restrict__ acc_L0,
+                               const int *__restrict__ acc_a, int kv_blocks, int B, int nh, int N, int S, int D1,
+                               int vec_per_row, long lo_vec, const T *__restrict__ hT, int H,
+                               T *__restrict__ pend_h, long lo, int *status) {
     wait_prior();
     allow_dependents();
     const int lkh = blockIdx.x, b = blockIdx.y;
+    const int a = acc_a[b];
+    if (lkh >= kv_blocks) {
+        const int j = lkh - kv_blocks;
+        if (j > a) return;
+        const T *s = hT + ((size_t)b * N + acc_path[b * D1 + j]) * H;
+        copy_row_split(pend_h + ((size_t)b * D1 + j) * H, lo, s, lo, H);
+        return;
+    }
     const int h = lkh % nh, lk = lkh / nh;           // lk = layer*2 + kv
-    const int a = acc_a[b], L0 = acc_L0[b];
+    const int L0 = acc_L0[b];
     if (L0 + a >= S) {
         if (threadIdx.x == 0) set_status(status, ST_RANGE);
         return;
@@ -774,26 +741,12 @@ __global__ void compact_kv_kernel(const uint4 *__restrict__ tree_kv, uint4 *__re
         const int node = acc_path[b * D1 + j];
         const size_t dst = (cb + L0 + j) * vec_per_row + v, src = (tb + node) * vec_per_row + v;
         const uint4 hi = tree_kv[src];
-        if (tree_lo) {
-            const uint4 lo = tree_kv[src + tree_lo];
-            cache[dst + cache_lo] = lo;
+        if (lo_vec) {
+            const uint4 l = tree_kv[src + lo_vec];
+            cache[dst + lo_vec] = l;
         }
         cache[dst] = hi;
     }
-}
-
-// Pending draft rows: target features h of the accepted nodes.
-template <typename T>
-__global__ void pend_h_kernel(const T *__restrict__ hT, const int *__restrict__ acc_path,
-                              const int *__restrict__ acc_a, int N, int D1, int H,
-                              T *__restrict__ pend_h, long lo) {
-    wait_prior();
-    allow_dependents();
-    const int b = blockIdx.x / D1, j = blockIdx.x - b * D1;
-    if (j > acc_a[b]) return;
-    const int node = acc_path[b * D1 + j];
-    const T *s = hT + ((size_t)b * N + node) * H;
-    copy_row_split(pend_h + ((size_t)b * D1 + j) * H, lo, s, lo, H);
 }
 
 // ---------------------------------------------------------------------------
@@ -903,14 +856,6 @@ void launch_tree_finalize(const TreeOut &t, const int *cand_tok, const int *cand
     note_launch();
 }
 
-void launch_verify_setup(const TreeIn &t, const int *seq_len, const int *root, int B, int N,
-                         int V, RowDesc *rows, int *src, uint64_t *vmask, int *status,
-                         cudaStream_t s) {
-    const int R = B * N;
-    launch_chain(verify_setup_kernel, (R + 127) / 128, 128, 0, s, t, seq_len, root, B, N, V, rows, src,
-                                                          vmask, status); note_launch();
-}
-
 void launch_tree_complete(const int *parent, int *depth, uint64_t *mask, const int *n_nodes, int b0, int nb,
                           int N, int *status, cudaStream_t s) {
     launch_chain(tree_complete_kernel, nb, 256, 0, s, parent, depth, mask, n_nodes, N, (N + 63) / 64, b0, status);
@@ -958,20 +903,14 @@ bool launch_accept_sample(const TreeIn &t, const float *logits, int B, int N, in
     return true;
 }
 
-void launch_compact_kv(const void *tree_kv, void *cache, const int *acc_path, const int *acc_L0,
-                       const int *acc_a, int n_layers, int B, int nh, int N, int S, int D1,
-                       int row_bytes, long lo_bytes, int *status, cudaStream_t s) {
-    dim3 grid(n_layers * 2 * nh, B);
-    const long lo_vec = lo_bytes / 16;      // both lo planes sit lo_bytes after their hi planes
-    launch_chain(compact_kv_kernel, grid, 128, 0, s, static_cast<const uint4 *>(tree_kv),
-                                           static_cast<uint4 *>(cache), acc_path, acc_L0, acc_a,
-                                           B, nh, N, S, D1, row_bytes / 16, lo_vec, lo_vec, status); note_launch();
-}
-
 template <typename T>
-void launch_pend_h(const T *hT, const int *acc_path, const int *acc_a, int B, int N, int D1,
-                   int H, T *pend_h, long lo, cudaStream_t s) {
-    launch_chain(pend_h_kernel<T>, B * D1, 256, 0, s, hT, acc_path, acc_a, N, D1, H, pend_h, lo); note_launch();
+void launch_compact(const void *tree_kv, void *cache, const int *acc_path, const int *acc_L0, const int *acc_a,
+                    int n_layers, int B, int nh, int N, int S, int D1, int row_bytes, long lo_bytes, const T *hT,
+                    int H, T *pend_h, long lo, int *status, cudaStream_t s) {
+    const int kv_blocks = n_layers * 2 * nh;
+    launch_chain(compact_kernel<T>, dim3(kv_blocks + D1, B), 128, 0, s, static_cast<const uint4 *>(tree_kv),
+                 static_cast<uint4 *>(cache), acc_path, acc_L0, acc_a, kv_blocks, B, nh, N, S, D1, row_bytes / 16,
+                 lo_bytes / 16, hT, H, pend_h, lo, status); note_launch();
 }
 
 template <typename T>
@@ -1006,8 +945,8 @@ void launch_prefill_finish(const int *argmax, const T *h_last, const int *L, int
                                        T *, long, cudaStream_t);                                \
     template void launch_tree_init<T>(const DraftArgs<T> &, int, cudaStream_t);                 \
     template void launch_tree_step<T>(const DraftArgs<T> &, int, int, cudaStream_t);            \
-    template void launch_pend_h<T>(const T *, const int *, const int *, int, int, int, int, T *, \
-                                   long, cudaStream_t);                                         \
+    template void launch_compact<T>(const void *, void *, const int *, const int *, const int *, int, int, int, \
+                                    int, int, int, int, long, const T *, int, T *, long, int *, cudaStream_t); \
     template void launch_prefill_draft_in<T>(const T *, const T *, const T *, const int *,      \
                                              const int *, int, int, T *, T *, long, cudaStream_t); \
     template void launch_select_visual<T>(float *, const T *, const T *, const int *, const int *, \

@@ -59,9 +59,12 @@ void launch_tree_step(const DraftArgs<T> &a, int B, int d, cudaStream_t s);
 void launch_tree_finalize(const TreeOut &t, const int *cand_tok, const int *cand_par,
                           const int *cand_depth, const float *cand_score, int *node_of,
                           const int *root, int B, int C, int N, int *status, cudaStream_t s);
-void launch_verify_setup(const TreeIn &t, const int *seq_len, const int *root, int B, int N,
-                         int V, RowDesc *rows, int *src, uint64_t *vmask, int *status,
-                         cudaStream_t s);
+// Verify rows, one per tree node: the node's checks, row descriptor and mask words,
+// x = its embedding and xn = the first layer's RMSNorm of it (gain g).
+template <typename T>
+void launch_verify_rows(const TreeIn &t, const int *seq_len, const int *root, int B, int N, int V, RowDesc *rows,
+                        uint64_t *vmask, const T *E, const T *g, int H, float eps, float *x, T *xn, long lo,
+                        int *status, cudaStream_t s);
 // Depths and ancestor-or-self masks of caller-planted trees from their parent
 // arrays, for requests b0 .. b0+nb-1 (n_nodes[b] nodes of request b; nodes
 // past it get depth 0 and an empty mask). A parent that does not precede its
@@ -90,13 +93,13 @@ bool launch_accept_sample(const TreeIn &t, const float *logits, int B, int N, in
                           int *n_pend, int *root, int *pend_next, int *acc_path, int *acc_L0, int *acc_a,
                           int *path_out, int *accept_len_out, int *bonus_out, int *index_map_out,
                           int *status, cudaStream_t s);
-// KV compaction; lo_bytes (0: none) = the lo planes' byte offset from their hi planes.
-void launch_compact_kv(const void *tree_kv, void *cache, const int *acc_path, const int *acc_L0,
-                       const int *acc_a, int n_layers, int B, int nh, int N, int S, int D1,
-                       int row_bytes, long lo_bytes, int *status, cudaStream_t s);
+// KV compaction; lo_bytes (0: none) = the lo planes' byte offset from their hi
+// planes. The same launch copies the accepted nodes' features hT to the draft's
+// pending rows pend_h (lo: their lo planes' element offset).
 template <typename T>
-void launch_pend_h(const T *hT, const int *acc_path, const int *acc_a, int B, int N, int D1,
-                   int H, T *pend_h, long lo, cudaStream_t s);
+void launch_compact(const void *tree_kv, void *cache, const int *acc_path, const int *acc_L0, const int *acc_a,
+                    int n_layers, int B, int nh, int N, int S, int D1, int row_bytes, long lo_bytes, const T *hT,
+                    int H, T *pend_h, long lo, int *status, cudaStream_t s);
 // Packed prefill chunks of R rows: the draft rows' inputs (and the requests' last
 // features), the visual rows' inputs, and the requests' state (one row per request).
 template <typename T>

@@ -43,7 +43,6 @@ struct msd_ctx {
     void *xn = nullptr, *q = nullptr, *attn = nullptr, *act = nullptr, *xfc = nullptr, *xr = nullptr;
     int *argmax_tmp = nullptr;
     RowDesc *rows = nullptr;
-    int *src = nullptr;
     uint64_t *vmask = nullptr;
     int *cand_tok = nullptr, *cand_par = nullptr, *cand_depth = nullptr, *frontier = nullptr,
         *node_of = nullptr;
@@ -302,22 +301,23 @@ GemmNorm norm_in(msd_ctx *c) {
 // One pre-norm decoder layer over R rows (target or draft). Rows come in
 // blocks of rows_per_req per request.
 // cache positions. in_folded: the layer's input norm was folded into the GEMM
-// that produced x; out_norm_g (nullable): the next layer's input-norm gain,
+// that produced x (xn_ready: it is in c->xn already); out_norm_g (nullable): the next layer's input-norm gain,
 // to fold into this layer's last GEMM. Returns whether it did.
 template <typename T>
 bool run_layer(msd_ctx *c, const msd_layer &lw, const msd_ctx::LayerPack &lp, int R,
                const RowDesc *rows, T *kdst, T *vdst, int dst_slots, const T *ck, const T *cv,
                int cslots, const T *tk, const T *tv, int tslots, const uint64_t *mask, int mw,
                int rows_per_req, cudaStream_t s, bool in_folded = false,
-               const void *out_norm_g = nullptr, const int2 *tiles = nullptr, int n_tiles = 0) {
+               const void *out_norm_g = nullptr, const int2 *tiles = nullptr, int n_tiles = 0,
+               bool xn_ready = false) {
     const int H = c->H, F = c->F;
     const float eps = c->cfg.rms_eps;
     const bool fold = folds(c, R, lp.o) && lp.qkv && lp.gu && lp.down;
     const GemmNorm nin = norm_in(c);
-    if (!(fold && in_folded))
+    if (!xn_ready && !(fold && in_folded))
         launch_rmsnorm<T>(c->x, static_cast<const T *>(lw.attn_norm), R, H, eps,
                           static_cast<T *>(c->xn), c->lo, s);
-    qkv_rope<T>(c, lw, lp, R, rows, kdst, vdst, dst_slots, s, fold && in_folded ? &nin : nullptr);
+    qkv_rope<T>(c, lw, lp, R, rows, kdst, vdst, dst_slots, s, fold && in_folded && !xn_ready ? &nin : nullptr);
     AttnArgs<T> a;
     a.q = static_cast<const T *>(c->q);
     a.rows = rows;
@@ -393,12 +393,12 @@ bool draft_fc(msd_ctx *c, int R, cudaStream_t s) {
 // to c->chunk rows of any requests: the GEMMs see full chunks whatever the
 // prompts' lengths (16 ragged prompts of 600 to 1660 rows in chunks of their own
 // cost a second, mostly empty chunk each), and large chunks fill the pairs of the
-// many-row GEMM (O at 7B: 64 of 76 in one round at 1024 rows, 304 in four at
-// 4864). A request's earlier rows are in the cache when a later chunk reads it.
+// many-row GEMM (O at 7B: 64 of 76 in one round at 1024 rows, 144 of 152 in two
+// at 2304). A request's earlier rows are in the cache when a later chunk reads it.
 // The draft rows of a chunk follow its target pass, since e_{i+1} is a gather by
 // the next position's source. All row metadata is built on the host first and
 // copied at once, so the launches run without a synchronisation between.
-constexpr int PREFILL_CHUNK = 4864;
+constexpr int PREFILL_CHUNK = 2304;
 
 // Byte offsets of the metadata arrays, for n rows in chunks of `chunk`, B requests.
 struct PrefillMeta {
@@ -530,11 +530,12 @@ msd_status prefill_impl(msd_ctx *c, int batch, const int32_t *seq_len_host, cons
     const bool feat = c->cfg.draft_input == MSD_DRAFT_FEATURE;
     for (const Chunk &k : chunks) {
         // target over the chunk, causal
-        launch_embed_rows<T>(E, vis, src_d + k.r0, k.n, H, c->x, V, c->status, s);
+        launch_embed_norm<T>(E, vis, src_d + k.r0, static_cast<const T *>(c->layers[0].attn_norm), k.n, H,
+                             c->cfg.rms_eps, c->x, static_cast<T *>(c->xn), c->lo, V, c->status, s);
         for (int l = 0; l < c->NL; ++l) {
             T *K = tkv<T>(c, c->target_kv, l, 0, c->S), *Vv = tkv<T>(c, c->target_kv, l, 1, c->S);
             run_layer<T>(c, c->layers[l], c->lpack[l], k.n, rows_d + k.r0, K, Vv, c->S, K, Vv, c->S, nullptr, nullptr,
-                         0, nullptr, 0, k.n, s, false, nullptr, tiles_d + k.t0, k.nt);
+                         0, nullptr, 0, k.n, s, false, nullptr, tiles_d + k.t0, k.nt, l == 0);
         }
         launch_rmsnorm<T>(c->x, static_cast<const T *>(c->w.final_norm), k.n, H, c->cfg.rms_eps, h, c->lo, s);
         // draft cache over positions 0 .. L-2 with the decoupled input (Eq. 7): text
@@ -655,15 +656,16 @@ msd_status verify_impl(msd_ctx *c, const msd_tree *tree, int32_t *argmax_dev, fl
                        cudaStream_t s) {
     const int B = c->B, N = c->N, H = c->H, V = c->V, R = B * N;
     TreeIn t{tree->tokens, tree->parent, tree->depth, tree->mask, tree->n_nodes};
-    launch_verify_setup(t, c->seq_len, c->root, B, N, V, c->rows, c->src, c->vmask, c->status, s);
-    launch_embed_rows<T>(static_cast<const T *>(c->w.embed), nullptr, c->src, R, H, c->x, V, c->status, s);
+    launch_verify_rows<T>(t, c->seq_len, c->root, B, N, V, c->rows, c->vmask, static_cast<const T *>(c->w.embed),
+                          static_cast<const T *>(c->layers[0].attn_norm), H, c->cfg.rms_eps, c->x,
+                          static_cast<T *>(c->xn), c->lo, c->status, s);
     bool folded = false;
     for (int l = 0; l < c->NL; ++l) {
         T *K = tkv<T>(c, c->target_kv, l, 0, c->S), *Vv = tkv<T>(c, c->target_kv, l, 1, c->S);
         T *tK = tkv<T>(c, c->tree_kv, l, 0, N), *tV = tkv<T>(c, c->tree_kv, l, 1, N);
         const void *next_g = l + 1 < c->NL ? c->layers[l + 1].attn_norm : nullptr;
         folded = run_layer<T>(c, c->layers[l], c->lpack[l], R, c->rows, tK, tV, N, K, Vv, c->S, tK, tV, N,
-                              c->vmask, c->W, N, s, folded, next_g);
+                              c->vmask, c->W, N, s, folded, next_g, nullptr, 0, l == 0);
     }
     launch_rmsnorm<T>(c->x, static_cast<const T *>(c->w.final_norm), R, H, c->cfg.rms_eps,
                       static_cast<T *>(c->hT), c->lo, s);
@@ -679,10 +681,9 @@ msd_status verify_impl(msd_ctx *c, const msd_tree *tree, int32_t *argmax_dev, fl
 // draft's pending rows.
 template <typename T>
 msd_status compact_impl(msd_ctx *c, cudaStream_t s, int grow) {
-    launch_compact_kv(c->tree_kv, c->target_kv, c->acc_path, c->acc_L0, c->acc_a, c->NL, c->B, c->nh,
-                      c->N, c->S, c->D1, (int)(c->hd * c->esz), c->lo * (long)c->esz, c->status, s);
-    launch_pend_h<T>(static_cast<const T *>(c->hT), c->acc_path, c->acc_a, c->B, c->N, c->D1, c->H,
-                     static_cast<T *>(c->pend_h), c->lo, s);
+    launch_compact<T>(c->tree_kv, c->target_kv, c->acc_path, c->acc_L0, c->acc_a, c->NL, c->B, c->nh, c->N, c->S,
+                      c->D1, (int)(c->hd * c->esz), c->lo * (long)c->esz, static_cast<const T *>(c->hT), c->H,
+                      static_cast<T *>(c->pend_h), c->lo, c->status, s);
     if (!c->capturing)
         for (int b = 0; b < c->B; ++b) c->L_bound[b] += grow < 0 ? c->D1 : grow;
     return post_status(c);
@@ -929,7 +930,6 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     ok &= dalloc(c, &c->logits, (size_t)c->Rlog * c->V * 4);
     ok &= dalloc(c, &c->argmax_tmp, sizeof(int) * c->B);
     ok &= dalloc(c, &c->rows, sizeof(RowDesc) * R);
-    ok &= dalloc(c, &c->src, sizeof(int) * R);
     ok &= dalloc(c, &c->vmask, sizeof(uint64_t) * c->B * c->N * c->W);
     ok &= dalloc(c, &c->cand_tok, sizeof(int) * c->B * c->C);
     ok &= dalloc(c, &c->cand_par, sizeof(int) * c->B * c->C);

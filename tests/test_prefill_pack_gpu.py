@@ -1,5 +1,5 @@
 """Prefill packs the prompts' rows into chunks of any requests: prompts that end
-inside a row tile, span two chunks (more than 4864 rows in all), or hold a single
+inside a row tile, span two chunks (more than 2304 rows in all), or hold a single
 token, against the oracle (caches, draft caches, root, one step)."""
 import pytest
 
@@ -16,7 +16,7 @@ TINY = synth.WORKLOADS["tiny"]
     (1, (0,), (1, 1), None),                # one row, no draft row
     (3, (0,), (1, 2), None),                # single-token prompts among others
     (4, (0, 64, 63), (1, 70), None),        # ends at, before and past row-tile edges
-    (3, (2000, 2300), (20, 300), (1,)),     # two chunks: request 1 spans them
+    (3, (2000, 2300), (20, 300), (1,)),     # three chunks: request 1 spans two
 ])
 def test_packed_prefill_matches_oracle(dtype, batch, vis, text, requests):
     wl = TINY.with_(dtype=dtype, batch=batch, n_vis=vis, n_text=text, n_sys=4)
