@@ -284,6 +284,62 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t *r, int gw
     else tmem_ld16(taddr, r);
 }
 
+// Two accumulators' columns with one round trip (a load and a wait each: the 7B verify
+// call 877 us against 867).
+__device__ __forceinline__ void tmem_ld16_two(uint32_t ta, uint32_t *a, uint32_t tb, uint32_t *b) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,"
+        "%31}, [%33];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(a[0]), "=&r"(a[1]), "=&r"(a[2]), "=&r"(a[3]), "=&r"(a[4]), "=&r"(a[5]), "=&r"(a[6]),
+          "=&r"(a[7]), "=&r"(a[8]), "=&r"(a[9]), "=&r"(a[10]), "=&r"(a[11]), "=&r"(a[12]), "=&r"(a[13]),
+          "=&r"(a[14]), "=&r"(a[15]),
+          "=&r"(b[0]), "=&r"(b[1]), "=&r"(b[2]), "=&r"(b[3]), "=&r"(b[4]), "=&r"(b[5]), "=&r"(b[6]),
+          "=&r"(b[7]), "=&r"(b[8]), "=&r"(b[9]), "=&r"(b[10]), "=&r"(b[11]), "=&r"(b[12]), "=&r"(b[13]),
+          "=&r"(b[14]), "=&r"(b[15])
+        : "r"(ta), "r"(tb)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld32_two(uint32_t ta, uint32_t *a, uint32_t tb, uint32_t *b) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,"
+        "%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%64];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,"
+        "%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%65];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(a[0]), "=&r"(a[1]), "=&r"(a[2]), "=&r"(a[3]), "=&r"(a[4]), "=&r"(a[5]), "=&r"(a[6]),
+          "=&r"(a[7]), "=&r"(a[8]), "=&r"(a[9]), "=&r"(a[10]), "=&r"(a[11]), "=&r"(a[12]), "=&r"(a[13]),
+          "=&r"(a[14]), "=&r"(a[15]), "=&r"(a[16]), "=&r"(a[17]), "=&r"(a[18]), "=&r"(a[19]), "=&r"(a[20]),
+          "=&r"(a[21]), "=&r"(a[22]), "=&r"(a[23]), "=&r"(a[24]), "=&r"(a[25]), "=&r"(a[26]), "=&r"(a[27]),
+          "=&r"(a[28]), "=&r"(a[29]), "=&r"(a[30]), "=&r"(a[31]),
+          "=&r"(b[0]), "=&r"(b[1]), "=&r"(b[2]), "=&r"(b[3]), "=&r"(b[4]), "=&r"(b[5]), "=&r"(b[6]),
+          "=&r"(b[7]), "=&r"(b[8]), "=&r"(b[9]), "=&r"(b[10]), "=&r"(b[11]), "=&r"(b[12]), "=&r"(b[13]),
+          "=&r"(b[14]), "=&r"(b[15]), "=&r"(b[16]), "=&r"(b[17]), "=&r"(b[18]), "=&r"(b[19]), "=&r"(b[20]),
+          "=&r"(b[21]), "=&r"(b[22]), "=&r"(b[23]), "=&r"(b[24]), "=&r"(b[25]), "=&r"(b[26]), "=&r"(b[27]),
+          "=&r"(b[28]), "=&r"(b[29]), "=&r"(b[30]), "=&r"(b[31])
+        : "r"(ta), "r"(tb)
+        : "memory");
+}
+
+// gw columns of n accumulators, acc_stride apart, added in order into r[0 .. gw).
+__device__ __forceinline__ void tmem_sum_cols(uint32_t taddr, int acc_stride, int n, uint32_t *r, int gw) {
+    if (n == 1) {
+        tmem_ld_cols(taddr, r, gw);
+        return;
+    }
+    uint32_t e[32];
+    if (gw > 16) tmem_ld32_two(taddr, r, taddr + acc_stride, e);
+    else tmem_ld16_two(taddr, r, taddr + acc_stride, e);
+    for (int q = 2;; ++q) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(e[j]));
+        if (q >= n) return;
+        tmem_ld_cols(taddr + q * acc_stride, e, gw);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Persistent two-SM variant (the context GEMM for many token rows).
 //
@@ -297,7 +353,7 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t *r, int gw
 // streams through one continuously running TMA -> MMA pipeline, across tile
 // boundaries. Roles (192 threads): warp 0 lane 0 issues TMA, warp 1
 // allocates TMEM and the even CTA's lane 0 issues the MMAs, warps 2-5 drain the
-// accumulators. Two TMEM accumulators let the epilogue of one tile overlap the
+// accumulators. Two groups of accumulators let the epilogue of one tile overlap the
 // MMAs of the next. A tile whose K range is cut between pairs ("pieces") is
 // fixed up through the workspace, each CTA its own 128 rows: each piece is
 // written to its CTA's slot (a CTA has at most two cut tiles, its first and its
@@ -306,7 +362,7 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t *r, int gw
 // ---------------------------------------------------------------------------
 constexpr int P_THREADS = 192;
 constexpr int P_MAX_STAGES = 12;
-constexpr int P_MAX_ACC = 8;
+constexpr int P_MAX_ACC = 2;       // accumulator groups
 constexpr int P_MAX_PIECES = 128;   // pieces of one cut tile (CTAs sharing it)
 
 struct PkParams {
@@ -320,8 +376,8 @@ struct PkParams {
     int T_sk, dp_rounds;    // stream-K tiles; rounds of whole tiles after them
     int T_all;              // all 256-row tiles x token tiles
     int kb_chunk;           // K-blocks of a whole tile accumulated before they are added to Y
-    int n_acc;              // accumulators the items take in turn
-    int fold;               // a pair's only tile: its chunks stay in their accumulators and are summed at the end
+    int n_acc;              // groups of accumulators the items take in turn (<= P_MAX_ACC)
+    int n_rot;              // accumulators of a group: an item's K-blocks take turns, the epilogue sums them
     float *Y;
     int ldy, epi;
     float *ws;
@@ -540,9 +596,11 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             for (; !stop && it.next(t, kb_b, kb_e); a = a + 1 == p.n_acc ? (aph ^= 1u, 0) : a + 1) {
                 if (!w_mbar_wait_cluster(acce0 + 8 * a, aph ^ 1u, &abort_flag, p.status)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t acc = tmem + a * p.acc_stride;
-                uint32_t more = 0;          // the item's first MMA starts the accumulator
-                for (int j = kb_b; j < kb_e; ++j) {
+                const uint32_t acc0 = tmem + a * p.n_rot * p.acc_stride;
+                for (int j = kb_b, rot = 0; j < kb_e; ++j) {
+                    const uint32_t acc = acc0 + rot * p.acc_stride;
+                    const uint32_t more = j - kb_b >= p.n_rot;      // its first block starts an accumulator
+                    if (++rot == p.n_rot) rot = 0;
                     if (!w_mbar_wait_cluster(full0 + 8 * s, ph, &abort_flag, p.status)) {
                         stop = true;
                         break;
@@ -562,7 +620,6 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                         for (int kk = 0; kk < BK / 16; ++kk)
                             w_mma_bf16_pair(on, acc, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : more);
                     }
-                    more = 1;
                     w_mma_commit_pair(on, empty0 + 8 * s, (uint16_t)3);
                     if (++s == stages) {
                         s = 0;
@@ -589,19 +646,19 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         int a = 0;
         uint32_t aph = 0;
         for (int item = 0; it.next(t, kb_b, kb_e); ++item, a = a + 1 == p.n_acc ? (aph ^= 1u, 0) : a + 1) {
-            if (p.fold && kb_e < KB) continue;      // (summed with the tile's last chunk)
             int wt, seg, row0, n0;
             tile_geom(t, wt, seg, row0, n0);
             const int o_local = row0 + row;
             const bool row_in = wt < p.tiles && o_local < p.seg_rows[seg];
             const int o = p.seg_out[seg] + o_local;
             const bool whole = t >= p.T_sk || (kb_b == 0 && kb_e == KB);
-            const uint32_t taddr = tmem + a * p.acc_stride + ((uint32_t)(q * 32) << 16);
+            const uint32_t taddr = tmem + a * p.n_rot * p.acc_stride + ((uint32_t)(q * 32) << 16);
+            const int n_sub = min(p.n_rot, kb_e - kb_b);
             // a CTA cuts at most two stream-K tiles: its first item and its last
             const int slot = 2 * (2 * cta + (item == 0 ? 0 : 1)) + half;
             float *part = p.ws + (size_t)slot * BN * BM;
             // (a whole tile's later chunks add to what this thread stored for the first)
-            const bool add = p.epi == EPI_ADD || (whole && kb_b > 0 && !p.fold);
+            const bool add = p.epi == EPI_ADD || (whole && kb_b > 0);
             const bool glu = p.epi == EPI_SWIGLU;
             float *stg = reinterpret_cast<float *>(smem_raw + p.stg_off);   // [32 columns][128 rows]
             // residual rows of 32 columns, requested one group ahead (the first
@@ -625,15 +682,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 for (int j = 0; j < 32; ++j) yin[j] = ynext[j];
                 if (g0 + 32 < BN) residual(g0 + 32, ynext);
                 uint32_t r[32];
-                tmem_ld_cols(taddr + g0, r, gw);
-                if (p.fold)             // the earlier chunks' accumulators, in K order before this one's
-                    for (int q = a - 1; q >= 0; --q) {
-                        uint32_t e[32];
-                        tmem_ld_cols(tmem + q * p.acc_stride + ((uint32_t)(32 * (warp & 3)) << 16) + g0, e, gw);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            r[j] = __float_as_uint(__uint_as_float(e[j]) + __uint_as_float(r[j]));
-                    }
+                tmem_sum_cols(taddr + g0, p.acc_stride, n_sub, r, gw);     // the item's accumulators
                 if (whole && glu) {
                     // gate row i and up row 64 + i of the tile sit in different
                     // warps: exchange through shared memory, then thread (i, h)
@@ -817,7 +866,11 @@ __global__ void __launch_bounds__(P_THREADS, 1)
 // (deterministic), and writes it. At most two CTAs share an SM, so every
 // launch of the decode step is a single wave.
 // ---------------------------------------------------------------------------
-constexpr int C_THREADS = 128;
+// Eight warps: past the last MMA a CTA runs a chain of tensor-memory reads, shared
+// memory, special functions and stores, which four warps left idle for most of it
+// (per launch in a replayed 7B step, four warps and then eight: gate/up 35.4 and
+// 34.1 us, q/k/v 20.9 and 20.1, down 19.1 and 18.0, O 11.8 and 11.1).
+constexpr int C_THREADS = 256;
 constexpr int C_STAGES = 4;
 
 struct CkParams {
@@ -924,29 +977,20 @@ __device__ __forceinline__ void c_epi_swiglu(const CkParams &p, const PartSrc &p
         const float o3 = __fdividef(a.w, 1.f + __expf(-a.w)) * b.w;
         Split<bf16>::store4(act + (size_t)m * F + j, lo, make_float4(o0, o1, o2, o3));
     };
-    for (int e0 = threadIdx.x; e0 < n; e0 += 2 * C_THREADS) {
-        int col[4], row[4];
-        bool use[4];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int e = e0 + u * C_THREADS;
-            col[2 * u] = col[2 * u + 1] = ps.c_lo + (e >> 4);
-            row[2 * u] = (e & 15) << 2;
-            row[2 * u + 1] = row[2 * u] + 64;
-            use[2 * u] = use[2 * u + 1] = e < n;
-        }
-        float4 v[4];
-        c_part_sums<4>(ps, col, row, use, v);
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-            if (use[2 * u]) emit(v[2 * u], v[2 * u + 1], col[2 * u], wt * 64 + row[2 * u]);
+    for (int e = threadIdx.x; e < n; e += C_THREADS) {
+        const int c = ps.c_lo + (e >> 4), r = (e & 15) << 2;
+        const int col[2] = {c, c}, row[2] = {r, r + 64};
+        const bool use[2] = {true, true};
+        float4 v[2];
+        c_part_sums<2>(ps, col, row, use, v);
+        emit(v[0], v[1], c, wt * 64 + r);
     }
 }
 
 // Global operands of the first EPI_PRE groups (RoPE) or columns (norm) of a
 // thread are requested before the split-K exchange, so that their round trip
 // overlaps it; later ones (large column shares only) are loaded in the loop.
-constexpr int EPI_PRE = 4;
+constexpr int EPI_PRE = 2;
 
 struct RopePre {
     RowDesc d[EPI_PRE];
@@ -1143,7 +1187,7 @@ __device__ __forceinline__ void c_reduce_norm(const CkParams &p, const PartSrc &
 // RAW: mw maps the caller's row-major weight, read only after the wait on the
 // previous kernel (which may have written it); otherwise the packed blocks.
 template <bool PAIR, bool RAW>
-__global__ void __launch_bounds__(C_THREADS)
+__global__ void __launch_bounds__(C_THREADS, 2)
     gemm_cluster_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mxl,
                         const __grid_constant__ CUtensorMap mw, const CkParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -1361,7 +1405,8 @@ __global__ void __launch_bounds__(C_THREADS)
             }
     }
 
-    // ---- epilogue: all 4 warps, TMEM lane quarter = warp -------------------
+    // ---- epilogue: all warps, TMEM lane quarter = warp mod 4; warps 0-3 and
+    // 4-7 take the tile's groups of 32 columns in turn ------------------------
     const bool ok = mbar_wait(done, 0, &abort_flag, p.status) && !abort_flag;
     // K split over the cluster: this CTA's MMAs are done, so its ring may now
     // receive the other ranks' slices. It arrives on the cluster barrier here
@@ -1373,8 +1418,9 @@ __global__ void __launch_bounds__(C_THREADS)
     }
     pdl_wait();                       // (every thread) before reading Y, rows or the table
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int row = warp * 32 + lane;
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const int g_first = (warp >> 2) * 32, g_step = C_THREADS / 4;
     const bool add = p.epi == EPI_ADD;
     const int rows_here = p.seg_rows[seg] - row0;           // valid weight rows in this tile
     const int o_base = p.seg_out[seg] + row0;
@@ -1382,17 +1428,9 @@ __global__ void __launch_bounds__(C_THREADS)
     const bool norm_out = p.nout.ss != nullptr;
     // columns [g0, g0 + gw) of the tile, the accumulators that took a K-block added in order
     const int n_acc = min(p.n_acc, nk);
-    auto acc_cols = [&](int g0, uint32_t *r, int gw) {
-        tmem_ld_cols(taddr + g0, r, gw);
-        for (int q = 1; q < n_acc; ++q) {
-            uint32_t t[32];
-            tmem_ld_cols(taddr + q * p.acc_stride + g0, t, gw);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(t[j]));
-        }
-    };
+    auto acc_cols = [&](int g0, uint32_t *r, int gw) { tmem_sum_cols(taddr + g0, p.acc_stride, n_acc, r, gw); };
     if (S == 1 && !paired && !norm_out) {
-        for (int g0 = 0; g0 < BN; g0 += 32) {
+        for (int g0 = g_first; g0 < BN; g0 += g_step) {
             const int gw = min(32, BN - g0);
             uint32_t r[32];
             acc_cols(g0, r, gw);
@@ -1417,7 +1455,7 @@ __global__ void __launch_bounds__(C_THREADS)
     } else {
         // partial [BN][128] fp32 in this CTA's (now idle) stage memory
         float *part = reinterpret_cast<float *>(smem_raw + (sbase - smem_u32(smem_raw)));
-        for (int g0 = 0; g0 < BN; g0 += 32) {
+        for (int g0 = g_first; g0 < BN; g0 += g_step) {
             const int gw = min(32, BN - g0);
             uint32_t r[32];
             acc_cols(g0, r, gw);
@@ -1454,18 +1492,17 @@ __global__ void __launch_bounds__(C_THREADS)
         if (S > 1) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");    // part, for the bulk copies
             asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-            if (threadIdx.x == 0) {
-                mbar_expect_tx(recv_bar, (uint32_t)((S - 1) * (ps.c_hi - ps.c_lo) * BM * 4));
-                for (int t = 0; t < S; ++t) {
-                    const int t_lo = t * BN / S, t_hi = (t + 1) * BN / S;
-                    if (t == (int)rank || t_hi == t_lo) continue;
-                    const int slot = (int)rank < t ? (int)rank : (int)rank - 1;
+            if (warp == 0) {
+                if (lane == 0) mbar_expect_tx(recv_bar, (uint32_t)((S - 1) * (ps.c_hi - ps.c_lo) * BM * 4));
+                const int t_lo = lane * BN / S, t_hi = (lane + 1) * BN / S;
+                if (lane < S && lane != (int)rank && t_hi > t_lo) {      // lane t: rank t's slice
+                    const int slot = (int)rank < lane ? (int)rank : (int)rank - 1;
                     const uint32_t src = smem_u32(part + t_lo * BM);
-                    const uint32_t dst = c_mapa(smem_u32(ps.recv + slot * span * BM), (uint32_t)t);
+                    const uint32_t dst = c_mapa(smem_u32(ps.recv + slot * span * BM), (uint32_t)lane);
                     asm volatile(
                         "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                             dst),
-                        "r"(src), "r"((uint32_t)((t_hi - t_lo) * BM * 4)), "r"(c_mapa(recv_bar, (uint32_t)t))
+                        "r"(src), "r"((uint32_t)((t_hi - t_lo) * BM * 4)), "r"(c_mapa(recv_bar, (uint32_t)lane))
                         : "memory");
                 }
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -1484,44 +1521,34 @@ __global__ void __launch_bounds__(C_THREADS)
         else {
             // plain reduction of this CTA's columns, float4 = 4 consecutive weight rows of one token
             const int n = (ps.c_hi - ps.c_lo) * (BM / 4);
-            for (int e0 = threadIdx.x; e0 < n; e0 += 2 * C_THREADS) {
-                int col[2], row[2];
-                bool use[2];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int e = e0 + u * C_THREADS;
-                    col[u] = ps.c_lo + e / (BM / 4);
-                    row[u] = (e % (BM / 4)) * 4;
-                    use[u] = e < n;
-                }
-                float4 v[2];
-                c_part_sums<2>(ps, col, row, use, v);
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int m = n0 + col[u], r4 = row[u];
-                    if (!use[u] || !okr || m >= p.M) continue;
-                    float4 acc = v[u];
-                    float *y = p.Y + (size_t)m * p.ldy + o_base + r4;
-                    if (r4 + 4 <= rows_here && ((reinterpret_cast<uintptr_t>(y) & 15u) == 0)) {
-                        if (add) {
-                            const float4 yi = *reinterpret_cast<const float4 *>(y);
-                            acc.x += yi.x; acc.y += yi.y; acc.z += yi.z; acc.w += yi.w;
-                        }
-                        *reinterpret_cast<float4 *>(y) = acc;
-                    } else {
-                        const float vv[4] = {acc.x, acc.y, acc.z, acc.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (r4 + e < rows_here) {
-                                if (add) y[e] = y[e] + vv[e];
-                                else y[e] = vv[e];
-                            }
+            for (int e = threadIdx.x; e < n; e += C_THREADS) {
+                const int col[1] = {ps.c_lo + e / (BM / 4)}, row[1] = {(e % (BM / 4)) * 4};
+                const bool use[1] = {true};
+                float4 v[1];
+                c_part_sums<1>(ps, col, row, use, v);
+                const int m = n0 + col[0], r4 = row[0];
+                if (!okr || m >= p.M) continue;
+                float4 acc = v[0];
+                float *y = p.Y + (size_t)m * p.ldy + o_base + r4;
+                if (r4 + 4 <= rows_here && ((reinterpret_cast<uintptr_t>(y) & 15u) == 0)) {
+                    if (add) {
+                        const float4 yi = *reinterpret_cast<const float4 *>(y);
+                        acc.x += yi.x; acc.y += yi.y; acc.z += yi.z; acc.w += yi.w;
                     }
+                    *reinterpret_cast<float4 *>(y) = acc;
+                } else {
+                    const float vv[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (r4 + q < rows_here) {
+                            if (add) y[q] = y[q] + vv[q];
+                            else y[q] = vv[q];
+                        }
                 }
             }
         }
         // this CTA's outgoing copies have read its partial before it exits
-        if (S > 1 && threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        if (S > 1 && warp == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1993,7 +2020,10 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     const int nb = X_lo ? 2 : 1;
     size_t stage = A_BYTES + (size_t)nb * BN * BK * 2;
     constexpr size_t HALF_SM = 104u * 1024u, FULL_SM = 200u * 1024u;
-    const int per_sm = 3 * stage <= HALF_SM ? 2 : 1;
+    int per_sm = 3 * stage <= HALF_SM ? 2 : 1;
+    // one-plane products over more than 64 rows that leave half of the CTAs unused: one
+    // per SM, whose stage memory holds the partials of up to eight splits
+    if (nb == 1 && BN > 64 && 2 * tiles <= p->num_sms) per_sm = 1;
     int stages = (int)((per_sm == 2 ? HALF_SM : FULL_SM) / stage);
     stages = std::max(2, std::min(stages, C_STAGES));
     int S = (per_sm * p->num_sms) / tiles;
@@ -2008,17 +2038,21 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         return (long)tiles * c * 304 <= (long)slots * per_sm * p->num_sms;
     };
     while (S > 1 && !one_wave(S)) --S;
-    // One-plane products (msd_linear): the accumulators truncate, so a chain of at
-    // most 16 K-blocks each -- as many of them as 256 TMEM columns hold take turns,
-    // and K is split further where that is not enough (17 x 4096 x 11008: 1.1e-6
+    // The accumulators truncate: the K-blocks take turns over two of them, in one-plane
+    // products (msd_linear) over as many as the CTA's TMEM columns hold, and there K is
+    // split further where that leaves chains past 16 blocks (17 x 4096 x 11008: 1.1e-6
     // relative in chains of 22, below 0.8e-6 in chains of 3)
     int acc_stride = 32;
     while (acc_stride < BN) acc_stride <<= 1;
-    const int n_acc = nb == 1 ? 256 / acc_stride : 1;
+    const int all_acc = 512 / per_sm / acc_stride;
+    const int n_acc = nb == 1 ? all_acc : std::min(kblocks <= 8 ? 4 : 2, all_acc);
     if (nb == 1) S = std::max(S, std::min(8, (kblocks + 16 * n_acc - 1) / (16 * n_acc)));
     // a short K runs in one CTA: four blocks take 3.5 us, 4.6 split and exchanged
-    // (16 x 256 x 256), eight 4.5 against 4.7
-    if (kblocks <= 8) S = 1;
+    // (16 x 256 x 256), eight 4.5 against 4.7; one-plane products split past n_acc blocks
+    if (kblocks <= 8) {
+        S = nb == 1 ? (kblocks + n_acc - 1) / n_acc : 1;
+        if (!one_wave(S)) S = 1;
+    }
     while (S > 1 && kblocks / S < 2) --S;
     // own partial [BN][128] fp32 plus the other ranks' slices of this rank's columns
     while (S > 1 && (size_t)BN * BM * 4 + (size_t)(S - 1) * ((BN + S - 1) / S) * BM * 4 > stages * stage) --S;
@@ -2174,7 +2208,7 @@ bool gemm_bf16(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int
 // pairs, T_sk of the T_all tiles stream-K, the others whole in chunks of
 // kb_chunk K-blocks.
 struct PersistShape {
-    int BN, nt, G, T_all, T_sk, dp_rounds, kb_chunk;
+    int BN, nt, G, T_all, T_sk, dp_rounds, kb_chunk, n_acc, n_rot;
 };
 constexpr uint32_t P_BUDGET = 220u * 1024u;     // ring and staging bytes of a CTA
 constexpr int P_STAGES = 6;
@@ -2187,34 +2221,37 @@ constexpr int P_STAGES = 6;
 // even, but the pieces' round trip through the workspace then costs 330 BN
 // where every tile is cut (O at 640 rows, 224 columns: 68 us against 40 in whole
 // tiles), about 180 BN where whole tiles follow to hide part of it.
-// A one-plane product (msd_linear) accumulates short chains of K-blocks: the
-// accumulators truncate, so the error grows with the chain (4096-long products:
-// 2.2e-6 relative in chains of 32 to 40 blocks, 4.4e-6 in one of 64). A pair's only
-// tile keeps its chunks in accumulators of their own, up to the 512 TMEM columns,
-// summed by its epilogue; otherwise chunks of 24 blocks are added to Y one after
-// another (576 x 4096 x 4096: 34 us added, 22 us kept).
+// The accumulators truncate, so the error grows with the chain of K-blocks that one
+// takes (one-plane products of 4096 terms: 2.2e-6 relative in chains of 32 to 40
+// blocks, 4.4e-6 in one of 64). The K-blocks of an item take turns over as many
+// accumulators as there is room for: 512 TMEM columns where a pair has one item,
+// half of them where its next item runs beside the epilogue. One-plane products
+// (msd_linear), which have no other error, are also cut into narrower tiles while
+// one round holds them: a K-block of 32 columns takes no longer than one of 96, and
+// 16 accumulators fit (1245 x 3664 x 129: 27.3 us and 9.0e-7 with tiles of 64 columns
+// or more, 23.2 us and 1.3e-7; 1000 x 512 x 1024: 15.0 to 12.9 us). Past 24
+// blocks in every accumulator, chunks of K are added to Y one after another.
 static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int pairs, size_t ws_bytes,
                                   int n_counters) {
     const int kblocks = (K + BK - 1) / BK, wt = (tiles + 1) / 2;
     PersistShape best{};
     double best_cost = 1e300;
-    for (int nt = (M + 255) / 256, n = 0; n < 6; ++nt, ++n) {
+    for (int nt = (M + 255) / 256, n = 0; n < 6 || (nb == 1 && (long long)wt * nt <= pairs); ++nt, ++n) {
         const int BN = ((M + nt - 1) / nt + 15) / 16 * 16;
-        if (n > 0 && BN < 64) break;
+        if (n > 0 && BN < (nb == 1 ? 32 : 64)) break;
         const long long T = (long long)wt * nt;
         const double tk = std::max(2.08 * nb * BN, 420.0 + 0.8 * nb * BN);
         // at least 4 K-blocks a pair
         const long long G = std::max<long long>(1, std::min<long long>(pairs, T * kblocks / 4));
-        int n_ch = 1;
-        if (nb == 1 && !glu) {
-            int stride = 32;
-            while (stride < BN) stride <<= 1;
-            const int most = T <= G ? std::min(512 / stride, P_MAX_ACC) : 1;    // accumulators of a pair's only tile
-            n_ch = (kblocks + 15) / 16;
-            if (n_ch > most) n_ch = (kblocks + 31) / 32 <= most ? most : (kblocks + 23) / 24;
-        }
+        int stride = 32;
+        while (stride < BN) stride <<= 1;
+        const int most = nb == 1 ? 16 : 4;
+        const bool chunked = nb == 1 && !glu;
+        const bool lone = T <= G && (!chunked || (kblocks + 31) / 32 <= 512 / stride);    // one item a pair
+        const int n_acc = lone ? 1 : 2, n_rot = std::min(512 / n_acc / stride, most);
+        const int n_ch = chunked && !lone ? (kblocks + 24 * n_rot - 1) / (24 * n_rot) : 1;
         const int chunk = (kblocks + n_ch - 1) / n_ch;
-        PersistShape g{BN, nt, (int)G, (int)T, 0, (int)((T + G - 1) / G), chunk};
+        PersistShape g{BN, nt, (int)G, (int)T, 0, (int)((T + G - 1) / G), chunk, n_acc, n_rot};
         double cost = g.dp_rounds * tk * kblocks;
         int rounds = (int)(T / G), T_sk = (int)(T - rounds * G);
         if (T_sk > 0) {
@@ -2231,6 +2268,8 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
                 2LL * T_sk <= n_counters) {
                 g.T_sk = T_sk;
                 g.dp_rounds = rounds;
+                g.n_acc = chunked && rounds == 0 ? 1 : 2;
+                g.n_rot = std::min(512 / g.n_acc / stride, most);
                 cost = sk;
             }
         }
@@ -2274,14 +2313,10 @@ static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     pk.n_tiles_n = nt;
     pk.stages = stages;
     pk.acc_stride = acc;
-    pk.n_acc = 2;
-    const int chunks = (kblocks + g.kb_chunk - 1) / g.kb_chunk;
-    if (chunks > 1 && g.T_sk == 0 && g.dp_rounds == 1 && chunks <= std::min(512 / acc, P_MAX_ACC)) {
-        pk.fold = 1;
-        pk.n_acc = std::max(2, chunks);
-    }
+    pk.n_acc = g.n_acc;
+    pk.n_rot = g.n_rot;
     pk.tmem_cols = 64;
-    while (pk.tmem_cols < pk.n_acc * acc) pk.tmem_cols <<= 1;
+    while (pk.tmem_cols < pk.n_acc * pk.n_rot * acc) pk.tmem_cols <<= 1;
     pk.grid = G;
     pk.tiles = tiles;
     pk.units = units;

@@ -21,6 +21,9 @@ SHAPES = [(129, 64, 128), (129, 8, 1), (144, 72, 300), (255, 4096, 129), (256, 2
 
 SHAPES += [(1, 8, 1), (7, 4096, 129), (16, 2048, 40000), (17, 72, 1000), (33, 11008, 64), (60, 4096, 4096),
            (128, 1032, 500), (100, 64, 20000)]
+# narrow tiles with up to 16 accumulators, cut short-K tiles, one CTA per SM past 64 rows
+SHAPES += [(349, 944, 216), (309, 456, 77), (1309, 7184, 68), (176, 11008, 4096), (129, 4096, 1000),
+           (119, 1520, 126), (80, 400, 300), (60, 304, 121), (7, 536, 19502)]
 
 
 @pytest.mark.parametrize("m,k,o", SHAPES)
