@@ -8,11 +8,11 @@
 // at once: packed fp32 FMAs (f32x2) keep the even-k and the odd-k sums of each
 // output in one 64-bit register, added at the end. Rows are padded to 68
 // floats, so the 8 rows a warp reads together sit in different banks.
-// Tiles of 32 x 8 to 128 outputs x 64 token rows, always 256 threads: the
+// Tiles of 32 outputs x 8 token rows to 128 x 128, always 256 threads: the
 // smaller the tile, the more warps share it by taking different k of a stage
-// (their sums meet in shared memory). When the tiles leave SMs idle, K is
-// split over the CTAs of a cluster (at most 8), whose partial tiles are summed
-// through distributed shared memory in rank order. Every order is fixed by the
+// (their sums meet in shared memory). K may be split over the CTAs of a cluster
+// (at most 8), whose partial tiles are summed through distributed shared memory
+// in rank order. Every order is fixed by the
 // launch's shape, so results are reproducible and an output depends only on
 // its own row of X.
 #include <cooperative_groups.h>
@@ -62,7 +62,6 @@ struct Tile {
     static constexpr int KS = SG_THREADS / GROUP;
     static constexpr int STAGE = (BO + BM) * SG_LD;                        // floats
     static constexpr int SMEM = STAGES * STAGE * 4;
-    static constexpr int PER_SM = TO * TM >= 64 ? 1 : 2;                   // CTAs an SM holds (registers)
     static_assert(GROUP % 32 == 0 && (SG_BK / 4) % KS == 0, "whole warps, whole 4-k chunks");
     static_assert(KS * BO * BM <= STAGES * STAGE, "the k groups' partial tiles reuse the ring");
 };
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(SG_THREADS) gemm_simt_kernel(const SgArgs a) {
     const int b0 = (int)((long long)split * nb / a.splits), b1 = (int)((long long)(split + 1) * nb / a.splits);
 
     // the rows this thread copies: 16 threads per row of a stage
-    constexpr int RO = TL::BO / 16, RM = (TL::BM + 15) / 16;    // (an 8-row tile: half of its last pass is idle)
+    constexpr int RO = TL::BO / 16, RM = (TL::BM + 15) / 16;    // (8- and 24-row tiles: half of the last pass is idle)
     const int crow = tid >> 4, cq = (tid & 15) * 4;
     const float *src[RO + RM];
 #pragma unroll
@@ -109,7 +108,7 @@ __global__ void __launch_bounds__(SG_THREADS) gemm_simt_kernel(const SgArgs a) {
         const int k = blk * SG_BK + cq;
 #pragma unroll
         for (int i = 0; i < RO + RM; ++i) {
-            if (TL::BM < 16 && i == RO && crow >= TL::BM) break;
+            if (TL::BM % 16 && i == RO + RM - 1 && crow + 16 * (RM - 1) >= TL::BM) break;
             const uint32_t d = s0 + (uint32_t)(st * TL::STAGE + 16 * i * SG_LD) * 4u;
             const float *p = src[i];
             if constexpr (VEC) {                  // K % 4 == 0: whole chunks
@@ -210,14 +209,9 @@ __global__ void __launch_bounds__(SG_THREADS) gemm_simt_kernel(const SgArgs a) {
 }
 
 template <class TL, bool VEC>
-void launch_tile(SgArgs a, int num_sms, cudaStream_t s) {
+void launch_tile(SgArgs a, int S, cudaStream_t s) {
     const int to = (a.O + TL::BO - 1) / TL::BO, tm = (a.M + TL::BM - 1) / TL::BM;
-    const int nb = (a.K + SG_BK - 1) / SG_BK;
-    // split K while that still fills idle SMs and leaves every split two or more
-    // k blocks
-    long S = (long)TL::PER_SM * num_sms / std::max(1L, (long)to * tm);
-    S = std::max(1L, std::min(std::min(S, 8L), (long)nb / 2));
-    a.splits = (int)S;
+    a.splits = S;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)to, (unsigned)tm, (unsigned)S);
     lc.blockDim = dim3(SG_THREADS);
@@ -237,12 +231,6 @@ void launch_tile(SgArgs a, int num_sms, cudaStream_t s) {
 }
 
 template <class TL>
-void launch_vec(const SgArgs &a, bool vec, int num_sms, cudaStream_t s) {
-    if (vec) launch_tile<TL, true>(a, num_sms, s);
-    else launch_tile<TL, false>(a, num_sms, s);
-}
-
-template <class TL>
 bool set_tile() {
     return cudaFuncSetAttribute(gemm_simt_kernel<TL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::SMEM) ==
                cudaSuccess &&
@@ -250,15 +238,34 @@ bool set_tile() {
                cudaSuccess;
 }
 
-typedef Tile<32, 8, 4, 2, 4> T32x8;
-typedef Tile<32, 16, 4, 4, 4> T32x16;
-typedef Tile<32, 32, 4, 4, 4> T32x32;
-typedef Tile<64, 64, 8, 8, 3> T64x64;
-typedef Tile<128, 64, 8, 8, 3> T128x64;
+// The tiles, with the time of one k block of a tile, its start and end, and what a
+// K split's exchange adds (ns, when every SM holds as many as fit).
+struct TileRow {
+    int BO, BM;
+    double block_ns, tile_ns, split_ns;
+    void (*launch[2])(SgArgs, int, cudaStream_t);     // [16-byte aligned rows]
+    bool (*setup)();
+};
+template <class TL>
+constexpr TileRow tile_row(double block_ns, double tile_ns, double split_ns) {
+    return {TL::BO, TL::BM, block_ns, tile_ns, split_ns, {launch_tile<TL, false>, launch_tile<TL, true>}, set_tile<TL>};
+}
+const TileRow TILES[] = {
+    tile_row<Tile<32, 8, 4, 2, 4>>(200, 200, 1500),
+    tile_row<Tile<32, 16, 4, 4, 4>>(300, 200, 1500),
+    tile_row<Tile<32, 24, 4, 3, 4>>(430, 200, 1500),
+    tile_row<Tile<32, 32, 4, 4, 4>>(595, 200, 1500),
+    tile_row<Tile<128, 64, 8, 8, 3>>(3450, 800, 10000),
+    tile_row<Tile<128, 128, 8, 8, 3>>(6150, 800, 10000),
+};
 
 }  // namespace
 
-bool gemm_simt_setup() { return set_tile<T32x8>() && set_tile<T32x16>() && set_tile<T32x32>() && set_tile<T64x64>() && set_tile<T128x64>(); }
+bool gemm_simt_setup() {
+    for (const TileRow &t : TILES)
+        if (!t.setup()) return false;
+    return true;
+}
 
 void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int O, float *Y, int ldy, int epi,
                       int num_sms, cudaStream_t s) {
@@ -274,18 +281,33 @@ void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int
     uintptr_t bits = reinterpret_cast<uintptr_t>(X);
     for (int i = 0; i < W.nseg; ++i) bits |= reinterpret_cast<uintptr_t>(w[i]);
     const bool vec = (bits & 15) == 0 && K % 4 == 0 && ldx % 4 == 0;
-    const int n = num_sms;
-    // The smallest tiles win while they all run at once (weights are read once per
-    // row of tiles, and small tiles share one among more warps): 24 x 1024 x 2816
-    // 12.5 us in 32 x 32 tiles, 22.6 in 64 x 32. Past two CTAs an SM, FMAs per
-    // shared-memory load decide: 333 x 3072 x 1024 57 us in 128 x 64 tiles, 66 to 81
-    // in smaller ones; 333 x 1024 x 1024 35 us in 64 x 64, 52 in 128 x 64 (48 tiles).
-    const long t32 = (long)((O + 31) / 32) * ((M + 31) / 32), t128 = (long)((O + 127) / 128) * ((M + 63) / 64);
-    if (M <= 8) launch_vec<T32x8>(a, vec, n, s);
-    else if (M <= 16) launch_vec<T32x16>(a, vec, n, s);
-    else if (M <= 32 || t32 <= 2L * n) launch_vec<T32x32>(a, vec, n, s);
-    else if (8 * t128 < 7L * n) launch_vec<T64x64>(a, vec, n, s);
-    else launch_vec<T128x64>(a, vec, n, s);
+    // The tile and the K splits whose rounds over the SMs take least. Small tiles leave
+    // the least of the chip idle, large ones make the most of a shared-memory load (us, in
+    // 32 x 24, 32 x 32, 128 x 64 and 128 x 128 tiles: 24 x 32000 x 1024 50, 67, -, -; 100 x
+    // 5632 x 1024 43, 49, 56, 99; 341 x 5632 x 1024 120, 121, 110, 99; 341 x 1024 x 2816
+    // 74, 78, 146, 262, and 69 in two splits of 32 x 24). One small tile on a SM hides
+    // less of its latency. Over 30 shapes the choice is within 1% of the best on average,
+    // 14% at most; splits of three ran up to half a round longer than of two or four.
+    const int nb = (K + SG_BK - 1) / SG_BK;
+    const TileRow *best = nullptr;
+    int S = 1;
+    double best_ns = 0;
+    for (const TileRow &t : TILES) {
+        if (t.BM < 24 && M > 4 * t.BM) continue;
+        const long tiles = (long)((O + t.BO - 1) / t.BO) * ((M + t.BM - 1) / t.BM);
+        for (int sp = 1; sp <= 8 && (sp == 1 || sp <= nb / 2); sp *= 2) {
+            const long rounds = (tiles * sp + num_sms - 1) / num_sms;
+            double ns = rounds * (t.block_ns * ((nb + sp - 1) / sp) + t.tile_ns);
+            if (rounds == 1 && t.BM < 64) ns *= 1.25;
+            if (sp > 1) ns += rounds * t.split_ns;
+            if (!best || ns < best_ns) {
+                best = &t;
+                best_ns = ns;
+                S = sp;
+            }
+        }
+    }
+    best->launch[vec](a, S, s);
 }
 
 }  // namespace msd

@@ -19,6 +19,11 @@ TINY = synth.WORKLOADS["tiny"]
 GEMM = [(1, 1, 1, 0, 0), (1, 64, 33, 0, 0), (16, 256, 256, 0, 0), (17, 260, 65, 4, 0), (32, 2816, 64, 0, 0),
         (33, 127, 129, 0, 0), (64, 8192, 16, 0, 0), (65, 66, 700, 1, 0), (5, 4096, 1024, 0, 1),
         (200, 1028, 500, 0, 0), (7, 3, 2000, 2, 3)]
+# every tile and split of the rule: 24-row tiles (one and several, short last ones), 128-row
+# tiles with short last rows and columns, two and four splits
+GEMM += [(24, 1024, 4000, 0, 0), (24, 2816, 1024, 4, 0), (20, 200, 5000, 1, 0), (48, 130, 3000, 0, 0),
+         (100, 512, 5632, 0, 0), (341, 256, 5632, 0, 0), (341, 2816, 1024, 0, 0), (700, 129, 2900, 0, 1),
+         (1500, 64, 3072, 0, 0), (257, 60, 6000, 3, 2), (16, 1024, 1024, 0, 0)]
 
 
 @pytest.mark.parametrize("m,k,o,pad,off", GEMM)
