@@ -280,30 +280,6 @@ __device__ __forceinline__ void copy_row_split(TD *__restrict__ dst, long dlo, c
     }
 }
 
-// One fp32 source row to an fp32 row (d1, nullable) and a split row (d2, lo
-// plane at dlo).
-template <typename TD2>
-__device__ __forceinline__ void copy_row_2dst_split(float *__restrict__ d1, TD2 *__restrict__ d2, long dlo,
-                                                    const float *__restrict__ src, int n) {
-    const int n4 = n >> 2;
-    for (int g0 = threadIdx.x; g0 < n4; g0 += 4 * blockDim.x) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) v[u] = *reinterpret_cast<const float4 *>(src + 4 * g);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) {
-                if (d1) *reinterpret_cast<float4 *>(d1 + 4 * g) = v[u];
-                Split<TD2>::store4(d2 + 4 * g, dlo, v[u]);
-            }
-        }
-    }
-}
-
 // Two row copies in one pass into split rows (lo planes at dlo): d1 <- s1 (a
 // split source with lo plane at s1lo, or fp32; null: zeros), d2 <- s2 (read
 // as its hi values alone: exact bf16 embeddings).

@@ -40,27 +40,26 @@ __global__ void catchup_setup_kernel(const int *__restrict__ seq_len, const int 
                      H, lo);
 }
 
-// h_hat of the root slot = draft output of the last pending row.
+// The root slot's row of the catch-up pass: request b's last pending row.
+__device__ __forceinline__ int root_row(const int *n_pend, int b, int D1) { return b * D1 + max(n_pend[b] - 1, 0); }
+
+// LM-head input of the root slot = draft output of the last pending row.
 template <typename T>
 __global__ void root_gather_kernel(const float *__restrict__ x, const int *__restrict__ n_pend, int D1,
-                                   int H, float *__restrict__ hhat_root, T *__restrict__ xr, long lo) {
+                                   int H, T *__restrict__ xr, long lo) {
     wait_prior();
     allow_dependents();
     const int b = blockIdx.x;
-    const int r = b * D1 + max(n_pend[b] - 1, 0);
-    copy_row_2dst_split(hhat_root + (size_t)b * H, xr + (size_t)b * H, lo, x + (size_t)r * H, H);
+    copy_row_split(xr + (size_t)b * H, lo, x + (size_t)root_row(n_pend, b, D1) * H, 0, H);
 }
 
-// Store h_hat of a tree pass's rows by slot, and a T copy for the LM head.
+// LM-head input of a tree pass's rows, where the last GEMM did not write it.
 template <typename T>
-__global__ void hhat_store_kernel(const float *__restrict__ x, const RowDesc *__restrict__ rows,
-                                  int Td, int H, float *__restrict__ hhat_slot, T *__restrict__ xb, long lo) {
+__global__ void draft_rows_kernel(const float *__restrict__ x, int H, T *__restrict__ xr, long lo) {
     wait_prior();
     allow_dependents();
     const int r = blockIdx.x;
-    const RowDesc d = rows[r];
-    copy_row_2dst_split(hhat_slot + ((size_t)d.req * Td + d.dst) * H, xb + (size_t)r * H, lo,
-                        x + (size_t)r * H, H);
+    copy_row_split(xr + (size_t)r * H, lo, x + (size_t)r * H, 0, H);
 }
 
 // Assemble the draft-pass row j of request b for a frontier node with token
@@ -123,7 +122,7 @@ __global__ void tree_init_kernel(DraftArgs<T> a) {
         for (int t = threadIdx.x; t < k; t += blockDim.x) a.frontier[(size_t)b * k + t] = front[t];
     if (a.D < 2) return;
     const int c = front[j];
-    emit_frontier_row(a, b, j, a.ids[(size_t)b * k + c], 1, a.hhat_root + (size_t)b * a.H, j,
+    emit_frontier_row(a, b, j, a.ids[(size_t)b * k + c], 1, a.x + (size_t)root_row(a.n_pend, b, a.D + 1) * a.H, j,
                       nullptr);
 }
 
@@ -172,7 +171,7 @@ __global__ void tree_step_kernel(DraftArgs<T> a, int d) {
     const int sp = (d - 2) * k + jp;                   // parent's slot
     const int slot = (d - 1) * k + j;
     emit_frontier_row(a, b, j, a.ids[((size_t)b * k + jp) * k + (e - jp * k)], d,
-                      a.hhat_slot + ((size_t)b * a.Td + sp) * a.H, slot,
+                      a.x + ((size_t)b * k + jp) * a.H, slot,
                       a.slot_mask + ((size_t)b * a.Td + sp) * a.Wd);
 }
 
@@ -821,15 +820,13 @@ void launch_catchup_setup(const int *seq_len, const int *n_pend, const T *pend_h
 }
 
 template <typename T>
-void launch_root_gather(const float *x, const int *n_pend, int B, int D1, int H, float *hhat_root,
-                        T *xr, long lo, cudaStream_t s) {
-    launch_chain(root_gather_kernel<T>, B, 256, 0, s, x, n_pend, D1, H, hhat_root, xr, lo); note_launch();
+void launch_root_gather(const float *x, const int *n_pend, int B, int D1, int H, T *xr, long lo, cudaStream_t s) {
+    launch_chain(root_gather_kernel<T>, B, 256, 0, s, x, n_pend, D1, H, xr, lo); note_launch();
 }
 
 template <typename T>
-void launch_hhat_store(const float *x, const RowDesc *rows, int R, int Td, int H,
-                       float *hhat_slot, T *xb, long lo, cudaStream_t s) {
-    launch_chain(hhat_store_kernel<T>, R, 256, 0, s, x, rows, Td, H, hhat_slot, xb, lo); note_launch();
+void launch_draft_rows(const float *x, int R, int H, T *xr, long lo, cudaStream_t s) {
+    launch_chain(draft_rows_kernel<T>, R, 256, 0, s, x, H, xr, lo); note_launch();
 }
 
 template <typename T>
@@ -939,10 +936,8 @@ void launch_prefill_finish(const int *argmax, const T *h_last, const int *L, int
     template void launch_catchup_setup<T>(const int *, const int *, const T *, const int *,     \
                                           const T *, int, int, int, int, T *, long, RowDesc *,  \
                                           int *, cudaStream_t);                                 \
-    template void launch_root_gather<T>(const float *, const int *, int, int, int, float *, T *, \
-                                        long, cudaStream_t);                                    \
-    template void launch_hhat_store<T>(const float *, const RowDesc *, int, int, int, float *,  \
-                                       T *, long, cudaStream_t);                                \
+    template void launch_root_gather<T>(const float *, const int *, int, int, int, T *, long, cudaStream_t); \
+    template void launch_draft_rows<T>(const float *, int, int, T *, long, cudaStream_t);       \
     template void launch_tree_init<T>(const DraftArgs<T> &, int, cudaStream_t);                 \
     template void launch_tree_step<T>(const DraftArgs<T> &, int, int, cudaStream_t);            \
     template void launch_compact<T>(const void *, void *, const int *, const int *, const int *, int, int, int, \

@@ -18,8 +18,8 @@ struct DraftArgs {
     int *cand_tok, *cand_par, *cand_depth;   // [B][C]
     float *cand_score;                       // [B][C]
     int *frontier;                           // [2][B][k] candidate ids, best first (by pass parity)
-    const float *hhat_root;                  // [B][H]
-    const float *hhat_slot;                  // [B][Td][H]
+    const float *x;             // h_hat: the pass's output rows (pass 1: B * (D + 1) catch-up rows, then B * k)
+    const int *n_pend;          // pending rows of each request (the root slot's is the last)
     const T *E;
     const int *seq_len;
     T *xfc;                     // next pass input rows [B*k][2H] (split: lo plane at +lo)
@@ -47,11 +47,9 @@ void launch_catchup_setup(const int *seq_len, const int *n_pend, const T *pend_h
                           const int *pend_next, const T *E, int B, int H, int D1, int V, T *xfc,
                           long lo, RowDesc *rows, int *status, cudaStream_t s);
 template <typename T>
-void launch_root_gather(const float *x, const int *n_pend, int B, int D1, int H, float *hhat_root,
-                        T *xr, long lo, cudaStream_t s);
+void launch_root_gather(const float *x, const int *n_pend, int B, int D1, int H, T *xr, long lo, cudaStream_t s);
 template <typename T>
-void launch_hhat_store(const float *x, const RowDesc *rows, int R, int Td, int H,
-                       float *hhat_slot, T *xb, long lo, cudaStream_t s);
+void launch_draft_rows(const float *x, int R, int H, T *xr, long lo, cudaStream_t s);
 template <typename T>
 void launch_tree_init(const DraftArgs<T> &a, int B, cudaStream_t s);
 template <typename T>

@@ -46,7 +46,8 @@ struct msd_ctx {
     uint64_t *vmask = nullptr;
     int *cand_tok = nullptr, *cand_par = nullptr, *cand_depth = nullptr, *frontier = nullptr,
         *node_of = nullptr;
-    float *cand_score = nullptr, *hhat_root = nullptr, *hhat_slot = nullptr;
+    float *cand_score = nullptr;
+    void *ones = nullptr;         // [H] unit gain (bf16)
     uint64_t *slot_mask = nullptr, *row_mask = nullptr;
     int *topk_ids = nullptr;
     float *topk_logp = nullptr;
@@ -576,7 +577,7 @@ DraftArgs<T> draft_args(msd_ctx *c) {
     a.B = c->B;
     a.cand_tok = c->cand_tok; a.cand_par = c->cand_par; a.cand_depth = c->cand_depth;
     a.cand_score = c->cand_score; a.frontier = c->frontier;
-    a.hhat_root = c->hhat_root; a.hhat_slot = c->hhat_slot;
+    a.x = c->x; a.n_pend = c->n_pend;
     a.E = static_cast<const T *>(c->w.embed);
     a.seq_len = c->seq_len;
     a.xfc = static_cast<T *>(c->xfc);
@@ -620,7 +621,7 @@ msd_status draft_impl(msd_ctx *c, const msd_tree *out, const msd_draft_record *r
     bool folded = draft_fc<T>(c, R1, s);
     run_layer<T>(c, c->w.draft, c->dpack, R1, c->rows, dK, dV, S, dK, dV, S, nullptr, nullptr, 0, nullptr, 0,
                  D1, s, folded);
-    launch_root_gather<T>(c->x, c->n_pend, B, D1, H, c->hhat_root, static_cast<T *>(c->xr), c->lo, s);
+    launch_root_gather<T>(c->x, c->n_pend, B, D1, H, static_cast<T *>(c->xr), c->lo, s);
     gemm<T>(c, static_cast<const T *>(c->xr), H, B, H, one(c->w.lm_head, V, c->pk_lm), V, c->logits, V,
             EPI_STORE, s);
     launch_topk_logp(c->logits, B, V, k, c->topk_ids, c->topk_logp, c->tks, s);
@@ -632,11 +633,16 @@ msd_status draft_impl(msd_ctx *c, const msd_tree *out, const msd_draft_record *r
     const int Rk = B * k;
     for (int d = 2; d <= c->D; ++d) {
         folded = draft_fc<T>(c, Rk, s);
-        run_layer<T>(c, c->w.draft, c->dpack, Rk, c->rows, tK, tV, c->Td, dK, dV, S, tK, tV, c->Td,
-                     c->row_mask, c->Wd, k, s, folded);
-        launch_hhat_store<T>(c->x, c->rows, Rk, c->Td, H, c->hhat_slot, static_cast<T *>(c->xr), c->lo, s);
-        gemm<T>(c, static_cast<const T *>(c->xr), H, Rk, H, one(c->w.lm_head, V, c->pk_lm), V, c->logits, V,
-                EPI_STORE, s);
+        // The LM head's input: x itself (fp32), or x as a split pair, which the layer's
+        // last GEMM writes like a folded norm of unit gain.
+        const T *head = reinterpret_cast<const T *>(c->x);
+        folded = run_layer<T>(c, c->w.draft, c->dpack, Rk, c->rows, tK, tV, c->Td, dK, dV, S, tK, tV, c->Td,
+                              c->row_mask, c->Wd, k, s, folded, c->ones);
+        if (c->esz == 2) {
+            if (!folded) launch_draft_rows<T>(c->x, Rk, H, static_cast<T *>(c->xr), c->lo, s);
+            head = static_cast<const T *>(folded ? c->xn : c->xr);
+        }
+        gemm<T>(c, head, H, Rk, H, one(c->w.lm_head, V, c->pk_lm), V, c->logits, V, EPI_STORE, s);
         launch_topk_logp(c->logits, Rk, V, k, c->topk_ids, c->topk_logp, c->tks, s);
         st = record_pass(c, rec, d - 1, k, s);
         if (st != MSD_OK) return st;
@@ -937,8 +943,7 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
     ok &= dalloc(c, &c->cand_score, sizeof(float) * c->B * c->C);
     ok &= dalloc(c, &c->node_of, sizeof(int) * c->B * c->C);
     ok &= dalloc(c, &c->frontier, sizeof(int) * 2 * c->B * c->k);
-    ok &= dalloc(c, &c->hhat_root, sizeof(float) * c->B * H);
-    ok &= dalloc(c, &c->hhat_slot, sizeof(float) * c->B * c->Td * H);
+    if (cfg->dtype == MSD_BF16) ok &= dalloc(c, &c->ones, 2 * (size_t)H);
     ok &= dalloc(c, &c->slot_mask, sizeof(uint64_t) * c->B * c->Td * c->Wd);
     ok &= dalloc(c, &c->row_mask, sizeof(uint64_t) * c->B * c->k * c->Wd);
     ok &= dalloc(c, &c->topk_ids, sizeof(int) * c->Rlog * c->k);
@@ -985,7 +990,9 @@ msd_status msd_create(const msd_config *cfg, const msd_weights *w, msd_ctx **out
             const double ang = (double)p * th;
             tab[(size_t)p * (c->hd / 2) + i] = make_float2((float)std::cos(ang), (float)std::sin(ang));
         }
-    if (cudaMemcpy(c->rope_tab, tab.data(), sizeof(float2) * tab.size(), cudaMemcpyHostToDevice) !=
+    const std::vector<uint16_t> ones(c->ones ? H : 0, 0x3F80);      // bf16 1.0
+    if (cudaMemcpy(c->ones, ones.data(), 2 * ones.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(c->rope_tab, tab.data(), sizeof(float2) * tab.size(), cudaMemcpyHostToDevice) !=
             cudaSuccess ||
         cudaDeviceSynchronize() != cudaSuccess) {
         msd_destroy(c);
