@@ -136,18 +136,22 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
         }
     };
 
-    // score tile: lanes run 8 keys x 4 rows, warps 2 (keys) x 4 (rows)
+    // score tile: lanes run 8 keys (lane bits 0, 2, 3) x 4 rows (bits 1, 4), warps 2 (keys)
+    // x 4 (rows): neighbouring lanes share every address of one operand, so that a
+    // 16-byte load serves more lanes at a time
     constexpr int SR = QR / 16, SKEYS = 4;                      // rows and keys per thread
     const int warp = tid >> 5, lane = tid & 31;
-    const int sk = (warp & 1) * 8 + (lane & 7), sr = (warp >> 1) * 4 + (lane >> 3);     // + 16 * i
+    const int sk = (warp & 1) * 8 + ((lane & 1) | (lane >> 1 & 6));                     // + 16 * i
+    const int sr = (warp >> 1) * 4 + ((lane >> 1 & 1) | (lane >> 3 & 2));
     // softmax: GT neighbouring threads per row
     constexpr int GT = AS_THREADS / QR, KPT = AS_KT / GT;
     const int xr = tid / GT, xk = tid % GT;
     const int xplen = xr < nrows ? min(a.rows[r0 + xr].plen, k_hi) : 0;
     const uint64_t *xmask = a.mask && xr < nrows ? a.mask + (size_t)(r0 + xr) * a.mask_words : nullptr;
-    // output tile: DT threads along the head dim, 4 dims each; rows or_ + OG * i
+    // output tile: DT threads along the head dim, 4 dims each; rows orow + OG * i (16
+    // threads a row: two rows side by side in neighbouring lanes)
     constexpr int DT = HD / 4, OG = AS_THREADS / DT, OR = QR / OG > 0 ? QR / OG : 1;
-    const int od = (tid % DT) * 4, orow = tid / DT;
+    const int od = (DT == 16 ? lane >> 1 : tid % DT) * 4, orow = DT == 16 ? warp * 2 + (lane & 1) : tid / DT;
     unsigned long long o01[OR] = {}, o23[OR] = {};
 
     if (nt > 0) load(0);
