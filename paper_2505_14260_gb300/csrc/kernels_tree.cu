@@ -90,6 +90,11 @@ __device__ void emit_frontier_row(const DraftArgs<T> &a, int b, int j, int tok, 
     copy_rows2_split(dst, parent_h, 0, dst + H, a.E + (size_t)tok * H, H, a.lo);
 }
 
+// The value a candidate is ranked by: its score, or -infinity where that is NaN (the
+// row's logits were not finite). Ties go to the lower index, so the order is total and
+// every rank is taken exactly once: the frontiers and the tree index by it.
+__device__ __forceinline__ float rank_value(float s) { return s == s ? s : -INFINITY; }
+
 // Depth-1 candidates from the root slot's top-k; the frontier of pass 2 is all
 // of them, best first. Grid (k, B): CTA j emits row j of pass 2; CTA 0 writes
 // the candidate arrays and the frontier (buffer 0).
@@ -102,7 +107,7 @@ __global__ void tree_init_kernel(DraftArgs<T> a) {
     __shared__ int front[TREE_MAXK];
     for (int t = threadIdx.x; t < k; t += blockDim.x) {
         const float s = a.logp[(size_t)b * k + t];
-        sc[t] = s;
+        sc[t] = rank_value(s);
         if (j == 0) {
             const size_t c = (size_t)b * a.C + t;
             a.cand_tok[c] = a.ids[(size_t)b * k + t];
@@ -147,7 +152,7 @@ __global__ void tree_step_kernel(DraftArgs<T> a, int d) {
         const int p = fin[jr];
         const size_t src = ((size_t)b * k + jr) * k + t;
         const float s = __fadd_rn(a.cand_score[(size_t)b * a.C + p], a.logp[src]);
-        sc[e] = s;
+        sc[e] = rank_value(s);
         if (j == 0) {
             const size_t c = (size_t)b * a.C + base + e;
             a.cand_tok[c] = a.ids[src];
@@ -192,7 +197,7 @@ __global__ void tree_finalize_kernel(TreeOut t, const int *__restrict__ cand_tok
     const int b = blockIdx.x, W = (N + 63) / 64;
     const size_t cb = (size_t)b * C;
     for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        ssc[c] = cand_score[cb + c];
+        ssc[c] = rank_value(cand_score[cb + c]);
         spar[c] = cand_par[cb + c];
     }
     __syncthreads();

@@ -182,3 +182,31 @@ def test_argmax_of_unaligned_rows(vocab, depth):
     am = eng.verify(logits=logits).cpu().numpy()
     assert np.array_equal(am, np.argmax(logits.cpu().numpy(), 1))
     eng.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("depth,nodes,topk", [(1, 5, 4), (4, 16, 4), (5, 60, 10)])
+def test_nonfinite_prompt_gives_a_well_formed_tree(dtype, bad, depth, nodes, topk):
+    """Logits that are not finite score every candidate NaN: the tree is still one (each
+    parent before its child, tokens of the vocabulary), and later calls go on."""
+    wl = synth.WORKLOADS["tiny"].with_(dtype=dtype, tree_depth=depth, tree_nodes=nodes, topk=topk, steps=2)
+    eng, _ = open_engine(wl)
+    p = synth.make_prompts(wl)[0]
+    p.vis[20] = bad
+    eng.prefill(*msd.upload_prompts([p]))
+    for _ in range(2):
+        eng.draft_tree()
+        torch.cuda.synchronize()
+        tok, par = eng.tree.tokens.cpu().numpy(), eng.tree.parent.cpu().numpy()
+        assert par[0] == -1 and all(0 <= par[i] < i for i in range(1, nodes))
+        assert ((tok >= 0) & (tok < wl.vocab)).all()
+        dep = [0]
+        for i in range(1, nodes):
+            dep.append(dep[par[i]] + 1)
+        assert eng.tree.depth.cpu().numpy().tolist() == dep and max(dep) <= depth
+        eng.verify()
+        eng.accept_compact()
+    torch.cuda.synchronize()
+    eng.draft_tree()                        # (a status word set above would be reported here)
+    eng.close()
