@@ -8,14 +8,17 @@
 // decode; 64 otherwise) and walks its keys in tiles of 64, copied by cp.async
 // into a two-stage ring: scores S = Q K^T as register tiles (packed fp32 FMAs
 // over even and odd elements), an online softmax over the tile in shared
-// memory, O += P V in registers. When the (row tile, head) CTAs leave SMs idle
-// the keys are cut into splits of whole tiles, one cluster per (row tile,
-// head), combined through distributed shared memory in split order; the last
-// split takes the tree keys. Rows are padded to HD + 4 floats, so the rows a
-// warp reads together sit in different banks.
+// memory, O += P V in registers. A key that a row does not see is left out of
+// that row's sums, not multiplied by zero: its K/V may hold a NaN or an infinity
+// (of another row, or of an earlier tree in a slot not written yet). When the
+// (row tile, head) CTAs leave SMs idle the keys are cut into splits of whole
+// tiles, one cluster per (row tile, head), combined through distributed shared
+// memory in split order; the last split takes the tree keys. Rows are padded to
+// HD + 4 floats, so the rows a warp reads together sit in different banks.
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -29,6 +32,7 @@ constexpr int AS_THREADS = 256;
 constexpr int AS_KT = 64;               // keys per tile
 constexpr int AS_PLD = AS_KT + 4;       // padded score row
 constexpr int AS_MAX_SPLITS = 8;
+constexpr float HIDDEN = -1.f;          // in place of the weight of a key that the row does not see
 
 struct AsArgs {
     AttnArgs<float> a;
@@ -187,15 +191,21 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                     sP[(sr + 16 * u) * AS_PLD + sk + 16 * v] = as_lo(s[u][v]) + as_hi(s[u][v]);
         }
         __syncthreads();
+        bool hidden = false;                    // a row does not see a key of the tile
         {
             const bool tree = i >= nc;
             const uint64_t bits = !tree ? ~0ull : (xmask && i - nc < a.mask_words ? xmask[i - nc] : 0ull);
             const int lim = tree ? (xr < nrows ? a.tree_slots - (i - nc) * AS_KT : 0) : xplen - (k_lo + i * AS_KT);
+            // keys of the tile that were copied (the rest of the stage is zeros)
+            const int held = xr < nrows ? (tree ? a.tree_slots - (i - nc) * AS_KT : k_hi - (k_lo + i * AS_KT)) : 0;
             float v[KPT], mx = -INFINITY;
+            unsigned seen = 0;
 #pragma unroll
             for (int j = 0; j < KPT; ++j) {
                 const int key = xk + GT * j;
                 const bool vis = key < lim && ((bits >> key) & 1ull);
+                seen |= (unsigned)vis << j;
+                hidden |= !vis && key < held;
                 v[j] = vis ? sP[xr * AS_PLD + key] * p.scale_log2 : -INFINITY;
                 mx = fmaxf(mx, v[j]);
             }
@@ -208,7 +218,7 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
             for (int j = 0; j < KPT; ++j) {
                 const float e = as_exp2(v[j] - use);
                 sum += e;
-                sP[xr * AS_PLD + xk + GT * j] = e;
+                sP[xr * AS_PLD + xk + GT * j] = (seen >> j & 1u) || xk + GT * j >= held ? e : HIDDEN;
             }
 #pragma unroll
             for (int o = GT / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -220,15 +230,9 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                 s_l[xr] = s_l[xr] * f + sum;
             }
         }
-        __syncthreads();
-        if (orow < QR) {
-#pragma unroll
-            for (int u = 0; u < OR; ++u) {
-                const float f = s_scale[orow + OG * u];
-                const unsigned long long ff = as_pack(f, f);
-                o01[u] = as_fma2(o01[u], ff, 0ull);
-                o23[u] = as_fma2(o23[u], ff, 0ull);
-            }
+        const bool skip = __syncthreads_or(hidden);
+        // O += P V, without the keys that are hidden from a row (skip: there are some)
+        auto pv = [&](auto skips) {
 #pragma unroll 4
             for (int k = 0; k < AS_KT; k += 4) {
                 ulonglong2 vv[4];
@@ -240,12 +244,24 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                     const float pk[4] = {pr.x, pr.y, pr.z, pr.w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
+                        if (decltype(skips)::value && pk[j] == HIDDEN) continue;
                         const unsigned long long pp = as_pack(pk[j], pk[j]);
                         o01[u] = as_fma2(pp, vv[j].x, o01[u]);
                         o23[u] = as_fma2(pp, vv[j].y, o23[u]);
                     }
                 }
             }
+        };
+        if (orow < QR) {
+#pragma unroll
+            for (int u = 0; u < OR; ++u) {
+                const float f = s_scale[orow + OG * u];
+                const unsigned long long ff = as_pack(f, f);
+                o01[u] = as_fma2(o01[u], ff, 0ull);
+                o23[u] = as_fma2(o23[u], ff, 0ull);
+            }
+            if (skip) pv(std::true_type());
+            else pv(std::false_type());
         }
         __syncthreads();                        // the stage and the scores may be overwritten
     }

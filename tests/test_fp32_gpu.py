@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from paper_2505_14260_gb300 import msd, synth
-from tests.gpu_support import open_engine
+from tests.gpu_support import open_engine, record_buffers
 from tests.parity_support import run_parity
 
 pytestmark = pytest.mark.gpu
@@ -76,3 +76,80 @@ def test_fp32_linear_rows_do_not_depend_on_each_other():
     eng.linear(x2, w, y2)
     assert np.array_equal(y[17].cpu().numpy(), y2[17].cpu().numpy())
     eng.close()
+
+
+# A key that a row does not see takes no part in that row's attention, whatever its K/V
+# hold: a NaN or an infinity stays with the rows that see it. (The prompts run over
+# several row and key tiles and, with few rows, over several key splits.)
+NONFINITE = [float("nan"), float("inf")]
+
+
+def _prompt(wl, bad=None, at=0):
+    p = synth.make_prompts(wl)[0]
+    if bad is not None:
+        p.vis[at] = bad
+    return msd.upload_prompts([p])
+
+
+@pytest.mark.parametrize("bad", NONFINITE)
+@pytest.mark.parametrize("hd,vis,at", [(64, 40, 30), (64, 200, 70), (128, 100, 60), (128, 700, 555)])
+def test_fp32_prefill_rows_before_a_nonfinite_one(hd, vis, at, bad):
+    wl = TINY.with_(n_heads=256 // hd, head_dim=hd, n_vis=(vis,), n_text=(30, 30), n_sys=8)
+    eng, _ = open_engine(wl, steps=1)
+    kv = []
+    for b in (None, bad):
+        eng.prefill(*_prompt(wl, b, at))
+        s = eng.state()
+        kv.append((s["target_kv"].clone(), s["draft_kv"].clone()))
+    pos = 8 + at                            # the row's position (the draft row before it holds its embedding)
+    assert torch.isnan(kv[1][0][-1, :, 0, :, pos]).all()
+    for c, n in ((0, pos), (1, pos - 1)):
+        assert torch.equal(kv[0][c][..., :n, :], kv[1][c][..., :n, :])
+    eng.close()
+
+
+@pytest.mark.parametrize("bad", NONFINITE)
+@pytest.mark.parametrize("hd,nodes,vis", [(64, 16, 64), (64, 70, 300), (128, 33, 500)])
+def test_fp32_verify_siblings_of_a_nonfinite_node(hd, nodes, vis, bad):
+    wl = TINY.with_(n_heads=256 // hd, head_dim=hd, tree_nodes=nodes, topk=8, n_vis=(vis,))
+    eng, w = open_engine(wl, steps=1)
+    prompt = _prompt(wl)
+    root = int(eng.prefill(*prompt)[0])
+    used = set(prompt[0][0].tolist()) | {root}
+    toks = [t for t in range(wl.vocab) if t not in used][:nodes]
+    bad_tok, toks[0] = toks[0], root
+    parent = [-1] + [(i - 1) // 3 for i in range(1, nodes)]
+    under = {2}                             # node 2 and what hangs below it
+    for i in range(3, nodes):
+        if parent[i] in under:
+            under.add(i)
+    eng.w["embed"][bad_tok] = bad
+    out = []
+    for t2 in (toks[2], bad_tok):
+        logits = torch.zeros(nodes, wl.vocab, device="cuda")
+        eng.plant(eng.tree, 0, toks[:2] + [t2] + toks[3:], parent)
+        eng.verify(logits=logits)
+        out.append(logits)
+    keep = [i for i in range(nodes) if i not in under]
+    assert torch.isnan(out[1][2]).all() and not torch.isnan(out[0]).any()
+    assert torch.equal(out[0][keep], out[1][keep])
+    eng.close()
+
+
+def test_fp32_draft_after_a_nonfinite_prompt():
+    """Slots of the draft tree that a pass has not written yet hold the last tree's values."""
+    wl = TINY.with_(n_sys=8, tree_nodes=40, tree_depth=5, topk=6)
+    recs = []
+    for first in (None, float("nan")):
+        eng, w = open_engine(wl, steps=1)
+        if first is not None:
+            eng.prefill(*_prompt(wl, first, 20))
+            eng.draft_tree()
+        eng.prefill(*_prompt(wl))
+        rec = record_buffers(wl)
+        eng.draft_tree(record=rec)
+        torch.cuda.synchronize()
+        recs.append((rec["logits"].cpu(), eng.tree.tokens.cpu(), eng.tree.parent.cpu()))
+        eng.close()
+    assert not torch.isnan(recs[0][0]).any()
+    assert all(torch.equal(a, b) for a, b in zip(*recs))
