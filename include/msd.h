@@ -341,6 +341,20 @@ msd_status msd_linear_noalloc(const void *x_dev, int32_t ldx, int32_t m, int32_t
  * Errors: MSD_ERR_INVALID (limit out of range), MSD_ERR_CUDA. */
 msd_status msd_test_wait_timeout(msd_ctx *ctx, int64_t limit_ns, void *stream);
 
+/* Test hook of the tensor-core GEMMs' launch rules (host only, needs no GPU): how
+ * a product of m token rows, inner dimension k and o outputs would be launched on
+ * a device of `sms` SMs. planes: 1 the caller's row-major weight (msd_linear), 2 a
+ * context's packed weight and split token rows; glu != 0: the fused gate/up product
+ * (planes 2). Errors: MSD_ERR_INVALID. */
+typedef struct {
+    int32_t ctas;         /* CTAs of the launch */
+    int32_t cluster;      /* CTAs that wait for one another */
+    int32_t smem_bytes;   /* dynamic shared memory of a CTA */
+    int32_t tmem_cols;    /* tensor-memory columns of a CTA */
+} msd_gemm_shape;
+msd_status msd_test_gemm_shape(int32_t m, int32_t k, int32_t o, int32_t planes, int32_t glu, int32_t sms,
+                               msd_gemm_shape *out);
+
 /* Profiling counters (tracing subsystem). kernel_launches counts every kernel
  * the library has run in this process (kernels executed by step graphs
  * included, kernels merely recorded into graphs excluded).

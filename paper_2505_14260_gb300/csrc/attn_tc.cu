@@ -67,6 +67,8 @@ struct Lay {
     static constexpr uint32_t T_QH = 0, T_QL = HD / 2, T_S = HD, T_O = HD + 2 * KT;
     static constexpr uint32_t T_COLS = T_O + HD <= 256 ? 256 : 512;
     static constexpr int LD = HD + 4;                     // fp32 partial row stride (floats)
+    static constexpr uint32_t SMEM = 1024 + STAGES * STAGE;
+    static_assert(SMEM >= tmem_smem_floor((int)T_COLS), "CTAs that share an SM fit its tensor memory");
 };
 
 struct AttnTcParams {
@@ -927,12 +929,10 @@ bool launch_attention_tc(AttnTcPlan *p, const AttnArgs<bf16> &a, int B, int rows
         }
         tp.n_order = n_blocks;
     }
-    const size_t smem = 1024 + (a.hd == 128 ? (size_t)STAGES * Lay<128>::STAGE : (size_t)STAGES * Lay<64>::STAGE);
+    const size_t smem = a.hd == 128 ? Lay<128>::SMEM : Lay<64>::SMEM;
     if (!p->attr_set) {
-        cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(1024 + STAGES * Lay<128>::STAGE));
-        cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(1024 + STAGES * Lay<64>::STAGE));
+        cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<128>::SMEM);
+        cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<64>::SMEM);
         cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         p->attr_set = true;

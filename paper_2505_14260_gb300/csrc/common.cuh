@@ -87,6 +87,15 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
 }
 
+// The dynamic shared memory that a CTA holding `cols` tensor-memory columns asks for
+// at least. A CTA of a cluster keeps its columns while it waits for its peers, and an
+// allocation waits, without a limit, for columns that the SM's other CTAs hold: two
+// such launches (other streams, other contexts) that each hold one SM and wait for
+// the other's would never end. So CTAs that share an SM have to fit its 512 columns
+// together. With 78 KB or more apiece at most two share one (228 KB), and a CTA of
+// more than 256 columns leaves no room for a second.
+constexpr uint32_t tmem_smem_floor(int cols) { return cols > 256 ? 193u * 1024u : 78u * 1024u; }
+
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<bf16>(bf16 v) { return __bfloat162float(v); }

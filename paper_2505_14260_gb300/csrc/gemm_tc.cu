@@ -1994,39 +1994,29 @@ void gemm_pack_glu(const void *gate, const void *up, int F, int K, void *dst, cu
     note_launch();
 }
 
-// Launch of the cluster split-K kernel: s K-splits per tile (a cluster), chosen
-// so that tiles * s fills the CTAs the SMs hold at once, s <= 8 and >= 2
+constexpr size_t HALF_SM = 104u * 1024u, FULL_SM = 200u * 1024u;     // ring bytes of two CTAs / one CTA per SM
+
+// How the cluster split-K kernel runs: S K-splits per tile (a cluster), chosen
+// so that tiles * S fills the CTAs the SMs hold at once, S <= 8 and >= 2
 // K-blocks each. Two CTAs share an SM when three stages fit in half of its
 // shared memory (token tiles of up to 64 split rows), otherwise one with up to
 // four stages; the split count keeps every split's partial slices within the
 // stage memory they reuse.
-static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
-                         int tiles, int BN, int kblocks, float *Y, int ldy, int epi, int *status,
-                         cudaStream_t s, int O, const GemmFused *fx = nullptr,
-                         const GemmNorm *nout = nullptr, const GemmNorm *nin = nullptr) {
-    CkParams ck;
-    memset(&ck, 0, sizeof ck);
-    if (fx) ck.fx = *fx;
-    if (nout) ck.nout = *nout;
-    if (nin) ck.nin = *nin;
-    ck.n_seg = W.nseg;
-    int out_off = 0;
-    for (int i = 0; i < W.nseg; ++i) {
-        ck.seg_rows[i] = W.rows[i];
-        ck.seg_tiles[i] = (W.rows[i] + BM - 1) / BM;
-        ck.seg_out[i] = out_off;
-        out_off += W.rows[i];
-    }
-    const int nb = X_lo ? 2 : 1;
+struct ClusterShape {
+    int S, stages, n_acc, acc_stride, tmem_cols;
+    bool pair;
+    size_t smem;
+};
+
+static ClusterShape cluster_shape(int tiles, int BN, int kblocks, int nb, bool packed, int num_sms) {
     size_t stage = A_BYTES + (size_t)nb * BN * BK * 2;
-    constexpr size_t HALF_SM = 104u * 1024u, FULL_SM = 200u * 1024u;
     int per_sm = 3 * stage <= HALF_SM ? 2 : 1;
     // one-plane products over more than 64 rows that leave half of the CTAs unused: one
     // per SM, whose stage memory holds the partials of up to eight splits
-    if (nb == 1 && BN > 64 && 2 * tiles <= p->num_sms) per_sm = 1;
+    if (nb == 1 && BN > 64 && 2 * tiles <= num_sms) per_sm = 1;
     int stages = (int)((per_sm == 2 ? HALF_SM : FULL_SM) / stage);
     stages = std::max(2, std::min(stages, C_STAGES));
-    int S = (per_sm * p->num_sms) / tiles;
+    int S = (per_sm * num_sms) / tiles;
     S = std::max(1, std::min(S, 8));
     // Clusters stay within a GPC, so fewer CTAs run at once the larger they are, and
     // a launch past that runs a second wave. Two CTAs per SM on 152 SMs: 32 clusters
@@ -2035,7 +2025,7 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     // in sixes, 14.8 in fives).
     auto one_wave = [&](int c) {
         const int slots = c >= 6 ? 256 : (c >= 4 ? 280 : (c == 3 ? 288 : 304));
-        return (long)tiles * c * 304 <= (long)slots * per_sm * p->num_sms;
+        return (long)tiles * c * 304 <= (long)slots * per_sm * num_sms;
     };
     while (S > 1 && !one_wave(S)) --S;
     // The accumulators truncate: the K-blocks take turns over two of them, in one-plane
@@ -2059,12 +2049,37 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     // Two-SM tiles for unsplit launches whose token stage is as large as the
     // weight block (split token rows, 32 or more): each CTA of a pair holds
     // half the token columns, so the ring gets a fourth stage.
-    const bool pair = S == 1 && nb == 2 && BN >= 32 && tiles % 2 == 0 && per_sm == 2 && W.packed;
-    const int BNs = pair ? BN / 2 : BN;
+    const bool pair = S == 1 && nb == 2 && BN >= 32 && tiles % 2 == 0 && per_sm == 2 && packed;
     if (pair) {
-        stage = A_BYTES + (size_t)nb * BNs * BK * 2;
+        stage = A_BYTES + (size_t)nb * (BN / 2) * BK * 2;
         stages = std::max(2, std::min((int)(HALF_SM / stage), C_STAGES));
     }
+    const int tmem_cols = n_acc * acc_stride;
+    const size_t smem = std::max<size_t>(1024 + (size_t)stages * stage, tmem_smem_floor(tmem_cols));
+    return ClusterShape{S, stages, n_acc, acc_stride, tmem_cols, pair, smem};
+}
+
+static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
+                         int tiles, int BN, int kblocks, float *Y, int ldy, int epi, int *status,
+                         cudaStream_t s, int O, const GemmFused *fx = nullptr,
+                         const GemmNorm *nout = nullptr, const GemmNorm *nin = nullptr) {
+    CkParams ck;
+    memset(&ck, 0, sizeof ck);
+    if (fx) ck.fx = *fx;
+    if (nout) ck.nout = *nout;
+    if (nin) ck.nin = *nin;
+    ck.n_seg = W.nseg;
+    int out_off = 0;
+    for (int i = 0; i < W.nseg; ++i) {
+        ck.seg_rows[i] = W.rows[i];
+        ck.seg_tiles[i] = (W.rows[i] + BM - 1) / BM;
+        ck.seg_out[i] = out_off;
+        out_off += W.rows[i];
+    }
+    const int nb = X_lo ? 2 : 1;
+    const ClusterShape g = cluster_shape(tiles, BN, kblocks, nb, W.packed != nullptr, p->num_sms);
+    const int S = g.S, stages = g.stages, BNs = g.pair ? BN / 2 : BN;
+    const bool pair = g.pair;
     ck.M = M;
     ck.kblocks = kblocks;
     ck.BN = BN;
@@ -2072,9 +2087,9 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     ck.splits = S;
     ck.stages = stages;
     ck.has_lo = X_lo ? 1 : 0;
-    ck.n_acc = n_acc;
-    ck.acc_stride = acc_stride;
-    ck.tmem_cols = n_acc * acc_stride;
+    ck.n_acc = g.n_acc;
+    ck.acc_stride = g.acc_stride;
+    ck.tmem_cols = g.tmem_cols;
     ck.wpacked = static_cast<const bf16 *>(W.packed);
     ck.Y = Y;
     ck.ldy = ldy;
@@ -2094,7 +2109,6 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         flag_kernel<<<1, 1, 0, s>>>(status, ST_RANGE);
         return false;
     }
-    const size_t smem = 1024 + (size_t)stages * stage;
     if (!p->cluster_attr_set) {
         auto set = [](const void *f) {
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(1024 + FULL_SM));
@@ -2117,7 +2131,7 @@ static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     memset(&lc, 0, sizeof lc);
     lc.gridDim = dim3((unsigned)tiles, 1, (unsigned)S);
     lc.blockDim = dim3(C_THREADS);
-    lc.dynamicSmemBytes = smem;
+    lc.dynamicSmemBytes = g.smem;
     lc.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2209,6 +2223,9 @@ bool gemm_bf16(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int
 // kb_chunk K-blocks.
 struct PersistShape {
     int BN, nt, G, T_all, T_sk, dp_rounds, kb_chunk, n_acc, n_rot;
+    int stages, acc_stride, tmem_cols;
+    uint32_t stage_bytes, stg_off;      // a ring stage; where the SwiGLU staging tile starts
+    size_t smem;
 };
 constexpr uint32_t P_BUDGET = 220u * 1024u;     // ring and staging bytes of a CTA
 constexpr int P_STAGES = 6;
@@ -2278,6 +2295,16 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
             best = g;
         }
     }
+    // the fused SwiGLU epilogue takes 16 KB of staging from the ring's budget
+    const uint32_t stg_bytes = glu ? 32u * BM * 4u : 0u;
+    best.stage_bytes = A_BYTES + (uint32_t)nb * (best.BN / 2) * BK * 2;
+    best.stages = std::max(2, std::min((int)((P_BUDGET - stg_bytes) / best.stage_bytes), P_STAGES));
+    best.stg_off = (uint32_t)(1024 + (size_t)best.stages * best.stage_bytes);
+    best.acc_stride = 32;
+    while (best.acc_stride < best.BN) best.acc_stride <<= 1;
+    best.tmem_cols = 64;
+    while (best.tmem_cols < best.n_acc * best.n_rot * best.acc_stride) best.tmem_cols <<= 1;
+    best.smem = std::max<size_t>(best.stg_off + stg_bytes, tmem_smem_floor(best.tmem_cols));
     return best;
 }
 
@@ -2298,25 +2325,18 @@ static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     const int nb = X_lo ? 2 : 1;
     const PersistShape g = persist_shape(tiles, M, K, nb, glu, p->num_sms / 2, p->ws_bytes, p->n_counters);
     const int BN = g.BN, nt = g.nt, kblocks = (K + BK - 1) / BK, G = g.G;
-    // the fused SwiGLU epilogue takes 16 KB of staging from the ring's budget
-    const uint32_t stg_bytes = glu ? 32u * BM * 4u : 0u;
-    const uint32_t stage_bytes = A_BYTES + (uint32_t)nb * (BN / 2) * BK * 2;
-    const int stages = std::max(2, std::min((int)((P_BUDGET - stg_bytes) / stage_bytes), P_STAGES));
-    const size_t smem = 1024 + (size_t)stages * stage_bytes + stg_bytes;
+    const int stages = g.stages;
     const long long units = (long long)g.T_sk * kblocks;
     const long long all_units = (long long)g.T_all * kblocks;
-    int acc = 32;
-    while (acc < BN) acc <<= 1;
     pk.M = M;
     pk.kblocks = kblocks;
     pk.BN = BN;
     pk.n_tiles_n = nt;
     pk.stages = stages;
-    pk.acc_stride = acc;
+    pk.acc_stride = g.acc_stride;
     pk.n_acc = g.n_acc;
     pk.n_rot = g.n_rot;
-    pk.tmem_cols = 64;
-    while (pk.tmem_cols < pk.n_acc * pk.n_rot * acc) pk.tmem_cols <<= 1;
+    pk.tmem_cols = g.tmem_cols;
     pk.grid = G;
     pk.tiles = tiles;
     pk.units = units;
@@ -2336,7 +2356,7 @@ static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
         pk.act = fx->act;
         pk.F = fx->F;
         pk.lo = fx->lo;
-        pk.stg_off = (uint32_t)(1024 + (size_t)stages * stage_bytes);
+        pk.stg_off = g.stg_off;
     }
     const bool raw = !W.packed;
     CUtensorMap rawx, raww;
@@ -2376,7 +2396,7 @@ static bool gemm_persist(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, 
     memset(&lc, 0, sizeof lc);
     lc.gridDim = dim3((unsigned)(2 * G));
     lc.blockDim = dim3(P_THREADS);
-    lc.dynamicSmemBytes = smem;
+    lc.dynamicSmemBytes = g.smem;
     lc.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2571,4 +2591,20 @@ extern "C" msd_status msd_linear_noalloc(const void *x, int32_t ldx, int32_t m, 
                                             (k + BK - 1) / BK, y, ldy, epi, d.status, s, o)
                              : gemm_persist(d.plan, X, nullptr, ldx, m, k, W, o, y, ldy, epi, nullptr, d.status, s);
     return ok && cudaGetLastError() == cudaSuccess ? OK : CUDA_ERR;
+}
+
+extern "C" msd_status msd_test_gemm_shape(int32_t m, int32_t k, int32_t o, int32_t planes, int32_t glu, int32_t sms,
+                                          msd_gemm_shape *out) {
+    using namespace msd;
+    if (m <= 0 || k <= 0 || o <= 0 || (planes != 1 && planes != 2) || (glu && planes == 1) || sms < 2 || !out)
+        return MSD_ERR_INVALID;
+    const int kblocks = (k + BK - 1) / BK, tiles = (o + BM - 1) / BM;
+    if (m <= 128) {
+        const ClusterShape g = cluster_shape(tiles, (m + 15) / 16 * 16, kblocks, planes, planes == 2, sms);
+        *out = msd_gemm_shape{tiles * g.S, g.pair ? 2 : g.S, (int32_t)g.smem, g.tmem_cols};
+    } else {
+        const PersistShape g = persist_shape(tiles, m, k, planes, glu != 0, sms / 2, WS_BYTES, N_COUNTERS);
+        *out = msd_gemm_shape{2 * g.G, 2, (int32_t)g.smem, g.tmem_cols};
+    }
+    return MSD_OK;
 }

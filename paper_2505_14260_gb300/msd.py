@@ -71,6 +71,10 @@ class msd_kernel_slot(ctypes.Structure):
                 ("span_ms", ctypes.c_double)]
 
 
+class msd_gemm_shape(ctypes.Structure):
+    _fields_ = [("ctas", c_int32), ("cluster", c_int32), ("smem_bytes", c_int32), ("tmem_cols", c_int32)]
+
+
 _SIGNATURES = {
     "msd_create": (c_int32, [POINTER(msd_config), POINTER(msd_weights), POINTER(c_void_p)]),
     "msd_destroy": (c_int32, [c_void_p]),
@@ -93,6 +97,7 @@ _SIGNATURES = {
                                      c_void_p, c_int32, c_int32, c_void_p]),
     "msd_tree_complete": (c_int32, [c_void_p, POINTER(msd_tree), c_int32, c_void_p]),
     "msd_test_wait_timeout": (c_int32, [c_void_p, c_int64, c_void_p]),
+    "msd_test_gemm_shape": (c_int32, [c_int32] * 6 + [POINTER(msd_gemm_shape)]),
     "msd_profile_enable": (c_int32, [c_void_p, c_int32]),
     "msd_profile_read": (c_int32, [c_void_p, POINTER(msd_profile)]),
     "msd_profile_slots": (c_int32, [c_void_p, POINTER(msd_kernel_slot), c_int32, POINTER(c_int32)]),
