@@ -351,6 +351,9 @@ typedef struct {
     int32_t cluster;      /* CTAs that wait for one another */
     int32_t smem_bytes;   /* dynamic shared memory of a CTA */
     int32_t tmem_cols;    /* tensor-memory columns of a CTA */
+    int32_t chain;        /* K-blocks (of 64) that one accumulator adds up, at most */
+    int32_t chunks;       /* chunks of K of a whole tile (0: no tile is whole) */
+    int32_t cut_tiles;    /* tiles whose K is cut between CTA pairs */
 } msd_gemm_shape;
 msd_status msd_test_gemm_shape(int32_t m, int32_t k, int32_t o, int32_t planes, int32_t glu, int32_t sms,
                                msd_gemm_shape *out);

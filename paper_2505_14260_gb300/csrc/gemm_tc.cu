@@ -2003,7 +2003,7 @@ constexpr size_t HALF_SM = 104u * 1024u, FULL_SM = 200u * 1024u;     // ring byt
 // four stages; the split count keeps every split's partial slices within the
 // stage memory they reuse.
 struct ClusterShape {
-    int S, stages, n_acc, acc_stride, tmem_cols;
+    int S, stages, n_acc, acc_stride, tmem_cols, chain;     // chain: K-blocks that one accumulator takes, at most
     bool pair;
     size_t smem;
 };
@@ -2031,7 +2031,9 @@ static ClusterShape cluster_shape(int tiles, int BN, int kblocks, int nb, bool p
     // The accumulators truncate: the K-blocks take turns over two of them, in one-plane
     // products (msd_linear) over as many as the CTA's TMEM columns hold, and there K is
     // split further where that leaves chains past 16 blocks (17 x 4096 x 11008: 1.1e-6
-    // relative in chains of 22, below 0.8e-6 in chains of 3)
+    // relative in chains of 22, below 0.8e-6 in chains of 3), as far as the partial slices
+    // have room: past 64 rows with a CTA on every half SM that is two splits of two
+    // accumulators (128 x 11008 x 20000: chains of 43, 2.9e-6)
     int acc_stride = 32;
     while (acc_stride < BN) acc_stride <<= 1;
     const int all_acc = 512 / per_sm / acc_stride;
@@ -2056,7 +2058,8 @@ static ClusterShape cluster_shape(int tiles, int BN, int kblocks, int nb, bool p
     }
     const int tmem_cols = n_acc * acc_stride;
     const size_t smem = std::max<size_t>(1024 + (size_t)stages * stage, tmem_smem_floor(tmem_cols));
-    return ClusterShape{S, stages, n_acc, acc_stride, tmem_cols, pair, smem};
+    const int chain = ((kblocks + S - 1) / S + n_acc - 1) / n_acc;
+    return ClusterShape{S, stages, n_acc, acc_stride, tmem_cols, chain, pair, smem};
 }
 
 static bool gemm_cluster(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int K, const GemmW &W,
@@ -2224,11 +2227,13 @@ bool gemm_bf16(GemmPlan *p, const bf16 *X, const bf16 *X_lo, int ldx, int M, int
 struct PersistShape {
     int BN, nt, G, T_all, T_sk, dp_rounds, kb_chunk, n_acc, n_rot;
     int stages, acc_stride, tmem_cols;
+    int chain;                          // K-blocks that one accumulator takes, at most
     uint32_t stage_bytes, stg_off;      // a ring stage; where the SwiGLU staging tile starts
     size_t smem;
 };
 constexpr uint32_t P_BUDGET = 220u * 1024u;     // ring and staging bytes of a CTA
 constexpr int P_STAGES = 6;
+constexpr int P_CHAIN = 32, P_CHUNK_CHAIN = 24;
 
 // Clocks, measured at 333 to 1024 rows and K = 4096, 11008. A K-block of a 256 x
 // BN tile takes 2.08 nb BN (4% above the MMAs' own time: 0.35 us at 160 columns
@@ -2246,8 +2251,12 @@ constexpr int P_STAGES = 6;
 // (msd_linear), which have no other error, are also cut into narrower tiles while
 // one round holds them: a K-block of 32 columns takes no longer than one of 96, and
 // 16 accumulators fit (1245 x 3664 x 129: 27.3 us and 9.0e-7 with tiles of 64 columns
-// or more, 23.2 us and 1.3e-7; 1000 x 512 x 1024: 15.0 to 12.9 us). Past 24
-// blocks in every accumulator, chunks of K are added to Y one after another.
+// or more, 23.2 us and 1.3e-7; 1000 x 512 x 1024: 15.0 to 12.9 us). Where a pair has
+// several whole tiles, chunks of K are added to Y one after another, with at most 24
+// blocks in every accumulator; a lone tile takes up to 32. Tiles whose pieces would put
+// more than 32 into one stay whole (500 x 11008 x 14336 in pieces of 82 blocks: 3.0e-6
+// and 158 us, 1.4e-6 and 186 us whole; 576 x 11008 x 9728, 86: 3.7e-6 and 113 us,
+// 1.4e-6 and 126 us; the pieces in chunks added to the workspace: 209 and 144 us).
 static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int pairs, size_t ws_bytes,
                                   int n_counters) {
     const int kblocks = (K + BK - 1) / BK, wt = (tiles + 1) / 2;
@@ -2264,11 +2273,12 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
         while (stride < BN) stride <<= 1;
         const int most = nb == 1 ? 16 : 4;
         const bool chunked = nb == 1 && !glu;
-        const bool lone = T <= G && (!chunked || (kblocks + 31) / 32 <= 512 / stride);    // one item a pair
+        const bool lone = T <= G && (!chunked || (kblocks + P_CHAIN - 1) / P_CHAIN <= 512 / stride);    // one item a pair
         const int n_acc = lone ? 1 : 2, n_rot = std::min(512 / n_acc / stride, most);
-        const int n_ch = chunked && !lone ? (kblocks + 24 * n_rot - 1) / (24 * n_rot) : 1;
+        const int n_ch = chunked && !lone ? (kblocks + P_CHUNK_CHAIN * n_rot - 1) / (P_CHUNK_CHAIN * n_rot) : 1;
         const int chunk = (kblocks + n_ch - 1) / n_ch;
         PersistShape g{BN, nt, (int)G, (int)T, 0, (int)((T + G - 1) / G), chunk, n_acc, n_rot};
+        g.chain = (chunk + n_rot - 1) / n_rot;
         double cost = g.dp_rounds * tk * kblocks;
         int rounds = (int)(T / G), T_sk = (int)(T - rounds * G);
         if (T_sk > 0) {
@@ -2280,13 +2290,17 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
                 T_sk += (int)G;
             }
             const double sk = T * tk * kblocks / G + (rounds == 0 ? 330.0 : 180.0) * BN;
+            const int sk_acc = chunked && rounds == 0 ? 1 : 2, sk_rot = std::min(512 / sk_acc / stride, most);
+            const long long piece = std::min<long long>(kblocks, (T_sk * (long long)kblocks + G - 1) / G);
+            const int sk_chain = (int)((piece + sk_rot - 1) / sk_rot);
             // (every pair holds a unit, and the pieces and tickets have their place)
             if (sk < cost && (long long)T_sk * kblocks >= G && 16ull * G * BN * BM <= ws_bytes &&
-                2LL * T_sk <= n_counters) {
+                2LL * T_sk <= n_counters && (!chunked || sk_chain <= P_CHAIN)) {
                 g.T_sk = T_sk;
                 g.dp_rounds = rounds;
-                g.n_acc = chunked && rounds == 0 ? 1 : 2;
-                g.n_rot = std::min(512 / g.n_acc / stride, most);
+                g.n_acc = sk_acc;
+                g.n_rot = sk_rot;
+                g.chain = std::max(sk_chain, rounds > 0 ? (chunk + sk_rot - 1) / sk_rot : 0);
                 cost = sk;
             }
         }
@@ -2601,10 +2615,11 @@ extern "C" msd_status msd_test_gemm_shape(int32_t m, int32_t k, int32_t o, int32
     const int kblocks = (k + BK - 1) / BK, tiles = (o + BM - 1) / BM;
     if (m <= 128) {
         const ClusterShape g = cluster_shape(tiles, (m + 15) / 16 * 16, kblocks, planes, planes == 2, sms);
-        *out = msd_gemm_shape{tiles * g.S, g.pair ? 2 : g.S, (int32_t)g.smem, g.tmem_cols};
+        *out = msd_gemm_shape{tiles * g.S, g.pair ? 2 : g.S, (int32_t)g.smem, g.tmem_cols, g.chain, 1, 0};
     } else {
         const PersistShape g = persist_shape(tiles, m, k, planes, glu != 0, sms / 2, WS_BYTES, N_COUNTERS);
-        *out = msd_gemm_shape{2 * g.G, 2, (int32_t)g.smem, g.tmem_cols};
+        const int chunks = (kblocks + g.kb_chunk - 1) / g.kb_chunk;
+        *out = msd_gemm_shape{2 * g.G, 2, (int32_t)g.smem, g.tmem_cols, g.chain, g.dp_rounds > 0 ? chunks : 0, g.T_sk};
     }
     return MSD_OK;
 }

@@ -72,7 +72,8 @@ class msd_kernel_slot(ctypes.Structure):
 
 
 class msd_gemm_shape(ctypes.Structure):
-    _fields_ = [("ctas", c_int32), ("cluster", c_int32), ("smem_bytes", c_int32), ("tmem_cols", c_int32)]
+    _fields_ = [("ctas", c_int32), ("cluster", c_int32), ("smem_bytes", c_int32), ("tmem_cols", c_int32),
+                ("chain", c_int32), ("chunks", c_int32), ("cut_tiles", c_int32)]
 
 
 _SIGNATURES = {

@@ -56,6 +56,47 @@ def test_linear_matches_float64(m, k, o):
     eng.close()
 
 
+# (m, k, o, chunks of a whole tile, cut tiles): whole tiles in chunks, cut tiles beside
+# them, cut tiles alone, and products whose pieces would be too long; cluster shapes of
+# 65 to 128 rows whose CTAs hold 512 columns, and the longest chain of the rule
+CHAINS = [(131, 1560, 20225, 2, 0), (700, 4096, 11000, 3, 0), (264, 4208, 9927, 3, 2), (275, 3352, 19573, 3, 0),
+          (500, 11008, 14336, 8, 0), (1953, 15728, 259, 0, 36), (72, 11008, 9472, 1, 0), (65, 8192, 1001, 1, 0),
+          (80, 11008, 500, 1, 0), (128, 11008, 20000, 1, 0)]
+
+
+@pytest.mark.parametrize("accumulate", [False, True])
+@pytest.mark.parametrize("m,k,o,chunks,cut", CHAINS)
+def test_linear_error_follows_the_chains(m, k, o, chunks, cut, accumulate):
+    """The accumulators truncate: a step of 16 terms loses half a unit in the last place on
+    average, at most 2^-24 of the partial sum, which grows like the square root of the
+    terms (2/3 of the result on average). Four steps a K-block over the launch's longest
+    chain bound every output column's error; the sums of accumulators, pieces and chunks
+    and the residual round once each (2^-24, some ten of them)."""
+    shape = msd.msd_gemm_shape()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert msd.lib().msd_test_gemm_shape(m, k, o, 1, 0, sms, ctypes.byref(shape)) == msd.MSD_OK
+    if sms == 152:
+        assert (shape.chunks, shape.cut_tiles) == (chunks, cut)
+    eng, _ = open_engine(synth.WORKLOADS["tiny"].with_(dtype="bf16"), steps=1)
+    g = torch.Generator(device="cuda").manual_seed(m + k + o)
+    x = torch.randn(m, k, generator=g, device="cuda").bfloat16()
+    w = torch.randn(o, k, generator=g, device="cuda").bfloat16()
+    y = torch.randn(m, o, generator=g, device="cuda") if accumulate else torch.full((m, o), float("nan"), device="cuda")
+    yn = y.clone()
+    ref = x.double() @ w.double().T
+    if accumulate:
+        ref += y
+    eng.linear(x, w, y, accumulate=accumulate)
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert msd.lib().msd_linear_noalloc(x.data_ptr(), k, m, k, w.data_ptr(), o, yn.data_ptr(), o, int(accumulate),
+                                        stream) == msd.MSD_OK
+    bound = 4 * shape.chain * 2.0 ** -24 * 2 / 3 + 10 * 2.0 ** -24
+    for out in (y, yn):         # (the scratch of the second call may cut fewer tiles: no longer chains)
+        err = (out.double() - ref).norm(dim=0) / ref.norm(dim=0)
+        assert float(err.max()) <= bound, (float(err.max()), bound)
+    eng.close()
+
+
 def test_linear_reads_a_weight_written_just_before():
     """The weight and the rows come from kernels launched right before the call."""
     eng, _ = open_engine(synth.WORKLOADS["tiny"].with_(dtype="bf16"), steps=1)

@@ -1,5 +1,5 @@
 """The launch rules of the tensor-core GEMMs, on the host: no two launches can hold
-tensor memory that each other's CTAs wait for."""
+tensor memory that each other's CTAs wait for, and the accumulators' chains stay short."""
 import ctypes
 import itertools
 import random
@@ -50,6 +50,16 @@ def test_ctas_that_share_an_sm_fit_its_tensor_memory(shape):
         for cols in itertools.combinations_with_replacement(sorted(least), n):
             if sum(least[c] + RESERVED for c in cols) <= SM_SMEM:
                 assert sum(cols) <= TMEM_COLS, (cols, least)
+
+
+def test_accumulator_chains_are_short(shape):
+    """One-plane products (msd_linear): no accumulator of the many-row kernel adds up more
+    than 32 K-blocks, none of the few-row kernel more than 16, or past 64 rows a quarter
+    of K (two accumulators, two K splits: the room that the partial slices have)."""
+    for m, k, o in _shapes():
+        g = shape(m, k, o, 1)
+        quarter = -(-(-(-k // 64)) // 4)
+        assert g.chain <= (16 if m <= 64 else max(16, quarter) if m <= 128 else 32), (m, k, o, g.chain)
 
 
 def test_shape_hook_refuses_bad_arguments():
