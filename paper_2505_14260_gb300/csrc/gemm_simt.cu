@@ -18,6 +18,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <iterator>
 
 #include "kernels.h"
 
@@ -294,7 +295,9 @@ void launch_gemm_simt(const float *X, int ldx, int M, int K, const GemmW &W, int
     double best_ns = 0;
     for (const TileRow &t : TILES) {
         if (t.BM < 24 && M > 4 * t.BM) continue;
-        const long tiles = (long)((O + t.BO - 1) / t.BO) * ((M + t.BM - 1) / t.BM);
+        const long row_tiles = (M + t.BM - 1) / t.BM, tiles = (O + t.BO - 1) / t.BO * row_tiles;
+        // (the grid's y; rows past the last, largest tile's 65535 are refused by the launch)
+        if (row_tiles > 65535 && &t != &TILES[std::size(TILES) - 1]) continue;
         for (int sp = 1; sp <= 8 && (sp == 1 || sp <= nb / 2); sp *= 2) {
             const long rounds = (tiles * sp + num_sms - 1) / num_sms;
             double ns = rounds * (t.block_ns * ((nb + sp - 1) / sp) + t.tile_ns);

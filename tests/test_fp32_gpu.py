@@ -46,6 +46,20 @@ def test_fp32_linear_matches_float64(m, k, o, pad, off, accumulate):
     eng.close()
 
 
+# more rows than the grid's 65535 row tiles of 24, and the most that 65535 of 64 hold
+@pytest.mark.parametrize("m,o", [(65535 * 24 + 1, 8), (65535 * 64, 3), (65535 * 32 + 5, 80)])
+def test_fp32_linear_takes_many_rows(m, o):
+    eng, _ = open_engine(TINY, steps=1)
+    g = torch.Generator(device="cuda").manual_seed(o)
+    x = torch.randn(m, 4, generator=g, device="cuda")
+    w = torch.randn(o, 4, generator=g, device="cuda")
+    y = torch.full((m, o), float("nan"), device="cuda")
+    eng.linear(x, w, y)
+    ref = x.double() @ w.double().T
+    assert bool(((y.double() - ref).abs() <= 5 * 2.0 ** -24 * (x.double().abs() @ w.double().abs().T) + 1e-30).all())
+    eng.close()
+
+
 # N over the 16-row tiles (one, two, a remainder) and the 64-row ones, prefixes
 # below a key tile, at its edge, past it, and over every split; hd 64 and 128
 @pytest.mark.parametrize("hd,nodes,vis,text", [(64, 7, 0, 9), (64, 33, 100, 28), (64, 70, 600, 41),
