@@ -367,9 +367,11 @@ bool launch_attention(const AttnArgs<float> &a, int rows_per_req, int num_sms, c
     p.rows_per_req = rows_per_req;
     p.tiles_per_req = p.nsplit = 1;
     p.scale_log2 = a.scale * 1.4426950408889634f;
-    if ((a.tiles ? (long)a.n_tiles : (long)a.R / 16 + a.R / rows_per_req) > 65535) return false;   // the grid's row tiles
+    const int qr = !a.tiles && rows_per_req <= 32 ? 16 : 64;
+    const long row_tiles = a.tiles ? a.n_tiles : (long)(a.R / rows_per_req) * ((rows_per_req + qr - 1) / qr);
+    if (row_tiles > 65535) return false;        // the grid's y
     cudaError_t e;
-    if (!a.tiles && rows_per_req <= 32)
+    if (qr == 16)
         e = a.hd == 128 ? launch_as<128, 16>(p, num_sms, s) : launch_as<64, 16>(p, num_sms, s);
     else
         e = a.hd == 128 ? launch_as<128, 64>(p, num_sms, s) : launch_as<64, 64>(p, num_sms, s);

@@ -167,3 +167,21 @@ def test_fp32_draft_after_a_nonfinite_prompt():
         eng.close()
     assert not torch.isnan(recs[0][0]).any()
     assert all(torch.equal(a, b) for a, b in zip(*recs))
+
+
+def test_fp32_one_row_of_very_many_requests():
+    """Plain decoding of more requests than 15/16 of the grid's 65535 row tiles."""
+    wl = TINY.with_(n_layers=1, hidden=64, n_heads=1, ffn=64, vocab=64, tree_nodes=1, tree_depth=1, topk=1,
+                    n_vis=(0,), n_text=(2, 2), steps=2)
+    g = torch.Generator().manual_seed(1)
+    ids = torch.randint(0, 64, (62000, 2), generator=g, dtype=torch.int32).cuda()
+    out = []
+    for b in (62000, 5):
+        eng, _ = open_engine(wl, steps=2, batch=b)
+        eng.prefill(ids[:b].contiguous(), [2] * b, None, [0] * b)
+        out.append([eng.ar_step().clone() for _ in range(2)])
+        torch.cuda.synchronize()
+        eng.ar_step()
+        eng.close()
+    for many, few in zip(*out):
+        assert torch.equal(many[:5], few)
