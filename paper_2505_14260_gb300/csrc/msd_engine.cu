@@ -272,9 +272,13 @@ void gate_up_swiglu(msd_ctx *c, const msd_layer &lw, const msd_ctx::LayerPack &l
         fx.act = static_cast<bf16 *>(c->act);
         fx.F = F;
         fx.lo = c->lo;
-        // (ffn is a multiple of 16 and the weights are packed: the fused GEMM takes every shape)
-        gemm_bf16_fused(c->gplan, static_cast<const bf16 *>(c->xn), lo_of(c, c->xn), H, R, H, wgu, O, fx, c->status, s,
-                        norm_in);
+        // (ffn is a multiple of 16, the weights are packed and a norm is folded for at most
+        // 128 rows only: the fused GEMM takes every shape)
+        if (!gemm_bf16_fused(c->gplan, static_cast<const bf16 *>(c->xn), lo_of(c, c->xn), H, R, H, wgu, O, fx,
+                             c->status, s, norm_in)) {
+            c->err = "gate/up GEMM: unsupported shape";
+            launch_flag(c->status, ST_RANGE, s);     // reported by the next call
+        }
     } else {
         GemmW wgu = {{lw.w_gate, lw.w_up, nullptr}, {F, F, 0}, 2, nullptr};
         gemm<T>(c, static_cast<const T *>(c->xn), H, R, H, wgu, 2 * F, c->gu, 2 * F, EPI_STORE, s);
