@@ -96,14 +96,6 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 // more than 256 columns leaves no room for a second.
 constexpr uint32_t tmem_smem_floor(int cols) { return cols > 256 ? 193u * 1024u : 78u * 1024u; }
 
-template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f<bf16>(bf16 v) { return __bfloat162float(v); }
-
-template <typename T> __device__ __forceinline__ T from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ bf16 from_f<bf16>(float v) { return __float2bfloat16_rn(v); }
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -145,12 +137,10 @@ __device__ __forceinline__ float block_max(float v, float *red) {
     return red[0];
 }
 
-// Total order used for every top-k / argmax decision: larger value first,
-// then lower index.
+// Four consecutive values as fp32, in one 16- or 8-byte access.
 template <typename T> struct Vec4;
 template <> struct Vec4<float> {
     static __device__ __forceinline__ float4 load(const float *g) { return *reinterpret_cast<const float4 *>(g); }
-    static __device__ __forceinline__ void store(float *o, float4 v) { *reinterpret_cast<float4 *>(o) = v; }
 };
 template <> struct Vec4<bf16> {
     static __device__ __forceinline__ float4 load(const bf16 *g) {
@@ -158,13 +148,6 @@ template <> struct Vec4<bf16> {
         const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162 *>(&u.x);
         const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162 *>(&u.y);
         return make_float4(__low2float(a), __high2float(a), __low2float(b), __high2float(b));
-    }
-    static __device__ __forceinline__ void store(bf16 *o, float4 v) {
-        __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-        uint2 u;
-        u.x = *reinterpret_cast<uint32_t *>(&a);
-        u.y = *reinterpret_cast<uint32_t *>(&b);
-        *reinterpret_cast<uint2 *>(o) = u;
     }
 };
 
@@ -178,8 +161,6 @@ template <> struct Vec4<bf16> {
 // caller-owned operands). For T = float the pair is the value itself.
 template <typename T> struct Split;
 template <> struct Split<float> {
-    static __device__ __forceinline__ void store(float *o, long, float v) { *o = v; }
-    static __device__ __forceinline__ float load(const float *g, long) { return *g; }
     static __device__ __forceinline__ void store4(float *o, long, float4 v) {
         *reinterpret_cast<float4 *>(o) = v;
     }
@@ -192,9 +173,6 @@ template <> struct Split<bf16> {
         const bf16 h = __float2bfloat16_rn(v);
         *o = h;
         if (lo) o[lo] = __float2bfloat16_rn(v - __bfloat162float(h));
-    }
-    static __device__ __forceinline__ float load(const bf16 *g, long lo) {
-        return lo ? __bfloat162float(g[0]) + __bfloat162float(g[lo]) : __bfloat162float(g[0]);
     }
     static __device__ __forceinline__ void store4(bf16 *o, long lo, float4 v) {
         const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
@@ -224,50 +202,7 @@ template <> struct Split<bf16> {
 // aligned: every thread of the CTA requests up to 4 groups of 4 elements (16-
 // or 8-byte accesses) before it stores any, so one pass costs about one memory
 // round trip instead of one per element.
-template <typename TD, typename TS>
-__device__ __forceinline__ void copy_row(TD *__restrict__ dst, const TS *__restrict__ src, int n) {
-    const int n4 = n >> 2;
-    for (int g0 = threadIdx.x; g0 < n4; g0 += 4 * blockDim.x) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) v[u] = Vec4<TS>::load(src + 4 * g);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) Vec4<TD>::store(dst + 4 * g, v[u]);
-        }
-    }
-}
-
-// Two independent row copies in one pass (s1 null: d1 gets zeros).
-template <typename TD1, typename TS1, typename TD2, typename TS2>
-__device__ __forceinline__ void copy_rows2(TD1 *__restrict__ d1, const TS1 *__restrict__ s1,
-                                           TD2 *__restrict__ d2, const TS2 *__restrict__ s2, int n) {
-    const int n4 = n >> 2;
-    for (int g0 = threadIdx.x; g0 < n4; g0 += 2 * blockDim.x) {
-        float4 a[2], b[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) {
-                a[u] = s1 ? Vec4<TS1>::load(s1 + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
-                b[u] = Vec4<TS2>::load(s2 + 4 * g);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int g = g0 + u * blockDim.x;
-            if (g < n4) {
-                Vec4<TD1>::store(d1 + 4 * g, a[u]);
-                Vec4<TD2>::store(d2 + 4 * g, b[u]);
-            }
-        }
-    }
-}
-
+//
 // Row copy between split buffers (source lo plane at slo, destination at dlo;
 // 0 = none): the pair's sum is re-split, so an exact bf16 source gets lo = 0.
 template <typename TD, typename TS>
@@ -318,6 +253,8 @@ __device__ __forceinline__ void copy_rows2_split(TD *__restrict__ d1, const TS1 
     }
 }
 
+// Total order used for every top-k / argmax decision: larger value first,
+// then lower index.
 __device__ __forceinline__ bool better(float va, int ia, float vb, int ib) {
     return va > vb || (va == vb && ia < ib);
 }

@@ -82,9 +82,6 @@ void launch_topk_logp(const float *logits, int R, int V, int k, int *ids, float 
 // candidates <= 256 in its row merge).
 bool topk_supported(int V, int k);
 
-template <typename T>
-void launch_convert(const float *x, T *y, long n, cudaStream_t s);
-
 // Sets the device status word (first code wins), in stream order.
 void launch_flag(int *status, int code, cudaStream_t s);
 

@@ -596,22 +596,6 @@ void launch_argmax(const float *logits, int R, int V, int *out, cudaStream_t s) 
     note_launch();
 }
 
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void convert_kernel(const float *__restrict__ x, T *__restrict__ y, long n) {
-    wait_prior();
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        y[i] = from_f<T>(x[i]);
-}
-
-template <typename T>
-void launch_convert(const float *x, T *y, long n, cudaStream_t s) {
-    if (n <= 0) return;
-    long blocks = (n + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    launch_chain(convert_kernel<T>, (int)blocks, 256, 0, s, x, y, n); note_launch();
-}
-
 __global__ void flag_status_kernel(int *status, int code) { wait_prior(); set_status(status, code); }
 
 void launch_flag(int *status, int code, cudaStream_t s) {
@@ -630,8 +614,7 @@ void launch_flag(int *status, int code, cudaStream_t s) {
                                     cudaStream_t);                                           \
     template void launch_rope_kv<T>(const float *, const RowDesc *, int, int, int,           \
                                     const float2 *, int, T *, T *, T *, int, long, int *,    \
-                                    cudaStream_t);                                           \
-    template void launch_convert<T>(const float *, T *, long, cudaStream_t);
+                                    cudaStream_t);
 MSD_INST(float)
 MSD_INST(bf16)
 #undef MSD_INST
