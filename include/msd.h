@@ -325,7 +325,7 @@ msd_status msd_linear(msd_ctx *ctx, const void *x_dev, int32_t ldx, int32_t m, i
  * is set, the call clears it, launches nothing and returns MSD_ERR_DEVICE: the
  * failed call's y is not to be trusted.
  * Errors: MSD_ERR_INVALID (null pointer, non-positive size, bad stride or
- * alignment), MSD_ERR_CAPACITY (m > 65535 * 256, the token-tile grid limit),
+ * alignment), MSD_ERR_CAPACITY (m > 65535 * 256, the limit of its tile counts),
  * MSD_ERR_DEVICE (see above), MSD_ERR_CUDA (a runtime call failed). */
 msd_status msd_linear_noalloc(const void *x_dev, int32_t ldx, int32_t m, int32_t k,
                               const void *w_dev, int32_t o, float *y_dev, int32_t ldy,

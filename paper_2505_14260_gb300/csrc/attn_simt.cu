@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
 
     // score tile: lanes run 8 keys (lane bits 0, 2, 3) x 4 rows (bits 1, 4), warps 2 (keys)
     // x 4 (rows): neighbouring lanes share every address of one operand, so that a
-    // 16-byte load serves more lanes at a time (24 rows over 333 keys, 16 heads: 14.9 us
+    // 16-byte load serves more lanes at a time (24 rows over 341 keys, 16 heads: 14.9 us
     // with bits 0-2 and 3-4, 12.2)
     constexpr int SR = QR / 16, SKEYS = 4;                      // rows and keys per thread
     const int warp = tid >> 5, lane = tid & 31;

@@ -9,9 +9,10 @@
 //
 // A CTA takes 64 query rows of one request and one head (the MMA's M = 64)
 // and one range of keys (a split). Roles (320 threads):
-//   warp 0 lane 0   TMA: K and V tiles of 64 keys (hi and lo planes, 128-byte
+//   warp 0          TMA: K and V tiles of 64 keys (hi and lo planes, 128-byte
 //                   swizzle) into a three-stage shared-memory ring
-//   warp 1          allocates tensor memory; lane 0 issues the MMAs
+//   warp 1          allocates tensor memory and issues the MMAs
+//                   (both loops run in the whole warp; one elected lane issues)
 //   warps 2-9       two per TMEM lane quarter (an M = 64 accumulator keeps
 //                   rows 16q .. 16q+15 in lanes 0-15 of quarter q, read in matrix
 //                   fragments so that all 32 threads of a warp have work), each

@@ -351,10 +351,12 @@ __device__ __forceinline__ void tmem_sum_cols(uint32_t taddr, int acc_stride, in
 // The work is the list of (tile, K-block) units, tile-major; pair c of G takes
 // units [c*U/G, (c+1)*U/G) of the cut tiles, then whole tiles, so every pair
 // streams through one continuously running TMA -> MMA pipeline, across tile
-// boundaries. Roles (192 threads): warp 0 lane 0 issues TMA, warp 1
-// allocates TMEM and the even CTA's lane 0 issues the MMAs, warps 2-5 drain the
-// accumulators. Two groups of accumulators let the epilogue of one tile overlap the
-// MMAs of the next. A tile whose K range is cut between pairs ("pieces") is
+// boundaries. Roles (192 threads): warp 0 issues TMA, warp 1 allocates TMEM and, in
+// the even CTA, issues the MMAs (whole warps, one elected lane), warps 2-5 drain the
+// accumulators. The accumulators come in groups: the K-blocks of an item (a tile, a
+// chunk or a piece of one) take turns over those of a group, and where a pair has
+// several items they take turns over two groups, so that the epilogue of one overlaps
+// the MMAs of the next. A tile whose K range is cut between pairs ("pieces") is
 // fixed up through the workspace, each CTA its own 128 rows: each piece is
 // written to its CTA's slot (a CTA has at most two cut tiles, its first and its
 // last), and the CTA that takes the tile's last ticket sums the pieces in pair
@@ -362,7 +364,7 @@ __device__ __forceinline__ void tmem_sum_cols(uint32_t taddr, int acc_stride, in
 // ---------------------------------------------------------------------------
 constexpr int P_THREADS = 192;
 constexpr int P_MAX_STAGES = 12;
-constexpr int P_MAX_ACC = 2;       // accumulator groups
+constexpr int P_MAX_ACC = 2;        // groups of accumulators
 constexpr int P_MAX_PIECES = 128;   // pieces of one cut tile (CTAs sharing it)
 
 struct PkParams {
@@ -376,8 +378,8 @@ struct PkParams {
     int T_sk, dp_rounds;    // stream-K tiles; rounds of whole tiles after them
     int T_all;              // all 256-row tiles x token tiles
     int kb_chunk;           // K-blocks of a whole tile accumulated before they are added to Y
-    int n_acc;              // groups of accumulators the items take in turn (<= P_MAX_ACC)
-    int n_rot;              // accumulators of a group: an item's K-blocks take turns, the epilogue sums them
+    int n_acc;              // groups of accumulators (<= P_MAX_ACC)
+    int n_rot;              // accumulators of a group, summed by the epilogue
     float *Y;
     int ldy, epi;
     float *ws;
@@ -2475,7 +2477,9 @@ constexpr int NOALLOC_COUNTERS = 4096;
 constexpr size_t NOALLOC_PARTIAL_BYTES = 16ull << 20;
 constexpr size_t NOALLOC_BYTES = NOALLOC_STATUS_BYTES + NOALLOC_COUNTERS * sizeof(int) + NOALLOC_PARTIAL_BYTES;
 constexpr int NOALLOC_MAX_DEVICES = 64;
-constexpr long NOALLOC_MAX_ROWS = 65535L * 256;   // token-tile grid dimension limit
+// 65535 token tiles of 256 rows: with up to 2^15 pairs of weight tiles (8 million
+// outputs) the launch's tile counts stay within an int.
+constexpr long NOALLOC_MAX_ROWS = 65535L * 256;
 }  // namespace
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];

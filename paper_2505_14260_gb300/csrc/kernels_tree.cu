@@ -711,9 +711,9 @@ accept_sample_kernel(TreeIn t, const float *__restrict__ logits, const float *__
 }
 
 // K/V of accepted node path[j] -> cache position L0 + j, all layers and heads.
-// grid (n_layers*2*nh, B); 16-byte vector copies.
-// Blocks past the KV rows (kv_blocks of a request) copy its pending draft rows:
-// the target features h of the accepted nodes.
+// grid (kv_blocks + D1, B): kv_blocks = n_layers*2*nh blocks copy K/V in 16-byte
+// vectors, the others one pending draft row each: the target features h of the
+// accepted nodes.
 template <typename T>
 __global__ void compact_kernel(const uint4 *__restrict__ tree_kv, uint4 *__restrict__ cache,
                                const int *__restrict__ acc_path, const int *__restrict__ acc_L0,

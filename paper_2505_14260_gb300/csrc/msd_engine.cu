@@ -304,10 +304,12 @@ GemmNorm norm_in(msd_ctx *c) {
 }
 
 // One pre-norm decoder layer over R rows (target or draft). Rows come in
-// blocks of rows_per_req per request.
-// cache positions. in_folded: the layer's input norm was folded into the GEMM
-// that produced x (xn_ready: it is in c->xn already); out_norm_g (nullable): the next layer's input-norm gain,
-// to fold into this layer's last GEMM. Returns whether it did.
+// blocks of rows_per_req per request, or (tiles) in n_tiles row tiles of one
+// request each; they see the cache ck/cv up to their prefix lengths and, with a
+// mask, the tree slots tk/tv. in_folded: the layer's input norm was folded into the
+// GEMM that produced x (xn_ready: it is in c->xn already); out_norm_g (nullable):
+// the next layer's input-norm gain, to fold into this layer's last GEMM. Returns
+// whether it did.
 template <typename T>
 bool run_layer(msd_ctx *c, const msd_layer &lw, const msd_ctx::LayerPack &lp, int R,
                const RowDesc *rows, T *kdst, T *vdst, int dst_slots, const T *ck, const T *cv,
