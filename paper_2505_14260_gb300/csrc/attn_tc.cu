@@ -66,7 +66,7 @@ struct Lay {
     static constexpr uint32_t STAGE = 4 * TILE;           // K hi, K lo, V hi, V lo
     // tensor-memory columns: Q hi, Q lo (bf16 pairs), two S/P buffers, O
     static constexpr uint32_t T_QH = 0, T_QL = HD / 2, T_S = HD, T_O = HD + 2 * KT;
-    static constexpr uint32_t T_COLS = T_O + HD <= 256 ? 256 : 512;
+    static constexpr uint32_t T_COLS = tmem_columns(T_O + HD);
     static constexpr int LD = HD + 4;                     // fp32 partial row stride (floats)
     static constexpr uint32_t SMEM = 1024 + STAGES * STAGE;
     static_assert(SMEM >= tmem_smem_floor((int)T_COLS), "CTAs that share an SM fit its tensor memory");

@@ -93,7 +93,9 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 // such launches (other streams, other contexts) that each hold one SM and wait for
 // the other's would never end. So CTAs that share an SM have to fit its 512 columns
 // together. With 78 KB or more apiece at most two share one (228 KB), and a CTA of
-// more than 256 columns leaves no room for a second.
+// more than 256 columns leaves no room for a second. All allocate a half or the
+// whole, so that none finds the free columns in two places.
+constexpr int tmem_columns(int used) { return used > 256 ? 512 : 256; }
 constexpr uint32_t tmem_smem_floor(int cols) { return cols > 256 ? 193u * 1024u : 78u * 1024u; }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -2058,7 +2058,7 @@ static ClusterShape cluster_shape(int tiles, int BN, int kblocks, int nb, bool p
         stage = A_BYTES + (size_t)nb * (BN / 2) * BK * 2;
         stages = std::max(2, std::min((int)(HALF_SM / stage), C_STAGES));
     }
-    const int tmem_cols = n_acc * acc_stride;
+    const int tmem_cols = tmem_columns(n_acc * acc_stride);
     const size_t smem = std::max<size_t>(1024 + (size_t)stages * stage, tmem_smem_floor(tmem_cols));
     const int chain = ((kblocks + S - 1) / S + n_acc - 1) / n_acc;
     return ClusterShape{S, stages, n_acc, acc_stride, tmem_cols, chain, pair, smem};
@@ -2318,8 +2318,7 @@ static PersistShape persist_shape(int tiles, int M, int K, int nb, bool glu, int
     best.stg_off = (uint32_t)(1024 + (size_t)best.stages * best.stage_bytes);
     best.acc_stride = 32;
     while (best.acc_stride < best.BN) best.acc_stride <<= 1;
-    best.tmem_cols = 64;
-    while (best.tmem_cols < best.n_acc * best.n_rot * best.acc_stride) best.tmem_cols <<= 1;
+    best.tmem_cols = tmem_columns(best.n_acc * best.n_rot * best.acc_stride);
     best.smem = std::max<size_t>(best.stg_off + stg_bytes, tmem_smem_floor(best.tmem_cols));
     return best;
 }

@@ -44,7 +44,7 @@ def test_ctas_that_share_an_sm_fit_its_tensor_memory(shape):
     for m, k, o in _shapes():
         for planes, glu in ((1, 0), (2, 0), (2, 1)):
             g = shape(m, k, o, planes, glu)
-            assert g.tmem_cols <= TMEM_COLS and g.smem_bytes <= 227 * 1024
+            assert g.tmem_cols in (256, TMEM_COLS) and g.smem_bytes <= 227 * 1024     # (free columns are never scattered)
             least[g.tmem_cols] = min(least.get(g.tmem_cols, SM_SMEM), g.smem_bytes)
     for n in range(2, 9):
         for cols in itertools.combinations_with_replacement(sorted(least), n):
