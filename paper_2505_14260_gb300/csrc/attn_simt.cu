@@ -191,22 +191,23 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                     sP[(sr + 16 * u) * AS_PLD + sk + 16 * v] = as_lo(s[u][v]) + as_hi(s[u][v]);
         }
         __syncthreads();
-        bool hidden = false;                    // a row does not see a key of the tile
+        bool hidden;                            // the row does not see a key of the tile
         {
             const bool tree = i >= nc;
-            const uint64_t bits = !tree ? ~0ull : (xmask && i - nc < a.mask_words ? xmask[i - nc] : 0ull);
-            const int lim = tree ? (xr < nrows ? a.tree_slots - (i - nc) * AS_KT : 0) : xplen - (k_lo + i * AS_KT);
-            // keys of the tile that were copied (the rest of the stage is zeros)
-            const int held = xr < nrows ? (tree ? a.tree_slots - (i - nc) * AS_KT : k_hi - (k_lo + i * AS_KT)) : 0;
+            auto below = [](int n) { return n >= AS_KT ? ~0ull : n <= 0 ? 0ull : (1ull << n) - 1ull; };
+            const int key0 = tree ? (i - nc) * AS_KT : k_lo + i * AS_KT;
+            // the tile's keys that the row sees, and those that were copied but it does
+            // not (the rest of the stage is zeros)
+            const uint64_t held = xr < nrows ? below((tree ? a.tree_slots : k_hi) - key0) : 0ull;
+            uint64_t vis = !tree ? below(xplen - key0) : (xmask && i - nc < a.mask_words ? xmask[i - nc] & held : 0ull);
+            uint64_t hid = held & ~vis;
+            hidden = hid != 0ull;
+            vis >>= xk;
+            hid >>= xk;
             float v[KPT], mx = -INFINITY;
-            unsigned seen = 0;
 #pragma unroll
             for (int j = 0; j < KPT; ++j) {
-                const int key = xk + GT * j;
-                const bool vis = key < lim && ((bits >> key) & 1ull);
-                seen |= (unsigned)vis << j;
-                hidden |= !vis && key < held;
-                v[j] = vis ? sP[xr * AS_PLD + key] * p.scale_log2 : -INFINITY;
+                v[j] = (vis >> (GT * j)) & 1ull ? sP[xr * AS_PLD + xk + GT * j] * p.scale_log2 : -INFINITY;
                 mx = fmaxf(mx, v[j]);
             }
 #pragma unroll
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
             for (int j = 0; j < KPT; ++j) {
                 const float e = as_exp2(v[j] - use);
                 sum += e;
-                sP[xr * AS_PLD + xk + GT * j] = (seen >> j & 1u) || xk + GT * j >= held ? e : HIDDEN;
+                sP[xr * AS_PLD + xk + GT * j] = (hid >> (GT * j)) & 1ull ? HIDDEN : e;
             }
 #pragma unroll
             for (int o = GT / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
