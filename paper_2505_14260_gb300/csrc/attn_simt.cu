@@ -8,13 +8,14 @@
 // decode; 64 otherwise) and walks its keys in tiles of 64, copied by cp.async
 // into a two-stage ring: scores S = Q K^T as register tiles (packed fp32 FMAs
 // over even and odd elements), an online softmax over the tile in shared
-// memory, O += P V in registers. A key that a row does not see is left out of
-// that row's sums, not multiplied by zero: its K/V may hold a NaN or an infinity
-// (of another row, or of an earlier tree in a slot not written yet). When the
-// (row tile, head) CTAs leave SMs idle the keys are cut into splits of whole
-// tiles, one cluster per (row tile, head), combined through distributed shared
-// memory in split order; the last split takes the tree keys. Rows are padded to
-// HD + 4 floats, so the rows a warp reads together sit in different banks.
+// memory, O += P V in registers. A key that a row does not see takes no part in
+// that row's sums: its weight is -0, and in a tile whose V holds a NaN or an
+// infinity (of another row, or of an earlier tree in a slot not written yet) it is
+// skipped. When the (row tile, head) CTAs leave SMs idle the keys are cut into
+// splits of whole tiles, one cluster per (row tile, head), combined through
+// distributed shared memory in split order; the last split takes the tree keys.
+// Rows are padded to HD + 4 floats, so the rows a warp reads together sit in
+// different banks.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -32,7 +33,7 @@ constexpr int AS_THREADS = 256;
 constexpr int AS_KT = 64;               // keys per tile
 constexpr int AS_PLD = AS_KT + 4;       // padded score row
 constexpr int AS_MAX_SPLITS = 8;
-constexpr float HIDDEN = -1.f;          // in place of the weight of a key that the row does not see
+constexpr float HIDDEN = -0.f;          // weight of a key that the row does not see (of one that it sees: +0 or more)
 
 struct AsArgs {
     AttnArgs<float> a;
@@ -75,7 +76,7 @@ template <int HD, int QR>
 __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
     using L = AsLay<HD, QR>;
     extern __shared__ __align__(16) float sm[];
-    __shared__ int s_live;
+    __shared__ int s_live, s_least;         // longest and shortest prefix of the rows
     wait_prior();
     allow_dependents();
     const AttnArgs<float> &a = p.a;
@@ -95,7 +96,10 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
     const int req = a.rows[r0].req;
 
     // query rows (zero past the tile's end), the rows' prefix lengths
-    if (tid == 0) s_live = 0;
+    if (tid == 0) {
+        s_live = 0;
+        s_least = 0x7fffffff;
+    }
     __syncthreads();
     float *sQ = sm + L::Q, *sP = sm + L::P, *s_scale = sm + L::ST, *s_m = s_scale + QR, *s_l = s_m + QR;
     for (int e = tid; e < QR * (HD / 4); e += AS_THREADS) {
@@ -104,13 +108,17 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
         if (r < nrows) v = *reinterpret_cast<const float4 *>(a.q + (size_t)(r0 + r) * H + h * HD + c);
         *reinterpret_cast<float4 *>(sQ + r * L::LD + c) = v;
     }
-    if (tid < nrows) atomicMax(&s_live, a.rows[r0 + tid].plen);
+    if (tid < nrows) {
+        const int plen = a.rows[r0 + tid].plen;
+        atomicMax(&s_live, plen);
+        atomicMin(&s_least, plen);
+    }
     if (tid < QR) {
         s_m[tid] = -INFINITY;
         s_l[tid] = 0.f;
     }
     __syncthreads();
-    const int live = min(s_live, a.cache_slots);
+    const int live = min(s_live, a.cache_slots), least = s_least;
     const int per = ((live + AS_KT - 1) / AS_KT + p.nsplit - 1) / p.nsplit * AS_KT;
     const int k_lo = split * per, k_hi = min(k_lo + per, live);
     const int nc = k_hi > k_lo ? (k_hi - k_lo + AS_KT - 1) / AS_KT : 0;
@@ -191,7 +199,7 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                     sP[(sr + 16 * u) * AS_PLD + sk + 16 * v] = as_lo(s[u][v]) + as_hi(s[u][v]);
         }
         __syncthreads();
-        bool hidden;                            // the row does not see a key of the tile
+        bool odd = false;                       // a value of V that is not finite, in a tile with hidden keys
         {
             const bool tree = i >= nc;
             auto below = [](int n) { return n >= AS_KT ? ~0ull : n <= 0 ? 0ull : (1ull << n) - 1ull; };
@@ -201,7 +209,6 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
             const uint64_t held = xr < nrows ? below((tree ? a.tree_slots : k_hi) - key0) : 0ull;
             uint64_t vis = !tree ? below(xplen - key0) : (xmask && i - nc < a.mask_words ? xmask[i - nc] & held : 0ull);
             uint64_t hid = held & ~vis;
-            hidden = hid != 0ull;
             vis >>= xk;
             hid >>= xk;
             float v[KPT], mx = -INFINITY;
@@ -231,8 +238,18 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                 s_l[xr] = s_l[xr] * f + sum;
             }
         }
-        const bool skip = __syncthreads_or(hidden);
-        // O += P V, without the keys that are hidden from a row (skip: there are some)
+        if (i >= nc || min(k_lo + (i + 1) * AS_KT, k_hi) > least) {
+            unsigned top = 0u;
+#pragma unroll
+            for (int e = tid; e < AS_KT * (HD / 4); e += AS_THREADS) {
+                const int r = e / (HD / 4), c = (e - r * (HD / 4)) * 4;
+                const uint4 w = *reinterpret_cast<const uint4 *>(sV + r * L::LD + c);
+                top = max(max(max(top, w.x << 1), max(w.y << 1, w.z << 1)), w.w << 1);
+            }
+            odd = top >= 0xff000000u;
+        }
+        const bool skip = __syncthreads_or(odd);
+        // O += P V; a hidden key adds -0 * V, nothing, or is skipped where that may be NaN
         auto pv = [&](auto skips) {
 #pragma unroll 4
             for (int k = 0; k < AS_KT; k += 4) {
@@ -245,7 +262,7 @@ __global__ void __launch_bounds__(AS_THREADS) attn_simt_kernel(const AsArgs p) {
                     const float pk[4] = {pr.x, pr.y, pr.z, pr.w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        if (decltype(skips)::value && pk[j] == HIDDEN) continue;
+                        if (decltype(skips)::value && __float_as_uint(pk[j]) == 0x80000000u) continue;
                         const unsigned long long pp = as_pack(pk[j], pk[j]);
                         o01[u] = as_fma2(pp, vv[j].x, o01[u]);
                         o23[u] = as_fma2(pp, vv[j].y, o23[u]);
